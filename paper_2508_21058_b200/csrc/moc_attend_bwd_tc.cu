@@ -533,8 +533,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
         // so the two instruction streams need no ordering between them and one's waits and commits are
         // covered by the other's MMAs.  Warps 14 and 15 idle.
         asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
-        if (warp <= 13 && lane == 0) {
-            const bool side1 = warp == 12;
+        if (warp <= 13) {                       // the warp stays together, one lane of it issues
+            const bool side1 = uniform(warp) == 12;
+            const int n_tiles = uniform(w_ntiles);
             constexpr uint32_t IDESC_T = idesc_bf16_f32(128, 128, 0, 0);      // T = X Y^T, both K-major
             constexpr uint32_t IDESC_ACC = idesc_bf16_f32(128, D, 0, 1);      // ACC += (TMEM) Y, Y MN-major
             constexpr uint64_t STAGE = TILE_BYTES >> 4;
@@ -545,14 +546,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
             auto lo = [](uint64_t d) { return (uint32_t)d; };
             auto hi = [](uint64_t d) { return (uint32_t)(d >> 32); };
             bool ok = true;
-            auto wait = [&](int b, int parity, int code) { ok = ok && mbar_wait_spin(bar(b), parity, abort_flag, p.status, code); };
+            auto wait = [&](int b, int parity, int code) { ok = ok && __all_sync(0xffffffffu, mbar_wait_spin(bar(b), parity, abort_flag, p.status, code)); };
             // the MMA groups, without their waits and commits
-            // (s3 = j mod the Y1 stage count is carried along by the callers: no division on this thread)
+            // (s3 = j mod the Y1 stage count is carried along by the callers: no division on this warp)
             auto t1 = [&](int j, int s3) {  // T1(j) = X1 Y1(j)^T
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks) {
                     const uint32_t o = ((ks >> 2) * SUB_BYTES + (ks & 3) * 32) >> 4;
-                    mma_ss_lo(tmem, lo(x1) + o, hi(x1), lo(y1k) + s3 * (uint32_t)STAGE + o, hi(y1k), IDESC_T, ks > 0);
+                    mma_ss_elect(tmem, lo(x1) + o, hi(x1), lo(y1k) + s3 * (uint32_t)STAGE + o, hi(y1k), IDESC_T, ks > 0);
                 }
             };
             auto t2 = [&](int j) {          // T2(j) = X2 Y2(j)^T
@@ -561,20 +562,20 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks) {
                     const uint32_t o = ((ks >> 2) * SUB_BYTES + (ks & 3) * 32) >> 4;
-                    mma_ss_lo(d, lo(x2) + o, hi(x2), lo(y2k) + s2 * (uint32_t)STAGE + o, hi(y2k), IDESC_T, ks > 0);
+                    mma_ss_elect(d, lo(x2) + o, hi(x2), lo(y2k) + s2 * (uint32_t)STAGE + o, hi(y2k), IDESC_T, ks > 0);
                 }
             };
             auto acc1 = [&](int j, int s3) {   // ACC1 += dS(j) Y1(j)
                 const uint32_t ds = tmem + ((MODE != DKV && (j & 1)) ? 384u : 128u);
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)
-                    mma_ts_lo(tmem + 256, ds + ks * 8, lo(y1m) + s3 * (uint32_t)STAGE + ks * (2048 >> 4), hi(y1m), IDESC_ACC, j > 0 || ks > 0);
+                    mma_ts_elect(tmem + 256, ds + ks * 8, lo(y1m) + s3 * (uint32_t)STAGE + ks * (2048 >> 4), hi(y1m), IDESC_ACC, j > 0 || ks > 0);
             };
             auto acc2 = [&](int j, int half) {   // ACC2 += P(j) Y2(j), the K steps of one half of P
                 const int s2 = j & 1;
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks)
-                    mma_ts_lo(tmem + 384, tmem + (half * 4 + ks) * 8, lo(y2m) + s2 * (uint32_t)STAGE + (half * 4 + ks) * (2048 >> 4), hi(y2m),
+                    mma_ts_elect(tmem + 384, tmem + (half * 4 + ks) * 8, lo(y2m) + s2 * (uint32_t)STAGE + (half * 4 + ks) * (2048 >> 4), hi(y2m),
                               IDESC_ACC, j > 0 || half > 0 || ks > 0);
             };
             // A wait, a fence or a commit between two groups leaves the pipe idle for longer than it takes, so each
@@ -589,7 +590,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                     if (ok) {
                         tc_fence_after();
                         t1(0, 0);
-                        tc_commit(bar(T1_FULL));
+                        tc_commit_elect(bar(T1_FULL));
                     }
                 }
                 int s3n = 1 % kY1Stages, ph3n = 0;                       // stage and phase of tile j + 1
@@ -608,12 +609,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                     if (MODE == DKV) acc2(j, 1);
                     if (more) {
                         t1(j + 1, s3n);
-                        tc_commit(bar(T1_FULL + ((j + 1) & 1)));
+                        tc_commit_elect(bar(T1_FULL + ((j + 1) & 1)));
                     }
                     if (++s3n == kY1Stages) { s3n = 0; ph3n ^= 1; }
                     if (MODE == DKV) {
-                        tc_commit(bar(Y2_EMPTY + (j & 1)));                 // the second of two arrivals
-                        if (more) mbar_arrive(bar(T1_ISSUED));              // the other side may use the pipe again
+                        tc_commit_elect(bar(Y2_EMPTY + (j & 1)));                 // the second of two arrivals
+                        if (more && lane == 0) mbar_arrive(bar(T1_ISSUED));              // the other side may use the pipe again
                     }
                 }
             } else {
@@ -626,8 +627,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                     if (!ok) break;
                     tc_fence_after();
                     t2(j);
-                    tc_commit(bar(T2_FULL + (j & 1)));
-                    tc_commit(bar(Y2_EMPTY + (j & 1)));
+                    tc_commit_elect(bar(T2_FULL + (j & 1)));
+                    tc_commit_elect(bar(Y2_EMPTY + (j & 1)));
                 }
                 int s3 = 0;                                               // Y1 stage of tile j
                 for (int j = 0; ok && j < n_tiles; ++j) {
@@ -638,18 +639,18 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                     if (!ok) break;
                     tc_fence_after();
                     acc1(j, s3);
-                    tc_commit(bar(Y1_EMPTY + s3));                  // at once: the next K tile waits for this stage
+                    tc_commit_elect(bar(Y1_EMPTY + s3));                  // at once: the next K tile waits for this stage
                     if (++s3 == kY1Stages) s3 = 0;
                     if (more) {
                         wait(Y2_FULL + (jn & 1), (jn >> 1) & 1, BW_YFULL);
                         if (!ok) break;
                         t2(jn);
-                        tc_commit(bar(T2_FULL + (jn & 1)));
-                        tc_commit(bar(Y2_EMPTY + (jn & 1)));    // dQ modes: V is read here only; dK/dV: the first of two arrivals
+                        tc_commit_elect(bar(T2_FULL + (jn & 1)));
+                        tc_commit_elect(bar(Y2_EMPTY + (jn & 1)));    // dQ modes: V is read here only; dK/dV: the first of two arrivals
                     }
                 }
             }
-            if (ok) tc_commit(bar(ACC_FULL));
+            if (ok) tc_commit_elect(bar(ACC_FULL));
         }
     }
     tc_fence_before();

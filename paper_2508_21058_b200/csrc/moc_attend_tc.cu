@@ -27,7 +27,7 @@
 //              runs across items.  Lane 16, bookkeeping: waits for what an item depends on, and when the item's
 //              rows are stored adds them to the queue's count of completed rows (the one thread that pays for
 //              a device-wide fence per item);
-//   warps 9, 10  one MMA-issuing thread per query tile g:  S_g(0), then  O_g += P_g V(j),  S_g(j + 1)  per key
+//   warps 9, 10  one MMA-issuing warp per query tile g:  S_g(0), then  O_g += P_g V(j),  S_g(j + 1)  per key
 //              tile.  S = Q K^T takes both operands from shared memory, O += P V takes P from TMEM and V as an
 //              MN-major shared-memory operand; all accumulators live in TMEM (S0, S1, O0, O1 = 512 columns);
 //   warp 11    scheduler and Q loader: lane 0 claims the next item and hands its description to the others
@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
     // barrier indices (pairs: per query tile g, per K/V stage, or per item slot)
     constexpr int Q_FULL = 0, Q_EMPTY = 3, K_FULL = 6, K_EMPTY = 8, V_FULL = 10, V_EMPTY = 12, S_FULL = 14, P_HALF = 16, P_FULL = 18,
                   O_FULL = 20, O_FREE = 22, TURN = 24, ITEM_FULL = 26, ITEM_EMPTY = 28, ROWS_DONE = 30, DEPEND = 32;
-    constexpr int kItemReaders = 2 + 2 + 256;          // producer and bookkeeping lanes, two issuers, every softmax thread
+    constexpr int kItemReaders = 2 + 2 + 256;          // producer and bookkeeping lanes, two issuing warps, every softmax thread
 
     if (threadIdx.x == 0) {
         s_abort = 0;
@@ -587,12 +587,13 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
         }
     } else if (warp < 11) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
-        // ------------------------------------------------------------ MMA issuers (one per query tile)
-        const int g = warp - 9;
-        if (lane == 0) {
+        // ------------------------------------------------------------ MMA issuers (one warp per query tile; the warp stays
+        // together, one lane of it issues)
+        const int g = uniform(warp - 9);
+        {
             constexpr uint32_t IDESC_PV = idesc_bf16_f32(128, D, 0, 1);
             // Descriptors are built once; inside the issue loops only the 14-bit start-address field
-            // (low word, 16-byte units) moves, so one tcgen05.mma costs the issuing thread a few
+            // (low word, 16-byte units) moves, so one tcgen05.mma costs the issuing warp a few
             // integer instructions.
             const uint64_t q_desc0 = smem_desc_sw128(sQ, 16, 1024), k_desc0 = smem_desc_sw128(sK, 16, 1024);
             const uint64_t v_desc0 = smem_desc_sw128(sV, SUB_BYTES, 1024);
@@ -607,7 +608,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks) {
                     const uint32_t o = ((ks >> 2) * SUB_BYTES + (ks & 3) * 32) >> 4;     // never carries out of the address field
-                    mma_ss_lo(d_s, q_lo + o, q_hi, k_lo + o, k_hi, idesc_qk, ks > 0);
+                    mma_ss_elect(d_s, q_lo + o, q_hi, k_lo + o, k_hi, idesc_qk, ks > 0);
                 }
             };
             // k-steps [ks0, ks1) of  O_g += P_g V(stage st)  (16 keys each)
@@ -618,35 +619,41 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                 if (ks1 - ks0 == 4) {
 #pragma unroll
                     for (int ks = 0; ks < 4; ++ks)
-                        mma_ts_lo(d_o, a_p + (ks0 + ks) * 8, v_lo + (ks0 + ks) * (2048 >> 4), v_hi, IDESC_PV, accumulate || ks > 0);
+                        mma_ts_elect(d_o, a_p + (ks0 + ks) * 8, v_lo + (ks0 + ks) * (2048 >> 4), v_hi, IDESC_PV, accumulate || ks > 0);
                 } else {
-                    for (int ks = ks0; ks < ks1; ++ks) mma_ts_lo(d_o, a_p + ks * 8, v_lo + ks * (2048 >> 4), v_hi, IDESC_PV, accumulate || ks > ks0);
+                    for (int ks = ks0; ks < ks1; ++ks) mma_ts_elect(d_o, a_p + ks * 8, v_lo + ks * (2048 >> 4), v_hi, IDESC_PV, accumulate || ks > ks0);
                 }
             };
             // items seen, items with this tile, K/V tiles seen, P tiles consumed, query tiles loaded before this item
             int n_item = 0, n_mine = 0, n_kv = 0, n_p = 0, n_qtile = 0;
             bool ok = true;
+            // the whole warp waits, and goes on or gives up together
+            auto wait = [&](int b, uint32_t parity, int code) {
+                return __all_sync(0xffffffffu, mbar_wait(bar(b), parity, abort_flag, p.status, code)) != 0;
+            };
             while (ok) {
                 const int sl = n_item & 1;
-                if (!mbar_wait(bar(ITEM_FULL + sl), (n_item >> 1) & 1, abort_flag, p.status, W_ITEMFULL)) break;
+                if (!wait(ITEM_FULL + sl, (n_item >> 1) & 1, W_ITEMFULL)) break;
                 const ItemSlot it_ = s_item[sl];
-                mbar_arrive(bar(ITEM_EMPTY + sl));
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(ITEM_EMPTY + sl));
                 ++n_item;
-                if (!it_.valid) break;
-                const int n_tiles = it_.ntiles;
+                if (!uniform(it_.valid)) break;
+                const int rows = uniform(it_.rows), n_tiles = uniform(it_.ntiles);
                 const int q_seq = n_qtile + g;                      // this tile's place in the sequence of Q loads
-                n_qtile += it_.rows > 128 ? 2 : 1;
-                if (g == 1 && it_.rows <= 128) {
+                n_qtile += rows > 128 ? 2 : 1;
+                if (g == 1 && rows <= 128) {
                     // no second query tile: this issuer only keeps the K/V ring's accounting (each stage is
                     // released by two arrivals)
                     for (int jt = 0; ok && jt < n_tiles; ++jt) {
                         const int st = n_kv & 1;
                         const uint32_t ph = (n_kv >> 1) & 1;
-                        ok = mbar_wait(bar(K_FULL + st), ph, abort_flag, p.status, W_KFULL) &&
-                             mbar_wait(bar(V_FULL + st), ph, abort_flag, p.status, W_VFULL);
+                        ok = wait(K_FULL + st, ph, W_KFULL) && wait(V_FULL + st, ph, W_VFULL);
                         if (!ok) break;
-                        mbar_arrive(bar(K_EMPTY + st));
-                        mbar_arrive(bar(V_EMPTY + st));
+                        if (lane == 0) {
+                            mbar_arrive(bar(K_EMPTY + st));
+                            mbar_arrive(bar(V_EMPTY + st));
+                        }
                         ++n_kv;
                     }
                     continue;
@@ -656,39 +663,41 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                 TileIter it(it_.rng, it_.nrng);
                 int t0, valid, valid_next = 0;
                 ok = it.next(t0, valid);
-                ok = ok && mbar_wait(bar(Q_FULL + qb), (q_seq / 3) & 1, abort_flag, p.status, W_QFULL);
-                ok = ok && mbar_wait(bar(K_FULL + (n_kv & 1)), (n_kv >> 1) & 1, abort_flag, p.status, W_KFULL);
+                valid = uniform(valid);
+                ok = ok && wait(Q_FULL + qb, (q_seq / 3) & 1, W_QFULL);
+                ok = ok && wait(K_FULL + (n_kv & 1), (n_kv >> 1) & 1, W_KFULL);
                 if (!ok) break;
                 tc_fence_after();
                 issue_qk(n_kv & 1, valid);
-                tc_commit(bar(S_FULL + g));
-                tc_commit(bar(K_EMPTY + (n_kv & 1)));
-                if (n_tiles == 1) tc_commit(bar(Q_EMPTY + qb));       // that was the item's only S: its Q buffer may be refilled
+                tc_commit_elect(bar(S_FULL + g));
+                tc_commit_elect(bar(K_EMPTY + (n_kv & 1)));
+                if (n_tiles == 1) tc_commit_elect(bar(Q_EMPTY + qb));       // that was the item's only S: its Q buffer may be refilled
                 for (int jt = 0; ok && jt < n_tiles; ++jt) {
                     const int st = n_kv & 1, sn = (n_kv + 1) & 1;
                     const uint32_t ph = (n_kv >> 1) & 1, phn = ((n_kv + 1) >> 1) & 1;
-                    const bool more = it.next(t0, valid_next);
-                    if (!mbar_wait(bar(V_FULL + st), ph, abort_flag, p.status, W_VFULL)) { ok = false; break; }
-                    if (more && !mbar_wait(bar(K_FULL + sn), phn, abort_flag, p.status, W_KFULL)) { ok = false; break; }
+                    const bool more = jt + 1 < n_tiles;
+                    if (more) { it.next(t0, valid_next); valid_next = uniform(valid_next); }
+                    if (!wait(V_FULL + st, ph, W_VFULL)) { ok = false; break; }
+                    if (more && !wait(K_FULL + sn, phn, W_KFULL)) { ok = false; break; }
                     const int steps = (valid + 15) >> 4, half = min(steps, 4);
-                    if (!mbar_wait(bar(P_HALF + g), n_p & 1, abort_flag, p.status, W_PHALF)) { ok = false; break; }
+                    if (!wait(P_HALF + g, n_p & 1, W_PHALF)) { ok = false; break; }
                     // the first P V of an item overwrites O: the previous item's epilogue must have read it
-                    if (jt == 0 && n_mine > 0 && !mbar_wait(bar(O_FREE + g), (n_mine - 1) & 1, abort_flag, p.status, W_OFREE)) { ok = false; break; }
+                    if (jt == 0 && n_mine > 0 && !wait(O_FREE + g, (n_mine - 1) & 1, W_OFREE)) { ok = false; break; }
                     tc_fence_after();
                     issue_pv(st, 0, half, jt > 0);
-                    if (!mbar_wait(bar(P_FULL + g), n_p & 1, abort_flag, p.status, W_PFULL)) { ok = false; break; }
+                    if (!wait(P_FULL + g, n_p & 1, W_PFULL)) { ok = false; break; }
                     tc_fence_after();
                     if (steps > half) issue_pv(st, half, steps, true);
                     // a commit between two groups of MMAs leaves the pipe idle: the next S goes out first, then all commits
                     if (more) {
                         issue_qk(sn, valid_next);
-                        tc_commit(bar(S_FULL + g));
-                        tc_commit(bar(V_EMPTY + st));
-                        tc_commit(bar(K_EMPTY + sn));
-                        if (jt + 2 == n_tiles) tc_commit(bar(Q_EMPTY + qb));      // the item's last S: its Q buffer may be refilled
+                        tc_commit_elect(bar(S_FULL + g));
+                        tc_commit_elect(bar(V_EMPTY + st));
+                        tc_commit_elect(bar(K_EMPTY + sn));
+                        if (jt + 2 == n_tiles) tc_commit_elect(bar(Q_EMPTY + qb));      // the item's last S: its Q buffer may be refilled
                     } else {
-                        tc_commit(bar(V_EMPTY + st));
-                        tc_commit(bar(O_FULL + g));
+                        tc_commit_elect(bar(V_EMPTY + st));
+                        tc_commit_elect(bar(O_FULL + g));
                     }
                     valid = valid_next;
                     ++n_kv;

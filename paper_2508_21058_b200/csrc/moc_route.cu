@@ -298,8 +298,8 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
         // MMAs; when blocks are streamed, warp 1 serves every unit and follows the reloads.
         const bool dual = resident && NG > 1;          // one selection group has one accumulator: one issuer
         const int first = warp == 1 ? 0 : 1, stride = dual ? 2 : 1;
-        if (lane == 0 && (warp == 1 || dual)) {
-            // descriptors are built once: issuing an MMA should cost this thread a few integer instructions
+        if (warp == 1 || dual) {               // the warp stays together, one lane of it issues
+            // descriptors are built once: issuing an MMA should cost this warp a few integer instructions
             const uint64_t q_desc0 = smem_desc_sw128(sQ, 16, 1024);
             uint64_t d_term[3 * SUB];
 #pragma unroll
@@ -310,6 +310,10 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
 #pragma unroll
             for (int x = 0; x < NG; ++x) nacc_total[x] = 0;
             bool ok = true;
+            // the whole warp waits, and goes on or gives up together
+            auto wait = [&](int b, uint32_t parity, int code) {
+                return __all_sync(0xffffffffu, mbar_wait(bar(b), parity, abort_flag, p.status, code)) != 0;
+            };
             // a round: one unit (resident block; the two issuers take alternate units), or NG consecutive units that
             // share every streamed block
             const int grp = resident ? 1 : NG;
@@ -318,11 +322,11 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                 int n_sb = 1;
                 for (int n = n0; n < n1; ++n) n_sb = max(n_sb, steps_of(n));
                 for (int n = n0; ok && n < n1; ++n)
-                    ok = mbar_wait(bar(Q_FULL + qstage_of(n)), qparity_of(n), abort_flag, p.status, RW_QFULL);
+                    ok = wait(Q_FULL + qstage_of(n), qparity_of(n), RW_QFULL);
                 for (int rep = 0; ok && rep < n_pass; ++rep)
                 for (int sb = 0; ok && sb < n_sb; ++sb) {
                     if (resident ? dn == 0 : sb != res_sb) {
-                        ok = mbar_wait(bar(D_FULL), dn & 1, abort_flag, p.status, RW_DFULL);
+                        ok = wait(D_FULL, dn & 1, RW_DFULL);
                         if (!ok) break;
                         ++dn;
                         res_sb = sb;
@@ -334,7 +338,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                         int uses = 0;                          // how often this accumulator has been filled (no indexed array:
 #pragma unroll                                                 // the counters stay in registers)
                         for (int x = 0; x < NG; ++x) uses = x == buf ? nacc_total[x] : uses;
-                        ok = mbar_wait(bar(ACC_EMPTY + buf), (uses & 1) ^ 1, abort_flag, p.status, RW_ACCEMPTY);
+                        ok = wait(ACC_EMPTY + buf, (uses & 1) ^ 1, RW_ACCEMPTY);
                         if (!ok) break;
                         tc_fence_after();
                         const int rows_sb = max(16, min(min(p.sb_rows, p.c_pad - sb * p.sb_rows), (reach - sb * p.sb_rows + 15) & ~15));
@@ -345,7 +349,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                             const uint32_t acc = tmem + buf * ACC_COLS;
 #pragma unroll
                             for (int ks = 0; ks < D / 16; ++ks)
-                                mma_ss_lo(acc, (uint32_t)qd + (((ks >> 2) * Q_SUB_BYTES + (ks & 3) * 32) >> 4), (uint32_t)(qd >> 32),
+                                mma_ss_elect(acc, (uint32_t)qd + (((ks >> 2) * Q_SUB_BYTES + (ks & 3) * 32) >> 4), (uint32_t)(qd >> 32),
                                           (uint32_t)d_term[ks >> 2] + (((ks & 3) * 32) >> 4), (uint32_t)(d_term[ks >> 2] >> 32), idesc, ks != 0);
                         } else {
                             // one instruction spans the step's columns (at most 256)
@@ -356,12 +360,12 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                             for (int term = 0; term < 3; ++term) {
 #pragma unroll
                                 for (int ks = 0; ks < D / 16; ++ks)
-                                    mma_ss_lo(acc, (uint32_t)qd + (((ks >> 2) * Q_SUB_BYTES + (ks & 3) * 32) >> 4), (uint32_t)(qd >> 32),
+                                    mma_ss_elect(acc, (uint32_t)qd + (((ks >> 2) * Q_SUB_BYTES + (ks & 3) * 32) >> 4), (uint32_t)(qd >> 32),
                                               (uint32_t)d_term[term * SUB + (ks >> 2)] + nofs + (((ks & 3) * 32) >> 4),
                                               (uint32_t)(d_term[term * SUB + (ks >> 2)] >> 32), idesc, (term | ks) != 0);
                             }
                         }
-                        tc_commit(bar(ACC_FULL + buf));
+                        tc_commit_elect(bar(ACC_FULL + buf));
 #pragma unroll
                         for (int x = 0; x < NG; ++x) nacc_total[x] += x == buf ? 1 : 0;
                     }
@@ -371,10 +375,10 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                         int nsb = sb + 1;
                         bool more = true;
                         if (nsb >= n_sb) { nsb = 0; more = rep + 1 < n_pass || n1 < nu; }
-                        if (more && nsb != sb) tc_commit(bar(D_EMPTY));
+                        if (more && nsb != sb) tc_commit_elect(bar(D_EMPTY));
                     }
                 }
-                for (int n = n0; ok && n < n1; ++n) tc_commit(bar(Q_EMPTY + qstage_of(n)));
+                for (int n = n0; ok && n < n1; ++n) tc_commit_elect(bar(Q_EMPTY + qstage_of(n)));
             }
         }
     } else if (warp < 2 + 4 * NG) {
