@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
     // barrier indices (pairs: per query tile g, per K/V stage, or per item slot)
     constexpr int Q_FULL = 0, Q_EMPTY = 3, K_FULL = 6, K_EMPTY = 8, V_FULL = 10, V_EMPTY = 12, S_FULL = 14, P_HALF = 16, P_FULL = 18,
-                  O_FULL = 20, O_FREE = 22, TURN = 24, ITEM_FULL = 26, ITEM_EMPTY = 28, ROWS_DONE = 30, DEPEND = 32;
+                  O_FULL = 20, O_FREE = 22, TURN = 24, ITEM_FULL = 26, ITEM_EMPTY = 28, ROWS_DONE = 30, DEPEND = 34;
     constexpr int kItemReaders = 2 + 2 + 256;          // producer and bookkeeping lanes, two issuing warps, every softmax thread
 
     if (threadIdx.x == 0) {
@@ -186,7 +186,8 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
             mbar_init(bar(TURN + t), 128);
             mbar_init(bar(ITEM_FULL + t), 1);
             mbar_init(bar(ITEM_EMPTY + t), kItemReaders);
-            mbar_init(bar(ROWS_DONE + t), 128);
+            mbar_init(bar(ROWS_DONE + t), 128);        // [item slot][query tile]
+            mbar_init(bar(ROWS_DONE + 2 + t), 128);
         }
         fence_barrier_init();
     }
@@ -488,7 +489,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                 else p.lse[(size_t)h * p.L + qi] = (pl ? big + __logf(wsum) : lse_own);
             }
             // this tile's rows are stored; the bookkeeping lane counts them once all 128 threads are here
-            mbar_arrive(bar(ROWS_DONE + g));
+            mbar_arrive(bar(ROWS_DONE + 2 * sl + g));
             ++n_mine;
         }
     } else if (warp == 8) {
@@ -549,28 +550,34 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
             // the next item has been seen, so that the fence before the count (it waits for the item's stores to
             // land) is not in the way of the next item.  DEPEND is arrived on after the previous item's rows were
             // counted, that is after every softmax thread has passed its previous wait on it.
-            int n_item = 0, n_tile[2] = {0, 0};
+            // Its fence may take longer than the groups need for two items, and a barrier must not complete two phases
+            // that nobody has waited for in between: ROWS_DONE exists once per item slot, and the slot of item n + 1 is handed
+            // back only when item n has been counted, so item n + 3, the next to use the ROWS_DONE of item n + 1, is not
+            // published before this lane is about to wait for item n + 1.
+            int n_item = 0;
+            uint32_t rows_phase = 0;                            // bit 2 slot + tile: parity of the next phase of that ROWS_DONE
             int pend_phase = -1, pend_rows = 0;                 // the item whose rows are still to be counted
             bool ok = true;
             while (ok) {
                 const int sl = n_item & 1;
                 if (!mbar_wait(bar(ITEM_FULL + sl), (n_item >> 1) & 1, abort_flag, p.status, W_ITEMFULL)) break;
                 const ItemSlot it_ = s_item[sl];
-                mbar_arrive(bar(ITEM_EMPTY + sl));
                 ++n_item;
                 const int group = it_.phase >> 1;
                 const bool dep_anchor = it_.valid && !it_.routed && p.k > 0, dep_routed = it_.valid && it_.routed && group >= 2;
                 if (pend_phase >= 0) {
                     const int n_qt = pend_rows > 128 ? 2 : 1;
                     for (int g = 0; ok && g < n_qt; ++g) {
-                        ok = mbar_wait(bar(ROWS_DONE + g), n_tile[g] & 1, abort_flag, p.status, W_ROWSDONE);
-                        ++n_tile[g];
+                        const int b = 2 * (sl ^ 1) + g;          // the pending item used the other slot
+                        ok = mbar_wait(bar(ROWS_DONE + b), (rows_phase >> b) & 1, abort_flag, p.status, W_ROWSDONE);
+                        rows_phase ^= 1u << b;
                     }
                     if (!ok) break;
                     __threadfence();
                     atomicAdd(&phase_tab[3 * pend_phase + 2], pend_rows);
                     pend_phase = -1;
                 }
+                mbar_arrive(bar(ITEM_EMPTY + sl));
                 if (!it_.valid) break;
                 if (dep_anchor)
                     ok = wait_count(&phase_tab[3 * (2 * group) + 2], phase_tab[3 * (2 * group) + 1], abort_flag, p.status, W_DEPEND);

@@ -241,3 +241,16 @@ def test_debug_build_checks_every_workspace_index_and_finds_nothing():
     env = dict(os.environ, MOC_LIBRARY="debug", MOC_PARITY_DIR=os.path.join(PU.OUT_ROOT, "parity_debug"))
     res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, env=env, timeout=600)
     assert res.returncode == 0 and "DEBUG_BUILD_OK" in res.stdout, res.stdout[-2000:] + res.stderr[-4000:]
+
+
+def test_many_short_items_in_a_row_never_wait_for_good():
+    """256-token chunks with 30 picks per query: tens of thousands of attention items a few microseconds long, so that a
+    CTA's softmax, its bookkeeping and its loads drift apart as far as the hand-overs between them allow."""
+    wl = W.workload("cfg3-m256-p8")
+    wl.n_heads = 2
+    run = PU.GpuRun(wl).forward()
+    O, lse = run.O.clone(), run.lse.clone()
+    for _ in range(20):
+        run.ws.random_(0, 256)
+        run.forward()                                                # checks the device status
+        assert torch.equal(O, run.O) and torch.equal(lse, run.lse)
