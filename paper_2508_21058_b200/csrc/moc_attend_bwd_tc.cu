@@ -43,7 +43,7 @@ struct BwdParams {
     const float *lse, *delta;
     __nv_bfloat16 *dQ, *dK, *dV;
     __nv_bfloat16 *part;          // [Hg][L][k][d] routed dQ partials of the group of heads in flight
-    const float *part_lse;        // [H][L][k] the forward's routed log-sum-exps: -inf marks an empty slot
+    const float *part_lse;        // the forward's routed log-sum-exps (part_lse_at): -inf marks an empty slot
     const KeyRange *rng;          // dQ modes: key ranges the items index
     const WorkItem *items;
     const int *item_lo_dev, *item_hi_dev;   // routed mode: the group's item range [*lo, *hi) on the device
@@ -382,12 +382,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                     if (qi >= 0) {
                         // the routed partials of this query, four slots requested together; a slot is in use
                         // if the forward left a finite log-sum-exp for it
-                        const float *pl = p.part_lse + ((size_t)h * p.L + qi) * p.k;
+                        const float *pl = p.part_lse + part_lse_at(h, LB, p.k, qi, 0);      // slot s: pl[s * 128]
                         for (int s0 = 0; s0 < p.k; s0 += 4) {
                             uint4 raw[4][4];
 #pragma unroll
                             for (int u = 0; u < 4; ++u) {
-                                const bool used = s0 + u < p.k && pl[s0 + u] != -INFINITY;
+                                const bool used = s0 + u < p.k && pl[(s0 + u) * 128] != -INFINITY;
 #pragma unroll
                                 for (int q4 = 0; q4 < 4; q4 += 2) {
                                     raw[u][q4] = raw[u][q4 + 1] = make_uint4(0, 0, 0, 0);

@@ -51,7 +51,7 @@ struct AttendParams {
     float *lse;
     __nv_bfloat16 *part_o;      // [2 or 1] buffers of the group in flight's partials (even / odd groups alternate), laid
                                 // out query-innermost in blocks of 128 queries (part_piece)
-    float *part_lse;            // [H][L][k]
+    float *part_lse;            // log-sum-exps of the partials, query-innermost (part_lse_at)
     size_t part_stride;         // elements between the two partial buffers (0 with a single group)
     const KeyRange *chunk_rng;  // [C] key range of a routed item (its chunk)
     const KeyRange *anc_rng;    // merged anchor ranges, indexed by the anchor items
@@ -252,13 +252,16 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
             __nv_bfloat16 *part_o = p.part_o + (size_t)(group & 1) * p.part_stride;
             const int h_loc = h - group * p.hg;
             constexpr int NP = D / 8;                   // 16-byte pieces per row
+            constexpr int KW = 8;                       // slots whose merge weights live in registers
             const int LB = (p.L + 127) >> 7;
             uint4 *part16 = reinterpret_cast<uint4 *>(part_o);
             if (!routed && qi >= 0 && p.k > 0) {
                 // the epilogue will merge this row's routed partials: start them on their way into L2 now.  A 128-byte
-                // line holds one pair of pieces of four consecutive queries: every fourth query (and the tile's first) asks
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(p.part_lse + ((size_t)h * p.L + qi) * p.k));
-                if ((qi & 3) == 0 || r == 0)
+                // line holds one pair of pieces of four consecutive queries: every fourth query (and the tile's first) asks.
+                // (Few picks only: what all CTAs ask for ahead has to stay in L2 until it is read.)
+                if ((qi & 31) == 0 || r == 0)
+                    for (int s = 0; s < p.k; ++s) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.part_lse + part_lse_at(h, LB, p.k, qi, s)));
+                if (p.k <= KW && ((qi & 3) == 0 || r == 0))
                     for (int s = 0; s < p.k; ++s)
                         for (int cc = 0; cc < NP; cc += 2)
                             asm volatile("prefetch.global.L2 [%0];" ::"l"(part16 + part_piece(h_loc, LB, p.k, NP, qi, s, cc)));
@@ -364,7 +367,6 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
             const float inv_l = 1.f / l_run;
             const float lse_own = (m_run + log2f(l_run)) * kLn2;
             float w_own = inv_l, big = lse_own, wsum = 1.f;
-            constexpr int KW = 8;                     // slots whose weights live in registers
             float wslot[KW];
 #pragma unroll
             for (int s = 0; s < KW; ++s) wslot[s] = 0.f;
@@ -378,11 +380,11 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                 if (!ok) break;
             }
             if (!routed && qi >= 0 && p.k > 0) {
-                pl = p.part_lse + ((size_t)h * p.L + qi) * p.k;
+                pl = p.part_lse + part_lse_at(h, LB, p.k, qi, 0);        // slot s: pl[s * 128]
                 if (p.k <= KW) {
                     float plv[KW];
 #pragma unroll
-                    for (int s = 0; s < KW; ++s) plv[s] = s < p.k ? __ldcg(pl + s) : -INFINITY;
+                    for (int s = 0; s < KW; ++s) plv[s] = s < p.k ? __ldcg(pl + s * 128) : -INFINITY;
 #pragma unroll
                     for (int s = 0; s < KW; ++s) big = fmaxf(big, plv[s]);
                     wsum = __expf(lse_own - big);
@@ -391,9 +393,20 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
 #pragma unroll
                     for (int s = 0; s < KW; ++s) wslot[s] /= wsum;
                 } else {
-                    for (int s = 0; s < p.k; ++s) big = fmaxf(big, __ldcg(pl + s));
-                    wsum = __expf(lse_own - big);
-                    for (int s = 0; s < p.k; ++s) wsum += __expf(__ldcg(pl + s) - big);
+                    // eight slots requested together; running maximum and sum
+                    wsum = 1.f;
+#pragma unroll 1
+                    for (int s0 = 0; s0 < p.k; s0 += 8) {
+                        float plv[8], m = big;
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) plv[u] = s0 + u < p.k ? __ldcg(pl + (s0 + u) * 128) : -INFINITY;
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) m = fmaxf(m, plv[u]);
+                        wsum *= __expf(big - m);
+                        big = m;
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) wsum += __expf(plv[u] - big);
+                    }
                 }
                 w_own = __expf(lse_own - big) / wsum * inv_l;
             }
@@ -445,23 +458,41 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                         }
                     }
                 } else if (pl) {
-                    for (int s = 0; s < p.k; ++s) {
-                        const float ls = __ldcg(pl + s);
-                        if (ls == -INFINITY) continue;
-                        const float w = __expf(ls - big) / wsum;
-                        uint4 raw[4];
-                        ld_cg_256(part16 + part_piece(h_loc, LB, p.k, NP, qi, s, ch * 4), raw[0], raw[1]);
-                        ld_cg_256(part16 + part_piece(h_loc, LB, p.k, NP, qi, s, ch * 4 + 2), raw[2], raw[3]);
+                    // Four slots requested together, their log-sum-exps a batch ahead.  (One slot at a time kept 16 KB in flight
+                    // per SM: 9 bytes a cycle, 220k cycles for the 2 MB of a 256-row item with 30 picks.)
+                    const float inv_w = 1.f / wsum;
+                    const uint4 *src = part16 + part_piece(h_loc, LB, p.k, NP, qi, 0, ch * 4);
+                    constexpr int SLOT = (NP / 2) * 256;       // pieces from one slot to the next
+                    float ls[4];
 #pragma unroll
-                        for (int q4 = 0; q4 < 4; ++q4) {
-                            const __nv_bfloat162 *b = reinterpret_cast<const __nv_bfloat162 *>(&raw[q4]);
+                    for (int u = 0; u < 4; ++u) ls[u] = u < p.k ? __ldcg(pl + u * 128) : -INFINITY;
+#pragma unroll 1
+                    for (int s0 = 0; s0 < p.k; s0 += 4, src += 4 * SLOT) {
+                        uint4 raw[4][4];
+                        float w[4];
 #pragma unroll
-                            for (int y = 0; y < 4; ++y) {
-                                const float2 f = __bfloat1622float2(b[y]);
-                                acc[q4 * 8 + 2 * y] = fmaf(w, f.x, acc[q4 * 8 + 2 * y]);
-                                acc[q4 * 8 + 2 * y + 1] = fmaf(w, f.y, acc[q4 * 8 + 2 * y + 1]);
+                        for (int u = 0; u < 4; ++u) {
+                            w[u] = __expf(ls[u] - big) * inv_w;        // exp(-inf) = 0: empty slot
+#pragma unroll
+                            for (int q4 = 0; q4 < 4; q4 += 2) {
+                                raw[u][q4] = raw[u][q4 + 1] = make_uint4(0, 0, 0, 0);
+                                if (ls[u] != -INFINITY) ld_cg_256(src + u * SLOT + q4 * 128, raw[u][q4], raw[u][q4 + 1]);
                             }
                         }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) ls[u] = s0 + 4 + u < p.k ? __ldcg(pl + (s0 + 4 + u) * 128) : -INFINITY;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+#pragma unroll
+                            for (int q4 = 0; q4 < 4; ++q4) {
+                                const __nv_bfloat162 *b = reinterpret_cast<const __nv_bfloat162 *>(&raw[u][q4]);
+#pragma unroll
+                                for (int y = 0; y < 4; ++y) {
+                                    const float2 f = __bfloat1622float2(b[y]);
+                                    acc[q4 * 8 + 2 * y] = fmaf(w[u], f.x, acc[q4 * 8 + 2 * y]);
+                                    acc[q4 * 8 + 2 * y + 1] = fmaf(w[u], f.y, acc[q4 * 8 + 2 * y + 1]);
+                                }
+                            }
                     }
                 }
                 if (qi < 0) continue;
@@ -485,7 +516,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                 }
             }
             if (qi >= 0) {
-                if (routed) p.part_lse[((size_t)h * p.L + qi) * p.k + slot] = lse_own;
+                if (routed) p.part_lse[part_lse_at(h, LB, p.k, qi, slot)] = lse_own;
                 else p.lse[(size_t)h * p.L + qi] = (pl ? big + __logf(wsum) : lse_own);
             }
             // this tile's rows are stored; the bookkeeping lane counts them once all 128 threads are here

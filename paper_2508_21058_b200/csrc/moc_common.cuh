@@ -44,7 +44,7 @@ struct WsLayout {
     size_t queue;       // int32[kQueueHeader + 6 groups] work queue of the forward attention kernel
     size_t part_o;      // bf16 [1 or 2][Hg][L][k][d] routed partial outputs (normalised) of one group of Hg heads; with
                         // several groups, two buffers that consecutive groups alternate between
-    size_t part_lse;    // float[H][L][k]    routed partial log-sum-exp (-inf = unused slot)
+    size_t part_lse;    // float[H][ceil(L / 128)][k][128]  routed partial log-sum-exp (-inf = unused slot), see part_lse_at
     size_t fwd_end;
     size_t delta;       // float[H][L]       rowsum(dO * O)
     size_t bwd_end;
@@ -154,6 +154,12 @@ __device__ __forceinline__ bool index_ok(bool, int *, int) { return true; }
 //   LB = ceil(L / 128) blocks per head
 __device__ __forceinline__ size_t part_piece(int hl, int LB, int k, int NP, int qi, int s, int c) {
     return ((((((size_t)hl * LB + (qi >> 7)) * k + s) * (NP >> 1) + (c >> 1)) * 128 + (qi & 127)) << 1) + (c & 1);
+}
+
+// Index of the log-sum-exp of (head, query, slot): query-innermost like the partials, so that the lanes of an anchor
+// item, which hold consecutive queries, read 128 contiguous bytes per slot.
+__device__ __forceinline__ size_t part_lse_at(int h, int LB, int k, int qi, int s) {
+    return (((size_t)h * LB + (qi >> 7)) * k + s) * 128 + (qi & 127);
 }
 
 // A named range around a call of the boundary, for timeline tools (NVTX; a no-op when no tool is attached).

@@ -63,7 +63,7 @@ void layout_workspace(moc_plan *p) {
     w.pool_done = take(sizeof(int32_t) * H * C);
     w.queue = take(sizeof(int32_t) * (kQueueHeader + 6 * groups));
     w.part_o = take(per_head * (size_t)p->heads_per_group * buffers);
-    w.part_lse = take(sizeof(float) * H * L * (k ? k : 1));
+    w.part_lse = take(sizeof(float) * H * ((L + 127) / 128 * 128) * (k ? k : 1));
     w.fwd_end = o;
     w.delta = take(sizeof(float) * H * L);
     w.bwd_end = o;

@@ -794,13 +794,13 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
 #pragma unroll
             for (int x = 0; x < KR; ++x) top.j[x] = top.j[x] >= 0 ? s_col[top.j[x]] : -1;
             int32_t *out = p.sel + ((size_t)h * p.L + i) * p.k + pass * 64;
-            float *pl = p.part_lse + ((size_t)h * p.L + i) * p.k + pass * 64;
+            float *pl = p.part_lse + part_lse_at(h, (p.L + 127) >> 7, p.k, i, pass * 64);     // slot x: pl[x * 128]
             if (live) {
 #pragma unroll
                 for (int x = 0; x < KR; ++x)
                     if (x < kp) {
                         out[x] = top.j[x];
-                        if (top.j[x] < 0) pl[x] = -INFINITY;
+                        if (top.j[x] < 0) pl[x * 128] = -INFINITY;
                     }
             }
             if (deferred) {
@@ -985,7 +985,7 @@ __global__ void __launch_bounds__(256) lists_from_sel_kernel(int32_t *__restrict
     int32_t *row = sel + ((size_t)h * L + i) * k;
     if (i < L) {
         const int ci = tok_chunk[i];
-        float *pl = part_lse + ((size_t)h * L + i) * k;
+        float *pl = part_lse + part_lse_at(h, (L + 127) >> 7, k, i, 0);      // slot s: pl[s * 128]
         for (int s = 0; s < k; ++s) {
             const int j = row[s];
             bool ok = j >= 0 && j < C && (!causal || j < ci);
@@ -994,7 +994,7 @@ __global__ void __launch_bounds__(256) lists_from_sel_kernel(int32_t *__restrict
             if (ok) atomicAdd(&hist[j], 1);
             else {
                 if (j != -1) row[s] = -1;
-                pl[s] = -INFINITY;
+                pl[s * 128] = -INFINITY;
             }
         }
     }
