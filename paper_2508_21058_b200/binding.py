@@ -90,11 +90,12 @@ def _check(code: int):
 
 
 def _ptr(t):
-    return C.c_void_p(0) if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """The current stream's handle, without building a torch.cuda.Stream object for it (5 us a call)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 class MocPlan:

@@ -111,16 +111,18 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     }
     int dev = 0;
     MOC_CUDA_TRY(cudaGetDevice(&dev));
-    cudaDeviceProp prop;
-    MOC_CUDA_TRY(cudaGetDeviceProperties(&prop, dev));
-    if (prop.major != 10) return MOC_ERR_ARCH;
+    // two attributes, not the whole property structure, which takes the driver a millisecond or two to fill in
+    int cc_major = 0, n_sm = 0;
+    MOC_CUDA_TRY(cudaDeviceGetAttribute(&cc_major, cudaDevAttrComputeCapabilityMajor, dev));
+    MOC_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+    if (cc_major != 10) return MOC_ERR_ARCH;
 
     moc_plan *p = new (std::nothrow) moc_plan();
     if (!p) return MOC_ERR_CUDA;
     p->H = pr->n_heads; p->L = L; p->d = pr->head_dim; p->C = C; p->k = pr->top_k;
     p->win_back = pr->win_back; p->win_fwd = pr->win_fwd; p->flags = pr->flags;
     p->scale = pr->softmax_scale > 0.f ? pr->softmax_scale : 1.0f / sqrtf((float)pr->head_dim);
-    p->device = dev; p->n_sm = prop.multiProcessorCount;
+    p->device = dev; p->n_sm = n_sm;
     p->off.assign(pr->chunk_off, pr->chunk_off + C + 1);
     p->shot.assign(pr->chunk_shot, pr->chunk_shot + C);
     p->mod.assign(pr->chunk_mod, pr->chunk_mod + C);
@@ -253,22 +255,31 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     cudaError_t e = cudaMalloc(&p->d_blob, o);
     if (e != cudaSuccess) { set_cuda_error(e, "cudaMalloc(plan tables)"); delete p; return MOC_ERR_CUDA; }
     char *b = static_cast<char *>(p->d_blob);
-    auto up = [&](size_t at, const void *src, size_t bytes) {
-        return bytes ? cudaMemcpy(b + at, src, bytes, cudaMemcpyHostToDevice) : cudaSuccess;
-    };
-    cudaError_t es[] = {up(o_off, p->off.data(), 4 * (C + 1)), up(o_shot, p->shot.data(), 4 * C), up(o_mod, p->mod.data(), C),
-                        up(o_tok, tok_chunk.data(), 4 * (size_t)L), up(o_bits, bits.data(), 4 * bits.size()),
-                        up(o_aoff, p->anc_off.data(), 4 * (C + 1)), up(o_arng, p->anc_rng.data(), sizeof(KeyRange) * p->anc_rng.size()),
-                        up(o_roff, p->ranc_off.data(), 4 * (C + 1)), up(o_ranc, p->ranc.data(), 4 * p->ranc.size()),
-                        up(o_qt, p->qitems.data(), sizeof(WorkItem) * p->qitems.size()),
-                        up(o_puo, p->pool_unit_off.data(), 4 * (C + 1)), up(o_puc, unit_chunk.data(), 4 * unit_chunk.size()),
-                        up(o_cap, p->cap_off.data(), 4 * (C + 1)), up(o_crng, chunk_rng.data(), sizeof(KeyRange) * C),
-                        up(o_kt, p->ktiles.data(), sizeof(KTile) * p->ktiles.size()),
-                        up(o_candc, cand_c.data(), 4 * cand_c.size()), up(o_lim, lim.data(), 4 * C), up(o_reach, reach.data(), 4 * C),
-                        up(o_colc, col_chunk.data(), 4 * col_chunk.size()),
-                        up(o_shots, p->shot_chunks.data(), sizeof(KeyRange) * p->shot_chunks.size())};
-    for (cudaError_t x : es)
-        if (x != cudaSuccess) { set_cuda_error(x, "cudaMemcpy(plan tables)"); cudaFree(p->d_blob); delete p; return MOC_ERR_CUDA; }
+    // the tables are put together on the host and go over in one copy (twenty small ones took longer than everything else here)
+    std::vector<char> host(o);
+    auto up = [&](size_t at, const void *src, size_t bytes) { if (bytes) memcpy(host.data() + at, src, bytes); };
+    up(o_off, p->off.data(), 4 * (C + 1));
+    up(o_shot, p->shot.data(), 4 * C);
+    up(o_mod, p->mod.data(), C);
+    up(o_tok, tok_chunk.data(), 4 * (size_t)L);
+    up(o_bits, bits.data(), 4 * bits.size());
+    up(o_aoff, p->anc_off.data(), 4 * (C + 1));
+    up(o_arng, p->anc_rng.data(), sizeof(KeyRange) * p->anc_rng.size());
+    up(o_roff, p->ranc_off.data(), 4 * (C + 1));
+    up(o_ranc, p->ranc.data(), 4 * p->ranc.size());
+    up(o_qt, p->qitems.data(), sizeof(WorkItem) * p->qitems.size());
+    up(o_puo, p->pool_unit_off.data(), 4 * (C + 1));
+    up(o_puc, unit_chunk.data(), 4 * unit_chunk.size());
+    up(o_cap, p->cap_off.data(), 4 * (C + 1));
+    up(o_crng, chunk_rng.data(), sizeof(KeyRange) * C);
+    up(o_kt, p->ktiles.data(), sizeof(KTile) * p->ktiles.size());
+    up(o_candc, cand_c.data(), 4 * cand_c.size());
+    up(o_lim, lim.data(), 4 * C);
+    up(o_reach, reach.data(), 4 * C);
+    up(o_colc, col_chunk.data(), 4 * col_chunk.size());
+    up(o_shots, p->shot_chunks.data(), sizeof(KeyRange) * p->shot_chunks.size());
+    e = cudaMemcpy(b, host.data(), o, cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) { set_cuda_error(e, "cudaMemcpy(plan tables)"); cudaFree(p->d_blob); delete p; return MOC_ERR_CUDA; }
     p->d_off = (int32_t *)(b + o_off); p->d_shot = (int32_t *)(b + o_shot); p->d_mod = (uint8_t *)(b + o_mod);
     p->d_tok_chunk = (int32_t *)(b + o_tok); p->d_anc_bits = (uint32_t *)(b + o_bits);
     p->d_anc_off = (int32_t *)(b + o_aoff); p->d_anc_rng = (KeyRange *)(b + o_arng);
