@@ -15,8 +15,8 @@
 //     workspace; the anchor mode adds them to its own part and writes dQ.
 //   dK/dV mode (key stationary, one CTA per 128 keys of a chunk):  X = (K, V) rows of the key
 //     tile by TMA, Y = (Q, dO) rows of every query that attends to the chunk - the query rows of
-//     the chunks that have it as an anchor, then the chunk's routed query list - copied by four
-//     producer warps with 16-byte asynchronous copies; lse and delta belong to the column; ACC1 is
+//     the chunks that have it as an anchor, then the chunk's routed query list - brought by four
+//     producer warps, Q and dO each through a ring of its own; lse and delta belong to the column; ACC1 is
 //     dK, ACC2 is dV.  Each key tile is owned by one CTA: no atomics, no partial sums.
 // The tensor pipe and the lanes overlap across tiles.  dK/dV: the issue order is ACC2(j), T1(j+1),
 // ACC1(j), T2(j+1), so that while the lanes form P(j+1) the pipe runs ACC1(j) and T2(j+1), and T1 / T2
@@ -57,6 +57,7 @@ struct BwdParams {
     size_t cap_total;
     int *status;
     int H, L, C, k;
+    SlotDiv kdiv;
     float scale, scale_log2;
 };
 
@@ -67,6 +68,8 @@ constexpr float kLog2e = 1.4426950408889634f;
 template <int D, int MODE>
 __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __grid_constant__ CUtensorMap tmK,
                                                                        const __grid_constant__ CUtensorMap tmV,
+                                                                       const __grid_constant__ CUtensorMap tmQ,
+                                                                       const __grid_constant__ CUtensorMap tmdO,
                                                                        const BwdParams p) {
     constexpr int TILE_BYTES = 128 * D * 2;
     constexpr int SUB = D / 64;
@@ -79,9 +82,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
     __shared__ int s_abort;
     __shared__ int w_valid, w_h, w_rows, w_first, w_nrng, w_ntiles, w_chunk, w_t0;
     __shared__ const KeyRange *w_rng;
-    // dK/dV mode: per streamed query, (lse * log2(e), delta), for tiles j and j + 1;
+    // dK/dV mode: per streamed query, (-lse * log2(e), -delta), for tiles j and j + 1;
     // dQ modes: the first 128 words hold the item's query rows while they are staged
-    __shared__ __align__(8) float s_ld[2][2][128];
+    __shared__ __align__(16) float s_ld[2][2][128];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -155,11 +158,11 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
         w_valid = valid;
         mbar_init(bar(X_FULL), MODE == DKV ? 1 : 256);
         for (int t = 0; t < kY1Stages; ++t) {
-            mbar_init(bar(Y1_FULL + t), MODE == DKV ? 128 : 1);
+            mbar_init(bar(Y1_FULL + t), MODE == DKV ? 2 : 1);       // dK/dV: the ring's two producer warps
             mbar_init(bar(Y1_EMPTY + t), 1);
         }
         for (int t = 0; t < kY2Stages; ++t) {
-            mbar_init(bar(Y2_FULL + t), MODE == DKV ? 128 : 1);
+            mbar_init(bar(Y2_FULL + t), MODE == DKV ? 2 : 1);
             mbar_init(bar(Y2_EMPTY + t), MODE == DKV ? 2 : 1);     // dK/dV: T2 and ACC2 both read the stage
             mbar_init(bar(T1_FULL + t), 1);
             mbar_init(bar(T2_FULL + t), 1);
@@ -204,7 +207,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
             if (r < rows) {
                 if (MODE == DQ_ROUTED) {
                     const int e = p.qlist[(size_t)h * p.cap_total + w_first + r];
-                    qi = e / p.k;
+                    qi = p.kdiv.query(e);
                     slot = e - qi * p.k;
                     (void)index_ok(e >= 0 && qi < p.L, p.status, IX_BWD_LIST_ENTRY);
                     if ((unsigned)qi >= (unsigned)p.L) qi = -1;      // never follow an entry that is not a row of this head
@@ -238,7 +241,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
             fence_proxy_async_smem();
             mbar_arrive(bar(X_FULL));
         }
-        const float c = p.scale_log2;
+        const uint64_t c2 = pack2(p.scale_log2, p.scale_log2), nlse2 = pack2(-lse2, -lse2), ndlt2 = pack2(-dlt, -dlt);
         TileIter it(w_rng, MODE == DKV ? 0 : w_nrng);
         bool ok = true;
         int s3 = 0, ph3 = 0;                          // Y1 stage of tile jt and its phase
@@ -263,20 +266,26 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                 // dK/dV: P goes over T1 columns that the other thread of the lane reads in its first round; that
                 // read is announced here and waited for (bounded, like every wait) just before the first store
                 if (MODE == DKV && rd == 0) mbar_arrive(bar(RD1));
+                // two columns per packed instruction; in dK/dV mode four columns' (negated) lse per shared-memory load
 #pragma unroll
-                for (int x = 0; x < 32; x += 2) {
-                    float l0 = lse2, l1 = lse2;
+                for (int x = 0; x < 32; x += 4) {
+                    uint64_t nl[2] = {nlse2, nlse2};
                     if (MODE == DKV) {
-                        const float2 l = *reinterpret_cast<const float2 *>(&s_ld[st][0][ch * 32 + x]);
-                        l0 = l.x; l1 = l.y;
+                        const ulonglong2 l = *reinterpret_cast<const ulonglong2 *>(&s_ld[st][0][ch * 32 + x]);
+                        nl[0] = l.x; nl[1] = l.y;
                     }
-                    float p0 = ex2(fmaf(__uint_as_float(s[x]), c, -l0)), p1 = ex2(fmaf(__uint_as_float(s[x + 1]), c, -l1));
-                    if (MODE != DKV) {
-                        if (ch * 32 + x >= valid) p0 = 0.f;
-                        if (ch * 32 + x + 1 >= valid) p1 = 0.f;
+#pragma unroll
+                    for (int y = 0; y < 2; ++y) {
+                        float p0, p1;
+                        unpack2(fma2(pack2(__uint_as_float(s[x + 2 * y]), __uint_as_float(s[x + 2 * y + 1])), c2, nl[y]), p0, p1);
+                        pv[rd * 32 + x + 2 * y] = ex2(p0);
+                        pv[rd * 32 + x + 2 * y + 1] = ex2(p1);
                     }
-                    pv[rd * 32 + x] = p0;
-                    pv[rd * 32 + x + 1] = p1;
+                }
+                if (MODE != DKV && valid < 128) {               // keys past the end of the range
+#pragma unroll
+                    for (int x = 0; x < 32; ++x)
+                        if (ch * 32 + x >= valid) pv[rd * 32 + x] = 0.f;
                 }
                 if (MODE == DKV) {
                     uint32_t ups[16];
@@ -312,14 +321,19 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                 tmem_wait_ld();
                 if (rd == 0) mbar_arrive(bar(RD2));                     // this thread's first-round columns have been read
 #pragma unroll
-                for (int x = 0; x < 32; x += 2) {
-                    float d0 = dlt, d1 = dlt;
+                for (int x = 0; x < 32; x += 4) {
+                    uint64_t nd[2] = {ndlt2, ndlt2};
                     if (MODE == DKV) {
-                        const float2 d = *reinterpret_cast<const float2 *>(&s_ld[st][1][ch * 32 + x]);
-                        d0 = d.x; d1 = d.y;
+                        const ulonglong2 d = *reinterpret_cast<const ulonglong2 *>(&s_ld[st][1][ch * 32 + x]);
+                        nd[0] = d.x; nd[1] = d.y;
                     }
-                    uds[x >> 1] = bf16x2(pv[rd * 32 + x] * (__uint_as_float(dp[x]) - d0),
-                                         pv[rd * 32 + x + 1] * (__uint_as_float(dp[x + 1]) - d1));
+#pragma unroll
+                    for (int y = 0; y < 2; ++y) {
+                        float a0, a1;
+                        unpack2(mul2(pack2(pv[rd * 32 + x + 2 * y], pv[rd * 32 + x + 2 * y + 1]),
+                                     add2(pack2(__uint_as_float(dp[x + 2 * y]), __uint_as_float(dp[x + 2 * y + 1])), nd[y])), a0, a1);
+                        uds[(x >> 1) + y] = bf16x2(a0, a1);
+                    }
                 }
                 if (rd == 0) {
                     ok = mbar_wait_spin(bar(RD2), jt & 1, abort_flag, p.status, BW_READ);
@@ -464,67 +478,133 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                     tma_load_2d(sX + TILE_BYTES + sub * SUB_BYTES, &tmV, sub * 64, h * p.L + w_t0, bar(X_FULL));
                 }
             }
-            // the queries that attend to this chunk, 128 at a time: Q rows -> Y1, dO rows -> Y2; each of the
-            // four producer warps copies 32 rows of every tile
-            const int pw = warp - 8;
+            // The queries that attend to this chunk, 128 at a time: Q rows -> Y1 by the first two producer warps, dO rows -> Y2
+            // by the other two, each warp 64 rows of every tile.  The two rings run on their own: a tile's Q is fetched as
+            // soon as a Y1 stage is free, whatever Y2 waits for (one loop for both left T1 of the next tile waiting for
+            // 1400 of a tile's 3900 cycles).  Full tiles of consecutive queries come by TMA, the others by 16-byte
+            // asynchronous copies (36 bytes a cycle and SM; TMA row gathers reach 24).
+            const int pw = warp - 8, wsub = pw & 1;
+            const bool y1 = pw < 2;
             const int chunk = w_chunk;
             const int a1 = p.ranc_off[chunk + 1];
             int a = p.ranc_off[chunk], r0 = 0, r1 = 0;       // current row range [r0, r1)
             const int n_list = p.cnt[h * p.C + chunk];
             const int32_t *list = p.qlist + (size_t)h * p.cap_total + p.cap_off[chunk];
             int e0 = 0;                                        // next entry of the routed list
-            int s3 = 0, ph3 = 0;
             bool ok = true;
-            const int i = pw * 32 + lane;                      // this lane's row of every tile
-            // the query behind this lane's row of the next tile, with its lse and delta; loaded one tile ahead so
-            // that these dependent loads are never waited for
-            int q = -1;
-            float q_lse = INFINITY, q_del = 0.f;
-            auto next_rows = [&]() {
+            // This lane's two rows of a tile, in two steps so that no load is waited for: the list entries two tiles ahead,
+            // then, one tile ahead, the queries with their lse and delta.
+            int nx_whole = -1, nx_row = -1, nx_end = 0, nx_e[2] = {-1, -1};
+            auto look_ahead = [&]() {
                 if (r0 >= r1 && a < a1) {                      // next merged range of anchor query rows
                     int qc = p.ranc[a];
                     r0 = p.off[qc]; r1 = p.off[qc + 1];
                     for (++a; a < a1 && p.ranc[a] == qc + 1; ++a) { qc = p.ranc[a]; r1 = p.off[qc + 1]; }
                 }
-                q = -1;
-                if (r0 < r1) { if (r0 + i < r1) q = r0 + i; }
-                else if (e0 + i < n_list && index_ok((size_t)p.cap_off[chunk] + e0 + i < p.cap_total, p.status, IX_BWD_LIST_POSITION)) {
-                    q = list[e0 + i] / p.k;
-                    if (!index_ok((unsigned)q < (unsigned)p.L, p.status, IX_BWD_LIST_ENTRY)) q = -1;
+                const int i = wsub * 64 + lane;
+                nx_whole = -1; nx_row = -1; nx_e[0] = nx_e[1] = -1;
+                if (r0 < r1) {
+                    if (r0 + 128 <= r1) nx_whole = r0;         // a full tile of consecutive queries
+                    nx_row = r0 + i;
+                    nx_end = r1;
+                    r0 += 128;
+                } else {
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+                        const int e = e0 + i + 32 * x;
+                        if (e < n_list && index_ok((size_t)p.cap_off[chunk] + e < p.cap_total, p.status, IX_BWD_LIST_POSITION)) nx_e[x] = list[e];
+                    }
+                    e0 += 128;
                 }
-                if (r0 < r1) r0 += 128; else e0 += 128;
-                // a column without a query gets lse = +inf: its P and dS come out as exact zeros
-                q_lse = q >= 0 ? p.lse[(size_t)h * p.L + q] * kLog2e : INFINITY;
-                q_del = q >= 0 ? p.delta[(size_t)h * p.L + q] : 0.f;
             };
-            if (n_tiles > 0) next_rows();
+            int whole = -1, q[2] = {-1, -1};
+            float q_lse[2] = {INFINITY, INFINITY}, q_del[2] = {0.f, 0.f};
+            auto next_rows = [&]() {
+                whole = nx_whole;
+#pragma unroll
+                for (int x = 0; x < 2; ++x) {
+                    q[x] = -1;
+                    if (nx_row >= 0) {
+                        if (nx_row + 32 * x < nx_end) q[x] = nx_row + 32 * x;
+                    } else if (nx_e[x] >= 0) {
+                        q[x] = p.kdiv.query(nx_e[x]);
+                        if (!index_ok((unsigned)q[x] < (unsigned)p.L, p.status, IX_BWD_LIST_ENTRY)) q[x] = -1;
+                    }
+                    // a column without a query gets lse = +inf: its P and dS come out as exact zeros
+                    // (used, that is waited for, when the tile's turn comes)
+                    q_lse[x] = INFINITY;
+                    q_del[x] = 0.f;
+                    if (y1 && q[x] >= 0) {
+                        q_lse[x] = p.lse[(size_t)h * p.L + q[x]];
+                        q_del[x] = p.delta[(size_t)h * p.L + q[x]];
+                    }
+                }
+                look_ahead();
+            };
+            if (n_tiles > 0) { look_ahead(); next_rows(); }
+            int st = 0, ph = 0;                                // stage of tile jt in this warp's ring, and its phase
+            int issued = 0;                                    // tiles whose copies this warp has issued
+            const int n_st = y1 ? kY1Stages : kY2Stages, b_full = y1 ? Y1_FULL : Y2_FULL, b_empty = y1 ? Y1_EMPTY : Y2_EMPTY;
+            const uint32_t ring = y1 ? sY1 : sY2;
+            const CUtensorMap *tile_map = y1 ? &tmQ : &tmdO;
+            const __nv_bfloat16 *rows_src = (y1 ? p.Q : p.dO) + (size_t)h * p.L * D;
+            if (lane == 0) prefetch_tensormap(tile_map);
             for (int jt = 0; ok && jt < n_tiles; ++jt) {
-                const int s2 = jt & 1;
-                ok = mbar_wait(bar(Y1_EMPTY + s3), ph3 ^ 1, abort_flag, p.status, BW_YEMPTY);
-                ok = ok && mbar_wait(bar(Y2_EMPTY + s2), ((jt >> 1) & 1) ^ 1, abort_flag, p.status, BW_YEMPTY);
-                // the lanes have finished with the lse / delta of tile jt - 2
-                if (jt >= 2) ok = ok && mbar_wait(bar(DS_DONE + s2), ((jt - 2) >> 1) & 1, abort_flag, p.status, BW_DSDONE);
+                // the next tile's loads go out first: behind this tile's copies they would queue for a thousand cycles
+                const bool by_tile = whole >= 0;
+                const int t_whole = whole, t_q[2] = {q[0], q[1]};
+                const float t_lse[2] = {q_lse[0], q_lse[1]}, t_del[2] = {q_del[0], q_del[1]};
+                if (jt + 1 < n_tiles) next_rows();
+                ok = mbar_wait(bar(b_empty + st), ph ^ 1, abort_flag, p.status, BW_YEMPTY);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                s_ld[s2][0][i] = q_lse;
-                s_ld[s2][1][i] = q_del;
-                constexpr int RP = 32 / CH;                    // rows per instruction
-                const int c16 = lane % CH;
+                const uint32_t dst = ring + st * TILE_BYTES;
+                if (by_tile) {
+                    if (lane == 0) {
 #pragma unroll
-                for (int rb = 0; rb < 32; rb += RP) {
-                    const int rl = rb + lane / CH, rr = pw * 32 + rl;
-                    const int qq = __shfl_sync(0xffffffffu, q, rl);
-                    const size_t src = ((size_t)h * p.L + max(qq, 0)) * D + c16 * 8;
-                    const uint32_t dst = (c16 >> 3) * SUB_BYTES + sw128_offset(rr, c16 & 7);
-                    cp_async16(sY1 + s3 * TILE_BYTES + dst, p.Q + src, qq >= 0 ? 16u : 0u);
-                    cp_async16(sY2 + s2 * TILE_BYTES + dst, p.dO + src, qq >= 0 ? 16u : 0u);
+                        for (int sub = 0; sub < SUB; ++sub)
+                            tma_load_2d(dst + sub * SUB_BYTES + wsub * 64 * 128, tile_map, sub * 64, h * p.L + t_whole + wsub * 64, bar(b_full + st));
+                    }
+                } else {
+                    constexpr int RP = 32 / CH;                // rows per instruction
+                    const int c16 = lane % CH;
+#pragma unroll
+                    for (int rb = 0; rb < 64; rb += RP) {
+                        const int rl = rb + lane / CH;
+                        const int qq = __shfl_sync(0xffffffffu, t_q[rb >> 5], rl & 31);
+                        cp_async16(dst + (c16 >> 3) * SUB_BYTES + sw128_offset(wsub * 64 + rl, c16 & 7),
+                                   rows_src + (size_t)max(qq, 0) * D + c16 * 8, qq >= 0 ? 16u : 0u);
+                    }
                 }
-                if (jt + 1 < n_tiles) next_rows();
+                ++issued;
+                if (y1) {
+                    // the lanes have finished with the lse / delta of tile jt - 2
+                    if (jt >= 2) ok = mbar_wait(bar(DS_DONE + (jt & 1)), ((jt - 2) >> 1) & 1, abort_flag, p.status, BW_DSDONE);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+#pragma unroll
+                    for (int x = 0; x < 2; ++x) {
+                        s_ld[jt & 1][0][wsub * 64 + x * 32 + lane] = t_lse[x] * -kLog2e;
+                        s_ld[jt & 1][1][wsub * 64 + x * 32 + lane] = -t_del[x];
+                    }
+                }
+                if (!by_tile) {
+                    cp_async_wait_all();
+                    fence_proxy_async_smem();
+                }
+                __syncwarp();
+                // one of the ring's two warps
+                if (lane == 0) {
+                    if (by_tile) mbar_expect_tx(bar(b_full + st), TILE_BYTES / 2);
+                    else mbar_arrive(bar(b_full + st));
+                }
+                if (++st == n_st) { st = 0; ph ^= 1; }
+            }
+            if (*abort_flag) {      // copies already issued must land before the shared memory is released
                 cp_async_wait_all();
-                fence_proxy_async_smem();
-                mbar_arrive(bar(Y1_FULL + s3));
-                mbar_arrive(bar(Y2_FULL + s2));
-                if (++s3 == kY1Stages) { s3 = 0; ph3 ^= 1; }
+                int dummy_flag = 0;
+                for (int b = 1; b <= n_st; ++b)
+                    if (issued - b >= 0) mbar_wait(bar(b_full + (issued - b) % n_st), ((issued - b) / n_st) & 1, &dummy_flag, p.status, BW_YFULL);
             }
         }
     } else {
@@ -664,9 +744,11 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
                            __nv_bfloat16 *dQ, __nv_bfloat16 *dK, __nv_bfloat16 *dV, void *ws, cudaStream_t s) {
     float *delta = ws_ptr<float>(ws, p->ws.delta);
     if (int r = launch_delta(p, O, dO, delta, s)) return r;
-    CUtensorMap tmK, tmV;
+    CUtensorMap tmK, tmV, tmQ, tmdO;       // Q and dO: tiles of 64 rows
     if (int r = make_tmap_2d_bf16(&tmK, K, (uint64_t)p->H * p->L, D, 128)) return r;
     if (int r = make_tmap_2d_bf16(&tmV, V, (uint64_t)p->H * p->L, D, 128)) return r;
+    if (int r = make_tmap_2d_bf16(&tmQ, Q, (uint64_t)p->H * p->L, D, 64)) return r;
+    if (int r = make_tmap_2d_bf16(&tmdO, dO, (uint64_t)p->H * p->L, D, 64)) return r;
     BwdParams a;
     a.Q = Q; a.K = K; a.V = V; a.dO = dO; a.lse = lse; a.delta = delta;
     a.part_lse = ws_ptr<float>(ws, p->ws.part_lse);
@@ -678,7 +760,7 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
     a.qlist = ws_ptr<int32_t>(ws, p->ws.qlist);
     a.cap_total = (size_t)p->cap_off[p->C];
     a.status = ws_ptr<int>(ws, p->ws.status);
-    a.H = p->H; a.L = p->L; a.C = p->C; a.k = p->k;
+    a.H = p->H; a.L = p->L; a.C = p->C; a.k = p->k; a.kdiv = SlotDiv::of(p->k);
     a.scale = p->scale; a.scale_log2 = p->scale * kLog2e;
     // seven tiles (X1 X2, three Y1 stages, two Y2 stages) and the slack that aligns them to 1024 bytes; at
     // d = 128 that is all an SM has, so the request is what the kernel's static variables leave of the limit
@@ -709,16 +791,16 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
             a.item_lo_dev = tile_off + (size_t)h0 * p->C;
             a.item_hi_dev = tile_off + (size_t)(h0 + hg) * p->C;
             const long long bound = (long long)hg * (((long long)p->L * p->k + kQTileRows - 1) / kQTileRows + p->C);
-            attend_bwd_tc_kernel<D, DQ_ROUTED><<<(unsigned)(2 * bound), kBwdThreads, smem[DQ_ROUTED], s>>>(tmK, tmV, a);
+            attend_bwd_tc_kernel<D, DQ_ROUTED><<<(unsigned)(2 * bound), kBwdThreads, smem[DQ_ROUTED], s>>>(tmK, tmV, tmQ, tmdO, a);
             MOC_LAUNCH_CHECK();
         }
         a.rng = p->d_anc_rng;
         a.items = p->d_qitems;
         a.item_lo_dev = a.item_hi_dev = nullptr;
-        attend_bwd_tc_kernel<D, DQ_ANCHOR><<<dim3((unsigned)(2 * p->qitems.size()), (unsigned)hg), kBwdThreads, smem[DQ_ANCHOR], s>>>(tmK, tmV, a);
+        attend_bwd_tc_kernel<D, DQ_ANCHOR><<<dim3((unsigned)(2 * p->qitems.size()), (unsigned)hg), kBwdThreads, smem[DQ_ANCHOR], s>>>(tmK, tmV, tmQ, tmdO, a);
         MOC_LAUNCH_CHECK();
     }
-    attend_bwd_tc_kernel<D, DKV><<<(unsigned)(p->ktiles.size() * (size_t)p->H), kBwdThreads, smem[DKV], s>>>(tmK, tmV, a);
+    attend_bwd_tc_kernel<D, DKV><<<(unsigned)(p->ktiles.size() * (size_t)p->H), kBwdThreads, smem[DKV], s>>>(tmK, tmV, tmQ, tmdO, a);
     MOC_LAUNCH_CHECK();
     return MOC_OK;
 }

@@ -63,6 +63,7 @@ struct AttendParams {
     size_t cap_total;
     int *status;
     int H, L, C, k, hg, n_groups, n_aitems;
+    SlotDiv kdiv;
     float scale_log2;           // softmax scale * log2(e)
     uint32_t cookie;
 };
@@ -132,13 +133,6 @@ __device__ __forceinline__ bool wait_count(const int *ctr, int need, volatile in
             }
         }
     }
-}
-
-// four rows of a 2-D tensor, 64 columns from column x on, into four consecutive 128-byte rows of shared memory
-__device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap *map, int x, int r0, int r1, int r2, int r3, uint32_t bar) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cta.global.tile::gather4.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], [%7];"
-                 ::"r"(dst), "l"(map), "r"(x), "r"(r0), "r"(r1), "r"(r2), "r"(r3), "r"(bar)
-                 : "memory");
 }
 
 template <int D>
@@ -240,7 +234,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                 if (routed) {
                     const bool at_ok = index_ok((size_t)first + rt < p.cap_total, p.status, IX_LIST_POSITION);
                     const int e = at_ok ? p.qlist[(size_t)h * p.cap_total + first + rt] : -1;
-                    qi = e / p.k;
+                    qi = p.kdiv.query(e);
                     slot = e - qi * p.k;
                     (void)index_ok(e >= 0 && qi < p.L, p.status, IX_LIST_ENTRY);
                     if (e < 0 || qi >= p.L) qi = -1;         // never follow an entry that is not a row of this head
@@ -822,7 +816,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                         const int rt = g * 128 + lane * 4 + x;
                         const size_t at = (size_t)first + (rt < rows ? rt : 0);
                         const int e = at < p.cap_total ? p.qlist[(size_t)h * p.cap_total + at] : 0;
-                        int qi = e / p.k;
+                        int qi = p.kdiv.query(e);
                         if (e < 0 || qi >= p.L) qi = 0;
                         row[x] = h * p.L + qi;
                     }
@@ -895,7 +889,7 @@ static int attend_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfl
     a.queue = ws_ptr<int>(ws, p->ws.queue);
     a.cap_total = (size_t)p->cap_off[p->C];
     a.status = ws_ptr<int>(ws, p->ws.status);
-    a.H = p->H; a.L = p->L; a.C = p->C; a.k = p->k; a.hg = p->heads_per_group; a.n_groups = n_groups;
+    a.H = p->H; a.L = p->L; a.C = p->C; a.k = p->k; a.kdiv = SlotDiv::of(p->k); a.hg = p->heads_per_group; a.n_groups = n_groups;
     a.n_aitems = (int)p->qitems.size();
     a.scale_log2 = p->scale * 1.4426950408889634f;
     a.cookie = p->cookie;

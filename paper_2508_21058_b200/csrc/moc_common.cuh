@@ -128,6 +128,23 @@ static inline T *ws_ptr(void *ws, size_t off) { return reinterpret_cast<T *>(sta
 template <typename T>
 static inline const T *ws_ptr(const void *ws, size_t off) { return reinterpret_cast<const T *>(static_cast<const char *>(ws) + off); }
 
+// Division of a list entry (query * k + slot) by k without the division sequence, whose reciprocal queues behind the
+// exponentials of the same scheduler.  Exact for 0 <= e < 2^31: mul = ceil(2^(31 + s) / k) with 2^s >= k, so that
+// 0 <= mul * k - 2^(31 + s) < k <= 2^s.
+struct SlotDiv {
+    uint32_t mul;
+    int shift;
+    static SlotDiv of(int k) {
+        int s = 0;
+        while ((1 << s) < k) ++s;
+        const uint64_t two = 1ull << (31 + s), kk = k > 0 ? k : 1;
+        return SlotDiv{(uint32_t)((two + kk - 1) / kk), 31 + s};
+    }
+#ifdef __CUDACC__
+    __device__ __forceinline__ int query(int e) const { return e < 0 ? -1 : (int)(((uint64_t)(uint32_t)e * mul) >> shift); }
+#endif
+};
+
 #ifdef __CUDACC__
 // Debug build (-DMOC_DEBUG): every index a kernel takes from the workspace (list entries, list positions,
 // work-item fields) is checked before it is used as an address; a bad one records MOC_ERR_INDEX with `code`
