@@ -257,15 +257,22 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
             // ---- P = exp2(scale log2(e) S - lse log2(e)) from T1
             const uint32_t t2c = (MODE != DKV && st) ? 384u : 128u;       // T2 (then dS) of this tile
             float pv[64];
+            uint32_t sv[2][32];
+            tmem_ld32(tmem + lane_off + half * 32, sv[0]);
+            tmem_ld32(tmem + lane_off + (2 + half) * 32, sv[1]);
+            tmem_wait_ld();
+            if (MODE == DKV) {
+                // P goes over T1 columns that the other thread of the lane reads; that read is announced here and waited
+                // for (bounded, like every wait) just before the first store
+                mbar_arrive(bar(RD1));
+            } else {                                                      // T1 has been read and may be overwritten
+                tc_fence_before();
+                mbar_arrive(bar(P_DONE));
+            }
 #pragma unroll
             for (int rd = 0; rd < 2; ++rd) {
                 const int ch = rd * 2 + half;
-                uint32_t s[32];
-                tmem_ld32(tmem + lane_off + ch * 32, s);
-                tmem_wait_ld();
-                // dK/dV: P goes over T1 columns that the other thread of the lane reads in its first round; that
-                // read is announced here and waited for (bounded, like every wait) just before the first store
-                if (MODE == DKV && rd == 0) mbar_arrive(bar(RD1));
+                const uint32_t (&s)[32] = sv[rd];
                 // two columns per packed instruction; in dK/dV mode four columns' (negated) lse per shared-memory load
 #pragma unroll
                 for (int x = 0; x < 32; x += 4) {
@@ -304,22 +311,21 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                 }
             }
             if (!ok) break;
-            if (MODE != DKV) {                                            // T1 has been read and may be overwritten
-                tc_fence_before();
-                mbar_arrive(bar(P_DONE));
-            }
             // ---- dS = P (dP - delta) from T2, written over T2 columns that have been read
             ok = mbar_wait_spin(bar(T2_FULL + st), (jt >> 1) & 1, abort_flag, p.status, BW_T2FULL);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
+            uint32_t dpv[2][32];
+            tmem_ld32(tmem + lane_off + t2c + half * 32, dpv[0]);
+            tmem_ld32(tmem + lane_off + t2c + (2 + half) * 32, dpv[1]);
+            tmem_wait_ld();
+            mbar_arrive(bar(RD2));                                      // this thread's columns have been read
 #pragma unroll
             for (int rd = 0; rd < 2; ++rd) {
                 const int ch = rd * 2 + half;
-                uint32_t dp[32], uds[16];
-                tmem_ld32(tmem + lane_off + t2c + ch * 32, dp);
-                tmem_wait_ld();
-                if (rd == 0) mbar_arrive(bar(RD2));                     // this thread's first-round columns have been read
+                const uint32_t (&dp)[32] = dpv[rd];
+                uint32_t uds[16];
 #pragma unroll
                 for (int x = 0; x < 32; x += 4) {
                     uint64_t nd[2] = {ndlt2, ndlt2};
