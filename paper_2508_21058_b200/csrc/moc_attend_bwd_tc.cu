@@ -785,27 +785,7 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
             MOC_CUDA_TRY(cudaFuncSetAttribute(fn[m], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem[m]));
         }
     }
-    // dQ group by group of heads (the routed mode leaves the group's partials in the workspace, the
-    // anchor mode adds them up), then dK / dV of every key tile
-    const int *tile_off = ws_ptr<int>(ws, p->ws.tile_off);
-    for (int h0 = 0; h0 < p->H; h0 += p->heads_per_group) {
-        const int hg = std::min(p->heads_per_group, p->H - h0);
-        a.h0 = h0;
-        if (p->k > 0) {
-            a.rng = p->d_chunk_rng;
-            a.items = ws_ptr<WorkItem>(ws, p->ws.rtiles);
-            a.item_lo_dev = tile_off + (size_t)h0 * p->C;
-            a.item_hi_dev = tile_off + (size_t)(h0 + hg) * p->C;
-            const long long bound = (long long)hg * (((long long)p->L * p->k + kQTileRows - 1) / kQTileRows + p->C);
-            attend_bwd_tc_kernel<D, DQ_ROUTED><<<(unsigned)(2 * bound), kBwdThreads, smem[DQ_ROUTED], s>>>(tmK, tmV, tmQ, tmdO, a);
-            MOC_LAUNCH_CHECK();
-        }
-        a.rng = p->d_anc_rng;
-        a.items = p->d_qitems;
-        a.item_lo_dev = a.item_hi_dev = nullptr;
-        attend_bwd_tc_kernel<D, DQ_ANCHOR><<<dim3((unsigned)(2 * p->qitems.size()), (unsigned)hg), kBwdThreads, smem[DQ_ANCHOR], s>>>(tmK, tmV, tmQ, tmdO, a);
-        MOC_LAUNCH_CHECK();
-    }
+    if (int r = launch_dq_tc(p, Q, K, V, lse, delta, dO, dQ, ws, s)) return r;
     attend_bwd_tc_kernel<D, DKV><<<(unsigned)(p->ktiles.size() * (size_t)p->H), kBwdThreads, smem[DKV], s>>>(tmK, tmV, tmQ, tmdO, a);
     MOC_LAUNCH_CHECK();
     return MOC_OK;

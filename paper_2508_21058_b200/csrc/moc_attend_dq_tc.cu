@@ -1,0 +1,548 @@
+// Tensor-core dQ of the sparse attention's backward (selection held constant): two persistent launches per group of heads.
+//
+// For a selected (query i, key t) pair:  P = exp(scale q.k - lse_i),  dP = dO_i . v_t,  dS = P (dP - delta_i),
+// dQ_i += scale dS k_t.  A work item is 128 query rows against their key tiles, as in the forward: the ROUTED launch takes
+// the rows of one chunk's query list against that chunk's keys and leaves one partial per (query, slot) in the workspace,
+// the ANCHOR launch takes consecutive rows against their anchor ranges, adds the rows' partials and writes dQ.
+//
+//     T1 = Q K^T,  T2 = dO V^T          (both operands from shared memory, into TMEM)
+//     threads (two per TMEM lane) turn T1 into P, then (P, T2) into dS, written back to TMEM as bf16
+//     ACC += dS K                        (A from TMEM, the K tile as an MN-major operand)
+//
+// One CTA per SM walks its items (a fixed stride through the launch's items, which are much alike): the tensor memory, the
+// barriers and the K/V rings live for the whole launch, and the next item's rows are fetched while the last tile of the current
+// one and its results are in work.  With a CTA per item, the launch of the CTA, its dependent look-ups and the gather of its
+// rows took 8000 cycles before the first product, of 42000 for an item of 13 key tiles.
+// 16 warps:
+//   warps 0-7   lanes, two threads per TMEM lane: of the four 32-column chunks of a tile, thread `half` takes chunks half and
+//               2 + half, and keeps its 64 P values between T1 and T2;
+//   warp 8      lane 0, TMA producer of the K and V tiles (three and two stages, running across items);
+//   warps 9-11  row loaders: the Q and dO rows of the next item by 16-byte asynchronous copies, its lse and delta, and its
+//               description for the other warps;
+//   warps 12,13 MMA issuers: warp 12 T1, warp 13 T2 and ACC.  T1(j + 1) is issued once the lanes have read T1(j); T2 has two
+//               buffers, T2(j + 2) follows ACC(j), which reads the dS stored over T2(j);
+//   warps 14,15 idle (they complete the fourth warpgroup).
+// Every mbarrier wait is bounded; a wait that runs out flags the workspace status word and the CTA drains and leaves.
+#include <algorithm>
+
+#include "moc_common.cuh"
+#include "moc_tc.cuh"
+
+namespace moc {
+
+using namespace tc;
+
+enum DqWait { DW_XFULL = 96, DW_XEMPTY, DW_YFULL, DW_YEMPTY, DW_T1FULL, DW_T2FULL, DW_READ, DW_DSDONE, DW_ACCFULL, DW_ACCFREE, DW_SMEM };
+
+struct DqParams {
+    const __nv_bfloat16 *Q, *dO;
+    const float *lse, *delta;
+    __nv_bfloat16 *dQ;
+    __nv_bfloat16 *part;          // routed dQ partials of the group of heads in flight (part_piece)
+    const float *part_lse;        // the forward's routed log-sum-exps (part_lse_at): -inf marks an empty slot
+    const KeyRange *rng;          // key ranges the items index
+    const WorkItem *items;        // up to 256 rows each: two of this kernel's items
+    const int *item_lo, *item_hi; // routed: the group's item range on the device
+    const int32_t *qlist;
+    size_t cap_total;
+    int *status;
+    int H, L, k, h0, hg, n_items; // anchor: n_items items for each of the group's hg heads
+    SlotDiv kdiv;
+    float scale, scale_log2;
+    uint32_t cookie;
+};
+
+constexpr int kDqThreads = 512, kKStages = 3, kVStages = 2, kLoaders = 3;
+
+// description of an item, as the row loaders leave it for the other warps; rows = 0: no more items
+struct DqItem { int h, first, rows, nrng, ntiles, rng_off, t0, t1; };
+
+template <int D, bool ANCHOR>
+__global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __grid_constant__ CUtensorMap tmK,
+                                                                     const __grid_constant__ CUtensorMap tmV, const DqParams p) {
+    constexpr int TILE_BYTES = 128 * D * 2;
+    constexpr int SUB = D / 64;
+    constexpr int SUB_BYTES = 128 * 128;
+    constexpr int CH = D / 8;               // 16-byte pieces per row
+    constexpr int N_TILES_SMEM = 2 + kKStages + kVStages;
+    enum { X_FULL = 0, X_EMPTY, K_FULL, K_EMPTY = K_FULL + kKStages, V_FULL = K_EMPTY + kKStages, V_EMPTY = V_FULL + kVStages,
+           T1_FULL = V_EMPTY + kVStages, T1_READ, T2_FULL, RD2 = T2_FULL + 2, DS_DONE, ACC_FULL = DS_DONE + 2, ACC_FREE, N_BARS };
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t bars[N_BARS];
+    __shared__ __align__(16) float s_ld[2][2][128];      // per item parity: -lse * log2(e) and -delta of the item's rows
+    __shared__ DqItem s_item[2];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int s_abort, s_lo, s_total;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    // shared tiles: X1 (Q) X2 (dO) | K stages | V stages
+    const uint32_t sX = sbase, sK = sbase + 2 * TILE_BYTES, sV = sbase + (2 + kKStages) * TILE_BYTES;
+    auto bar = [&](int i) { return smem_u32(&bars[i]); };
+
+    if (threadIdx.x == 0) {
+        s_abort = 0;
+        bool valid = *(volatile int *)p.status == 0;
+        if (valid && (uint32_t)((volatile int *)p.status)[ST_COOKIE] != p.cookie) {
+            atomicCAS(p.status, 0, MOC_ERR_WORKSPACE);      // not this plan's lists: report, touch nothing else
+            valid = false;
+        }
+        uint32_t dyn_bytes;
+        asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn_bytes));
+        if (valid && (sbase - smem_u32(smem_raw)) + (uint32_t)N_TILES_SMEM * TILE_BYTES > dyn_bytes) {
+            // the launch gave less shared memory than the tiles need: report, touch nothing
+            if (atomicCAS(p.status, 0, MOC_ERR_TIMEOUT) == 0) p.status[ST_DETAIL] = DW_SMEM;
+            valid = false;
+        }
+        s_lo = (!ANCHOR && valid) ? *p.item_lo : 0;
+        s_total = !valid ? 0 : 2 * (ANCHOR ? p.n_items * p.hg : *p.item_hi - s_lo);
+        mbar_init(bar(X_FULL), kLoaders);
+        mbar_init(bar(X_EMPTY), 2 + 8);                     // both issuers, and each lane warp when it has the item's data
+        for (int t = 0; t < kKStages; ++t) { mbar_init(bar(K_FULL + t), 1); mbar_init(bar(K_EMPTY + t), 1); }
+        for (int t = 0; t < kVStages; ++t) { mbar_init(bar(V_FULL + t), 1); mbar_init(bar(V_EMPTY + t), 1); }
+        mbar_init(bar(T1_FULL), 1);
+        mbar_init(bar(T1_READ), 256);
+        for (int t = 0; t < 2; ++t) { mbar_init(bar(T2_FULL + t), 1); mbar_init(bar(DS_DONE + t), 256); }
+        mbar_init(bar(RD2), 256);
+        mbar_init(bar(ACC_FULL), 1);
+        mbar_init(bar(ACC_FREE), 256);
+        fence_barrier_init();
+    }
+    __syncthreads();
+    if (s_total <= (int)blockIdx.x) return;
+    if (warp == 8) {
+        tmem_alloc(smem_u32(&tmem_slot), 512);
+        tmem_relinquish();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+
+    // TMEM columns: T1 [0,128)  T2 of the even tiles [128,256)  ACC [256,384)  T2 of the odd tiles [384,512)
+    const uint32_t tmem = tmem_slot;
+    volatile int *abort_flag = &s_abort;
+    // item x of the launch (x counts halves of 256-row work items); false: it has no rows
+    auto fetch = [&](int x, DqItem &o) -> bool {
+        int item = x >> 1, h = 0;
+        if (ANCHOR) { h = p.h0 + item / p.n_items; item %= p.n_items; }
+        else item += s_lo;
+        const WorkItem w = p.items[item];
+        const int skip = (x & 1) * 128;
+        o.h = ANCHOR ? h : w.h;
+        o.first = w.first + skip;
+        o.rows = min(128, w.rows - skip);
+        o.nrng = w.nrng; o.ntiles = w.ntiles; o.rng_off = w.rng_off; o.t0 = w.t0; o.t1 = w.t1;
+        if (!ANCHOR && !index_ok((unsigned)w.h < (unsigned)p.H && w.rows > 0 && w.rows <= kQTileRows && w.first >= 0 &&
+                                 (size_t)w.first + w.rows <= p.cap_total && w.nrng == 1, p.status, IX_BWD_ITEM_FIELDS))
+            o.rows = 0;
+        return o.rows > 0;
+    };
+
+    if (warp < 8) {
+        // ------------------------------------------------------------ lane threads
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
+        const int r = threadIdx.x & 127;              // row of the item = TMEM lane
+        const int half = warp >> 2;
+        const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
+        const uint64_t c2 = pack2(p.scale_log2, p.scale_log2);
+        constexpr int NP = D / 8;
+        const int LB = (p.L + 127) >> 7;
+        uint4 *part16 = reinterpret_cast<uint4 *>(p.part);
+        int g = 0;                                    // tiles processed
+        bool ok = true;
+        for (int n = 0; ok; ++n) {
+            ok = mbar_wait(bar(X_FULL), n & 1, abort_flag, p.status, DW_XFULL);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            const int rows = s_item[n & 1].rows, h = s_item[n & 1].h, first = s_item[n & 1].first, n_tiles = s_item[n & 1].ntiles;
+            if (rows == 0) break;
+            TileIter it(p.rng + s_item[n & 1].rng_off, s_item[n & 1].nrng, s_item[n & 1].t0, s_item[n & 1].t1);
+            const float nlse = s_ld[n & 1][0][r], ndlt = s_ld[n & 1][1][r];
+            const uint64_t nlse2 = pack2(nlse, nlse), ndlt2 = pack2(ndlt, ndlt);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(X_EMPTY));
+            // the destination of this row's result, wanted at the end
+            int e = -1;
+            if (r < rows) e = ANCHOR ? first + r : p.qlist[(size_t)h * p.cap_total + first + r];
+            for (int jt = 0; jt < n_tiles; ++jt, ++g) {
+                const int st = g & 1;
+                int valid = 128, t0;
+                it.next(t0, valid);
+                ok = mbar_wait_spin(bar(T1_FULL), g & 1, abort_flag, p.status, DW_T1FULL);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_fence_after();
+                // ---- P = exp2(scale log2(e) S - lse log2(e)) from T1
+                const uint32_t t2c = st ? 384u : 128u;       // T2 (then dS) of this tile
+                float pv[64];
+                uint32_t sv[2][32];
+                tmem_ld32(tmem + lane_off + half * 32, sv[0]);
+                tmem_ld32(tmem + lane_off + (2 + half) * 32, sv[1]);
+                tmem_wait_ld();
+                tc_fence_before();
+                mbar_arrive(bar(T1_READ));                   // T1 may be overwritten
+#pragma unroll
+                for (int rd = 0; rd < 2; ++rd) {
+                    const int ch = rd * 2 + half;
+#pragma unroll
+                    for (int x = 0; x < 32; x += 2) {
+                        float p0, p1;
+                        unpack2(fma2(pack2(__uint_as_float(sv[rd][x]), __uint_as_float(sv[rd][x + 1])), c2, nlse2), p0, p1);
+                        pv[rd * 32 + x] = ex2(p0);
+                        pv[rd * 32 + x + 1] = ex2(p1);
+                    }
+                    if (valid < 128) {                       // keys past the end of the range
+#pragma unroll
+                        for (int x = 0; x < 32; ++x)
+                            if (ch * 32 + x >= valid) pv[rd * 32 + x] = 0.f;
+                    }
+                }
+                // ---- dS = P (dP - delta) from T2, written over T2 columns that have been read
+                ok = mbar_wait_spin(bar(T2_FULL + st), (g >> 1) & 1, abort_flag, p.status, DW_T2FULL);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_fence_after();
+                uint32_t dpv[2][32];
+                tmem_ld32(tmem + lane_off + t2c + half * 32, dpv[0]);
+                tmem_ld32(tmem + lane_off + t2c + (2 + half) * 32, dpv[1]);
+                tmem_wait_ld();
+                mbar_arrive(bar(RD2));                       // this thread's columns have been read
+#pragma unroll
+                for (int rd = 0; rd < 2; ++rd) {
+                    const int ch = rd * 2 + half;
+                    uint32_t uds[16];
+#pragma unroll
+                    for (int x = 0; x < 32; x += 2) {
+                        float a0, a1;
+                        unpack2(mul2(pack2(pv[rd * 32 + x], pv[rd * 32 + x + 1]),
+                                     add2(pack2(__uint_as_float(dpv[rd][x]), __uint_as_float(dpv[rd][x + 1])), ndlt2)), a0, a1);
+                        uds[x >> 1] = bf16x2(a0, a1);
+                    }
+                    if (rd == 0) {                           // the other thread of the lane has read the columns stored over
+                        ok = mbar_wait_spin(bar(RD2), g & 1, abort_flag, p.status, DW_READ);
+                        ok = __all_sync(0xffffffffu, ok);
+                    }
+                    if (ok) tmem_st16(tmem + lane_off + t2c + ch * 16, uds);
+                }
+                if (!ok) break;
+                tmem_wait_st();
+                tc_fence_before();
+                mbar_arrive(bar(DS_DONE + st));
+            }
+            if (!ok) break;
+            // ---- epilogue
+            ok = mbar_wait(bar(ACC_FULL), n & 1, abort_flag, p.status, DW_ACCFULL);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            uint32_t v[D / 64][32];
+#pragma unroll
+            for (int c = 0; c < D / 64; ++c) tmem_ld32(tmem + lane_off + 256 + (2 * c + half) * 32, v[c]);
+            tmem_wait_ld();
+            tc_fence_before();
+            mbar_arrive(bar(ACC_FREE));                      // the next item's dQ may be accumulated
+            if (e < 0) continue;
+            int qi = e, slot = 0;
+            if (!ANCHOR) {
+                qi = p.kdiv.query(e);
+                slot = e - qi * p.k;
+                if (!index_ok((unsigned)qi < (unsigned)p.L, p.status, IX_BWD_LIST_ENTRY) || (unsigned)qi >= (unsigned)p.L) continue;
+            }
+#pragma unroll 1
+            for (int c = 0; c < D / 64; ++c) {
+                const int ch = 2 * c + half;
+                float acc[32];
+#pragma unroll
+                for (int x = 0; x < 32; ++x) acc[x] = __uint_as_float(D == 64 || c == 0 ? v[0][x] : v[D / 64 - 1][x]) * p.scale;
+                if (ANCHOR) {
+                    // the routed partials of this query, four slots requested together; a slot is in use
+                    // if the forward left a finite log-sum-exp for it
+                    const float *pl = p.part_lse + part_lse_at(h, LB, p.k, qi, 0);      // slot s: pl[s * 128]
+#pragma unroll 1
+                    for (int s0 = 0; s0 < p.k; s0 += 4) {
+                        uint4 raw[4][4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            const bool used = s0 + u < p.k && pl[(s0 + u) * 128] != -INFINITY;
+#pragma unroll
+                            for (int q4 = 0; q4 < 4; q4 += 2) {
+                                raw[u][q4] = raw[u][q4 + 1] = make_uint4(0, 0, 0, 0);
+                                if (used) ld_cg_256(part16 + part_piece(h - p.h0, LB, p.k, NP, qi, s0 + u, ch * 4 + q4), raw[u][q4], raw[u][q4 + 1]);
+                            }
+                        }
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+#pragma unroll
+                            for (int q4 = 0; q4 < 4; ++q4) {
+                                const __nv_bfloat162 *b = reinterpret_cast<const __nv_bfloat162 *>(&raw[u][q4]);
+#pragma unroll
+                                for (int y = 0; y < 4; ++y) {
+                                    const float2 f = __bfloat1622float2(b[y]);
+                                    acc[q4 * 8 + 2 * y] += f.x;
+                                    acc[q4 * 8 + 2 * y + 1] += f.y;
+                                }
+                            }
+                    }
+                }
+                uint4 out[4];
+                uint32_t *o32 = reinterpret_cast<uint32_t *>(out);
+#pragma unroll
+                for (int x = 0; x < 16; ++x) o32[x] = bf16x2(acc[2 * x], acc[2 * x + 1]);
+                if (ANCHOR) {
+                    uint4 *dst = reinterpret_cast<uint4 *>(p.dQ + ((size_t)h * p.L + qi) * D + ch * 32);
+#pragma unroll
+                    for (int q4 = 0; q4 < 4; ++q4) dst[q4] = out[q4];
+                } else {                                     // whole 32-byte sectors (pairs of pieces)
+                    st_256(part16 + part_piece(h - p.h0, LB, p.k, NP, qi, slot, ch * 4), out[0], out[1]);
+                    st_256(part16 + part_piece(h - p.h0, LB, p.k, NP, qi, slot, ch * 4 + 2), out[2], out[3]);
+                }
+            }
+        }
+    } else if (warp == 8) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+        // ------------------------------------------------------------ TMA producer of the K and V tiles
+        if (lane == 0) {
+            prefetch_tensormap(&tmK);
+            prefetch_tensormap(&tmV);
+            int n_k = 0, n_v = 0, s3 = 0, ph3 = 0;           // K and V tiles issued; K stage and its phase
+            bool ok = true;
+            for (int x = blockIdx.x; ok && x < s_total; x += gridDim.x) {
+                DqItem w;
+                if (!fetch(x, w)) continue;
+                TileIter it(p.rng + w.rng_off, w.nrng, w.t0, w.t1);
+                int t0, valid;
+                while (it.next(t0, valid)) {
+                    const int s2 = n_v & 1;
+                    ok = mbar_wait(bar(K_EMPTY + s3), ph3 ^ 1, abort_flag, p.status, DW_YEMPTY);
+                    if (!ok) break;
+                    mbar_expect_tx(bar(K_FULL + s3), TILE_BYTES);
+#pragma unroll
+                    for (int sub = 0; sub < SUB; ++sub)
+                        tma_load_2d(sK + s3 * TILE_BYTES + sub * SUB_BYTES, &tmK, sub * 64, w.h * p.L + t0, bar(K_FULL + s3));
+                    ++n_k;
+                    ok = mbar_wait(bar(V_EMPTY + s2), ((n_v >> 1) & 1) ^ 1, abort_flag, p.status, DW_YEMPTY);
+                    if (!ok) break;
+                    mbar_expect_tx(bar(V_FULL + s2), TILE_BYTES);
+#pragma unroll
+                    for (int sub = 0; sub < SUB; ++sub)
+                        tma_load_2d(sV + s2 * TILE_BYTES + sub * SUB_BYTES, &tmV, sub * 64, w.h * p.L + t0, bar(V_FULL + s2));
+                    ++n_v;
+                    if (++s3 == kKStages) { s3 = 0; ph3 ^= 1; }
+                }
+            }
+            if (*abort_flag) {      // copies already issued must land before the shared memory is released
+                int dummy_flag = 0;
+                for (int b = 1; b <= kKStages; ++b)
+                    if (n_k - b >= 0) mbar_wait(bar(K_FULL + (n_k - b) % kKStages), ((n_k - b) / kKStages) & 1, &dummy_flag, p.status, DW_YFULL);
+                for (int b = 1; b <= kVStages; ++b)
+                    if (n_v - b >= 0) mbar_wait(bar(V_FULL + ((n_v - b) & 1)), ((n_v - b) >> 1) & 1, &dummy_flag, p.status, DW_YFULL);
+            }
+        }
+    } else if (warp < 12) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+        // ------------------------------------------------------------ row loaders.  The eight pieces of an item's rows - 32-row
+        // block b & 3 of Q (b < 4) or dO - are dealt to the three warps; who brings a block of Q also brings its lse and
+        // delta.  Everything an item needs is looked up before its buffers are free.
+        const int lw = warp - 9;
+        int n = 0;
+        bool ok = true;
+        int x = blockIdx.x;
+        for (bool more = true; ok && more; ++n) {
+            DqItem w = {};
+            more = false;
+            for (; x < s_total && !more; x += gridDim.x) more = fetch(x, w);
+            if (!more) w.rows = 0;
+            int q[3];
+            float lse[3], del[3];
+#pragma unroll
+            for (int y = 0; y < 3; ++y) {
+                const int b = lw + 3 * y, i = (b & 3) * 32 + lane;
+                q[y] = -1; lse[y] = INFINITY; del[y] = 0.f;
+                if (b < 8 && i < w.rows) {
+                    q[y] = w.first + i;
+                    if (!ANCHOR) {
+                        q[y] = p.kdiv.query(p.qlist[(size_t)w.h * p.cap_total + w.first + i]);
+                        if ((unsigned)q[y] >= (unsigned)p.L) q[y] = -1;      // never follow an entry that is not a row of this head
+                    }
+                    if (b < 4 && q[y] >= 0) {
+                        lse[y] = p.lse[(size_t)w.h * p.L + q[y]];
+                        del[y] = p.delta[(size_t)w.h * p.L + q[y]];
+                    }
+                }
+            }
+            if (n > 0) {
+                ok = mbar_wait(bar(X_EMPTY), (n - 1) & 1, abort_flag, p.status, DW_XEMPTY);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+            }
+            if (more) {
+#pragma unroll
+                for (int y = 0; y < 3; ++y) {
+                    const int b = lw + 3 * y;
+                    if (b >= 8) break;
+                    const __nv_bfloat16 *src = (b < 4 ? p.Q : p.dO) + (size_t)w.h * p.L * D;
+                    const uint32_t dst = sX + (b >> 2) * TILE_BYTES;
+                    constexpr int RP = 32 / CH;                // rows per instruction
+                    const int c16 = lane % CH;
+#pragma unroll
+                    for (int rb = 0; rb < 32; rb += RP) {
+                        const int rl = rb + lane / CH, qq = __shfl_sync(0xffffffffu, q[y], rl);
+                        cp_async16(dst + (c16 >> 3) * SUB_BYTES + sw128_offset((b & 3) * 32 + rl, c16 & 7), src + (size_t)max(qq, 0) * D + c16 * 8,
+                                   qq >= 0 ? 16u : 0u);
+                    }
+                    if (b < 4) {                               // a row without a query gets lse = +inf: P and dS are zero
+                        s_ld[n & 1][0][b * 32 + lane] = lse[y] * -1.4426950408889634f;
+                        s_ld[n & 1][1][b * 32 + lane] = -del[y];
+                    }
+                }
+            }
+            if (lw == 0 && lane == 0) s_item[n & 1] = w;
+            cp_async_wait_all();
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(X_FULL));
+        }
+        cp_async_wait_all();
+    } else {
+        // ------------------------------------------------------------ MMA issuers (a warp stays together, one lane of it issues)
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+        if (warp <= 13) {
+            constexpr uint32_t IDESC_T = idesc_bf16_f32(128, 128, 0, 0);      // T = X Y^T, both K-major
+            constexpr uint32_t IDESC_ACC = idesc_bf16_f32(128, D, 0, 1);      // ACC += dS K, K MN-major
+            constexpr uint32_t STAGE = TILE_BYTES >> 4;
+            auto lo = [](uint64_t d) { return (uint32_t)d; };
+            auto hi = [](uint64_t d) { return (uint32_t)(d >> 32); };
+            bool ok = true;
+            auto wait = [&](int b, int parity, int code) { ok = ok && __all_sync(0xffffffffu, mbar_wait_spin(bar(b), parity, abort_flag, p.status, code)); };
+            int g = 0, s3 = 0, ph3 = 0;                        // tile, its K stage and phase
+            if (uniform(warp) == 12) {
+                const uint64_t x1 = smem_desc_sw128(sX, 16, 1024), kk = smem_desc_sw128(sK, 16, 1024);
+                for (int n = 0; ok; ++n) {
+                    wait(X_FULL, n & 1, DW_XFULL);
+                    if (!ok) break;
+                    const int n_tiles = uniform(s_item[n & 1].rows) ? uniform(s_item[n & 1].ntiles) : 0;
+                    if (n_tiles == 0) break;
+                    for (int j = 0; ok && j < n_tiles; ++j, ++g) {
+                        wait(K_FULL + s3, ph3, DW_YFULL);
+                        if (g > 0) wait(T1_READ, (g - 1) & 1, DW_READ);
+                        if (!ok) break;
+                        tc_fence_after();
+#pragma unroll
+                        for (int ks = 0; ks < D / 16; ++ks) {
+                            const uint32_t o = ((ks >> 2) * SUB_BYTES + (ks & 3) * 32) >> 4;
+                            mma_ss_elect(tmem, lo(x1) + o, hi(x1), lo(kk) + s3 * STAGE + o, hi(kk), IDESC_T, ks > 0);
+                        }
+                        tc_commit_elect(bar(T1_FULL));
+                        if (j + 1 == n_tiles) tc_commit_elect(bar(X_EMPTY));
+                        if (++s3 == kKStages) { s3 = 0; ph3 ^= 1; }
+                    }
+                }
+            } else {
+                const uint64_t x2 = smem_desc_sw128(sX + TILE_BYTES, 16, 1024), vv = smem_desc_sw128(sV, 16, 1024);
+                const uint64_t km = smem_desc_sw128(sK, SUB_BYTES, 1024);
+                // T2(t) = dO V(t)^T for tile t of the launch; `last`: it is the item's last
+                auto t2 = [&](int t, bool last) {
+                    const int s2 = t & 1;
+                    wait(V_FULL + s2, (t >> 1) & 1, DW_YFULL);
+                    if (!ok) return;
+                    tc_fence_after();
+                    const uint32_t d = tmem + (s2 ? 384u : 128u);
+#pragma unroll
+                    for (int ks = 0; ks < D / 16; ++ks) {
+                        const uint32_t o = ((ks >> 2) * SUB_BYTES + (ks & 3) * 32) >> 4;
+                        mma_ss_elect(d, lo(x2) + o, hi(x2), lo(vv) + s2 * STAGE + o, hi(vv), IDESC_T, ks > 0);
+                    }
+                    tc_commit_elect(bar(T2_FULL + s2));
+                    tc_commit_elect(bar(V_EMPTY + s2));
+                    if (last) tc_commit_elect(bar(X_EMPTY));
+                };
+                for (int n = 0; ok; ++n) {
+                    wait(X_FULL, n & 1, DW_XFULL);
+                    if (!ok) break;
+                    const int n_tiles = uniform(s_item[n & 1].rows) ? uniform(s_item[n & 1].ntiles) : 0;
+                    if (n_tiles == 0) break;
+                    t2(g, n_tiles == 1);
+                    if (n_tiles > 1) t2(g + 1, n_tiles == 2);
+                    for (int j = 0; ok && j < n_tiles; ++j, ++g) {
+                        wait(DS_DONE + (g & 1), (g >> 1) & 1, DW_DSDONE);
+                        if (j == 0 && n > 0) wait(ACC_FREE, (n - 1) & 1, DW_ACCFREE);      // the previous item's dQ has been read
+                        if (!ok) break;
+                        tc_fence_after();
+                        const uint32_t ds = tmem + ((g & 1) ? 384u : 128u);
+#pragma unroll
+                        for (int ks = 0; ks < 8; ++ks)
+                            mma_ts_elect(tmem + 256, ds + ks * 8, lo(km) + s3 * STAGE + ks * (2048 >> 4), hi(km), IDESC_ACC, j > 0 || ks > 0);
+                        tc_commit_elect(bar(K_EMPTY + s3));
+                        if (++s3 == kKStages) s3 = 0;
+                        if (j + 2 < n_tiles) t2(g + 2, j + 3 == n_tiles);
+                    }
+                    if (ok) tc_commit_elect(bar(ACC_FULL));
+                }
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 8) tmem_dealloc(tmem, 512);
+}
+
+template <int D>
+static int dq_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat16 *K, const __nv_bfloat16 *V, const float *lse,
+                   const float *delta, const __nv_bfloat16 *dO, __nv_bfloat16 *dQ, void *ws, cudaStream_t s) {
+    CUtensorMap tmK, tmV;
+    if (int r = make_tmap_2d_bf16(&tmK, K, (uint64_t)p->H * p->L, D, 128)) return r;
+    if (int r = make_tmap_2d_bf16(&tmV, V, (uint64_t)p->H * p->L, D, 128)) return r;
+    DqParams a;
+    a.Q = Q; a.dO = dO; a.lse = lse; a.delta = delta; a.dQ = dQ;
+    a.part = ws_ptr<__nv_bfloat16>(ws, p->ws.part_o);      // the forward's partial outputs are no longer needed
+    a.part_lse = ws_ptr<float>(ws, p->ws.part_lse);
+    a.qlist = ws_ptr<int32_t>(ws, p->ws.qlist);
+    a.cap_total = (size_t)p->cap_off[p->C];
+    a.status = ws_ptr<int>(ws, p->ws.status);
+    a.H = p->H; a.L = p->L; a.k = p->k; a.kdiv = SlotDiv::of(p->k);
+    a.n_items = (int)p->qitems.size();
+    a.scale = p->scale; a.scale_log2 = p->scale * 1.4426950408889634f;
+    a.cookie = p->cookie;
+    // seven tiles (Q, dO, three K and two V stages; always the d = 128 footprint, so that CTAs, which each take all of the
+    // tensor memory, never share an SM): all an SM has, so the request is what the static variables leave of the limit
+    const size_t tiles = (size_t)(2 + kKStages + kVStages) * 128 * 128 * 2;
+    size_t smem[2];
+    int optin = 0;
+    MOC_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
+    const void *fn[2] = {(const void *)attend_dq_tc_kernel<D, false>, (const void *)attend_dq_tc_kernel<D, true>};
+    for (int m = 0; m < 2; ++m) {
+        cudaFuncAttributes fa;
+        MOC_CUDA_TRY(cudaFuncGetAttributes(&fa, fn[m]));
+        smem[m] = std::min(tiles + 1024, (size_t)optin - fa.sharedSizeBytes);
+        if (smem[m] < tiles) return MOC_ERR_SHAPE;
+        MOC_CUDA_TRY(cudaFuncSetAttribute(fn[m], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem[m]));
+    }
+    const int *tile_off = ws_ptr<int>(ws, p->ws.tile_off);
+    for (int h0 = 0; h0 < p->H; h0 += p->heads_per_group) {
+        const int hg = std::min(p->heads_per_group, p->H - h0);
+        a.h0 = h0; a.hg = hg;
+        if (p->k > 0) {
+            a.rng = p->d_chunk_rng;
+            a.items = ws_ptr<WorkItem>(ws, p->ws.rtiles);
+            a.item_lo = tile_off + (size_t)h0 * p->C;
+            a.item_hi = tile_off + (size_t)(h0 + hg) * p->C;
+            const long long most = 2LL * hg * (((long long)p->L * p->k + kQTileRows - 1) / kQTileRows + p->C);
+            attend_dq_tc_kernel<D, false><<<(unsigned)std::min<long long>(p->n_sm, most), kDqThreads, smem[0], s>>>(tmK, tmV, a);
+            MOC_LAUNCH_CHECK();
+        }
+        a.rng = p->d_anc_rng;
+        a.items = p->d_qitems;
+        a.item_lo = a.item_hi = nullptr;
+        const long long n_anc = 2LL * a.n_items * hg;
+        attend_dq_tc_kernel<D, true><<<(unsigned)std::min<long long>(p->n_sm, n_anc), kDqThreads, smem[1], s>>>(tmK, tmV, a);
+        MOC_LAUNCH_CHECK();
+    }
+    return MOC_OK;
+}
+
+int launch_dq_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat16 *K, const __nv_bfloat16 *V, const float *lse,
+                 const float *delta, const __nv_bfloat16 *dO, __nv_bfloat16 *dQ, void *ws, cudaStream_t s) {
+    return p->d == 128 ? dq_tc_d<128>(p, Q, K, V, lse, delta, dO, dQ, ws, s) : dq_tc_d<64>(p, Q, K, V, lse, delta, dO, dQ, ws, s);
+}
+
+}  // namespace moc

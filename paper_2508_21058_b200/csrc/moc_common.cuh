@@ -192,6 +192,8 @@ struct TileIter {
     const KeyRange *rng;
     int n, ri, t, end;      // the current range's end is kept: one load per range, not per tile
     __device__ TileIter(const KeyRange *r, int n_) : rng(r), n(n_), ri(0), t(n_ > 0 ? r[0].t0 : 0), end(n_ > 0 ? r[0].t1 : 0) {}
+    // the first range given by value
+    __device__ TileIter(const KeyRange *r, int n_, int t0, int t1) : rng(r), n(n_), ri(0), t(t0), end(t1) {}
     __device__ bool next(int &t0, int &valid) {
         if (ri >= n) return false;
         t0 = t;
@@ -224,6 +226,8 @@ int launch_attend_bwd_scalar(const moc_plan *p, const __nv_bfloat16 *Q, const __
 int launch_attend_bwd_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat16 *K, const __nv_bfloat16 *V,
                          const __nv_bfloat16 *O, const float *lse, const __nv_bfloat16 *dO, const int32_t *sel,
                          __nv_bfloat16 *dQ, __nv_bfloat16 *dK, __nv_bfloat16 *dV, void *ws, cudaStream_t s);
+int launch_dq_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat16 *K, const __nv_bfloat16 *V, const float *lse,
+                 const float *delta, const __nv_bfloat16 *dO, __nv_bfloat16 *dQ, void *ws, cudaStream_t s);
 int launch_delta(const moc_plan *p, const __nv_bfloat16 *O, const __nv_bfloat16 *dO, float *delta, cudaStream_t s);
 int launch_attend_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat16 *K, const __nv_bfloat16 *V,
                      const int32_t *sel, __nv_bfloat16 *O, float *lse, void *ws, cudaStream_t s);
