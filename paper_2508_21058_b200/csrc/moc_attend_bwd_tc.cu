@@ -1,28 +1,21 @@
-// Tensor-core backward of the sparse attention (selection held constant): dQ, dK, dV from
-// Q, K, V, dO, the forward's log-sum-exp and delta_i = sum_x dO_ix O_ix.
+// Tensor-core backward of the sparse attention (selection held constant): dK and dV, and the launch of the whole backward
+// (dQ: moc_attend_dq_tc.cu; delta_i = sum_x dO_ix O_ix: moc_attend_scalar.cu).
 //
 // For a selected (query i, key t) pair:  P = exp(scale q.k - lse_i),  dP = dO_i . v_t,
-// dS = P (dP - delta_i);  dV_t += P dO_i,  dK_t += scale dS q_i,  dQ_i += scale dS k_t.
+// dS = P (dP - delta_i);  dV_t += P dO_i,  dK_t += scale dS q_i.
 //
-// One kernel, three modes, one tile engine.  A CTA holds a STATIONARY pair of 128-row tiles
-// (X1, X2) in shared memory and streams pairs of 128-row tiles (Y1, Y2) through three and two stages:
-//     T1 = X1 Y1^T,  T2 = X2 Y2^T        (both operands from shared memory, into TMEM)
+// Key stationary: a CTA holds 128 keys of a chunk, X = (K, V), and streams Y = (Q, dO), 128 rows at a time, of every query
+// that attends to the chunk - the query rows of the chunks that have it as an anchor, then the chunk's routed query list -
+// through rings of three and two stages:
+//     T1 = K Q^T,  T2 = V dO^T          (both operands from shared memory, into TMEM)
 //     threads (two per TMEM lane) turn T1 into P, then (P, T2) into dS, written back to TMEM as bf16
-//     ACC1 += dS Y1,  ACC2 += P Y2       (A from TMEM, B the streamed tile as an MN-major operand)
-//   dQ modes (query stationary, the forward's work items, 128 rows per CTA):  X = (Q, dO) rows of
-//     the item, Y = (K, V) tiles of its key ranges by TMA; lse and delta belong to the lane;
-//     ACC1 is the item's dQ.  The routed mode leaves one partial per (query, slot) in the
-//     workspace; the anchor mode adds them to its own part and writes dQ.
-//   dK/dV mode (key stationary, one CTA per 128 keys of a chunk):  X = (K, V) rows of the key
-//     tile by TMA, Y = (Q, dO) rows of every query that attends to the chunk - the query rows of
-//     the chunks that have it as an anchor, then the chunk's routed query list - brought by four
-//     producer warps, Q and dO each through a ring of its own; lse and delta belong to the column; ACC1 is
-//     dK, ACC2 is dV.  Each key tile is owned by one CTA: no atomics, no partial sums.
-// The tensor pipe and the lanes overlap across tiles.  dK/dV: the issue order is ACC2(j), T1(j+1),
-// ACC1(j), T2(j+1), so that while the lanes form P(j+1) the pipe runs ACC1(j) and T2(j+1), and T1 / T2
-// are rewritten only after the contraction that reads the P / dS stored over them; ACC2(j) starts on the
-// first half of P(j) while the lanes form the second.  dQ: no ACC2, so its columns serve as a second T2:
-// T1(j+1) and T2(j+1) are issued once the lanes have read T1(j) and run while they form dS(j).
+//     ACC1 += dS Q,  ACC2 += P dO       (A from TMEM, the streamed tile as an MN-major operand)
+// lse and delta belong to the column; ACC1 is dK, ACC2 is dV.  Each key tile is owned by one CTA: no atomics, no partial
+// sums.  Issue order: ACC2(j), T1(j+1), ACC1(j), T2(j+1), so that while the lanes form P(j+1) the pipe runs ACC1(j) and
+// T2(j+1), and T1 / T2 are rewritten only after the contraction that reads the P / dS stored over them; ACC2(j) starts on the
+// first half of P(j) while the lanes form the second.
+// A tile takes 3300 cycles (33k-token clip) for 2048 cycles of MMAs at the pipe's best rate: P, dS and the wait for T1(j+1)
+// between them are one chain per tile (two tiles in flight would need 1024 columns of tensor memory).
 // 16 warps: 0-7 the lane threads (two per TMEM lane), 8-11 the producers, 12 and 13 the MMA issuers,
 // 14-15 idle (they complete the fourth warpgroup; the lanes take the registers the others give up).  Every mbarrier wait is
 // bounded; a wait that runs out flags the workspace status word and the CTA drains and leaves.
@@ -35,21 +28,14 @@ namespace moc {
 
 using namespace tc;
 
-enum BwdMode { DQ_ROUTED = 0, DQ_ANCHOR = 1, DKV = 2 };
 enum BwdWait { BW_XFULL = 64, BW_YFULL, BW_YEMPTY, BW_T1FULL, BW_T2FULL, BW_PDONE, BW_DSDONE, BW_ACCFULL, BW_SMEM, BW_READ };
 
 struct BwdParams {
     const __nv_bfloat16 *Q, *K, *V, *dO;
     const float *lse, *delta;
-    __nv_bfloat16 *dQ, *dK, *dV;
-    __nv_bfloat16 *part;          // [Hg][L][k][d] routed dQ partials of the group of heads in flight
-    const float *part_lse;        // the forward's routed log-sum-exps (part_lse_at): -inf marks an empty slot
-    const KeyRange *rng;          // dQ modes: key ranges the items index
-    const WorkItem *items;
-    const int *item_lo_dev, *item_hi_dev;   // routed mode: the group's item range [*lo, *hi) on the device
-    int h0;                       // first head of the group in flight
+    __nv_bfloat16 *dK, *dV;
     uint32_t cookie;              // what the workspace's status area must hold
-    const KTile *ktiles;          // dK/dV mode
+    const KTile *ktiles;
     int n_ktiles, n_long;         // tiles per head, and how many of them come first for every head
     const int32_t *off, *ranc_off, *ranc, *cap_off;
     const int *cnt;
@@ -65,12 +51,12 @@ constexpr int kY1Stages = 3, kY2Stages = 2;   // stages of the streamed tiles Y1
 constexpr int kBwdThreads = 512;
 constexpr float kLog2e = 1.4426950408889634f;
 
-template <int D, int MODE>
-__global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __grid_constant__ CUtensorMap tmK,
-                                                                       const __grid_constant__ CUtensorMap tmV,
-                                                                       const __grid_constant__ CUtensorMap tmQ,
-                                                                       const __grid_constant__ CUtensorMap tmdO,
-                                                                       const BwdParams p) {
+template <int D>
+__global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __grid_constant__ CUtensorMap tmK,
+                                                                      const __grid_constant__ CUtensorMap tmV,
+                                                                      const __grid_constant__ CUtensorMap tmQ,
+                                                                      const __grid_constant__ CUtensorMap tmdO,
+                                                                      const BwdParams p) {
     constexpr int TILE_BYTES = 128 * D * 2;
     constexpr int SUB = D / 64;
     constexpr int SUB_BYTES = 128 * 128;
@@ -80,15 +66,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
     __shared__ __align__(8) uint64_t bars[23];
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort;
-    __shared__ int w_valid, w_h, w_rows, w_first, w_nrng, w_ntiles, w_chunk, w_t0;
-    __shared__ const KeyRange *w_rng;
-    // dK/dV mode: per streamed query, (-lse * log2(e), -delta), for tiles j and j + 1;
-    // dQ modes: the first 128 words hold the item's query rows while they are staged
+    __shared__ int w_valid, w_h, w_rows, w_ntiles, w_chunk, w_t0;
+    // per streamed query, (-lse * log2(e), -delta), for tiles j and j + 1
     __shared__ __align__(16) float s_ld[2][2][128];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
-    uint8_t *gbase = smem_raw + (sbase - smem_u32(smem_raw));
     // shared tiles: X1 X2 | Y1 stages | Y2 stages
     const uint32_t sX = sbase, sY1 = sbase + 2 * TILE_BYTES, sY2 = sbase + (2 + kY1Stages) * TILE_BYTES;
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
@@ -109,61 +92,36 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
             if (atomicCAS(p.status, 0, MOC_ERR_TIMEOUT) == 0) p.status[1] = BW_SMEM;
             valid = 0;
         }
-        if (MODE != DKV) {
-            int item = blockIdx.x >> 1;
-            const int half = blockIdx.x & 1;
-            if (MODE == DQ_ROUTED && valid) {
-                item += *p.item_lo_dev;
-                if (item >= *p.item_hi_dev) valid = 0;
-            }
-            WorkItem w = {};
-            if (valid) {
-                w = p.items[item];
-                if (MODE == DQ_ROUTED && !index_ok((unsigned)w.h < (unsigned)p.H && w.rows > 0 && w.rows <= kQTileRows && w.first >= 0 &&
-                                                   (size_t)w.first + w.rows <= p.cap_total && w.nrng == 1, p.status, IX_BWD_ITEM_FIELDS))
-                    valid = 0;
-            }
-            if (valid) {
-                w_h = MODE == DQ_ROUTED ? w.h : p.h0 + (int)blockIdx.y;
-                w_first = w.first + half * 128;
-                w_rows = min(128, w.rows - half * 128);
-                w_rng = p.rng + w.rng_off;
-                w_nrng = w.nrng;
-                w_ntiles = w.ntiles;
-                if (w_rows <= 0) valid = 0;
-            }
-        } else {
-            // block order: the long key tiles of every head, then the others head by head (tiles of one chunk next
-            // to each other: they stream the same query rows)
-            const int n_long_all = p.n_long * p.H;
-            int b = blockIdx.x, hh, ti;
-            if (b < n_long_all) { hh = b / p.n_long; ti = b - hh * p.n_long; }
-            else { b -= n_long_all; const int n_rest = p.n_ktiles - p.n_long; hh = b / n_rest; ti = p.n_long + b - hh * n_rest; }
-            const KTile kt = p.ktiles[ti];
-            w_h = hh;
-            w_chunk = kt.chunk;
-            w_t0 = kt.t0;
-            w_rows = kt.valid;
-            // query tiles: merged row ranges of the chunks that have this chunk as an anchor, then the routed list
-            int nt = 0;
-            const int a0 = p.ranc_off[kt.chunk], a1 = p.ranc_off[kt.chunk + 1];
-            for (int a = a0; a < a1;) {
-                int qc = p.ranc[a], r0 = p.off[qc], r1 = p.off[qc + 1];
-                for (++a; a < a1 && p.ranc[a] == qc + 1; ++a) { qc = p.ranc[a]; r1 = p.off[qc + 1]; }
-                nt += (r1 - r0 + 127) / 128;
-            }
-            nt += (p.cnt[w_h * p.C + kt.chunk] + 127) / 128;
-            w_ntiles = nt;
+        // block order: the long key tiles of every head, then the others head by head (tiles of one chunk next
+        // to each other: they stream the same query rows)
+        const int n_long_all = p.n_long * p.H;
+        int b = blockIdx.x, hh, ti;
+        if (b < n_long_all) { hh = b / p.n_long; ti = b - hh * p.n_long; }
+        else { b -= n_long_all; const int n_rest = p.n_ktiles - p.n_long; hh = b / n_rest; ti = p.n_long + b - hh * n_rest; }
+        const KTile kt = p.ktiles[ti];
+        w_h = hh;
+        w_chunk = kt.chunk;
+        w_t0 = kt.t0;
+        w_rows = kt.valid;
+        // query tiles: merged row ranges of the chunks that have this chunk as an anchor, then the routed list
+        int nt = 0;
+        const int a0 = p.ranc_off[kt.chunk], a1 = p.ranc_off[kt.chunk + 1];
+        for (int a = a0; a < a1;) {
+            int qc = p.ranc[a], r0 = p.off[qc], r1 = p.off[qc + 1];
+            for (++a; a < a1 && p.ranc[a] == qc + 1; ++a) { qc = p.ranc[a]; r1 = p.off[qc + 1]; }
+            nt += (r1 - r0 + 127) / 128;
         }
+        nt += (p.cnt[w_h * p.C + kt.chunk] + 127) / 128;
+        w_ntiles = nt;
         w_valid = valid;
-        mbar_init(bar(X_FULL), MODE == DKV ? 1 : 256);
+        mbar_init(bar(X_FULL), 1);
         for (int t = 0; t < kY1Stages; ++t) {
-            mbar_init(bar(Y1_FULL + t), MODE == DKV ? 2 : 1);       // dK/dV: the ring's two producer warps
+            mbar_init(bar(Y1_FULL + t), 2);       // the ring's two producer warps
             mbar_init(bar(Y1_EMPTY + t), 1);
         }
         for (int t = 0; t < kY2Stages; ++t) {
-            mbar_init(bar(Y2_FULL + t), MODE == DKV ? 2 : 1);
-            mbar_init(bar(Y2_EMPTY + t), MODE == DKV ? 2 : 1);     // dK/dV: T2 and ACC2 both read the stage
+            mbar_init(bar(Y2_FULL + t), 2);
+            mbar_init(bar(Y2_EMPTY + t), 2);      // T2 and ACC2 both read the stage
             mbar_init(bar(T1_FULL + t), 1);
             mbar_init(bar(T2_FULL + t), 1);
             mbar_init(bar(DS_DONE + t), 256);
@@ -186,8 +144,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
     __syncthreads();
     tc_fence_after();
 
-    // TMEM columns: T1 [0,128)  T2 [128,256)  ACC1 [256,384)  ACC2 [384,512); the dQ modes have no ACC2
-    // and use its columns as a second T2, for the odd tiles
+    // TMEM columns: T1 [0,128)  T2 [128,256)  ACC1 [256,384)  ACC2 [384,512)
     const uint32_t tmem = tmem_slot;
     const int h = w_h, rows = w_rows, n_tiles = w_ntiles;
     volatile int *abort_flag = &s_abort;
@@ -201,86 +158,35 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
         const int r = threadIdx.x & 127;              // row of the stationary tile = TMEM lane
         const int half = warp >> 2;
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
-        int qi = -1, slot = 0;
-        float lse2 = INFINITY, dlt = 0.f;             // dQ modes: this lane's query
-        if (MODE != DKV) {
-            if (r < rows) {
-                if (MODE == DQ_ROUTED) {
-                    const int e = p.qlist[(size_t)h * p.cap_total + w_first + r];
-                    qi = p.kdiv.query(e);
-                    slot = e - qi * p.k;
-                    (void)index_ok(e >= 0 && qi < p.L, p.status, IX_BWD_LIST_ENTRY);
-                    if ((unsigned)qi >= (unsigned)p.L) qi = -1;      // never follow an entry that is not a row of this head
-                } else {
-                    qi = w_first + r;
-                }
-                if (qi >= 0) {
-                    lse2 = p.lse[(size_t)h * p.L + qi] * kLog2e;
-                    dlt = p.delta[(size_t)h * p.L + qi];
-                }
-            }
-            // stage the item's rows, one half Q and the other dO: consecutive threads take consecutive 16-byte pieces
-            int *s_row = reinterpret_cast<int *>(&s_ld[0][0][0]);
-            if (half == 0) s_row[r] = qi;
-            asm volatile("bar.sync 1, 256;" ::: "memory");
-            constexpr int RP = 128 / CH;
-            const int c16 = r % CH;
-            {
-                const __nv_bfloat16 *src = half ? p.dO : p.Q;
-                uint8_t *dst = gbase + half * TILE_BYTES + (c16 >> 3) * SUB_BYTES;
-                uint4 v[CH];
-#pragma unroll
-                for (int ps = 0; ps < CH; ++ps) {
-                    const int rr = ps * RP + r / CH, q = s_row[rr];
-                    v[ps] = make_uint4(0, 0, 0, 0);
-                    if (q >= 0) v[ps] = __ldg(reinterpret_cast<const uint4 *>(src + ((size_t)h * p.L + q) * D) + c16);
-                }
-#pragma unroll
-                for (int ps = 0; ps < CH; ++ps) *reinterpret_cast<uint4 *>(dst + sw128_offset(ps * RP + r / CH, c16 & 7)) = v[ps];
-            }
-            fence_proxy_async_smem();
-            mbar_arrive(bar(X_FULL));
-        }
-        const uint64_t c2 = pack2(p.scale_log2, p.scale_log2), nlse2 = pack2(-lse2, -lse2), ndlt2 = pack2(-dlt, -dlt);
-        TileIter it(w_rng, MODE == DKV ? 0 : w_nrng);
+        const uint64_t c2 = pack2(p.scale_log2, p.scale_log2);
         bool ok = true;
         int s3 = 0, ph3 = 0;                          // Y1 stage of tile jt and its phase
         for (int jt = 0; jt < n_tiles; ++jt) {
             const int st = jt & 1;
-            int valid = 128, t0;
-            if (MODE != DKV) it.next(t0, valid);
             ok = mbar_wait_spin(bar(T1_FULL + st), (jt >> 1) & 1, abort_flag, p.status, BW_T1FULL);
-            if (MODE == DKV) ok = ok && mbar_wait(bar(Y1_FULL + s3), ph3, abort_flag, p.status, BW_YFULL);
+            ok = ok && mbar_wait(bar(Y1_FULL + s3), ph3, abort_flag, p.status, BW_YFULL);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
             // ---- P = exp2(scale log2(e) S - lse log2(e)) from T1
-            const uint32_t t2c = (MODE != DKV && st) ? 384u : 128u;       // T2 (then dS) of this tile
+            constexpr uint32_t t2c = 128u;                // T2, then dS
             float pv[64];
             uint32_t sv[2][32];
             tmem_ld32(tmem + lane_off + half * 32, sv[0]);
             tmem_ld32(tmem + lane_off + (2 + half) * 32, sv[1]);
             tmem_wait_ld();
-            if (MODE == DKV) {
-                // P goes over T1 columns that the other thread of the lane reads; that read is announced here and waited
-                // for (bounded, like every wait) just before the first store
-                mbar_arrive(bar(RD1));
-            } else {                                                      // T1 has been read and may be overwritten
-                tc_fence_before();
-                mbar_arrive(bar(P_DONE));
-            }
+            // P goes over T1 columns that the other thread of the lane reads; that read is announced here and waited
+            // for (bounded, like every wait) just before the first store
+            mbar_arrive(bar(RD1));
 #pragma unroll
             for (int rd = 0; rd < 2; ++rd) {
                 const int ch = rd * 2 + half;
                 const uint32_t (&s)[32] = sv[rd];
-                // two columns per packed instruction; in dK/dV mode four columns' (negated) lse per shared-memory load
+                // two columns per packed instruction; four columns' (negated) lse per shared-memory load
 #pragma unroll
                 for (int x = 0; x < 32; x += 4) {
-                    uint64_t nl[2] = {nlse2, nlse2};
-                    if (MODE == DKV) {
-                        const ulonglong2 l = *reinterpret_cast<const ulonglong2 *>(&s_ld[st][0][ch * 32 + x]);
-                        nl[0] = l.x; nl[1] = l.y;
-                    }
+                    const ulonglong2 l = *reinterpret_cast<const ulonglong2 *>(&s_ld[st][0][ch * 32 + x]);
+                    const uint64_t nl[2] = {l.x, l.y};
 #pragma unroll
                     for (int y = 0; y < 2; ++y) {
                         float p0, p1;
@@ -289,12 +195,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                         pv[rd * 32 + x + 2 * y + 1] = ex2(p1);
                     }
                 }
-                if (MODE != DKV && valid < 128) {               // keys past the end of the range
-#pragma unroll
-                    for (int x = 0; x < 32; ++x)
-                        if (ch * 32 + x >= valid) pv[rd * 32 + x] = 0.f;
-                }
-                if (MODE == DKV) {
+                {
                     uint32_t ups[16];
 #pragma unroll
                     for (int x = 0; x < 16; ++x) ups[x] = bf16x2(pv[rd * 32 + 2 * x], pv[rd * 32 + 2 * x + 1]);
@@ -328,11 +229,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                 uint32_t uds[16];
 #pragma unroll
                 for (int x = 0; x < 32; x += 4) {
-                    uint64_t nd[2] = {ndlt2, ndlt2};
-                    if (MODE == DKV) {
-                        const ulonglong2 d = *reinterpret_cast<const ulonglong2 *>(&s_ld[st][1][ch * 32 + x]);
-                        nd[0] = d.x; nd[1] = d.y;
-                    }
+                    const ulonglong2 d = *reinterpret_cast<const ulonglong2 *>(&s_ld[st][1][ch * 32 + x]);
+                    const uint64_t nd[2] = {d.x, d.y};
 #pragma unroll
                     for (int y = 0; y < 2; ++y) {
                         float a0, a1;
@@ -380,238 +278,155 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                         reinterpret_cast<uint4 *>(dst)[q4] = out;
                     }
                 };
-                // the routed dQ partials use the forward's layout of routed partials: query-innermost pieces
-                constexpr int NP = D / 8;
-                const int LB = (p.L + 127) >> 7;
-                uint4 *part16 = reinterpret_cast<uint4 *>(p.part);
-                if (MODE == DQ_ROUTED) {
-                    if (qi >= 0) {
-                        uint4 out[4];
+                if (r < rows) store_row(p.dK + ((size_t)h * p.L + w_t0 + r) * D + ch * 32);
+                // dV = ACC2, not scaled
+                __syncwarp();
+                tmem_ld32(tmem + lane_off + 384 + ch * 32, v);
+                tmem_wait_ld();
 #pragma unroll
-                        for (int q4 = 0; q4 < 4; ++q4) {
-                            out[q4].x = bf16x2(acc[q4 * 8 + 0], acc[q4 * 8 + 1]);
-                            out[q4].y = bf16x2(acc[q4 * 8 + 2], acc[q4 * 8 + 3]);
-                            out[q4].z = bf16x2(acc[q4 * 8 + 4], acc[q4 * 8 + 5]);
-                            out[q4].w = bf16x2(acc[q4 * 8 + 6], acc[q4 * 8 + 7]);
-                        }
-                        // whole 32-byte sectors (pairs of pieces)
-                        st_256(part16 + part_piece(h - p.h0, LB, p.k, NP, qi, slot, ch * 4), out[0], out[1]);
-                        st_256(part16 + part_piece(h - p.h0, LB, p.k, NP, qi, slot, ch * 4 + 2), out[2], out[3]);
-                    }
-                } else if (MODE == DQ_ANCHOR) {
-                    if (qi >= 0) {
-                        // the routed partials of this query, four slots requested together; a slot is in use
-                        // if the forward left a finite log-sum-exp for it
-                        const float *pl = p.part_lse + part_lse_at(h, LB, p.k, qi, 0);      // slot s: pl[s * 128]
-                        for (int s0 = 0; s0 < p.k; s0 += 4) {
-                            uint4 raw[4][4];
-#pragma unroll
-                            for (int u = 0; u < 4; ++u) {
-                                const bool used = s0 + u < p.k && pl[(s0 + u) * 128] != -INFINITY;
-#pragma unroll
-                                for (int q4 = 0; q4 < 4; q4 += 2) {
-                                    raw[u][q4] = raw[u][q4 + 1] = make_uint4(0, 0, 0, 0);
-                                    if (used) ld_cg_256(part16 + part_piece(h - p.h0, LB, p.k, NP, qi, s0 + u, ch * 4 + q4), raw[u][q4], raw[u][q4 + 1]);
-                                }
-                            }
-#pragma unroll
-                            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                                for (int q4 = 0; q4 < 4; ++q4) {
-                                    const __nv_bfloat162 *b = reinterpret_cast<const __nv_bfloat162 *>(&raw[u][q4]);
-#pragma unroll
-                                    for (int y = 0; y < 4; ++y) {
-                                        const float2 f = __bfloat1622float2(b[y]);
-                                        acc[q4 * 8 + 2 * y] += f.x;
-                                        acc[q4 * 8 + 2 * y + 1] += f.y;
-                                    }
-                                }
-                        }
-                        store_row(p.dQ + ((size_t)h * p.L + qi) * D + ch * 32);
-                    }
-                } else {
-                    if (r < rows) store_row(p.dK + ((size_t)h * p.L + w_t0 + r) * D + ch * 32);
-                    // dV = ACC2, not scaled
-                    __syncwarp();
-                    tmem_ld32(tmem + lane_off + 384 + ch * 32, v);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int x = 0; x < 32; ++x) acc[x] = __uint_as_float(v[x]);
-                    if (r < rows) store_row(p.dV + ((size_t)h * p.L + w_t0 + r) * D + ch * 32);
-                }
+                for (int x = 0; x < 32; ++x) acc[x] = __uint_as_float(v[x]);
+                if (r < rows) store_row(p.dV + ((size_t)h * p.L + w_t0 + r) * D + ch * 32);
             }
         }
     } else if (warp < 12) {
         // ------------------------------------------------------------ producers
         asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
-        if (MODE != DKV) {
-            if (warp == 8 && lane == 0) {
-                prefetch_tensormap(&tmK);
-                prefetch_tensormap(&tmV);
-                TileIter it(w_rng, w_nrng);
-                int t0, valid, jt = 0, s3 = 0, ph3 = 0, n_k = 0;      // jt counts the V copies issued, n_k the K copies
-                while (it.next(t0, valid)) {
-                    const int s2 = jt & 1;
-                    if (!mbar_wait(bar(Y1_EMPTY + s3), ph3 ^ 1, abort_flag, p.status, BW_YEMPTY)) break;
-                    mbar_expect_tx(bar(Y1_FULL + s3), TILE_BYTES);
+        // the key tile itself: K -> X1, V -> X2
+        if (warp == 8 && lane == 0) {
+            mbar_expect_tx(bar(X_FULL), 2 * TILE_BYTES);
 #pragma unroll
-                    for (int sub = 0; sub < SUB; ++sub)
-                        tma_load_2d(sY1 + s3 * TILE_BYTES + sub * SUB_BYTES, &tmK, sub * 64, h * p.L + t0, bar(Y1_FULL + s3));
-                    ++n_k;
-                    if (!mbar_wait(bar(Y2_EMPTY + s2), ((jt >> 1) & 1) ^ 1, abort_flag, p.status, BW_YEMPTY)) break;
-                    mbar_expect_tx(bar(Y2_FULL + s2), TILE_BYTES);
-#pragma unroll
-                    for (int sub = 0; sub < SUB; ++sub)
-                        tma_load_2d(sY2 + s2 * TILE_BYTES + sub * SUB_BYTES, &tmV, sub * 64, h * p.L + t0, bar(Y2_FULL + s2));
-                    ++jt;
-                    if (++s3 == kY1Stages) { s3 = 0; ph3 ^= 1; }
-                }
-                if (*abort_flag) {      // copies already issued must land before the shared memory is released
-                    int dummy_flag = 0;
-                    for (int b = 1; b <= kY1Stages; ++b)
-                        if (n_k - b >= 0) mbar_wait(bar(Y1_FULL + ((n_k - b) % kY1Stages)), ((n_k - b) / kY1Stages) & 1, &dummy_flag, p.status, BW_YFULL);
-                    for (int b = 1; b <= kY2Stages; ++b)
-                        if (jt - b >= 0) mbar_wait(bar(Y2_FULL + ((jt - b) & 1)), ((jt - b) >> 1) & 1, &dummy_flag, p.status, BW_YFULL);
-                }
+            for (int sub = 0; sub < SUB; ++sub) {
+                tma_load_2d(sX + sub * SUB_BYTES, &tmK, sub * 64, h * p.L + w_t0, bar(X_FULL));
+                tma_load_2d(sX + TILE_BYTES + sub * SUB_BYTES, &tmV, sub * 64, h * p.L + w_t0, bar(X_FULL));
             }
-        } else {
-            // the key tile itself: K -> X1, V -> X2
-            if (warp == 8 && lane == 0) {
-                mbar_expect_tx(bar(X_FULL), 2 * TILE_BYTES);
-#pragma unroll
-                for (int sub = 0; sub < SUB; ++sub) {
-                    tma_load_2d(sX + sub * SUB_BYTES, &tmK, sub * 64, h * p.L + w_t0, bar(X_FULL));
-                    tma_load_2d(sX + TILE_BYTES + sub * SUB_BYTES, &tmV, sub * 64, h * p.L + w_t0, bar(X_FULL));
-                }
+        }
+        // The queries that attend to this chunk, 128 at a time: Q rows -> Y1 by the first two producer warps, dO rows -> Y2
+        // by the other two, each warp 64 rows of every tile.  The two rings run on their own: a tile's Q is fetched as
+        // soon as a Y1 stage is free, whatever Y2 waits for (one loop for both left T1 of the next tile waiting for
+        // 1400 of a tile's 3900 cycles).  Full tiles of consecutive queries come by TMA, the others by 16-byte
+        // asynchronous copies (36 bytes a cycle and SM; TMA row gathers reach 24).
+        const int pw = warp - 8, wsub = pw & 1;
+        const bool y1 = pw < 2;
+        const int chunk = w_chunk;
+        const int a1 = p.ranc_off[chunk + 1];
+        int a = p.ranc_off[chunk], r0 = 0, r1 = 0;       // current row range [r0, r1)
+        const int n_list = p.cnt[h * p.C + chunk];
+        const int32_t *list = p.qlist + (size_t)h * p.cap_total + p.cap_off[chunk];
+        int e0 = 0;                                        // next entry of the routed list
+        bool ok = true;
+        // This lane's two rows of a tile, in two steps so that no load is waited for: the list entries two tiles ahead,
+        // then, one tile ahead, the queries with their lse and delta.
+        int nx_whole = -1, nx_row = -1, nx_end = 0, nx_e[2] = {-1, -1};
+        auto look_ahead = [&]() {
+            if (r0 >= r1 && a < a1) {                      // next merged range of anchor query rows
+                int qc = p.ranc[a];
+                r0 = p.off[qc]; r1 = p.off[qc + 1];
+                for (++a; a < a1 && p.ranc[a] == qc + 1; ++a) { qc = p.ranc[a]; r1 = p.off[qc + 1]; }
             }
-            // The queries that attend to this chunk, 128 at a time: Q rows -> Y1 by the first two producer warps, dO rows -> Y2
-            // by the other two, each warp 64 rows of every tile.  The two rings run on their own: a tile's Q is fetched as
-            // soon as a Y1 stage is free, whatever Y2 waits for (one loop for both left T1 of the next tile waiting for
-            // 1400 of a tile's 3900 cycles).  Full tiles of consecutive queries come by TMA, the others by 16-byte
-            // asynchronous copies (36 bytes a cycle and SM; TMA row gathers reach 24).
-            const int pw = warp - 8, wsub = pw & 1;
-            const bool y1 = pw < 2;
-            const int chunk = w_chunk;
-            const int a1 = p.ranc_off[chunk + 1];
-            int a = p.ranc_off[chunk], r0 = 0, r1 = 0;       // current row range [r0, r1)
-            const int n_list = p.cnt[h * p.C + chunk];
-            const int32_t *list = p.qlist + (size_t)h * p.cap_total + p.cap_off[chunk];
-            int e0 = 0;                                        // next entry of the routed list
-            bool ok = true;
-            // This lane's two rows of a tile, in two steps so that no load is waited for: the list entries two tiles ahead,
-            // then, one tile ahead, the queries with their lse and delta.
-            int nx_whole = -1, nx_row = -1, nx_end = 0, nx_e[2] = {-1, -1};
-            auto look_ahead = [&]() {
-                if (r0 >= r1 && a < a1) {                      // next merged range of anchor query rows
-                    int qc = p.ranc[a];
-                    r0 = p.off[qc]; r1 = p.off[qc + 1];
-                    for (++a; a < a1 && p.ranc[a] == qc + 1; ++a) { qc = p.ranc[a]; r1 = p.off[qc + 1]; }
-                }
-                const int i = wsub * 64 + lane;
-                nx_whole = -1; nx_row = -1; nx_e[0] = nx_e[1] = -1;
-                if (r0 < r1) {
-                    if (r0 + 128 <= r1) nx_whole = r0;         // a full tile of consecutive queries
-                    nx_row = r0 + i;
-                    nx_end = r1;
-                    r0 += 128;
-                } else {
-#pragma unroll
-                    for (int x = 0; x < 2; ++x) {
-                        const int e = e0 + i + 32 * x;
-                        if (e < n_list && index_ok((size_t)p.cap_off[chunk] + e < p.cap_total, p.status, IX_BWD_LIST_POSITION)) nx_e[x] = list[e];
-                    }
-                    e0 += 128;
-                }
-            };
-            int whole = -1, q[2] = {-1, -1};
-            float q_lse[2] = {INFINITY, INFINITY}, q_del[2] = {0.f, 0.f};
-            auto next_rows = [&]() {
-                whole = nx_whole;
+            const int i = wsub * 64 + lane;
+            nx_whole = -1; nx_row = -1; nx_e[0] = nx_e[1] = -1;
+            if (r0 < r1) {
+                if (r0 + 128 <= r1) nx_whole = r0;         // a full tile of consecutive queries
+                nx_row = r0 + i;
+                nx_end = r1;
+                r0 += 128;
+            } else {
 #pragma unroll
                 for (int x = 0; x < 2; ++x) {
-                    q[x] = -1;
-                    if (nx_row >= 0) {
-                        if (nx_row + 32 * x < nx_end) q[x] = nx_row + 32 * x;
-                    } else if (nx_e[x] >= 0) {
-                        q[x] = p.kdiv.query(nx_e[x]);
-                        if (!index_ok((unsigned)q[x] < (unsigned)p.L, p.status, IX_BWD_LIST_ENTRY)) q[x] = -1;
-                    }
-                    // a column without a query gets lse = +inf: its P and dS come out as exact zeros
-                    // (used, that is waited for, when the tile's turn comes)
-                    q_lse[x] = INFINITY;
-                    q_del[x] = 0.f;
-                    if (y1 && q[x] >= 0) {
-                        q_lse[x] = p.lse[(size_t)h * p.L + q[x]];
-                        q_del[x] = p.delta[(size_t)h * p.L + q[x]];
-                    }
+                    const int e = e0 + i + 32 * x;
+                    if (e < n_list && index_ok((size_t)p.cap_off[chunk] + e < p.cap_total, p.status, IX_BWD_LIST_POSITION)) nx_e[x] = list[e];
                 }
-                look_ahead();
-            };
-            if (n_tiles > 0) { look_ahead(); next_rows(); }
-            int st = 0, ph = 0;                                // stage of tile jt in this warp's ring, and its phase
-            int issued = 0;                                    // tiles whose copies this warp has issued
-            const int n_st = y1 ? kY1Stages : kY2Stages, b_full = y1 ? Y1_FULL : Y2_FULL, b_empty = y1 ? Y1_EMPTY : Y2_EMPTY;
-            const uint32_t ring = y1 ? sY1 : sY2;
-            const CUtensorMap *tile_map = y1 ? &tmQ : &tmdO;
-            const __nv_bfloat16 *rows_src = (y1 ? p.Q : p.dO) + (size_t)h * p.L * D;
-            if (lane == 0) prefetch_tensormap(tile_map);
-            for (int jt = 0; ok && jt < n_tiles; ++jt) {
-                // the next tile's loads go out first: behind this tile's copies they would queue for a thousand cycles
-                const bool by_tile = whole >= 0;
-                const int t_whole = whole, t_q[2] = {q[0], q[1]};
-                const float t_lse[2] = {q_lse[0], q_lse[1]}, t_del[2] = {q_del[0], q_del[1]};
-                if (jt + 1 < n_tiles) next_rows();
-                ok = mbar_wait(bar(b_empty + st), ph ^ 1, abort_flag, p.status, BW_YEMPTY);
+                e0 += 128;
+            }
+        };
+        int whole = -1, q[2] = {-1, -1};
+        float q_lse[2] = {INFINITY, INFINITY}, q_del[2] = {0.f, 0.f};
+        auto next_rows = [&]() {
+            whole = nx_whole;
+#pragma unroll
+            for (int x = 0; x < 2; ++x) {
+                q[x] = -1;
+                if (nx_row >= 0) {
+                    if (nx_row + 32 * x < nx_end) q[x] = nx_row + 32 * x;
+                } else if (nx_e[x] >= 0) {
+                    q[x] = p.kdiv.query(nx_e[x]);
+                    if (!index_ok((unsigned)q[x] < (unsigned)p.L, p.status, IX_BWD_LIST_ENTRY)) q[x] = -1;
+                }
+                // a column without a query gets lse = +inf: its P and dS come out as exact zeros
+                // (used, that is waited for, when the tile's turn comes)
+                q_lse[x] = INFINITY;
+                q_del[x] = 0.f;
+                if (y1 && q[x] >= 0) {
+                    q_lse[x] = p.lse[(size_t)h * p.L + q[x]];
+                    q_del[x] = p.delta[(size_t)h * p.L + q[x]];
+                }
+            }
+            look_ahead();
+        };
+        if (n_tiles > 0) { look_ahead(); next_rows(); }
+        int st = 0, ph = 0;                                // stage of tile jt in this warp's ring, and its phase
+        int issued = 0;                                    // tiles whose copies this warp has issued
+        const int n_st = y1 ? kY1Stages : kY2Stages, b_full = y1 ? Y1_FULL : Y2_FULL, b_empty = y1 ? Y1_EMPTY : Y2_EMPTY;
+        const uint32_t ring = y1 ? sY1 : sY2;
+        const CUtensorMap *tile_map = y1 ? &tmQ : &tmdO;
+        const __nv_bfloat16 *rows_src = (y1 ? p.Q : p.dO) + (size_t)h * p.L * D;
+        if (lane == 0) prefetch_tensormap(tile_map);
+        for (int jt = 0; ok && jt < n_tiles; ++jt) {
+            // the next tile's loads go out first: behind this tile's copies they would queue for a thousand cycles
+            const bool by_tile = whole >= 0;
+            const int t_whole = whole, t_q[2] = {q[0], q[1]};
+            const float t_lse[2] = {q_lse[0], q_lse[1]}, t_del[2] = {q_del[0], q_del[1]};
+            if (jt + 1 < n_tiles) next_rows();
+            ok = mbar_wait(bar(b_empty + st), ph ^ 1, abort_flag, p.status, BW_YEMPTY);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            const uint32_t dst = ring + st * TILE_BYTES;
+            if (by_tile) {
+                if (lane == 0) {
+#pragma unroll
+                    for (int sub = 0; sub < SUB; ++sub)
+                        tma_load_2d(dst + sub * SUB_BYTES + wsub * 64 * 128, tile_map, sub * 64, h * p.L + t_whole + wsub * 64, bar(b_full + st));
+                }
+            } else {
+                constexpr int RP = 32 / CH;                // rows per instruction
+                const int c16 = lane % CH;
+#pragma unroll
+                for (int rb = 0; rb < 64; rb += RP) {
+                    const int rl = rb + lane / CH;
+                    const int qq = __shfl_sync(0xffffffffu, t_q[rb >> 5], rl & 31);
+                    cp_async16(dst + (c16 >> 3) * SUB_BYTES + sw128_offset(wsub * 64 + rl, c16 & 7),
+                               rows_src + (size_t)max(qq, 0) * D + c16 * 8, qq >= 0 ? 16u : 0u);
+                }
+            }
+            ++issued;
+            if (y1) {
+                // the lanes have finished with the lse / delta of tile jt - 2
+                if (jt >= 2) ok = mbar_wait(bar(DS_DONE + (jt & 1)), ((jt - 2) >> 1) & 1, abort_flag, p.status, BW_DSDONE);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                const uint32_t dst = ring + st * TILE_BYTES;
-                if (by_tile) {
-                    if (lane == 0) {
 #pragma unroll
-                        for (int sub = 0; sub < SUB; ++sub)
-                            tma_load_2d(dst + sub * SUB_BYTES + wsub * 64 * 128, tile_map, sub * 64, h * p.L + t_whole + wsub * 64, bar(b_full + st));
-                    }
-                } else {
-                    constexpr int RP = 32 / CH;                // rows per instruction
-                    const int c16 = lane % CH;
-#pragma unroll
-                    for (int rb = 0; rb < 64; rb += RP) {
-                        const int rl = rb + lane / CH;
-                        const int qq = __shfl_sync(0xffffffffu, t_q[rb >> 5], rl & 31);
-                        cp_async16(dst + (c16 >> 3) * SUB_BYTES + sw128_offset(wsub * 64 + rl, c16 & 7),
-                                   rows_src + (size_t)max(qq, 0) * D + c16 * 8, qq >= 0 ? 16u : 0u);
-                    }
+                for (int x = 0; x < 2; ++x) {
+                    s_ld[jt & 1][0][wsub * 64 + x * 32 + lane] = t_lse[x] * -kLog2e;
+                    s_ld[jt & 1][1][wsub * 64 + x * 32 + lane] = -t_del[x];
                 }
-                ++issued;
-                if (y1) {
-                    // the lanes have finished with the lse / delta of tile jt - 2
-                    if (jt >= 2) ok = mbar_wait(bar(DS_DONE + (jt & 1)), ((jt - 2) >> 1) & 1, abort_flag, p.status, BW_DSDONE);
-                    ok = __all_sync(0xffffffffu, ok);
-                    if (!ok) break;
-#pragma unroll
-                    for (int x = 0; x < 2; ++x) {
-                        s_ld[jt & 1][0][wsub * 64 + x * 32 + lane] = t_lse[x] * -kLog2e;
-                        s_ld[jt & 1][1][wsub * 64 + x * 32 + lane] = -t_del[x];
-                    }
-                }
-                if (!by_tile) {
-                    cp_async_wait_all();
-                    fence_proxy_async_smem();
-                }
-                __syncwarp();
-                // one of the ring's two warps
-                if (lane == 0) {
-                    if (by_tile) mbar_expect_tx(bar(b_full + st), TILE_BYTES / 2);
-                    else mbar_arrive(bar(b_full + st));
-                }
-                if (++st == n_st) { st = 0; ph ^= 1; }
             }
-            if (*abort_flag) {      // copies already issued must land before the shared memory is released
+            if (!by_tile) {
                 cp_async_wait_all();
-                int dummy_flag = 0;
-                for (int b = 1; b <= n_st; ++b)
-                    if (issued - b >= 0) mbar_wait(bar(b_full + (issued - b) % n_st), ((issued - b) / n_st) & 1, &dummy_flag, p.status, BW_YFULL);
+                fence_proxy_async_smem();
             }
+            __syncwarp();
+            // one of the ring's two warps
+            if (lane == 0) {
+                if (by_tile) mbar_expect_tx(bar(b_full + st), TILE_BYTES / 2);
+                else mbar_arrive(bar(b_full + st));
+            }
+            if (++st == n_st) { st = 0; ph ^= 1; }
+        }
+        if (*abort_flag) {      // copies already issued must land before the shared memory is released
+            cp_async_wait_all();
+            int dummy_flag = 0;
+            for (int b = 1; b <= n_st; ++b)
+                if (issued - b >= 0) mbar_wait(bar(b_full + (issued - b) % n_st), ((issued - b) / n_st) & 1, &dummy_flag, p.status, BW_YFULL);
         }
     } else {
         // ------------------------------------------------------------ MMA issuers: warp 12 owns the T1 / P side
@@ -644,7 +459,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
             };
             auto t2 = [&](int j) {          // T2(j) = X2 Y2(j)^T
                 const int s2 = j & 1;
-                const uint32_t d = tmem + ((MODE != DKV && s2) ? 384u : 128u);
+                const uint32_t d = tmem + 128;
 #pragma unroll
                 for (int ks = 0; ks < D / 16; ++ks) {
                     const uint32_t o = ((ks >> 2) * SUB_BYTES + (ks & 3) * 32) >> 4;
@@ -652,7 +467,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                 }
             };
             auto acc1 = [&](int j, int s3) {   // ACC1 += dS(j) Y1(j)
-                const uint32_t ds = tmem + ((MODE != DKV && (j & 1)) ? 384u : 128u);
+                const uint32_t ds = tmem + 128;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)
                     mma_ts_elect(tmem + 256, ds + ks * 8, lo(y1m) + s3 * (uint32_t)STAGE + ks * (2048 >> 4), hi(y1m), IDESC_ACC, j > 0 || ks > 0);
@@ -664,13 +479,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                     mma_ts_elect(tmem + 384, tmem + (half * 4 + ks) * 8, lo(y2m) + s2 * (uint32_t)STAGE + (half * 4 + ks) * (2048 >> 4), hi(y2m),
                               IDESC_ACC, j > 0 || half > 0 || ks > 0);
             };
-            // A wait, a fence or a commit between two groups leaves the pipe idle for longer than it takes, so each
-            // side waits early for the tiles it will read, fences once per hand-over from the lanes, and commits
-            // after the last group it has to issue at that point.
+            // MMAs queue up behind one another, so a group goes out as soon as what it reads is there
             wait(X_FULL, 0, BW_XFULL);
             if (side1) {
-                // dK/dV: ACC2(j) starts on the first half of P(j); T1(j+1) follows ACC2(j), which reads the P
-                // written over T1(j).  dQ: T1(j+1) follows the lanes' read of T1(j).
+                // ACC2(j) starts on the first half of P(j); T1(j+1) follows ACC2(j), which reads the P written over T1(j)
                 if (n_tiles > 0) {
                     wait(Y1_FULL, 0, BW_YFULL);
                     if (ok) {
@@ -682,57 +494,52 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_bwd_tc_kernel(const __g
                 int s3n = 1 % kY1Stages, ph3n = 0;                       // stage and phase of tile j + 1
                 for (int j = 0; ok && j < n_tiles; ++j) {
                     const bool more = j + 1 < n_tiles;
-                    if (MODE == DKV) {
-                        wait(P_HALF, j & 1, BW_PDONE);
-                        if (!ok) break;
-                        tc_fence_after();
-                        acc2(j, 0);
-                    }
-                    if (more) wait(Y1_FULL + s3n, ph3n, BW_YFULL);
-                    if (MODE == DKV || more) wait(P_DONE, j & 1, BW_PDONE);
+                    wait(P_HALF, j & 1, BW_PDONE);
                     if (!ok) break;
                     tc_fence_after();
-                    if (MODE == DKV) acc2(j, 1);
+                    acc2(j, 0);
+                    if (more) wait(Y1_FULL + s3n, ph3n, BW_YFULL);
+                    wait(P_DONE, j & 1, BW_PDONE);
+                    if (!ok) break;
+                    tc_fence_after();
+                    acc2(j, 1);
                     if (more) {
                         t1(j + 1, s3n);
                         tc_commit_elect(bar(T1_FULL + ((j + 1) & 1)));
                     }
                     if (++s3n == kY1Stages) { s3n = 0; ph3n ^= 1; }
-                    if (MODE == DKV) {
-                        tc_commit_elect(bar(Y2_EMPTY + (j & 1)));                 // the second of two arrivals
-                        if (more && lane == 0) mbar_arrive(bar(T1_ISSUED));              // the other side may use the pipe again
-                    }
+                    tc_commit_elect(bar(Y2_EMPTY + (j & 1)));                    // the second of two arrivals
+                    if (more && lane == 0) mbar_arrive(bar(T1_ISSUED));          // the other side may use the pipe again
                 }
             } else {
                 // The lanes wait for T1(j+1) as soon as dS(j) is done, so this side keeps out of the pipe while the
-                // other issues it.  dK/dV: ACC1(j) waits for that issue, and T2(j+1) follows ACC1(j), which reads the
-                // dS written over T2(j).  dQ: two T2 buffers; ACC1(j) then T2(j+2), both while the lanes form P(j+1).
-                constexpr int AHEAD = MODE == DKV ? 1 : 2;
-                for (int j = 0; ok && j < AHEAD && j < n_tiles; ++j) {
-                    wait(Y2_FULL + (j & 1), 0, BW_YFULL);
-                    if (!ok) break;
-                    tc_fence_after();
-                    t2(j);
-                    tc_commit_elect(bar(T2_FULL + (j & 1)));
-                    tc_commit_elect(bar(Y2_EMPTY + (j & 1)));
+                // other issues it: ACC1(j) waits for that issue, and T2(j+1) follows ACC1(j), which reads the dS written over T2(j).
+                if (n_tiles > 0) {
+                    wait(Y2_FULL, 0, BW_YFULL);
+                    if (ok) {
+                        tc_fence_after();
+                        t2(0);
+                        tc_commit_elect(bar(T2_FULL));
+                        tc_commit_elect(bar(Y2_EMPTY));
+                    }
                 }
                 int s3 = 0;                                               // Y1 stage of tile j
                 for (int j = 0; ok && j < n_tiles; ++j) {
-                    const int jn = j + AHEAD;
+                    const int jn = j + 1;
                     const bool more = jn < n_tiles;
-                    if (MODE == DKV && j + 1 < n_tiles) wait(T1_ISSUED, j & 1, BW_T1FULL);
+                    if (more) wait(T1_ISSUED, j & 1, BW_T1FULL);
                     wait(DS_DONE + (j & 1), (j >> 1) & 1, BW_DSDONE);
                     if (!ok) break;
                     tc_fence_after();
                     acc1(j, s3);
-                    tc_commit_elect(bar(Y1_EMPTY + s3));                  // at once: the next K tile waits for this stage
+                    tc_commit_elect(bar(Y1_EMPTY + s3));                  // at once: a later Q tile waits for this stage
                     if (++s3 == kY1Stages) s3 = 0;
                     if (more) {
                         wait(Y2_FULL + (jn & 1), (jn >> 1) & 1, BW_YFULL);
                         if (!ok) break;
                         t2(jn);
                         tc_commit_elect(bar(T2_FULL + (jn & 1)));
-                        tc_commit_elect(bar(Y2_EMPTY + (jn & 1)));    // dQ modes: V is read here only; dK/dV: the first of two arrivals
+                        tc_commit_elect(bar(Y2_EMPTY + (jn & 1)));    // the first of two arrivals
                     }
                 }
             }
@@ -757,10 +564,8 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
     if (int r = make_tmap_2d_bf16(&tmdO, dO, (uint64_t)p->H * p->L, D, 64)) return r;
     BwdParams a;
     a.Q = Q; a.K = K; a.V = V; a.dO = dO; a.lse = lse; a.delta = delta;
-    a.part_lse = ws_ptr<float>(ws, p->ws.part_lse);
-    a.cookie = p->cookie; a.h0 = 0; a.item_lo_dev = a.item_hi_dev = nullptr;
-    a.dQ = dQ; a.dK = dK; a.dV = dV;
-    a.part = ws_ptr<__nv_bfloat16>(ws, p->ws.part_o);      // the forward's partial outputs are no longer needed
+        a.cookie = p->cookie;
+    a.dK = dK; a.dV = dV;
     a.ktiles = p->d_ktiles; a.n_ktiles = (int)p->ktiles.size(); a.n_long = p->n_long_ktiles; a.off = p->d_off; a.ranc_off = p->d_ranc_off; a.ranc = p->d_ranc; a.cap_off = p->d_cap_off;
     a.cnt = ws_ptr<int>(ws, p->ws.cnt);
     a.qlist = ws_ptr<int32_t>(ws, p->ws.qlist);
@@ -771,22 +576,15 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
     // seven tiles (X1 X2, three Y1 stages, two Y2 stages) and the slack that aligns them to 1024 bytes; at
     // d = 128 that is all an SM has, so the request is what the kernel's static variables leave of the limit
     const size_t tiles = (size_t)(2 + kY1Stages + kY2Stages) * 128 * D * 2;
-    size_t smem[3];
-    {
-        int optin = 0;
-        MOC_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
-        const void *fn[3] = {(const void *)attend_bwd_tc_kernel<D, DQ_ROUTED>, (const void *)attend_bwd_tc_kernel<D, DQ_ANCHOR>,
-                             (const void *)attend_bwd_tc_kernel<D, DKV>};
-        for (int m = 0; m < 3; ++m) {
-            cudaFuncAttributes fa;
-            MOC_CUDA_TRY(cudaFuncGetAttributes(&fa, fn[m]));
-            smem[m] = std::min(tiles + 1024, (size_t)optin - fa.sharedSizeBytes);
-            if (smem[m] < tiles) return MOC_ERR_SHAPE;
-            MOC_CUDA_TRY(cudaFuncSetAttribute(fn[m], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem[m]));
-        }
-    }
+    int optin = 0;
+    cudaFuncAttributes fa;
+    MOC_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device));
+    MOC_CUDA_TRY(cudaFuncGetAttributes(&fa, attend_dkv_tc_kernel<D>));
+    const size_t smem = std::min(tiles + 1024, (size_t)optin - fa.sharedSizeBytes);
+    if (smem < tiles) return MOC_ERR_SHAPE;
+    MOC_CUDA_TRY(cudaFuncSetAttribute(attend_dkv_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (int r = launch_dq_tc(p, Q, K, V, lse, delta, dO, dQ, ws, s)) return r;
-    attend_bwd_tc_kernel<D, DKV><<<(unsigned)(p->ktiles.size() * (size_t)p->H), kBwdThreads, smem[DKV], s>>>(tmK, tmV, tmQ, tmdO, a);
+    attend_dkv_tc_kernel<D><<<(unsigned)(p->ktiles.size() * (size_t)p->H), kBwdThreads, smem, s>>>(tmK, tmV, tmQ, tmdO, a);
     MOC_LAUNCH_CHECK();
     return MOC_OK;
 }
