@@ -84,39 +84,6 @@ struct ItemSlot {
     const KeyRange *rng;
 };
 
-// Queue bookkeeping in the workspace (kQueueHeader ints, then three per phase: first item, rows that must
-// complete, rows completed), written before the persistent kernel starts.  Phase 2 g is the routed items of head
-// group g (rows = the group's list entries), phase 2 g + 1 its anchor items (rows = its query rows).  One block.
-__global__ void attend_queue_kernel(int *__restrict__ queue, const int *__restrict__ tile_off, const int *__restrict__ cnt,
-                                    const int *__restrict__ status, uint32_t cookie, int H, int L, int C, int k, int hg, int n_groups,
-                                    int n_aitems) {
-    __shared__ int red[256];
-    const bool routed_ok = status[ST_STATUS] == 0 && (uint32_t)status[ST_COOKIE] == cookie;     // else nothing may be read
-    int first = 0;
-    for (int g = 0; g < n_groups; ++g) {
-        const int h0 = g * hg, h1 = min(H, h0 + hg);
-        int entries = 0;
-        if (routed_ok && k > 0)
-            for (int x = h0 * C + threadIdx.x; x < h1 * C; x += blockDim.x) entries += cnt[x];
-        red[threadIdx.x] = entries;
-        __syncthreads();
-        for (int o = 128; o > 0; o >>= 1) {
-            if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            const int n_r = (routed_ok && k > 0) ? tile_off[h1 * C] - tile_off[h0 * C] : 0;
-            int *ph = queue + kQueueHeader + 3 * (2 * g);
-            ph[0] = first; ph[1] = red[0]; ph[2] = 0;
-            first += n_r;
-            ph[3] = first; ph[4] = (h1 - h0) * L; ph[5] = 0;
-            first += (h1 - h0) * n_aitems;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) { queue[0] = 0; queue[1] = routed_ok ? first : 0; queue[2] = 2 * n_groups; queue[3] = 0; }
-}
-
 // a bounded wait on a counter in global memory (another CTA adds to it)
 __device__ __forceinline__ bool wait_count(const int *ctr, int need, volatile int *abort_flag, int *status, int code) {
     if (*(volatile const int *)ctr >= need) return true;
@@ -147,7 +114,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
     extern __shared__ uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bars[36];
     __shared__ uint32_t tmem_slot;
-    __shared__ int s_abort;
+    __shared__ int s_abort, s_usable;      // s_usable: the workspace holds this plan's lists
     __shared__ ItemSlot s_item[2];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -161,7 +128,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
     constexpr int kItemReaders = 2 + 2 + 256;          // producer and bookkeeping lanes, two issuing warps, every softmax thread
 
     if (threadIdx.x == 0) {
-        s_abort = 0;
+        s_abort = s_usable = 0;
         for (int t = 0; t < 3; ++t) {
             mbar_init(bar(Q_FULL + t), 1);
             mbar_init(bar(Q_EMPTY + t), 1);
@@ -748,6 +715,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
         if (lane == 0) {
             usable = *(volatile int *)p.status == 0 && (uint32_t)((volatile int *)p.status)[ST_COOKIE] == p.cookie;
             if (!usable) atomicCAS(p.status, 0, MOC_ERR_WORKSPACE);      // not this plan's lists: report, touch nothing else
+            s_usable = usable;
             total = usable ? p.queue[1] : 0;
             n_phases = p.queue[2];
             prefetch_tensormap(&tmQ);
@@ -840,6 +808,14 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
     tc_fence_before();
     __syncthreads();
     if (warp == 8) tmem_dealloc(tmem, kTmemCols);
+    // the last CTA to leave rewinds the queue, so that the next call on this workspace needs no launch that prepares it
+    if (threadIdx.x == 0 && s_usable) {
+        __threadfence();
+        if (atomicAdd(&p.queue[3], 1) == (int)gridDim.x - 1) {
+            p.queue[0] = p.queue[3] = 0;
+            for (int ph = 0; ph < 2 * p.n_groups; ++ph) phase_tab[3 * ph + 2] = 0;
+        }
+    }
 }
 
 // ---- host side
@@ -893,15 +869,12 @@ static int attend_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfl
     a.n_aitems = (int)p->qitems.size();
     a.scale_log2 = p->scale * 1.4426950408889634f;
     a.cookie = p->cookie;
-    attend_queue_kernel<<<1, 256, 0, s>>>(a.queue, a.tile_off, ws_ptr<int>(ws, p->ws.cnt), a.status, p->cookie, p->H, p->L, p->C, p->k,
-                                          p->heads_per_group, n_groups, a.n_aitems);
-    MOC_LAUNCH_CHECK();
     // always the d = 128 footprint: more than half an SM's shared memory, so CTAs (which each
     // take all 512 TMEM columns) never share an SM
     const size_t smem = 7 * (size_t)128 * 128 * 2 + 1024;      // Q ring of three, K and V two stages each
     MOC_CUDA_TRY(cudaFuncSetAttribute(attend_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    // one CTA per SM, never more than there are anchor items (the least the queue can hold)
-    const long long most = (long long)p->H * a.n_aitems;
+    // one CTA per SM, never more than there can be items
+    const long long most = (long long)p->H * (a.n_aitems + ((long long)p->L * p->k + kQTileRows - 1) / kQTileRows + (p->k ? p->C : 0));
     const unsigned grid = (unsigned)std::max(1LL, std::min<long long>(p->n_sm, most));
     attend_tc_kernel<D><<<grid, kThreads, smem, s>>>(tmQ, tmQrow, tmK, tmV, a);
     MOC_LAUNCH_CHECK();

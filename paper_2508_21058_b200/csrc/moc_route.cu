@@ -28,7 +28,7 @@
 //   operand, the selection adds the three column groups and every candidate sinks through the sorted
 //   list in one pass (template parameter FEW).
 // route_tiles_kernel  running count of attention tiles over (head, chunk) from the pick counts;
-// route_items_kernel  the routed attention work items (one per 256 picks of a chunk).
+// route_items_kernel  the routed attention work items (one per 256 picks of a chunk) and the attention's work queue.
 // Every mbarrier wait is bounded; a wait that runs out flags the workspace status word.
 #include <float.h>
 #include <algorithm>
@@ -939,9 +939,43 @@ __global__ void __launch_bounds__(1024) route_tiles_kernel(const int *__restrict
     if (t == 1023) { gtile[HC] = st[1023]; status[ST_COOKIE] = (int)cookie; }
 }
 
-// The routed work items of (head, chunk) pair i: one per kQTileRows entries of its query list.
+// What the attention kernels' work queue needs to know, written once per selection (kQueueHeader ints, then three per
+// phase: first item, rows that must complete, rows completed).  Phase 2 g is the routed items of head group g (rows = the
+// group's list entries), phase 2 g + 1 its anchor items (rows = its query rows).  The forward kernel leaves the counters
+// rewound.  One block: a warp adds up a group's pick counts, one thread then lays the phases out.
+__device__ void write_queue(int *__restrict__ queue, const int *__restrict__ cnt, const int *__restrict__ gtile, int H, int L, int C, int k,
+                            int hg, int n_groups, int n_aitems) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int g = warp; g < n_groups; g += blockDim.x >> 5) {
+        const int h0 = g * hg, h1 = min(H, h0 + hg);
+        int entries = 0;
+        if (k > 0)
+            for (int x = h0 * C + lane; x < h1 * C; x += 32) entries += cnt[x];
+        entries = __reduce_add_sync(0xffffffffu, entries);
+        if (lane == 0) queue[kQueueHeader + 6 * g + 1] = entries;
+    }
+    if (threadIdx.x != 0) return;
+    int first = 0;
+    for (int g = 0; g < n_groups; ++g) {
+        const int h0 = g * hg, h1 = min(H, h0 + hg);
+        int *ph = queue + kQueueHeader + 6 * g;
+        ph[0] = first; ph[2] = 0;
+        if (k > 0) first += gtile[h1 * C] - gtile[h0 * C];
+        ph[3] = first; ph[4] = (h1 - h0) * L; ph[5] = 0;
+        first += (h1 - h0) * n_aitems;
+    }
+    queue[0] = 0; queue[1] = first; queue[2] = 2 * n_groups; queue[3] = 0;
+}
+
+// The routed work items of (head, chunk) pair i: one per kQTileRows entries of its query list; the last block writes the
+// work queue.
 __global__ void route_items_kernel(const int *__restrict__ cnt, const int *__restrict__ gtile, WorkItem *__restrict__ items,
-                                   const int32_t *__restrict__ off, const int32_t *__restrict__ cap_off, int H, int C) {
+                                   const int32_t *__restrict__ off, const int32_t *__restrict__ cap_off, int *__restrict__ queue, int H, int L,
+                                   int C, int k, int hg, int n_groups, int n_aitems) {
+    if (blockIdx.x == gridDim.x - 1) {
+        write_queue(queue, cnt, gtile, H, L, C, k, hg, n_groups, n_aitems);
+        return;
+    }
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;     // one warp per pair
     if (i >= H * C) return;
     const int h = i / C, c = i % C, n = cnt[i];
@@ -959,12 +993,11 @@ static int finish_lists(const moc_plan *p, void *ws, cudaStream_t s, bool count_
         route_tiles_kernel<<<1, 1024, 0, s>>>(cnt, ws_ptr<int>(ws, p->ws.tile_off), ws_ptr<int>(ws, p->ws.status), p->H * p->C, p->cookie);
         MOC_LAUNCH_CHECK();
     }
-    if (p->k > 0) {
-        route_items_kernel<<<(unsigned)((p->H * p->C + 3) / 4), 128, 0, s>>>(cnt, ws_ptr<int>(ws, p->ws.tile_off),
-                                                                               ws_ptr<WorkItem>(ws, p->ws.rtiles), p->d_off,
-                                                                               p->d_cap_off, p->H, p->C);
-        MOC_LAUNCH_CHECK();
-    }
+    const unsigned pairs = p->k > 0 ? (unsigned)((p->H * p->C + 3) / 4) : 0;
+    route_items_kernel<<<pairs + 1, 128, 0, s>>>(cnt, ws_ptr<int>(ws, p->ws.tile_off), ws_ptr<WorkItem>(ws, p->ws.rtiles), p->d_off,
+                                                 p->d_cap_off, ws_ptr<int>(ws, p->ws.queue), p->H, p->L, p->C, p->k, p->heads_per_group,
+                                                 (p->H + p->heads_per_group - 1) / p->heads_per_group, (int)p->qitems.size());
+    MOC_LAUNCH_CHECK();
     return MOC_OK;
 }
 
