@@ -63,7 +63,6 @@ struct AttendParams {
     size_t cap_total;
     int *status;
     int H, L, C, k, hg, n_groups, n_aitems;
-    SlotDiv kdiv;
     float scale_log2;           // softmax scale * log2(e)
     uint32_t cookie;
 };
@@ -201,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                 if (routed) {
                     const bool at_ok = index_ok((size_t)first + rt < p.cap_total, p.status, IX_LIST_POSITION);
                     const int e = at_ok ? p.qlist[(size_t)h * p.cap_total + first + rt] : -1;
-                    qi = p.kdiv.query(e);
+                    qi = e / p.k;
                     slot = e - qi * p.k;
                     (void)index_ok(e >= 0 && qi < p.L, p.status, IX_LIST_ENTRY);
                     if (e < 0 || qi >= p.L) qi = -1;         // never follow an entry that is not a row of this head
@@ -722,13 +721,18 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
             prefetch_tensormap(&tmQrow);
         }
         int n_item = 0, n_qtile = 0;
-        bool ok = true;
+        bool ok = true, late = false;
         while (ok) {
             const int sl = n_item & 1;
             ItemSlot s;
             s.valid = 0; s.routed = 0; s.h = 0; s.first = 0; s.rows = 0; s.nrng = 0; s.ntiles = 0; s.phase = 0; s.rng = nullptr;
             if (lane == 0) {
                 if (n_item >= 2) ok = mbar_wait(bar(ITEM_EMPTY + sl), ((n_item - 2) >> 1) & 1, abort_flag, p.status, W_ITEMEMPTY);
+                // Claimed early, an item's gathers are done before they are needed, but it is kept from a CTA that may be idle.
+                // After an anchor item (whose successors have plain tiles to load, and which end the queue), and when there
+                // are only a few items per CTA, the next one is claimed when the last S of this one has been issued.
+                if (ok && n_qtile > 0 && (late || total <= 2 * (int)gridDim.x))
+                    ok = mbar_wait(bar(Q_EMPTY + (n_qtile - 1) % 3), ((n_qtile - 1) / 3) & 1, abort_flag, p.status, W_QEMPTY);
                 const int t = (ok && usable && !*abort_flag && *(volatile int *)p.status == 0) ? atomicAdd(&p.queue[0], 1) : total;
                 if (t < total) {
                     int ph = 0;
@@ -754,6 +758,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                 s_item[sl] = s;
                 __threadfence_block();
                 mbar_arrive(bar(ITEM_FULL + sl));
+                late = !s.routed;
             }
             ++n_item;
             // the rest of the warp learns the item from lane 0
@@ -784,7 +789,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                         const int rt = g * 128 + lane * 4 + x;
                         const size_t at = (size_t)first + (rt < rows ? rt : 0);
                         const int e = at < p.cap_total ? p.qlist[(size_t)h * p.cap_total + at] : 0;
-                        int qi = p.kdiv.query(e);
+                        int qi = e / p.k;
                         if (e < 0 || qi >= p.L) qi = 0;
                         row[x] = h * p.L + qi;
                     }
@@ -865,7 +870,7 @@ static int attend_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfl
     a.queue = ws_ptr<int>(ws, p->ws.queue);
     a.cap_total = (size_t)p->cap_off[p->C];
     a.status = ws_ptr<int>(ws, p->ws.status);
-    a.H = p->H; a.L = p->L; a.C = p->C; a.k = p->k; a.kdiv = SlotDiv::of(p->k); a.hg = p->heads_per_group; a.n_groups = n_groups;
+    a.H = p->H; a.L = p->L; a.C = p->C; a.k = p->k; a.hg = p->heads_per_group; a.n_groups = n_groups;
     a.n_aitems = (int)p->qitems.size();
     a.scale_log2 = p->scale * 1.4426950408889634f;
     a.cookie = p->cookie;
