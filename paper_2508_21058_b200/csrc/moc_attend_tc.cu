@@ -33,7 +33,8 @@
 //   warp 11    scheduler and Q loader: lane 0 claims the next item and hands its description to the others
 //              through a two-slot ring; then the warp loads the item's Q tiles (plain tiles for anchor items,
 //              row gathers, four rows per lane, for routed ones) into a ring of three tile buffers, so the next
-//              item's first query tile is in place before the current item ends.
+//              item's first query tile is in place before the current item ends.  With short chunks four more warps,
+//              12 to 15, load the tiles, 32 rows each.
 // Every wait (mbarrier or global counter) is bounded; one that runs out flags the workspace status word and
 // the CTA drains its copies and leaves.
 #include <algorithm>
@@ -69,6 +70,7 @@ struct AttendParams {
 
 constexpr int kBN = 128;               // keys per tile
 constexpr int kThreads = 384;          // three warpgroups: softmax 0, softmax 1, {producer, two MMA issuers, scheduler}
+constexpr int kThreadsLoaders = 512;   // ... and a fourth one of Q loaders
 constexpr int kTmemCols = 512;         // S0/P0 [0,128) S1/P1 [128,256) O0 [256,384) O1 [384,512)
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleThreshold = 8.0f;    // log2 units: O is rescaled only when the row max grows by more
@@ -101,8 +103,9 @@ __device__ __forceinline__ bool wait_count(const int *ctr, int need, volatile in
     }
 }
 
-template <int D>
-__global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
+// LOADERS: four more warps load the query tiles, for short routed items (see the rule where the kernel is launched)
+template <int D, bool LOADERS>
+__global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
                                                                 const __grid_constant__ CUtensorMap tmQrow,
                                                                 const __grid_constant__ CUtensorMap tmK,
                                                                 const __grid_constant__ CUtensorMap tmV,
@@ -124,7 +127,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
     // barrier indices (pairs: per query tile g, per K/V stage, or per item slot)
     constexpr int Q_FULL = 0, Q_EMPTY = 3, K_FULL = 6, K_EMPTY = 8, V_FULL = 10, V_EMPTY = 12, S_FULL = 14, P_HALF = 16, P_FULL = 18,
                   O_FULL = 20, O_FREE = 22, TURN = 24, ITEM_FULL = 26, ITEM_EMPTY = 28, ROWS_DONE = 30, DEPEND = 34;
-    constexpr int kItemReaders = 2 + 2 + 256;          // producer and bookkeeping lanes, two issuing warps, every softmax thread
+    constexpr int kItemReaders = 2 + 2 + 256 + (LOADERS ? 4 : 0);      // producer and bookkeeping lanes, two issuing warps, every softmax thread, loading warps
 
     if (threadIdx.x == 0) {
         s_abort = s_usable = 0;
@@ -167,7 +170,8 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
         // ------------------------------------------------------------ softmax / epilogue groups
         // the row-per-thread softmax holds a whole 128-key row of S in registers: take the
         // registers the third warpgroup gives up
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+        if (LOADERS) asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
+        else asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
         const int g = warp >> 2;                       // query tile of this group
         const int r = threadIdx.x & 127;               // row within the tile = TMEM lane
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
@@ -484,7 +488,8 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
             ++n_mine;
         }
     } else if (warp == 8) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        if (LOADERS) asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         if (lane == 0) {
             // ------------------------------------------------------------ TMA producer of the K and V tiles
             prefetch_tensormap(&tmK);
@@ -584,7 +589,8 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
             }
         }
     } else if (warp < 11) {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        if (LOADERS) asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         // ------------------------------------------------------------ MMA issuers (one warp per query tile; the warp stays
         // together, one lane of it issues)
         const int g = uniform(warp - 9);
@@ -627,7 +633,9 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
             bool ok = true;
             // the whole warp waits, and goes on or gives up together
             auto wait = [&](int b, uint32_t parity, int code) {
-                return __all_sync(0xffffffffu, mbar_wait(bar(b), parity, abort_flag, p.status, code)) != 0;
+                // (with the loaders' traffic on every scheduler a parked issuer wakes later still: it polls)
+                return __all_sync(0xffffffffu, LOADERS ? mbar_wait_spin(bar(b), parity, abort_flag, p.status, code)
+                                                       : mbar_wait(bar(b), parity, abort_flag, p.status, code)) != 0;
             };
             while (ok) {
                 const int sl = n_item & 1;
@@ -704,8 +712,9 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                 ++n_mine;
             }
         }
-    } else {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    } else if (!LOADERS || warp == 11) {
+        if (LOADERS) asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         // ------------------------------------------------------------ scheduler (lane 0 claims items in queue order) and
         // Q loader (the whole warp): a claimed item is published at once, then its query tiles are loaded as their
         // buffers come free, which for the first tile is before the previous item has finished
@@ -767,6 +776,7 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
             ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
             if (!valid || !ok) break;
             const int n_qt = rows > 128 ? 2 : 1;
+            if (LOADERS) { n_qtile += n_qt; continue; }
             for (int g = 0; ok && g < n_qt; ++g) {
                 const int qb = n_qtile % 3;
                 ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.status, W_QEMPTY);
@@ -801,7 +811,71 @@ __global__ void __launch_bounds__(kThreads, 1) attend_tc_kernel(const __grid_con
                 ++n_qtile;
             }
         }
-        if (*abort_flag && lane == 0) {
+        if (!LOADERS && *abort_flag && lane == 0) {
+            // drain: the Q copies already issued must land before the CTA's shared memory is released
+            int dummy_flag = 0;
+            for (int b = 1; b <= 3; ++b) {
+                const int qj = n_qtile - b;
+                if (qj >= 0) mbar_wait(bar(Q_FULL + qj % 3), (qj / 3) & 1, &dummy_flag, p.status, W_QFULL);
+            }
+        }
+    } else {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        // ------------------------------------------------------------ Q loaders: rows 32 lw .. 32 lw + 31 of every query tile.
+        // All four warps load a part of every tile, so a buffer cannot be filled and released without one of them: none
+        // can miss a phase of Q_EMPTY.
+        const int lw = warp - 12;
+        int n_item = 0, n_qtile = 0;
+        bool ok = true;
+        while (ok) {
+            const int sl = n_item & 1;
+            ok = mbar_wait(bar(ITEM_FULL + sl), (n_item >> 1) & 1, abort_flag, p.status, W_ITEMFULL);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            const int valid = s_item[sl].valid, routed = s_item[sl].routed, h = s_item[sl].h, first = s_item[sl].first, rows = s_item[sl].rows;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(ITEM_EMPTY + sl));
+            ++n_item;
+            if (!valid) break;
+            const int n_qt = rows > 128 ? 2 : 1;
+            // the queries of this lane's rows (a row past the item's end fetches row 0 of the head: its result is never stored)
+            int qrow[2] = {0, 0};
+            if (routed) {
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    const int rt = g * 128 + lw * 32 + lane;
+                    const size_t at = (size_t)first + rt;
+                    const int e = rt < rows && at < p.cap_total ? p.qlist[(size_t)h * p.cap_total + at] : -1;
+                    qrow[g] = e < 0 ? 0 : e / p.k;
+                    if (qrow[g] >= p.L) qrow[g] = 0;
+                }
+            }
+            for (int g = 0; ok && g < n_qt; ++g) {
+                const int qb = n_qtile % 3;
+                int row[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) row[x] = h * p.L + __shfl_sync(0xffffffffu, qrow[g], (lane & 7) * 4 + x);
+                ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.status, W_QEMPTY);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (lw == 0 && lane == 0) mbar_expect_tx(bar(Q_FULL + qb), TILE_BYTES);
+                const uint32_t dst = sQ + qb * TILE_BYTES + lw * 32 * 128;
+                if (!routed) {
+                    if (lane == 0) {
+#pragma unroll
+                        for (int sub = 0; sub < SUB; ++sub)
+                            tma_load_2d(dst + sub * SUB_BYTES, &tmQ, sub * 64, h * p.L + first + g * 128 + lw * 32, bar(Q_FULL + qb));
+                    }
+                } else if (lane < 8) {                          // lane l gathers rows 4 l .. 4 l + 3 of the warp's 32
+#pragma unroll
+                    for (int sub = 0; sub < SUB; ++sub)
+                        tma_gather4(dst + sub * SUB_BYTES + lane * 512, &tmQrow, sub * 64, row[0], row[1], row[2], row[3], bar(Q_FULL + qb));
+                }
+                __syncwarp();
+                ++n_qtile;
+            }
+        }
+        if (*abort_flag && lw == 0 && lane == 0) {
             // drain: the Q copies already issued must land before the CTA's shared memory is released
             int dummy_flag = 0;
             for (int b = 1; b <= 3; ++b) {
@@ -848,11 +922,11 @@ int make_tmap_2d_bf16(CUtensorMap *map, const void *base, uint64_t rows, uint64_
     return MOC_OK;
 }
 
-template <int D>
+template <int D, bool LOADERS>
 static int attend_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat16 *K, const __nv_bfloat16 *V,
                        __nv_bfloat16 *O, float *lse, void *ws, cudaStream_t s) {
     CUtensorMap tmQ, tmQrow, tmK, tmV;
-    if (int r = make_tmap_2d_bf16(&tmQ, Q, (uint64_t)p->H * p->L, D, 128)) return r;
+    if (int r = make_tmap_2d_bf16(&tmQ, Q, (uint64_t)p->H * p->L, D, LOADERS ? 32 : 128)) return r;
     if (int r = make_tmap_2d_bf16(&tmQrow, Q, (uint64_t)p->H * p->L, D, 1)) return r;      // row gathers: a box one row high
     if (int r = make_tmap_2d_bf16(&tmK, K, (uint64_t)p->H * p->L, D, kBN)) return r;
     if (int r = make_tmap_2d_bf16(&tmV, V, (uint64_t)p->H * p->L, D, kBN)) return r;
@@ -877,18 +951,25 @@ static int attend_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfl
     // always the d = 128 footprint: more than half an SM's shared memory, so CTAs (which each
     // take all 512 TMEM columns) never share an SM
     const size_t smem = 7 * (size_t)128 * 128 * 2 + 1024;      // Q ring of three, K and V two stages each
-    MOC_CUDA_TRY(cudaFuncSetAttribute(attend_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    MOC_CUDA_TRY(cudaFuncSetAttribute(attend_tc_kernel<D, LOADERS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     // one CTA per SM, never more than there can be items
     const long long most = (long long)p->H * (a.n_aitems + ((long long)p->L * p->k + kQTileRows - 1) / kQTileRows + (p->k ? p->C : 0));
     const unsigned grid = (unsigned)std::max(1LL, std::min<long long>(p->n_sm, most));
-    attend_tc_kernel<D><<<grid, kThreads, smem, s>>>(tmQ, tmQrow, tmK, tmV, a);
+    attend_tc_kernel<D, LOADERS><<<grid, LOADERS ? kThreadsLoaders : kThreads, smem, s>>>(tmQ, tmQrow, tmK, tmV, a);
     MOC_LAUNCH_CHECK();
     return MOC_OK;
 }
 
 int launch_attend_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat16 *K, const __nv_bfloat16 *V,
                      const int32_t *, __nv_bfloat16 *O, float *lse, void *ws, cudaStream_t s) {
-    return p->d == 128 ? attend_tc_d<128>(p, Q, K, V, O, lse, ws, s) : attend_tc_d<64>(p, Q, K, V, O, lse, ws, s);
+    // Who loads the query tiles.  A row gather costs the warp that issues it some 65 cycles for four rows of 128 bytes: with
+    // one warp a 256-row routed item cannot start more often than every 13000 cycles (half that at d = 64), with four every
+    // 3000 to 4000 - but four loading warps, one on every scheduler, are in the way of the softmax.  The line lies at four
+    // key tiles a chunk, d = 128 (one warp -> four): 256-token chunks 24.4 -> 22.9 ms, 512-token chunks 27.2 -> 26.6 ms,
+    // 1560-token frames 3.42 -> 3.50 ms; 256-token chunks at d = 64: 462 -> 472 us (training step).
+    if (p->d == 64) return attend_tc_d<64, false>(p, Q, K, V, O, lse, ws, s);
+    const bool loaders = p->k > 0 && p->routed_key_tiles <= 4LL * p->ncol;
+    return loaders ? attend_tc_d<128, true>(p, Q, K, V, O, lse, ws, s) : attend_tc_d<128, false>(p, Q, K, V, O, lse, ws, s);
 }
 
 }  // namespace moc

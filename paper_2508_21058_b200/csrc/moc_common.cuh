@@ -76,6 +76,7 @@ struct moc_plan {
     // Routing scores only the chunks that can ever be picked: text chunks are anchors of every query, so the score
     // matrix has one column per non-text chunk ("column" = index among those, in chunk order).
     int ncol;                                // number of columns
+    int64_t routed_key_tiles;                // key tiles of all of them
     int cwords;                              // uint32 words per candidate bitmap row (over columns)
     int prefix_mode;                         // 1: every query chunk's candidates are exactly the columns [0, lim[c])
     int c_pad;                               // columns rounded up to a multiple of 16 (MMA N granularity)

@@ -214,6 +214,8 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     for (int j = 0; j < C; ++j)
         if (p->mod[j] != 1) { col_of[j] = (int32_t)col_chunk.size(); col_chunk.push_back(j); }
     p->ncol = (int)col_chunk.size();
+    p->routed_key_tiles = 0;
+    for (int j : col_chunk) p->routed_key_tiles += (p->off[j + 1] - p->off[j] + 127) / 128;
     p->cwords = std::max(1, (p->ncol + 31) / 32);
     p->c_pad = std::max(16, (p->ncol + 15) / 16 * 16);
     std::vector<uint32_t> cand_c((size_t)C * p->cwords, 0u);
