@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
         s_abort = s_usable = 0;
         for (int t = 0; t < 3; ++t) {
             mbar_init(bar(Q_FULL + t), 1);
-            mbar_init(bar(Q_EMPTY + t), 1);
+            mbar_init(bar(Q_EMPTY + t), 2);            // the issuer that reads it, and the other one when it has seen it
         }
         mbar_init(bar(DEPEND), 1);
         for (int t = 0; t < 2; ++t) {
@@ -646,8 +646,19 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 ++n_item;
                 if (!uniform(it_.valid)) break;
                 const int rows = uniform(it_.rows), n_tiles = uniform(it_.ntiles);
-                const int q_seq = n_qtile + g;                      // this tile's place in the sequence of Q loads
+                const int q_first = n_qtile, q_seq = q_first + g;   // the item's first and this tile's place in the sequence of Q loads
                 n_qtile += rows > 128 ? 2 : 1;
+                // Every query tile is waited for by both issuers, and a buffer is refilled only when both have: an issuer that
+                // left out the other's tiles could wait for a buffer whose previous load is still on its way, and take the
+                // barrier's phase for the one it waits for.  This is the other issuer's tile.
+                auto pass_tile = [&](int t) {
+                    ok = ok && wait(Q_FULL + t % 3, (t / 3) & 1, W_QFULL);
+                    if (ok && lane == 0) mbar_arrive(bar(Q_EMPTY + t % 3));
+                };
+                if (g == 1) {
+                    pass_tile(q_first);
+                    if (!ok) break;
+                }
                 if (g == 1 && rows <= 128) {
                     // no second query tile: this issuer only keeps the K/V ring's accounting (each stage is
                     // released by two arrivals)
@@ -709,6 +720,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                     ++n_kv;
                     ++n_p;
                 }
+                if (g == 0 && rows > 128) pass_tile(q_first + 1);
                 ++n_mine;
             }
         }
