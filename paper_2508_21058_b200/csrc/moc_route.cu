@@ -58,6 +58,36 @@ struct TopK {
     }
 };
 
+// ---- the first columns of a list of 17 to 32 picks: candidates as 64-bit keys, high word the score as an integer of
+// the same order (-0 and +0 alike), low word the complement of the column, so that one integer compare orders them as the
+// result is ordered (score descending, then column ascending).
+constexpr uint32_t kNoScore = 0x007fffffu;      // high word of a score of -inf: nothing there
+__device__ __forceinline__ uint64_t score_key(float f, int col) {
+    asm("add.rn.f32 %0, %0, 0f00000000;" : "+f"(f));
+    const int b = __float_as_int(f);
+    return (uint64_t)((uint32_t)b ^ ((uint32_t)(b >> 31) | 0x80000000u)) << 32 | (uint32_t)~col;
+}
+__device__ __forceinline__ float key_score(uint64_t key) {
+    const uint32_t u = (uint32_t)(key >> 32);
+    return __uint_as_float((u & 0x80000000u) ? u ^ 0x80000000u : ~u);
+}
+__device__ __forceinline__ void order_keys(uint64_t &a, uint64_t &b, bool desc) {
+    const bool lt = a < b;
+    const uint64_t hi = lt ? b : a, lo = lt ? a : b;
+    a = desc ? hi : lo;
+    b = desc ? lo : hi;
+}
+// sorted descending by a bitonic network (a fixed sequence of compare-exchange steps, every index a compile-time constant)
+__device__ __forceinline__ void sort32(uint64_t (&a)[32]) {
+#pragma unroll
+    for (int k2 = 2; k2 <= 32; k2 <<= 1)
+#pragma unroll
+        for (int jj = k2 >> 1; jj > 0; jj >>= 1)
+#pragma unroll
+            for (int ii = 0; ii < 32; ++ii)
+                if (!(ii & jj)) order_keys(a[ii], a[ii | jj], k2 == 32 || (ii & k2) == 0);
+}
+
 // desc3[h][t][col][:] for t = 0, 1, 2: bf16 terms of the descriptor of score column col (the col-th non-text
 // chunk; rows beyond the last column are zero); also clears the pick counters and the status words (the workspace holds no plan's lists until they
 // are complete) and states the limit of the bounded waits.  With desc == nullptr only the clearing is done.
@@ -104,6 +134,9 @@ struct RouteParams {
     int sb_rows;            // chunks per scoring step (one accumulator's worth)
     int d_rows;             // descriptor rows per term held in shared memory: c_pad (resident) or sb_rows (streamed)
     int q_stages;
+    int dual;               // two issuers (resident block, two accumulators or more).  The Q stages are then even in number: each
+                            // stage serves one issuer, which so waits for every use of it (an issuer that left out a use could
+                            // take the phase of a load still on its way for the one it waits for)
     int n_pass;             // selection passes over a tile's scores: 64 picks each (the scores are recomputed per pass)
     int surv_cap;           // threshold selection: survivor slots per query row in shared memory (0 = not used)
     int *tile_off;          // [H C + 1] running tile counts, written by the last block to finish
@@ -296,7 +329,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
         // With a resident descriptor block, warp 1 serves the even units and the last warpgroup's first warp
         // the odd ones (each its own accumulators), so one issuer's waits and instruction overhead hide behind the other's
         // MMAs; when blocks are streamed, warp 1 serves every unit and follows the reloads.
-        const bool dual = resident && NG > 1;          // one selection group has one accumulator: one issuer
+        const bool dual = p.dual != 0;
         const int first = warp == 1 ? 0 : 1, stride = dual ? 2 : 1;
         if (warp == 1 || dual) {               // the warp stays together, one lane of it issues
             // descriptors are built once: issuing an MMA should cost this warp a few integer instructions
@@ -764,17 +797,42 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                         for (int b = 0; b < half; ++b) scan(b * 32, (b + half) * 32, b + half < nblk);
                         fast = drain();
                     } else {
-                        // Long lists: no group maxima (a list of k needs more groups than registers hold); the columns
-                        // go 64 at a time against the list's own k-th score, which rises as they go: after n columns
-                        // about k / n of the next ones survive.  A pair of blocks whose survivors do not fit the
-                        // queue (the first ones, when everything survives and the queue is short) is extracted
-                        // best-first instead.
+                        // Long lists: no group maxima (a list of k needs more groups than registers hold); the columns are
+                        // scanned against the list's own k-th score, which rises as they go: after n columns about k / n of
+                        // the next ones survive.  64 columns at a time, with a 64-entry queue from the start; with the
+                        // shorter queue of the 32-entry lists the first 32 columns are sorted by a network and are the
+                        // list, and the next ones go 32 at a time, which always fit, until 4 k have been seen.  (Taken best
+                        // first, as pairs of blocks whose survivors do not fit still are, the first 64 columns cost two thirds of
+                        // the selection: up to k rounds of 350 instructions a block.  264k tokens, 30 picks of 1008
+                        // columns, 6 heads: 4.26 -> 3.25 ms.)
+                        int b0 = 0;
+                        if constexpr (KMAX == 32) {
+                            if (sb == 0) {
+                                uint32_t v[32];
+                                uint64_t key[32];
+                                tmem_ld32(acc, v);
+                                const uint32_t cand = cand_bits(0);
+                                tmem_wait_ld();
+#pragma unroll
+                                for (int c = 0; c < 32; ++c) key[c] = score_key(((cand >> c) & 1u) ? __uint_as_float(v[c]) : -INFINITY, c);
+                                sort32(key);
+#pragma unroll
+                                for (int x = 0; x < 32; ++x) {
+                                    const bool some = (uint32_t)(key[x] >> 32) != kNoScore;
+                                    top.s[x] = some ? key_score(key[x]) : -INFINITY;
+                                    top.j[x] = some ? (int)~(uint32_t)key[x] : -1;
+                                }
+                                update_kth();
+                                b0 = 1;
+                            }
+                        }
 #pragma unroll 1
-                        for (int b0 = 0; b0 < nblk; b0 += 2) {
+                        while (b0 < nblk) {
                             thr = fmaxf(kth, -FLT_MAX);
-                            const bool two = b0 + 1 < nblk;
+                            const bool two = b0 + 1 < nblk && (KMAX == 64 || jb + b0 * 32 >= 4 * kp);
                             scan(b0 * 32, (b0 + 1) * 32, two);
-                            if (!drain()) extract_blocks(b0 * 32, min(rows_sb, (b0 + 2) * 32));
+                            if (!drain()) extract_blocks(b0 * 32, min(rows_sb, (b0 + 1 + two) * 32));
+                            b0 += 1 + two;
                         }
                     }
                 }
@@ -1128,6 +1186,8 @@ static int launch_route_d(const moc_plan *p, const __nv_bfloat16 *Q, const float
             surv = 16 + a.surv_cap * per_slot;
         }
         a.q_stages = (int)std::min<size_t>(4, (budget - d_block - hist - surv) / q_tile);
+        a.dual = a.d_rows == p->c_pad && ng > 1 && a.q_stages >= 2;
+        if (a.dual) a.q_stages &= ~1;
         if (a.d_rows != p->c_pad && a.q_stages < ng) return MOC_ERR_SHAPE;      // streamed blocks: a round's Q tiles are held together
         const size_t smem = 1024 + d_block + a.q_stages * q_tile + hist + surv;
         CUtensorMap tmQ, tmD;
