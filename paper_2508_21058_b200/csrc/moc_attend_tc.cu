@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
     constexpr int SUB = D / 64;            // 64-column (128-byte) sub-tiles per row
     constexpr int SUB_BYTES = 128 * 128;   // one sub-tile: 128 rows of 128 bytes
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bars[36];
+    __shared__ __align__(8) uint64_t bars[39];
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort, s_usable;      // s_usable: the workspace holds this plan's lists
     __shared__ ItemSlot s_item[2];
@@ -125,15 +125,19 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
     const uint32_t sQ = sbase, sK = sbase + 3 * TILE_BYTES, sV = sbase + 5 * TILE_BYTES;
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
     // barrier indices (pairs: per query tile g, per K/V stage, or per item slot)
-    constexpr int Q_FULL = 0, Q_EMPTY = 3, K_FULL = 6, K_EMPTY = 8, V_FULL = 10, V_EMPTY = 12, S_FULL = 14, P_HALF = 16, P_FULL = 18,
-                  O_FULL = 20, O_FREE = 22, TURN = 24, ITEM_FULL = 26, ITEM_EMPTY = 28, ROWS_DONE = 30, DEPEND = 34;
+    constexpr int Q_FULL = 0, Q_EMPTY = 6, K_FULL = 9, K_EMPTY = 11, V_FULL = 13, V_EMPTY = 15, S_FULL = 17, P_HALF = 19, P_FULL = 21,
+                  O_FULL = 23, O_FREE = 25, TURN = 27, ITEM_FULL = 29, ITEM_EMPTY = 31, ROWS_DONE = 33, DEPEND = 37;
     constexpr int kItemReaders = 2 + 2 + 256 + (LOADERS ? 4 : 0);      // producer and bookkeeping lanes, two issuing warps, every softmax thread, loading warps
 
     if (threadIdx.x == 0) {
         s_abort = s_usable = 0;
         for (int t = 0; t < 3; ++t) {
-            mbar_init(bar(Q_FULL + t), 1);
-            mbar_init(bar(Q_EMPTY + t), 2);            // the issuer that reads it, and the other one when it has seen it
+            // A Q buffer has one full barrier per query tile g, so that each issuer waits for every phase of its own ones: on
+            // a shared one, an issuer that leaves out the other's tiles could wait for a buffer whose previous load is still
+            // on its way, and take that phase for the one it waits for.
+            mbar_init(bar(Q_FULL + t), 1);             // [g][buffer]
+            mbar_init(bar(Q_FULL + 3 + t), 1);
+            mbar_init(bar(Q_EMPTY + t), 1);
         }
         mbar_init(bar(DEPEND), 1);
         for (int t = 0; t < 2; ++t) {
@@ -630,6 +634,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             };
             // items seen, items with this tile, K/V tiles seen, P tiles consumed, query tiles loaded before this item
             int n_item = 0, n_mine = 0, n_kv = 0, n_p = 0, n_qtile = 0;
+            uint32_t q_phase = 0;                         // bit b: parity of the next load of this tile into buffer b
             bool ok = true;
             // the whole warp waits, and goes on or gives up together
             auto wait = [&](int b, uint32_t parity, int code) {
@@ -646,19 +651,8 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 ++n_item;
                 if (!uniform(it_.valid)) break;
                 const int rows = uniform(it_.rows), n_tiles = uniform(it_.ntiles);
-                const int q_first = n_qtile, q_seq = q_first + g;   // the item's first and this tile's place in the sequence of Q loads
+                const int q_seq = n_qtile + g;                      // this tile's place in the sequence of Q loads
                 n_qtile += rows > 128 ? 2 : 1;
-                // Every query tile is waited for by both issuers, and a buffer is refilled only when both have: an issuer that
-                // left out the other's tiles could wait for a buffer whose previous load is still on its way, and take the
-                // barrier's phase for the one it waits for.  This is the other issuer's tile.
-                auto pass_tile = [&](int t) {
-                    ok = ok && wait(Q_FULL + t % 3, (t / 3) & 1, W_QFULL);
-                    if (ok && lane == 0) mbar_arrive(bar(Q_EMPTY + t % 3));
-                };
-                if (g == 1) {
-                    pass_tile(q_first);
-                    if (!ok) break;
-                }
                 if (g == 1 && rows <= 128) {
                     // no second query tile: this issuer only keeps the K/V ring's accounting (each stage is
                     // released by two arrivals)
@@ -681,7 +675,8 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 int t0, valid, valid_next = 0;
                 ok = it.next(t0, valid);
                 valid = uniform(valid);
-                ok = ok && wait(Q_FULL + qb, (q_seq / 3) & 1, W_QFULL);
+                ok = ok && wait(Q_FULL + 3 * g + qb, (q_phase >> qb) & 1, W_QFULL);
+                q_phase ^= 1u << qb;
                 ok = ok && wait(K_FULL + (n_kv & 1), (n_kv >> 1) & 1, W_KFULL);
                 if (!ok) break;
                 tc_fence_after();
@@ -720,7 +715,6 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                     ++n_kv;
                     ++n_p;
                 }
-                if (g == 0 && rows > 128) pass_tile(q_first + 1);
                 ++n_mine;
             }
         }
@@ -742,6 +736,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             prefetch_tensormap(&tmQrow);
         }
         int n_item = 0, n_qtile = 0;
+        uint32_t q_phase = 0;                          // bit 3 g + buffer: parity of the next phase of that Q_FULL
         bool ok = true, late = false;
         while (ok) {
             const int sl = n_item & 1;
@@ -790,17 +785,17 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             const int n_qt = rows > 128 ? 2 : 1;
             if (LOADERS) { n_qtile += n_qt; continue; }
             for (int g = 0; ok && g < n_qt; ++g) {
-                const int qb = n_qtile % 3;
+                const int qb = n_qtile % 3, qf = 3 * g + qb;
                 ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.status, W_QEMPTY);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                if (lane == 0) mbar_expect_tx(bar(Q_FULL + qb), TILE_BYTES);
+                if (lane == 0) mbar_expect_tx(bar(Q_FULL + qf), TILE_BYTES);
                 __syncwarp();
                 if (!routed) {
                     if (lane == 0) {
 #pragma unroll
                         for (int sub = 0; sub < SUB; ++sub)
-                            tma_load_2d(sQ + qb * TILE_BYTES + sub * SUB_BYTES, &tmQ, sub * 64, h * p.L + first + g * 128, bar(Q_FULL + qb));
+                            tma_load_2d(sQ + qb * TILE_BYTES + sub * SUB_BYTES, &tmQ, sub * 64, h * p.L + first + g * 128, bar(Q_FULL + qf));
                     }
                 } else {
                     // lane l gathers rows 4 l .. 4 l + 3 of the tile; a row past the item's end repeats the item's
@@ -818,18 +813,17 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
 #pragma unroll
                     for (int sub = 0; sub < SUB; ++sub)
                         tma_gather4(sQ + qb * TILE_BYTES + sub * SUB_BYTES + lane * 512, &tmQrow, sub * 64, row[0], row[1], row[2], row[3],
-                                    bar(Q_FULL + qb));
+                                    bar(Q_FULL + qf));
                 }
+                q_phase ^= 1u << qf;
                 ++n_qtile;
             }
         }
         if (!LOADERS && *abort_flag && lane == 0) {
             // drain: the Q copies already issued must land before the CTA's shared memory is released
             int dummy_flag = 0;
-            for (int b = 1; b <= 3; ++b) {
-                const int qj = n_qtile - b;
-                if (qj >= 0) mbar_wait(bar(Q_FULL + qj % 3), (qj / 3) & 1, &dummy_flag, p.status, W_QFULL);
-            }
+            // (a barrier that was never used is past the phase before its first)
+            for (int b = 0; b < 6; ++b) mbar_wait(bar(Q_FULL + b), ((q_phase >> b) & 1) ^ 1, &dummy_flag, p.status, W_QFULL);
         }
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
@@ -838,6 +832,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
         // can miss a phase of Q_EMPTY.
         const int lw = warp - 12;
         int n_item = 0, n_qtile = 0;
+        uint32_t q_phase = 0;                          // bit 3 g + buffer: parity of the next phase of that Q_FULL
         bool ok = true;
         while (ok) {
             const int sl = n_item & 1;
@@ -863,37 +858,36 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 }
             }
             for (int g = 0; ok && g < n_qt; ++g) {
-                const int qb = n_qtile % 3;
+                const int qb = n_qtile % 3, qf = 3 * g + qb;
                 int row[4];
 #pragma unroll
                 for (int x = 0; x < 4; ++x) row[x] = h * p.L + __shfl_sync(0xffffffffu, qrow[g], (lane & 7) * 4 + x);
                 ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.status, W_QEMPTY);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
-                if (lw == 0 && lane == 0) mbar_expect_tx(bar(Q_FULL + qb), TILE_BYTES);
+                if (lw == 0 && lane == 0) mbar_expect_tx(bar(Q_FULL + qf), TILE_BYTES);
                 const uint32_t dst = sQ + qb * TILE_BYTES + lw * 32 * 128;
                 if (!routed) {
                     if (lane == 0) {
 #pragma unroll
                         for (int sub = 0; sub < SUB; ++sub)
-                            tma_load_2d(dst + sub * SUB_BYTES, &tmQ, sub * 64, h * p.L + first + g * 128 + lw * 32, bar(Q_FULL + qb));
+                            tma_load_2d(dst + sub * SUB_BYTES, &tmQ, sub * 64, h * p.L + first + g * 128 + lw * 32, bar(Q_FULL + qf));
                     }
                 } else if (lane < 8) {                          // lane l gathers rows 4 l .. 4 l + 3 of the warp's 32
 #pragma unroll
                     for (int sub = 0; sub < SUB; ++sub)
-                        tma_gather4(dst + sub * SUB_BYTES + lane * 512, &tmQrow, sub * 64, row[0], row[1], row[2], row[3], bar(Q_FULL + qb));
+                        tma_gather4(dst + sub * SUB_BYTES + lane * 512, &tmQrow, sub * 64, row[0], row[1], row[2], row[3], bar(Q_FULL + qf));
                 }
                 __syncwarp();
+                q_phase ^= 1u << qf;
                 ++n_qtile;
             }
         }
         if (*abort_flag && lw == 0 && lane == 0) {
             // drain: the Q copies already issued must land before the CTA's shared memory is released
             int dummy_flag = 0;
-            for (int b = 1; b <= 3; ++b) {
-                const int qj = n_qtile - b;
-                if (qj >= 0) mbar_wait(bar(Q_FULL + qj % 3), (qj / 3) & 1, &dummy_flag, p.status, W_QFULL);
-            }
+            // (a barrier that was never used is past the phase before its first)
+            for (int b = 0; b < 6; ++b) mbar_wait(bar(Q_FULL + b), ((q_phase >> b) & 1) ^ 1, &dummy_flag, p.status, W_QFULL);
         }
     }
     tc_fence_before();
