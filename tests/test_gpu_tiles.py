@@ -1,0 +1,52 @@
+"""The attention and routing kernels at the edges of their tiles, lists and variants, against the CPU oracle, with the
+tolerances of the other parity tests; and a workspace used again gives the same bits."""
+import pytest
+import torch
+
+from oracle import Oracle
+from paper_2508_21058_b200 import workloads as W
+
+import parity_utils as PU
+
+pytestmark = pytest.mark.gpu
+
+# heads, head_dim, (shots, caption, frames, frame length), k
+SHAPES = {
+    "whole tiles only": (5, 128, (3, 128, 6, 128), 4),                 # one key tile a chunk; every dK/dV query tile from consecutive rows
+    "four key tiles a chunk": (2, 128, (2, 16, 4, 512), 2),            # the last size with four query-loading warps
+    "four key tiles and one key": (2, 128, (2, 16, 4, 513), 2),        # the first size with one
+    "one row past a tile": (7, 128, (2, 1, 11, 129), 9),               # items of 256 rows and of a few; a merge of 8 + 1 picks
+    "one row short of two tiles": (2, 64, (2, 31, 9, 255), 8),         # a full merge batch
+    "17 picks": (3, 64, (2, 1, 13, 65), 17),                           # the shortest sorted list, 26 columns
+    "32 picks of 33 columns and more": (2, 128, (3, 8, 15, 33), 32),   # a full list, and one column in the second block
+    "33 picks": (2, 64, (2, 8, 24, 33), 33),                           # the longer list
+    "fewer candidates than picks": (2, 128, (1, 8, 20, 40), 24),
+    "no picks": (3, 128, (2, 130, 3, 129), 0),                         # anchor items alone
+}
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_tile_and_list_edges(shape):
+    heads, d, lay, k = SHAPES[shape]
+    wl = W.Workload("edges", heads, d, W.make_layout(*lay), k, 1, 1)
+    run = PU.GpuRun(wl, tensors=("q", "k", "v", "do")).forward()
+    x, orc = run.host_inputs(), Oracle.from_workload(wl)
+    sel = run.sel.cpu().numpy()
+    if k:
+        PU.assert_routing(wl, orc, x["q"], orc.chunk_pool(x["k"]), sel)
+    O_ref, lse_ref = orc.attend(x["q"], x["k"], x["v"], sel)
+    O, lse = run.O.clone(), run.lse.clone()
+    PU.assert_attention_close(PU.attention_errors(O.float().cpu().numpy().reshape(-1, d), lse.cpu().numpy().reshape(-1), O_ref, lse_ref))
+    for again in range(30):                                # the work queue is rewound by the pass before
+        run.attend_only()
+        assert torch.equal(O, run.O) and torch.equal(lse, run.lse), again
+    run.backward()
+    rows = W.sample_rows(wl, 64)
+    dQ_g, dK_g, dV_g = (t.float().cpu().numpy() for t in (run.dQ, run.dK, run.dV))
+    off = wl.layout.chunk_off
+    for head, chunk in ((0, 1), (heads - 1, wl.n_chunks // 2)):
+        t0, t1 = int(off[chunk]), int(off[chunk + 1])
+        dQ, dK, dV = orc.attend_bwd(x["q"], x["k"], x["v"], x["do"], sel, rows, head, (t0, t1))
+        PU.assert_grad_close(dQ_g[rows[:, 0], rows[:, 1]], dQ)
+        PU.assert_grad_close(dK_g[head, t0:t1], dK)
+        PU.assert_grad_close(dV_g[head, t0:t1], dV)
