@@ -135,7 +135,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
         fence_barrier_init();
     }
     __syncthreads();
-    if (!w_valid) return;
+    if (!w_valid) {
+        if (blockIdx.x == gridDim.x - 1) previous_done();
+        return;
+    }
     if (warp == 8) {
         tmem_alloc(smem_u32(&tmem_slot), 512);
         tmem_relinquish();
@@ -549,6 +552,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
     tc_fence_before();
     __syncthreads();
     if (warp == 8) tmem_dealloc(tmem, 512);
+    if (blockIdx.x == gridDim.x - 1) previous_done();    // nothing here depends on dQ's launches, but what follows may
 }
 
 template <int D>
@@ -584,7 +588,7 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
     if (smem < tiles) return MOC_ERR_SHAPE;
     MOC_CUDA_TRY(cudaFuncSetAttribute(attend_dkv_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (int r = launch_dq_tc(p, Q, K, V, lse, delta, dO, dQ, ws, s)) return r;
-    attend_dkv_tc_kernel<D><<<(unsigned)(p->ktiles.size() * (size_t)p->H), kBwdThreads, smem, s>>>(tmK, tmV, tmQ, tmdO, a);
+    MOC_CUDA_TRY(launch_early(attend_dkv_tc_kernel<D>, (unsigned)(p->ktiles.size() * (size_t)p->H), kBwdThreads, smem, s, tmK, tmV, tmQ, tmdO, a));
     MOC_LAUNCH_CHECK();
     return MOC_OK;
 }

@@ -109,7 +109,11 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
         fence_barrier_init();
     }
     __syncthreads();
-    if (s_total <= (int)blockIdx.x) return;
+    next_may_start();
+    if (s_total <= (int)blockIdx.x) {
+        if (ANCHOR && blockIdx.x == 0) previous_done();
+        return;
+    }
     if (warp == 8) {
         tmem_alloc(smem_u32(&tmem_slot), 512);
         tmem_relinquish();
@@ -241,6 +245,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
             tmem_wait_ld();
             tc_fence_before();
             mbar_arrive(bar(ACC_FREE));                      // the next item's dQ may be accumulated
+            if (ANCHOR) previous_done();                     // the routed launch's partials are complete
             if (e < 0) continue;
             int qi = e, slot = 0;
             if (!ANCHOR) {
@@ -484,6 +489,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
     tc_fence_before();
     __syncthreads();
     if (warp == 8) tmem_dealloc(tmem, 512);
+    if (ANCHOR && blockIdx.x == 0) previous_done();      // an abandoned launch has not waited yet
 }
 
 template <int D>
@@ -534,7 +540,9 @@ static int dq_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat1
         a.items = p->d_qitems;
         a.item_lo = a.item_hi = nullptr;
         const long long n_anc = 2LL * a.n_items * hg;
-        attend_dq_tc_kernel<D, true><<<(unsigned)std::min<long long>(p->n_sm, n_anc), kDqThreads, smem[1], s>>>(tmK, tmV, a);
+        const unsigned anc_grid = (unsigned)std::min<long long>(p->n_sm, n_anc);
+        if (p->k > 0) MOC_CUDA_TRY(launch_early(attend_dq_tc_kernel<D, true>, anc_grid, kDqThreads, smem[1], s, tmK, tmV, a));
+        else attend_dq_tc_kernel<D, true><<<anc_grid, kDqThreads, smem[1], s>>>(tmK, tmV, a);
         MOC_LAUNCH_CHECK();
     }
     return MOC_OK;

@@ -124,6 +124,22 @@ void set_cuda_error(cudaError_t e, const char *where);
         }                                                          \
     } while (0)
 
+// A kernel that may start while the kernel before it in the stream still runs: once every block of that one has called
+// next_may_start() or has left.  It calls previous_done() where it needs the other's results; and a kernel has to see to it
+// that it does not finish before the previous one, for the sake of what follows in the stream.
+__device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void previous_done() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... P, typename... A>
+static inline cudaError_t launch_early(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A &&...args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid); c.blockDim = dim3(block); c.dynamicSmemBytes = smem; c.stream = s;
+    c.attrs = &at; c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
+}
+
 template <typename T>
 static inline T *ws_ptr(void *ws, size_t off) { return reinterpret_cast<T *>(static_cast<char *>(ws) + off); }
 template <typename T>
