@@ -588,7 +588,7 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
     if (smem < tiles) return MOC_ERR_SHAPE;
     MOC_CUDA_TRY(cudaFuncSetAttribute(attend_dkv_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (int r = launch_dq_tc(p, Q, K, V, lse, delta, dO, dQ, ws, s)) return r;
-    MOC_CUDA_TRY(launch_early(attend_dkv_tc_kernel<D>, (unsigned)(p->ktiles.size() * (size_t)p->H), kBwdThreads, smem, s, tmK, tmV, tmQ, tmdO, a));
+    MOC_CUDA_TRY(launch_early(backward_overlaps(p), attend_dkv_tc_kernel<D>, (unsigned)(p->ktiles.size() * (size_t)p->H), kBwdThreads, smem, s, tmK, tmV, tmQ, tmdO, a));
     MOC_LAUNCH_CHECK();
     return MOC_OK;
 }

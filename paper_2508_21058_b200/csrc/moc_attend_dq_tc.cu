@@ -541,8 +541,7 @@ static int dq_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat1
         a.item_lo = a.item_hi = nullptr;
         const long long n_anc = 2LL * a.n_items * hg;
         const unsigned anc_grid = (unsigned)std::min<long long>(p->n_sm, n_anc);
-        if (p->k > 0) MOC_CUDA_TRY(launch_early(attend_dq_tc_kernel<D, true>, anc_grid, kDqThreads, smem[1], s, tmK, tmV, a));
-        else attend_dq_tc_kernel<D, true><<<anc_grid, kDqThreads, smem[1], s>>>(tmK, tmV, a);
+        MOC_CUDA_TRY(launch_early(p->k > 0 && backward_overlaps(p), attend_dq_tc_kernel<D, true>, anc_grid, kDqThreads, smem[1], s, tmK, tmV, a));
         MOC_LAUNCH_CHECK();
     }
     return MOC_OK;
