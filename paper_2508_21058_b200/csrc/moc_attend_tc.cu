@@ -166,6 +166,9 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    // Launched early (see moc_common.cuh): barriers and tensor memory are set up while the routing's last launch runs; from
+    // here on what it wrote is read.
+    previous_done();
     const uint32_t tmem = tmem_slot;
     volatile int *abort_flag = &s_abort;
     int *phase_tab = p.queue + kQueueHeader;
@@ -961,7 +964,7 @@ static int attend_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfl
     // one CTA per SM, never more than there can be items
     const long long most = (long long)p->H * (a.n_aitems + ((long long)p->L * p->k + kQTileRows - 1) / kQTileRows + (p->k ? p->C : 0));
     const unsigned grid = (unsigned)std::max(1LL, std::min<long long>(p->n_sm, most));
-    attend_tc_kernel<D, LOADERS><<<grid, LOADERS ? kThreadsLoaders : kThreads, smem, s>>>(tmQ, tmQrow, tmK, tmV, a);
+    MOC_CUDA_TRY(launch_early(true, attend_tc_kernel<D, LOADERS>, grid, LOADERS ? kThreadsLoaders : kThreads, smem, s, tmQ, tmQrow, tmK, tmV, a));
     MOC_LAUNCH_CHECK();
     return MOC_OK;
 }
