@@ -974,8 +974,8 @@ int launch_attend_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloa
     // Who loads the query tiles.  A row gather costs the warp that issues it some 65 cycles for four rows of 128 bytes: with
     // one warp a 256-row routed item cannot start more often than every 13000 cycles (half that at d = 64), with four every
     // 3000 to 4000 - but four loading warps, one on every scheduler, are in the way of the softmax.  The line lies at four
-    // key tiles a chunk, d = 128 (one warp -> four): 256-token chunks 24.4 -> 22.9 ms, 512-token chunks 27.2 -> 26.6 ms,
-    // 1560-token frames 3.42 -> 3.50 ms; 256-token chunks at d = 64: 462 -> 472 us (training step).
+    // key tiles a chunk, d = 128 (one warp -> four): 256-token chunks 23.3 -> 21.8 ms, 512-token chunks 26.4 -> 25.5 ms,
+    // 1560-token frames 3.54 -> 3.65 ms; 256-token chunks at d = 64: 462 -> 472 us (training step).
     if (p->d == 64) return attend_tc_d<64, false>(p, Q, K, V, O, lse, ws, s);
     const bool loaders = p->k > 0 && p->routed_key_tiles <= 4LL * p->ncol;
     return loaders ? attend_tc_d<128, true>(p, Q, K, V, O, lse, ws, s) : attend_tc_d<128, false>(p, Q, K, V, O, lse, ws, s);
