@@ -433,9 +433,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
         }
     } else {
         // ------------------------------------------------------------ MMA issuers: warp 12 owns the T1 / P side
-        // (T1, ACC2), warp 13 the T2 / dS side (T2, ACC1); each side's TMEM columns are touched by its issuer only,
-        // so the two instruction streams need no ordering between them and one's waits and commits are
-        // covered by the other's MMAs.  Warps 14 and 15 idle.
+        // (T1, ACC2), warp 13 the T2 / dS side (T2, ACC1); each side's TMEM columns are touched by its issuer only, so the two
+        // instruction streams need no ordering between them and one's waits and commits are covered by the other's MMAs.
+        // The streamed tiles are read by both sides: each waits for every tile of either ring that it reads (Q: T1 and
+        // ACC1, whose dS(j) follows T1(j); dO: T2 and ACC2, which nothing else orders).  Warps 14 and 15 idle.
         asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
         if (warp <= 13) {                       // the warp stays together, one lane of it issues
             const bool side1 = uniform(warp) == 12;
@@ -497,6 +498,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                 int s3n = 1 % kY1Stages, ph3n = 0;                       // stage and phase of tile j + 1
                 for (int j = 0; ok && j < n_tiles; ++j) {
                     const bool more = j + 1 < n_tiles;
+                    wait(Y2_FULL + (j & 1), (j >> 1) & 1, BW_YFULL);             // dO of the tile: P(j) comes of Q alone
                     wait(P_HALF, j & 1, BW_PDONE);
                     if (!ok) break;
                     tc_fence_after();
