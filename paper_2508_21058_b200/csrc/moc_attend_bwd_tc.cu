@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
     constexpr int CH = D / 8;               // 16-byte pieces per row
     constexpr int N_TILES_SMEM = 2 + kY1Stages + kY2Stages;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bars[23];
+    __shared__ __align__(8) uint64_t bars[24];
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort;
     __shared__ int w_valid, w_h, w_rows, w_ntiles, w_chunk, w_t0;
@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
     const uint32_t sX = sbase, sY1 = sbase + 2 * TILE_BYTES, sY2 = sbase + (2 + kY1Stages) * TILE_BYTES;
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
     constexpr int X_FULL = 0, Y1_FULL = 1, Y1_EMPTY = 4, Y2_FULL = 7, Y2_EMPTY = 9, T1_FULL = 11, T2_FULL = 13,
-                  P_HALF = 15, P_DONE = 16, DS_DONE = 17, ACC_FULL = 19, T1_ISSUED = 20, RD1 = 21, RD2 = 22;
+                  P_HALF = 15, P_DONE = 16, DS_DONE = 17, ACC_FULL = 19, T1_ISSUED = 20, RD1 = 22, RD2 = 23;
 
     if (threadIdx.x == 0) {
         s_abort = 0;
@@ -125,10 +125,10 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             mbar_init(bar(T1_FULL + t), 1);
             mbar_init(bar(T2_FULL + t), 1);
             mbar_init(bar(DS_DONE + t), 256);
+            mbar_init(bar(T1_ISSUED + t), 1);
         }
         mbar_init(bar(P_HALF), 256);
         mbar_init(bar(P_DONE), 256);
-        mbar_init(bar(T1_ISSUED), 1);
         mbar_init(bar(RD1), 256);
         mbar_init(bar(RD2), 256);
         mbar_init(bar(ACC_FULL), 2);                                // both issuers
@@ -514,7 +514,9 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                     }
                     if (++s3n == kY1Stages) { s3n = 0; ph3n ^= 1; }
                     tc_commit_elect(bar(Y2_EMPTY + (j & 1)));                    // the second of two arrivals
-                    if (more && lane == 0) mbar_arrive(bar(T1_ISSUED));          // the other side may use the pipe again
+                    // the other side may use the pipe again.  Two barriers: nothing keeps this side from arriving for tile j + 1 before
+                    // the other has looked at tile j's, and a wait by parity misses a phase that another one has followed.
+                    if (more && lane == 0) mbar_arrive(bar(T1_ISSUED + (j & 1)));
                 }
             } else {
                 // The lanes wait for T1(j+1) as soon as dS(j) is done, so this side keeps out of the pipe while the
@@ -532,7 +534,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                 for (int j = 0; ok && j < n_tiles; ++j) {
                     const int jn = j + 1;
                     const bool more = jn < n_tiles;
-                    if (more) wait(T1_ISSUED, j & 1, BW_T1FULL);
+                    if (more) wait(T1_ISSUED + (j & 1), (j >> 1) & 1, BW_T1FULL);
                     wait(DS_DONE + (j & 1), (j >> 1) & 1, BW_DSDONE);
                     if (!ok) break;
                     tc_fence_after();

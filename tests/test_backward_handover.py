@@ -12,8 +12,8 @@ Y1, Y2 = 3, 2                                            # stages of the Q and d
 # what the loop of each issuing warp does per tile, in order: (wait | commit | arrive, barrier, parity) and its MMA groups;
 # "+": only where there is a next tile
 SIDE1 = ["wait Y2_FULL + (j & 1), (j >> 1) & 1", "wait P_HALF, j & 1", "acc2 0", "+wait Y1_FULL + s3n, ph3n", "wait P_DONE, j & 1", "acc2 1",
-         "+t1", "+commit T1_FULL + ((j + 1) & 1)", "commit Y2_EMPTY + (j & 1)", "+arrive T1_ISSUED"]
-SIDE2 = ["+wait T1_ISSUED, j & 1", "wait DS_DONE + (j & 1), (j >> 1) & 1", "acc1", "commit Y1_EMPTY + s3",
+         "+t1", "+commit T1_FULL + ((j + 1) & 1)", "commit Y2_EMPTY + (j & 1)", "+arrive T1_ISSUED + (j & 1)"]
+SIDE2 = ["+wait T1_ISSUED + (j & 1), (j >> 1) & 1", "wait DS_DONE + (j & 1), (j >> 1) & 1", "acc1", "commit Y1_EMPTY + s3",
          "+wait Y2_FULL + (jn & 1), (jn >> 1) & 1", "+t2", "+commit T2_FULL + (jn & 1)", "+commit Y2_EMPTY + (jn & 1)"]
 
 
@@ -168,11 +168,18 @@ def test_the_model_is_of_this_source():
     assert source_ops(side2) == [op.lstrip("+") for op in SIDE2] + ["commit ACC_FULL"]
 
 
-def test_every_reader_finds_its_tile():
-    assert any(list(_schedules(SIDE1, SIDE2)))
+def test_every_reader_finds_its_tile_and_every_warp_ends():
+    assert all(list(_schedules(SIDE1, SIDE2)))
 
 
 @pytest.mark.parametrize("missing", ["wait Y2_FULL + (j & 1), (j >> 1) & 1", "wait P_DONE, j & 1", "+wait Y1_FULL + s3n, ph3n"])
 def test_the_model_sees_a_missing_wait(missing):
     with pytest.raises(WrongTile):
         list(_schedules([op for op in SIDE1 if op != missing], SIDE2))
+
+
+def test_the_model_sees_a_barrier_that_gets_two_phases_ahead():
+    """One barrier in the place of the pair: the dS side, held back, misses a phase and waits for good."""
+    one = [[op.replace("T1_ISSUED + (j & 1), (j >> 1) & 1", "T1_ISSUED, j & 1").replace("T1_ISSUED + (j & 1)", "T1_ISSUED") for op in ops]
+           for ops in (SIDE1, SIDE2)]
+    assert not all(list(_schedules(*one)))
