@@ -280,7 +280,10 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     up(o_reach, reach.data(), 4 * C);
     up(o_colc, col_chunk.data(), 4 * col_chunk.size());
     up(o_shots, p->shot_chunks.data(), sizeof(KeyRange) * p->shot_chunks.size());
+    // A copy from pageable memory may return while the last of it is still on its way, and a caller's non-blocking stream is
+    // not ordered behind the stream of the copy: the plan is handed out when the tables are there.
     e = cudaMemcpy(b, host.data(), o, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) { set_cuda_error(e, "cudaMemcpy(plan tables)"); cudaFree(p->d_blob); delete p; return MOC_ERR_CUDA; }
     p->d_off = (int32_t *)(b + o_off); p->d_shot = (int32_t *)(b + o_shot); p->d_mod = (uint8_t *)(b + o_mod);
     p->d_tok_chunk = (int32_t *)(b + o_tok); p->d_anc_bits = (uint32_t *)(b + o_bits);

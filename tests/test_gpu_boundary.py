@@ -254,3 +254,26 @@ def test_many_short_items_in_a_row_never_wait_for_good():
         run.ws.random_(0, 256)
         run.forward()                                                # checks the device status
         assert torch.equal(O, run.O) and torch.equal(lse, run.lse)
+
+
+@pytest.mark.parametrize("name", ["mini2", "cfg1"])              # tables of 20 KB, and of 150 KB
+def test_a_new_plans_tables_are_there_for_a_stream_of_any_kind(name):
+    """A plan made while the copy engine is busy, and used at once on a non-blocking stream."""
+    wl = W.workload(name)
+    wl.n_heads = 2
+    x = W.generate(wl, "cuda", ("q", "k", "v"))
+    want = MocPlan.from_workload(wl).forward(x["q"], x["k"], x["v"])[:4]
+    host, dev = torch.empty(1 << 28, dtype=torch.uint8, pin_memory=True), torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+    copies, side = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    plans = []                                                   # closing one would wait for the whole device
+    for _ in range(6):
+        with torch.cuda.stream(copies):
+            for _ in range(4):
+                dev.copy_(host, non_blocking=True)
+        plan = MocPlan.from_workload(wl)
+        plans.append(plan)
+        with torch.cuda.stream(side):
+            *got, ws = plan.forward(x["q"], x["k"], x["v"])
+            assert plan.moc_get_status(ws)[0] == 0               # waits for the side stream alone
+            assert all(torch.equal(a, b) for a, b in zip(got, want))
