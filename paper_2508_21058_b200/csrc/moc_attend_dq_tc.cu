@@ -9,7 +9,7 @@
 //     threads (two per TMEM lane) turn T1 into P, then (P, T2) into dS, written back to TMEM as bf16
 //     ACC += dS K                        (A from TMEM, the K tile as an MN-major operand)
 //
-// One CTA per SM walks its items (a fixed stride through the launch's items, which are much alike): the tensor memory, the
+// One CTA per SM walks its items (an equal share of the launch's, which but for the empty ones are much alike): the tensor memory, the
 // barriers and the K/V rings live for the whole launch, and the next item's rows are fetched while the last tile of the current
 // one and its results are in work.  With a CTA per item, the launch of the CTA, its dependent look-ups and the gather of its
 // rows took 8000 cycles before the first product, of 42000 for an item of 13 key tiles.
@@ -140,6 +140,21 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
                                  (size_t)w.first + w.rows <= p.cap_total && w.nrng == 1, p.status, IX_BWD_ITEM_FIELDS))
             o.rows = 0;
         return o.rows > 0;
+    };
+    // The CTA's next item with rows, from `round` and `pos` on (which start at 0 and blockIdx.x).  Of an item of at most 128
+    // rows the second half has none, and such items come in patterns: a CTA that kept its place in every round would, the
+    // grid being even, take nothing but second halves, or, with chunks of 257 to 384 rows, only every other item.  So the
+    // place moves by three, an odd number, from round to round.  (Training steps, the place kept -> moved: 64 frames of 128
+    // tokens, 8 heads, no picks 484 -> 364 us; 256 of 64, 24 heads, 4 picks 3072 -> 2712 us.)
+    auto next_item = [&](int &round, int &pos, DqItem &o) -> bool {
+        while (round < s_total) {
+            const int x = round + pos;
+            round += gridDim.x;
+            pos += 3;
+            if (pos >= (int)gridDim.x) pos -= gridDim.x;
+            if (x < s_total && fetch(x, o)) return true;
+        }
+        return false;
     };
 
     if (warp < 8) {
@@ -311,9 +326,8 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
             prefetch_tensormap(&tmV);
             int n_k = 0, n_v = 0, s3 = 0, ph3 = 0;           // K and V tiles issued; K stage and its phase
             bool ok = true;
-            for (int x = blockIdx.x; ok && x < s_total; x += gridDim.x) {
-                DqItem w;
-                if (!fetch(x, w)) continue;
+            DqItem w;
+            for (int round = 0, pos = blockIdx.x; ok && next_item(round, pos, w);) {
                 TileIter it(p.rng + w.rng_off, w.nrng, w.t0, w.t1);
                 int t0, valid;
                 while (it.next(t0, valid)) {
@@ -351,11 +365,10 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
         const int lw = warp - 9;
         int n = 0;
         bool ok = true;
-        int x = blockIdx.x;
+        int round = 0, pos = blockIdx.x;
         for (bool more = true; ok && more; ++n) {
             DqItem w = {};
-            more = false;
-            for (; x < s_total && !more; x += gridDim.x) more = fetch(x, w);
+            more = next_item(round, pos, w);
             if (!more) w.rows = 0;
             int q[3];
             float lse[3], del[3];

@@ -134,3 +134,24 @@ def test_both_arms_describe_the_workload_with_the_same_config():
     wl = W.workload("cfg2")
     a, b = bench.config_of(wl, False, 1), bench.config_of(W.workload("cfg2"), False, 1)
     assert a == b and a["workload"] == "cfg2" and a["tokens"] == 264128 and a["top_k"] == 6 and a["backward"] is False
+
+
+@pytest.mark.parametrize("chunk", [64, 128, 300, 384, 640, 1560])
+def test_dq_rows_are_dealt_evenly_to_the_blocks(chunk):
+    """The walk of the dQ kernel's blocks (next_item): every 128-row half of the 256-row items is somebody's, once, and no
+    block has many more halves with rows in them than the mean, whatever the chunk length leaves empty."""
+    with open(os.path.join(ROOT, "paper_2508_21058_b200", "csrc", "moc_attend_dq_tc.cu")) as f:
+        step = int(re.search(r"pos \+= (\d+);", f.read()).group(1))
+    grid, per_chunk = 148, [min(256, chunk - r) for r in range(0, chunk, 256)]
+    for items in (100, 148, 1001, 7777):
+        seen, load = [], [0] * grid
+        for pos in range(grid):
+            block = pos
+            for first in range(0, 2 * items, grid):
+                x = first + pos
+                if x < 2 * items:
+                    seen.append(x)
+                    load[block] += per_chunk[(x >> 1) % len(per_chunk)] > 128 * (x & 1)
+                pos = (pos + step) % grid
+        assert sorted(seen) == list(range(2 * items))
+        assert max(load) <= 1.03 * sum(load) / grid + 2
