@@ -59,11 +59,11 @@ struct TopK {
 };
 
 // ---- the first columns of a list of 17 to 32 picks: candidates as 64-bit keys, high word the score as an integer of
-// the same order (-0 and +0 alike), low word the complement of the column, so that one integer compare orders them as the
-// result is ordered (score descending, then column ascending).
+// the same order (-0 and +0 alike, and a NaN, which is never picked, as -inf), low word the complement of the column, so that one
+// integer compare orders them as the result is ordered (score descending, then column ascending).
 constexpr uint32_t kNoScore = 0x007fffffu;      // high word of a score of -inf: nothing there
 __device__ __forceinline__ uint64_t score_key(float f, int col) {
-    asm("add.rn.f32 %0, %0, 0f00000000;" : "+f"(f));
+    asm("max.f32 %0, %0, 0fff800000;\n\tadd.rn.f32 %0, %0, 0f00000000;" : "+f"(f));
     const int b = __float_as_int(f);
     return (uint64_t)((uint32_t)b ^ ((uint32_t)(b >> 31) | 0x80000000u)) << 32 | (uint32_t)~col;
 }

@@ -76,3 +76,29 @@ def test_launches_that_overlap_leave_complete_results(name, heads):
     for again, ts in enumerate(got):
         for a, b in zip(want, ts):
             assert torch.equal(a, b), again
+
+
+@pytest.mark.parametrize("k", [9, 16, 17, 24, 31, 40])
+def test_a_nan_score_is_never_picked(k):
+    """Keys with a NaN make their chunk's descriptor NaN for every query of the head: the picks are what the clean stream gives
+    without that chunk (from a list one longer); a query with a NaN picks nothing."""
+    lay = W.make_layout(3, 8, 24, 33)                          # 72 score columns, the chunk among the first 32
+    wl = W.Workload("nan", 2, 64, lay, k, 1, 1)
+    longer = PU.GpuRun(W.Workload("nan", 2, 64, lay, k + 1, 1, 1)).forward().sel
+    run, chunk, row = PU.GpuRun(wl), 5, lay.n_tokens - 3
+    clean = run.forward().sel.clone()
+    t0, t1 = int(lay.chunk_off[chunk]), int(lay.chunk_off[chunk + 1])
+    run.x["k"][1, t0 + 1, 7] = float("nan")
+    run.x["q"][0, row, 3] = float("nan")
+    p = run.plan
+    p.moc_chunk_pool(run.x["k"], run.desc, run.ws)
+    p.moc_route(run.x["q"], run.desc, run.sel, run.ws)
+    run.check_status()
+    assert not bool((run.sel[1] == chunk).any()) and bool((clean[1] == chunk).any())
+    want = torch.full_like(run.sel[1], -1)
+    kept = longer[1] != chunk
+    for i in range(lay.n_tokens):
+        picks = longer[1, i][kept[i]][:k]
+        want[i, :len(picks)] = picks
+    assert torch.equal(run.sel[1], want)
+    assert bool((run.sel[0, row] == -1).all())
