@@ -83,7 +83,7 @@ struct moc_plan {
     int n_pool_units;
     int heads_per_group;                     // Hg: heads whose routed partials are held at once (attention runs group by group)
     size_t partials_budget;                  // bytes the routed partials may take; sets Hg
-    uint32_t cookie;                         // hash of the problem, written into a workspace this plan has routed on
+    uint32_t cookie;                         // hash of the problem and the heads per group, written into a workspace this plan has routed on
     uint32_t wait_us;                        // limit of the kernels' bounded waits (0 = default); tests shorten it
     // device tables (one allocation)
     void *d_blob;

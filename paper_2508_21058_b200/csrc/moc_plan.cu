@@ -33,6 +33,22 @@ static bool is_anchor(const moc_plan *p, int c, int j) {
     return true;
 }
 
+// FNV-1a over the problem and the heads per group: a workspace routed by one plan is not accepted by a plan of another problem,
+// nor under another budget (routing lays the attention's work queue out by groups of heads)
+static uint32_t plan_cookie(const moc_plan *p) {
+    uint32_t hsh = 2166136261u;
+    auto mix = [&](const void *data, size_t n) {
+        const unsigned char *b = static_cast<const unsigned char *>(data);
+        for (size_t i = 0; i < n; ++i) { hsh ^= b[i]; hsh *= 16777619u; }
+    };
+    const int32_t hdr[] = {p->H, p->L, p->d, p->C, p->k, p->win_back, p->win_fwd, (int32_t)(p->flags & MOC_FLAG_CAUSAL), p->heads_per_group};
+    mix(hdr, sizeof hdr);
+    mix(p->off.data(), p->off.size() * 4);
+    mix(p->shot.data(), p->shot.size() * 4);
+    mix(p->mod.data(), p->mod.size());
+    return hsh ? hsh : 1u;
+}
+
 // Workspace layout.  The routed partial outputs ([heads][L][k][d] bf16, k times the size of O) are held for
 // one group of Hg heads at a time; attention and its backward run group by group.  If all heads fit the plan's
 // budget there is one group and one buffer; otherwise two buffers of Hg heads each (consecutive groups
@@ -67,21 +83,7 @@ void layout_workspace(moc_plan *p) {
     w.fwd_end = o;
     w.delta = take(sizeof(float) * H * L);
     w.bwd_end = o;
-}
-
-// FNV-1a over the problem: a workspace routed by one plan is not accepted by a plan of another problem
-static uint32_t plan_cookie(const moc_plan *p) {
-    uint32_t hsh = 2166136261u;
-    auto mix = [&](const void *data, size_t n) {
-        const unsigned char *b = static_cast<const unsigned char *>(data);
-        for (size_t i = 0; i < n; ++i) { hsh ^= b[i]; hsh *= 16777619u; }
-    };
-    const int32_t hdr[] = {p->H, p->L, p->d, p->C, p->k, p->win_back, p->win_fwd, (int32_t)(p->flags & MOC_FLAG_CAUSAL)};
-    mix(hdr, sizeof hdr);
-    mix(p->off.data(), p->off.size() * 4);
-    mix(p->shot.data(), p->shot.size() * 4);
-    mix(p->mod.data(), p->mod.size());
-    return hsh ? hsh : 1u;
+    p->cookie = plan_cookie(p);
 }
 
 }  // namespace moc
@@ -240,7 +242,6 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     }
     p->partials_budget = (size_t)6 << 30;
     p->wait_us = 0;
-    p->cookie = plan_cookie(p);
     layout_workspace(p);
     // the fixed scratch of moc_chunk_pool_noalloc: its address is looked up here, where allocating is allowed
     if (int r = pool_scratch_prepare(dev)) { delete p; return r; }

@@ -214,6 +214,25 @@ def test_workspace_budget_groups_heads_and_results_do_not_change():
     assert e.value.code == ERR_TOO_LARGE
 
 
+def test_a_workspace_routed_under_another_budget_is_refused():
+    """The work queue in the workspace is laid out by groups of heads: with other groups it is not followed."""
+    wl = W.workload("mini2")
+    wl.n_heads = 5
+    run = PU.GpuRun(wl, tensors=("q", "k", "v", "do")).forward()
+    want = run.O.clone()
+    full = run.plan.workspace_bytes(False)
+    run.plan.moc_plan_set_workspace_budget(full - 3 * 2 * wl.n_tokens * wl.top_k * wl.head_dim)      # groups of 2, 2, 1
+    x, grads = run.x, [torch.full_like(run.O, 7.0) for _ in range(3)]
+    run.O.fill_(7.0)
+    run.plan.moc_attend(x["q"], x["k"], x["v"], run.sel, run.O, run.lse, run.ws)
+    run.plan.moc_attend_bwd(x["q"], x["k"], x["v"], run.O, run.lse, x["do"], run.sel, *grads, run.ws)
+    torch.cuda.synchronize()
+    assert run.plan.moc_get_status(run.ws)[0] == ERR_WORKSPACE
+    assert all(bool(torch.all(t == 7.0)) for t in (run.O, *grads))
+    run.forward()                                                    # routed again, it works
+    assert float((run.O.float() - want.float()).abs().max()) <= 1e-2
+
+
 def test_debug_build_checks_every_workspace_index_and_finds_nothing():
     """The same sources built with -DMOC_DEBUG check every index taken from the workspace; on a sound run
     they must stay silent (status 0) and give the same answers.  Runs in a child process: a process loads
