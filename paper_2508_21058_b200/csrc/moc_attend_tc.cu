@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
     constexpr int SUB = D / 64;            // 64-column (128-byte) sub-tiles per row
     constexpr int SUB_BYTES = 128 * 128;   // one sub-tile: 128 rows of 128 bytes
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bars[39];
+    __shared__ __align__(8) uint64_t bars[42];
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort, s_usable;      // s_usable: the workspace holds this plan's lists
     __shared__ ItemSlot s_item[2];
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
     // barrier indices (pairs: per query tile g, per K/V stage, or per item slot)
     constexpr int Q_FULL = 0, Q_EMPTY = 6, K_FULL = 9, K_EMPTY = 11, V_FULL = 13, V_EMPTY = 15, S_FULL = 17, P_HALF = 19, P_FULL = 21,
-                  O_FULL = 23, O_FREE = 25, TURN = 27, ITEM_FULL = 29, ITEM_EMPTY = 31, ROWS_DONE = 33, DEPEND = 37;
+                  O_FULL = 23, O_FREE = 25, TURN = 27, ITEM_FULL = 29, ITEM_EMPTY = 31, ROWS_DONE = 33, DEPEND = 41;
     constexpr int kItemReaders = 2 + 2 + 256 + (LOADERS ? 4 : 0);      // producer and bookkeeping lanes, two issuing warps, every softmax thread, loading warps
 
     if (threadIdx.x == 0) {
@@ -153,9 +153,8 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             mbar_init(bar(TURN + t), 128);
             mbar_init(bar(ITEM_FULL + t), 1);
             mbar_init(bar(ITEM_EMPTY + t), kItemReaders);
-            mbar_init(bar(ROWS_DONE + t), 128);        // [item slot][query tile]
-            mbar_init(bar(ROWS_DONE + 2 + t), 128);
         }
+        for (int t = 0; t < 8; ++t) mbar_init(bar(ROWS_DONE + t), 128);      // [item modulo 4][query tile]
         fence_barrier_init();
     }
     __syncthreads();
@@ -491,7 +490,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 else p.lse[(size_t)h * p.L + qi] = (pl ? big + __logf(wsum) : lse_own);
             }
             // this tile's rows are stored; the bookkeeping lane counts them once all 128 threads are here
-            mbar_arrive(bar(ROWS_DONE + 2 * sl + g));
+            mbar_arrive(bar(ROWS_DONE + 2 * ((n_item - 1) & 3) + g));
             ++n_mine;
         }
     } else if (warp == 8) {
@@ -554,11 +553,11 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             // land) is not in the way of the next item.  DEPEND is arrived on after the previous item's rows were
             // counted, that is after every softmax thread has passed its previous wait on it.
             // Its fence may take longer than the groups need for two items, and a barrier must not complete two phases
-            // that nobody has waited for in between: ROWS_DONE exists once per item slot, and the slot of item n + 1 is handed
-            // back only when item n has been counted, so item n + 3, the next to use the ROWS_DONE of item n + 1, is not
-            // published before this lane is about to wait for item n + 1.
+            // that nobody has waited for in between: the slot of item n + 2 is handed back only when item n + 1 has been
+            // counted, so item n + 4, the next to use the ROWS_DONE of item n, is not published before this lane has waited for
+            // item n.  (With one per slot, item n + 2 used it again, which is published while this lane may still be about to wait.)
             int n_item = 0;
-            uint32_t rows_phase = 0;                            // bit 2 slot + tile: parity of the next phase of that ROWS_DONE
+            uint32_t rows_phase = 0;                            // bit 2 (item modulo 4) + tile: parity of the next phase of that ROWS_DONE
             int pend_phase = -1, pend_rows = 0;                 // the item whose rows are still to be counted
             bool ok = true;
             while (ok) {
@@ -571,7 +570,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 if (pend_phase >= 0) {
                     const int n_qt = pend_rows > 128 ? 2 : 1;
                     for (int g = 0; ok && g < n_qt; ++g) {
-                        const int b = 2 * (sl ^ 1) + g;          // the pending item used the other slot
+                        const int b = 2 * ((n_item - 2) & 3) + g;          // the pending item is the one before this
                         ok = mbar_wait(bar(ROWS_DONE + b), (rows_phase >> b) & 1, abort_flag, p.status, W_ROWSDONE);
                         rows_phase ^= 1u << b;
                     }
