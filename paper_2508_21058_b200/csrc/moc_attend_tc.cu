@@ -737,7 +737,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             prefetch_tensormap(&tmQ);
             prefetch_tensormap(&tmQrow);
         }
-        int n_item = 0, n_qtile = 0;
+        int n_item = 0, n_qtile = 0, last_g = 0;       // last_g: query tile of the last one loaded or published
         uint32_t q_phase = 0;                          // bit 3 g + buffer: parity of the next phase of that Q_FULL
         bool ok = true, late = false;
         while (ok) {
@@ -749,8 +749,14 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 // Claimed early, an item's gathers are done before they are needed, but it is kept from a CTA that may be idle.
                 // After an anchor item (whose successors have plain tiles to load, and which end the queue), and when there
                 // are only a few items per CTA, the next one is claimed when the last S of this one has been issued.
-                if (ok && n_qtile > 0 && (late || total <= 2 * (int)gridDim.x))
-                    ok = mbar_wait(bar(Q_EMPTY + (n_qtile - 1) % 3), ((n_qtile - 1) / 3) & 1, abort_flag, p.status, W_QEMPTY);
+                if (ok && n_qtile > 0 && (late || total <= 2 * (int)gridDim.x)) {
+                    const int qb = (n_qtile - 1) % 3, qf = 3 * last_g + qb;
+                    // Where others load the tiles, the buffer's release before this one may be yet to come, and its phase would be
+                    // taken for this one's.  It has come when the item's last tile is there.  (That barrier's own phase
+                    // before was of an item that the softmax warps have left, and the next is of one not yet published.)
+                    if (LOADERS) ok = mbar_wait(bar(Q_FULL + qf), ((q_phase >> qf) & 1) ^ 1, abort_flag, p.status, W_QFULL);
+                    ok = ok && mbar_wait(bar(Q_EMPTY + qb), ((n_qtile - 1) / 3) & 1, abort_flag, p.status, W_QEMPTY);
+                }
                 const int t = (ok && usable && !*abort_flag && *(volatile int *)p.status == 0) ? atomicAdd(&p.queue[0], 1) : total;
                 if (t < total) {
                     int ph = 0;
@@ -785,7 +791,11 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
             if (!valid || !ok) break;
             const int n_qt = rows > 128 ? 2 : 1;
-            if (LOADERS) { n_qtile += n_qt; continue; }
+            last_g = n_qt - 1;
+            if (LOADERS) {
+                for (int g = 0; g < n_qt; ++g, ++n_qtile) q_phase ^= 1u << (3 * g + n_qtile % 3);
+                continue;
+            }
             for (int g = 0; ok && g < n_qt; ++g) {
                 const int qb = n_qtile % 3, qf = 3 * g + qb;
                 ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.status, W_QEMPTY);
