@@ -15,7 +15,8 @@
 // T2(j+1), and T1 / T2 are rewritten only after the contraction that reads the P / dS stored over them; ACC2(j) starts on the
 // first half of P(j) while the lanes form the second.
 // A tile takes 3300 cycles (33k-token clip) for 2048 cycles of MMAs at the pipe's best rate: P, dS and the wait for T1(j+1)
-// between them are one chain per tile (two tiles in flight would need 1024 columns of tensor memory).
+// between them are one chain per tile (at d = 128 two tiles in flight would need 768 columns of tensor memory, of 512; at d = 64,
+// where the accumulators take 64 columns each, a second T1 would fit).
 // 16 warps: 0-7 the lane threads (two per TMEM lane), 8-11 the producers, 12 and 13 the MMA issuers,
 // 14-15 idle (they complete the fourth warpgroup; the lanes take the registers the others give up).  Every mbarrier wait is
 // bounded; a wait that runs out flags the workspace status word and the CTA drains and leaves.
@@ -572,7 +573,7 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
     if (int r = make_tmap_2d_bf16(&tmdO, dO, (uint64_t)p->H * p->L, D, 64)) return r;
     BwdParams a;
     a.Q = Q; a.K = K; a.V = V; a.dO = dO; a.lse = lse; a.delta = delta;
-        a.cookie = p->cookie;
+    a.cookie = p->cookie;
     a.dK = dK; a.dV = dV;
     a.ktiles = p->d_ktiles; a.n_ktiles = (int)p->ktiles.size(); a.n_long = p->n_long_ktiles; a.off = p->d_off; a.ranc_off = p->d_ranc_off; a.ranc = p->d_ranc; a.cap_off = p->d_cap_off;
     a.cnt = ws_ptr<int>(ws, p->ws.cnt);

@@ -244,8 +244,8 @@ int launch_attend_bwd_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_b
                          const __nv_bfloat16 *O, const float *lse, const __nv_bfloat16 *dO, const int32_t *sel,
                          __nv_bfloat16 *dQ, __nv_bfloat16 *dK, __nv_bfloat16 *dV, void *ws, cudaStream_t s);
 // Whether the launches of the backward start while the one before still runs: up to 16 dK/dV blocks per SM.  Training steps,
-// in turn (one after another -> overlapping): 0.7 blocks per SM 178 -> 152 us, 4 464 -> 451 us; at 20 and 45 the two are alike
-// (6.42 / 6.47 and 14.3 / 14.4 ms), at 111 overlapping is the slower one (102.7 -> 103.2 ms, sixteen scenes).
+// in turn (one after another -> overlapping): 0.7 blocks per SM 158 -> 134 us, 4 447 -> 428 us; at 20, 45 and 111 the two are alike
+// (6.64 / 6.64, 14.16 / 14.16 and 102.9 / 102.3 ms, where the runs of one side differ by 0.7 %).
 inline bool backward_overlaps(const moc_plan *p) { return p->ktiles.size() * (size_t)p->H <= 16 * (size_t)p->n_sm; }
 int launch_dq_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat16 *K, const __nv_bfloat16 *V, const float *lse,
                  const float *delta, const __nv_bfloat16 *dO, __nv_bfloat16 *dQ, void *ws, cudaStream_t s);

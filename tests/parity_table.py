@@ -9,7 +9,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 def main():
-    src = os.environ.get("MOC_PARITY_DIR", os.path.join(ROOT, "gpurun_out", "parity"))      # the default of tests/parity_utils.py
+    src = os.environ.get("MOC_PARITY_DIR", os.path.join(ROOT, "build", "test_out", "parity"))      # the default of tests/parity_utils.py
     recs = {os.path.basename(f)[:-5]: json.load(open(f)) for f in sorted(glob.glob(os.path.join(src, "*.json")))}
     order = [n for n in ("cfg0", "cfg1", "cfg2", "cfg4") if n in recs] + sorted(n for n in recs if n.startswith("cfg3")) + \
         sorted(n for n in recs if not n.startswith("cfg"))

@@ -30,7 +30,7 @@ GUARD = 4096
 POISON = 0xA5
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-OUT_ROOT = os.path.join(ROOT, "gpurun_out")          # where a run leaves its outputs
+OUT_ROOT = os.path.join(ROOT, "build", "test_out")    # where a run leaves its outputs
 PARITY_DIR = os.environ.get("MOC_PARITY_DIR", os.path.join(OUT_ROOT, "parity"))
 
 
