@@ -983,16 +983,17 @@ int launch_attend_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloa
     // Who loads the query tiles.  A row gather costs the warp that issues it some 65 cycles for four rows of 128 bytes: with
     // one warp a 256-row routed item cannot start more often than every 13000 cycles (half that at d = 64), with four every
     // 3000 to 4000 - but four loading warps, one on every scheduler, are in the way of the softmax.  Measured, one warp -> four
-    // (d = 128; six heads of 264k tokens unless said otherwise):
+    // (d = 128; streams of 264k tokens):
     //   two key tiles a chunk and less: 24 heads of a clip in 64-, 128- and 256-token frames 688 -> 602, 644 -> 551, 722 -> 667 us;
-    //     256-token chunks, 2, 6, 12 and 23 picks 4.46 -> 4.37, 6.66 -> 6.36, 10.1 -> 9.7, 18.2 -> 17.2 ms;
-    //   three: 2, 6, 10, 15, 20 picks 5.14 -> 5.24, 7.63 -> 7.69, 10.12 -> 9.99, 13.35 -> 12.95, 17.5 -> 16.6 ms; 12 picks on a clip 1423 -> 1454 us;
-    //   four: 4, 8, 12, 16, 24, 32 picks 6.01 -> 6.09, 8.52 -> 8.80, 11.31 -> 11.40, 14.21 -> 14.09, 20.8 -> 20.0, 26.6 -> 25.3 ms; a clip, 4 picks
-    //     1136 -> 1184 us;
+    //     256-token chunks, 2, 6, 12 and 23 picks 4.46 -> 4.37, 6.66 -> 6.36, 10.1 -> 9.7, 18.2 -> 17.2 ms (6 heads);
+    //   three: 3 and 8 picks 11.52 -> 11.71, 18.08 -> 17.87 ms (12 heads); 2, 6, 10, 15 picks 5.14 -> 5.24, 7.63 -> 7.69, 10.12 -> 9.99,
+    //     13.35 -> 12.95 ms (6 heads);
+    //   four: 4, 8, 11, 14 picks 24.5 -> 25.1, 34.9 -> 35.9, 44.3 -> 44.1, 53.7 -> 52.2 ms (24 heads); 16, 24, 32 picks 14.21 -> 14.09, 20.8 -> 20.0,
+    //     26.6 -> 25.3 ms (6 heads); a clip, 4 picks 1136 -> 1184 us;
     //   five to twelve: 1 to 3 % slower with fewer than 16 picks, within 1 % with more (five, 32 picks: 3 % faster, in runs that differ by 4).
     // At d = 64 four are slower: 512-token chunks 16.0 -> 18.0 ms, a training step on 256-token chunks 429 -> 443 us.
     if (p->d == 64) return attend_tc_d<64, false>(p, Q, K, V, O, lse, ws, s);
-    const long long up_to = p->k >= 16 ? 4 : p->k > 8 ? 3 : 2;        // key tiles a chunk, on average
+    const long long up_to = p->k > 8 ? 4 : p->k > 6 ? 3 : 2;        // key tiles a chunk, on average
     const bool loaders = p->k > 0 && p->routed_key_tiles <= up_to * p->ncol;
     return loaders ? attend_tc_d<128, true>(p, Q, K, V, O, lse, ws, s) : attend_tc_d<128, false>(p, Q, K, V, O, lse, ws, s);
 }

@@ -16,10 +16,10 @@ SHAPES = {
     "four key tiles a chunk": (2, 128, (2, 16, 4, 512), 2),            # one query-loading warp: few picks
     "four key tiles and one key": (2, 128, (2, 16, 4, 513), 2),        # one, whatever the picks
     "two key tiles a chunk": (2, 128, (2, 16, 6, 256), 2),             # the last size with four loading warps whatever the picks
-    "two key tiles and one key": (2, 128, (2, 16, 10, 257), 8),        # the first size with one for up to 8 picks
-    "three key tiles, 9 picks": (2, 128, (2, 16, 9, 384), 9),          # the last size with four for 9 to 15 picks
-    "four key tiles, 15 picks": (1, 128, (2, 16, 10, 512), 15),        # the last number of picks with one at this size
-    "four key tiles, 16 picks": (1, 128, (2, 16, 10, 512), 16),        # the first with four
+    "two key tiles and one key": (2, 128, (2, 16, 8, 257), 6),         # the first size with one for up to 6 picks
+    "three key tiles, 7 picks": (2, 128, (2, 16, 8, 384), 7),          # the last size with four for 7 and 8
+    "four key tiles, 8 picks": (1, 128, (2, 16, 8, 512), 8),           # the last number of picks with one at this size
+    "four key tiles, 9 picks": (1, 128, (2, 16, 8, 512), 9),           # the first with four
     "one row past a tile": (7, 128, (2, 1, 11, 129), 9),               # items of 256 rows and of a few; a merge of 8 + 1 picks
     "one row short of two tiles": (2, 64, (2, 31, 9, 255), 8),         # a full merge batch
     "17 picks": (3, 64, (2, 1, 13, 65), 17),                           # the shortest sorted list, 26 columns
