@@ -26,12 +26,12 @@
 //   warp 8     lane 0, TMA producer: the K and V tiles of 128 keys, two stages each, 128-byte swizzle; the ring
 //              runs across items.  Lane 16, bookkeeping: waits for what an item depends on, and when the item's
 //              rows are stored adds them to the queue's count of completed rows (the one thread that pays for
-//              a device-wide fence per item);
+//              device-wide fences);
 //   warps 9, 10  one MMA-issuing warp per query tile g:  S_g(0), then  O_g += P_g V(j),  S_g(j + 1)  per key
 //              tile.  S = Q K^T takes both operands from shared memory, O += P V takes P from TMEM and V as an
 //              MN-major shared-memory operand; all accumulators live in TMEM (S0, S1, O0, O1 = 512 columns);
 //   warp 11    scheduler and Q loader: lane 0 claims the next item and hands its description to the others
-//              through a two-slot ring; then the warp loads the item's Q tiles (plain tiles for anchor items,
+//              through a ring of three slots; then the warp loads the item's Q tiles (plain tiles for anchor items,
 //              row gathers, four rows per lane, for routed ones) into a ring of three tile buffers, so the next
 //              item's first query tile is in place before the current item ends.  With short chunks four more warps,
 //              12 to 15, load the tiles, 32 rows each.
@@ -64,6 +64,7 @@ struct AttendParams {
     size_t cap_total;
     int *status;
     int H, L, C, k, hg, n_groups, n_aitems;
+    SlotDiv kdiv;
     float scale_log2;           // softmax scale * log2(e)
     uint32_t cookie;
 };
@@ -72,17 +73,28 @@ constexpr int kBN = 128;               // keys per tile
 constexpr int kThreads = 384;          // three warpgroups: softmax 0, softmax 1, {producer, two MMA issuers, scheduler}
 constexpr int kThreadsLoaders = 512;   // ... and a fourth one of Q loaders
 constexpr int kTmemCols = 512;         // S0/P0 [0,128) S1/P1 [128,256) O0 [256,384) O1 [384,512)
+constexpr int kItemSlots = 3;          // items handed over and not yet seen by every warp (no more than the ROWS_DONE allow)
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleThreshold = 8.0f;    // log2 units: O is rescaled only when the row max grows by more
 
 enum WaitCode { W_QFULL = 1, W_KFULL, W_VFULL, W_SFULL, W_PFULL, W_OFULL, W_KEMPTY, W_VEMPTY, W_TURN, W_PHALF,
-                W_QEMPTY, W_OFREE, W_ITEMFULL, W_ITEMEMPTY, W_ROWSDONE, W_DEPEND };
+                W_QEMPTY, W_OFREE, W_ITEMFULL, W_ITEMEMPTY, W_ROWSDONE, W_DEPEND, W_MERGE };
 
 // One claimed item, as the scheduler hands it over.
 struct ItemSlot {
     int valid;          // 0: the queue is empty, everyone leaves
     int routed, h, first, rows, nrng, ntiles, phase;
+    int qbuf;           // Q buffer of its first query tile
     const KeyRange *rng;
+};
+
+// Walks the ring of item slots: the slot of an item, and the phase of its barriers.
+struct SlotIter {
+    int at = 0;
+    uint32_t phase = 0;
+    __device__ __forceinline__ void next() {
+        if (++at == kItemSlots) { at = 0; phase ^= 1; }
+    }
 };
 
 // a bounded wait on a counter in global memory (another CTA adds to it)
@@ -103,6 +115,37 @@ __device__ __forceinline__ bool wait_count(const int *ctr, int need, volatile in
     }
 }
 
+constexpr float kLog2e = 1.4426950408889634f;
+
+// acc += w x (the bf16 pair u) where cond holds
+__device__ __forceinline__ void add_weighted_if(bool cond, uint64_t &acc, uint32_t u, float w) {
+    const uint64_t v = pack2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u)), w2 = pack2(w, w);
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t@p fma.rn.f32x2 %0, %1, %2, %0;\n\t}" : "+l"(acc) : "l"(v), "l"(w2), "r"((int)cond));
+}
+
+// Of a row's 64 columns lane i of four holds pairs 4 x + i (columns 8 x + 2 i, + 1) in word x; afterwards it holds
+// columns 16 i .. 16 i + 15.
+__device__ __forceinline__ void quad_transpose(uint32_t (&u)[8], int i) {
+    // word 2 y + z of lane i goes to word 4 z + i of lane y
+    uint32_t t[8];
+    // lanes two apart exchange the halves y / 2, then neighbours the words y % 2
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        const uint32_t other = __shfl_xor_sync(0xffffffffu, (i & 2) ? u[x] : u[4 + x], 2);
+        t[x] = (i & 2) ? other : u[x];                   // from the lane with bit 1 clear
+        t[4 + x] = (i & 2) ? u[4 + x] : other;           // from the lane with bit 1 set
+    }
+    // t[4 s + 2 b + z]: word 2 (2 (i / 2) + b) + z of lane (i & 1) + 2 s
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int z = 0; z < 2; ++z) {
+            const uint32_t other = __shfl_xor_sync(0xffffffffu, (i & 1) ? t[4 * s + z] : t[4 * s + 2 + z], 1);
+            u[4 * z + 2 * s] = (i & 1) ? other : t[4 * s + z];
+            u[4 * z + 2 * s + 1] = (i & 1) ? t[4 * s + 2 + z] : other;
+        }
+}
+
 // LOADERS: four more warps load the query tiles, for short routed items (see the rule where the kernel is launched)
 template <int D, bool LOADERS>
 __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
@@ -114,10 +157,10 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
     constexpr int SUB = D / 64;            // 64-column (128-byte) sub-tiles per row
     constexpr int SUB_BYTES = 128 * 128;   // one sub-tile: 128 rows of 128 bytes
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t bars[42];
+    __shared__ __align__(8) uint64_t bars[41 + 2 * kItemSlots + 8 * (D == 128 ? 2 : 3)];
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort, s_usable;      // s_usable: the workspace holds this plan's lists
-    __shared__ ItemSlot s_item[2];
+    __shared__ ItemSlot s_item[kItemSlots];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -126,7 +169,11 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
     // barrier indices (pairs: per query tile g, per K/V stage, or per item slot)
     constexpr int Q_FULL = 0, Q_EMPTY = 6, K_FULL = 9, K_EMPTY = 11, V_FULL = 13, V_EMPTY = 15, S_FULL = 17, P_HALF = 19, P_FULL = 21,
-                  O_FULL = 23, O_FREE = 25, TURN = 27, ITEM_FULL = 29, ITEM_EMPTY = 31, ROWS_DONE = 33, DEPEND = 41;
+                  O_FULL = 23, O_FREE = 25, TURN = 27, ROWS_DONE = 29, DEPEND = 37, ITEM_FULL = 38, ITEM_EMPTY = ITEM_FULL + kItemSlots,
+                  MERGED = ITEM_EMPTY + kItemSlots, MERGE = MERGED + 3;
+    constexpr int kMergeStages = D == 128 ? 2 : 3;                     // blocks of partials under way per softmax warp
+    // Who merges the routed partials how: see the epilogue of the anchor items.
+    constexpr bool kMergeInRegs = D == 128 && LOADERS;
     constexpr int kItemReaders = 2 + 2 + 256 + (LOADERS ? 4 : 0);      // producer and bookkeeping lanes, two issuing warps, every softmax thread, loading warps
 
     if (threadIdx.x == 0) {
@@ -151,9 +198,13 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             mbar_init(bar(O_FULL + t), 1);
             mbar_init(bar(O_FREE + t), 128);
             mbar_init(bar(TURN + t), 128);
+        }
+        for (int t = 0; t < kItemSlots; ++t) {
             mbar_init(bar(ITEM_FULL + t), 1);
             mbar_init(bar(ITEM_EMPTY + t), kItemReaders);
         }
+        for (int t = 0; t < 3; ++t) mbar_init(bar(MERGED + t), 4);            // the softmax warps of the tile
+        for (int t = 0; t < 8 * kMergeStages; ++t) mbar_init(bar(MERGE + t), 1);
         for (int t = 0; t < 8; ++t) mbar_init(bar(ROWS_DONE + t), 128);      // [item modulo 4][query tile]
         fence_barrier_init();
     }
@@ -171,77 +222,87 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
     const uint32_t tmem = tmem_slot;
     volatile int *abort_flag = &s_abort;
     int *phase_tab = p.queue + kQueueHeader;
+    // Before a query tile is loaded into a buffer (whose last S, Q_EMPTY, is done): the wait for the merge that its previous
+    // tile, if it was an anchor item's, did in it; `merges`: so will the tile to be loaded.
+    auto merged = [&](int qb, bool merges, uint32_t &used, uint32_t &phase) -> bool {
+        if (D != 128 || kMergeInRegs) return true;
+        bool done = true;
+        if ((used >> qb) & 1) {
+            done = mbar_wait(bar(MERGED + qb), (phase >> qb) & 1, abort_flag, p.status, W_MERGE);
+            phase ^= 1u << qb;
+        }
+        used = (used & ~(1u << qb)) | ((uint32_t)(merges && p.k > 0) << qb);
+        return done;
+    };
 
     if (warp < 8) {
         // ------------------------------------------------------------ softmax / epilogue groups
         // the row-per-thread softmax holds a whole 128-key row of S in registers: take the
         // registers the third warpgroup gives up
-        if (LOADERS) asm volatile("setmaxnreg.inc.sync.aligned.u32 208;");
-        else asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
         const int g = warp >> 2;                       // query tile of this group
         const int r = threadIdx.x & 127;               // row within the tile = TMEM lane
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t tS = tmem + g * 128 + lane_off, tP = tS, tO = tmem + 256 + g * 128 + lane_off;
         const float c = p.scale_log2;
-        // running counts that give every barrier's phase: items seen, items this group worked on, key tiles it
-        // processed, key tiles processed in two-tile items (the turn-taking of the exponentials)
-        int n_item = 0, n_mine = 0, n_s = 0, n_turn = 0, n_dep = 0;
+        // What gives every barrier's phase: of the running counts only the low bits, in one register.  (A row of S fills most of
+        // the registers: each one that lives through the loop over the tiles is one the loop lacks.)
+        enum : uint32_t { S_ODD = 1, TURN_ODD = 2, TURNED = 4, MINE_ODD = 8, DEP_ODD = 16, MERGE_AT = 5 };      // key tiles; key tiles in
+                                                       // two-tile items, any at all; items with this tile; DEPENDs; MERGE phases
+        uint32_t bits = 0;
+        int n_item = 0, last_phase = -1;               // items seen, modulo 12 (three slots, four ROWS_DONE)
         bool ok = true;
         while (ok) {
-            const int sl = n_item & 1;
-            ok = mbar_wait(bar(ITEM_FULL + sl), (n_item >> 1) & 1, abort_flag, p.status, W_ITEMFULL);
+            const int sl = n_item % kItemSlots;
+            ok = mbar_wait(bar(ITEM_FULL + sl), (n_item / kItemSlots) & 1, abort_flag, p.status, W_ITEMFULL);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             const ItemSlot it_ = s_item[sl];
             mbar_arrive(bar(ITEM_EMPTY + sl));
-            ++n_item;
+            n_item = n_item == 11 ? 0 : n_item + 1;
             if (!it_.valid) break;
             const int h = it_.h, rows = it_.rows, first = it_.first, group = it_.phase >> 1;
             const bool routed = it_.routed != 0, two = rows > 128;
-            // an item that depends on other items' rows (see the bookkeeping lane) is released through DEPEND, whose
-            // phase counts those items only
-            const bool dep = routed ? group >= 2 : p.k > 0;
-            const int dep_phase = n_dep & 1;
-            if (dep) ++n_dep;
-            if (g == 1 && !two) continue;               // this item has one query tile
-            const int rt = g * 128 + r;                 // row within the work item
-            int qi = -1, slot = 0;
-            if (rt < rows) {
-                if (routed) {
-                    const bool at_ok = index_ok((size_t)first + rt < p.cap_total, p.status, IX_LIST_POSITION);
-                    const int e = at_ok ? p.qlist[(size_t)h * p.cap_total + first + rt] : -1;
-                    qi = e / p.k;
-                    slot = e - qi * p.k;
-                    (void)index_ok(e >= 0 && qi < p.L, p.status, IX_LIST_ENTRY);
-                    if (e < 0 || qi >= p.L) qi = -1;         // never follow an entry that is not a row of this head
-                } else {
-                    qi = first + rt;
+            // an item that depends on other items' rows (see the bookkeeping lane) is released through DEPEND; the first of a
+            // phase speaks for the others
+            const bool dep = (routed ? group >= 2 : p.k > 0) && it_.phase != last_phase;
+            last_phase = it_.phase;
+            const uint32_t dep_phase = (bits & DEP_ODD) ? 1 : 0;
+            if (dep) bits ^= DEP_ODD;
+            if (g == 1 && !two) {                       // this item has one query tile
+                if (dep) {                              // ... and every thread sees every phase of DEPEND
+                    ok = mbar_wait(bar(DEPEND), dep_phase, abort_flag, p.status, W_DEPEND);
+                    ok = __all_sync(0xffffffffu, ok);
+                    const int b = ROWS_DONE + 2 * ((n_item - 1) & 3) + 1;
+                    mbar_arrive(bar(b));
                 }
+                continue;
+            }
+            const int rt = g * 128 + r;                 // row within the work item
+            // the list entry of a routed row is asked for here and looked at in the epilogue
+            int qi = -1, entry = -1;
+            if (rt < rows) {
+                if (!routed) qi = first + rt;
+                else if (index_ok((size_t)first + rt < p.cap_total, p.status, IX_LIST_POSITION))
+                    entry = p.qlist[(size_t)h * p.cap_total + first + rt];
             }
             // partials of the group in flight: even and odd groups alternate between two buffers
-            __nv_bfloat16 *part_o = p.part_o + (size_t)(group & 1) * p.part_stride;
-            const int h_loc = h - group * p.hg;
-            constexpr int NP = D / 8;                   // 16-byte pieces per row
-            constexpr int KW = 8;                       // slots whose merge weights live in registers
-            const int LB = (p.L + 127) >> 7;
-            uint4 *part16 = reinterpret_cast<uint4 *>(part_o);
+            const int h_loc = h - group * p.hg, LB = (p.L + 127) >> 7;
+            char *part = reinterpret_cast<char *>(p.part_o + (size_t)(group & 1) * p.part_stride);
             if (!routed && qi >= 0 && p.k > 0) {
-                // the epilogue will merge this row's routed partials: start them on their way into L2 now.  A 128-byte
-                // line holds one pair of pieces of four consecutive queries: every fourth query (and the tile's first) asks.
-                // (Few picks only: what all CTAs ask for ahead has to stay in L2 until it is read.)
+                // the epilogue will merge this row's routed partials: start them on their way into L2 now
+                // (few picks only: what all CTAs ask for ahead has to stay in L2 until it is read)
                 if ((qi & 31) == 0 || r == 0)
                     for (int s = 0; s < p.k; ++s) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.part_lse + part_lse_at(h, LB, p.k, qi, s)));
-                if (p.k <= KW && ((qi & 3) == 0 || r == 0))
-                    for (int s = 0; s < p.k; ++s)
-                        for (int cc = 0; cc < NP; cc += 2)
-                            asm volatile("prefetch.global.L2 [%0];" ::"l"(part16 + part_piece(h_loc, LB, p.k, NP, qi, s, cc)));
+                if (p.k <= 8)
+                    for (int x = 0; x < p.k * (D / 64); ++x) asm volatile("prefetch.global.L2 [%0];" ::"l"(part + part_line(h_loc, LB, p.k, D / 64, qi, 0) + ((size_t)x << 14)));
             }
 
             float m_run = -INFINITY, l_run = 0.f;
             TileIter it(it_.rng, it_.nrng);
             int t0, valid, jt = 0;
             while (it.next(t0, valid)) {
-                ok = mbar_wait(bar(S_FULL + g), n_s & 1, abort_flag, p.status, W_SFULL);
+                ok = mbar_wait(bar(S_FULL + g), bits & S_ODD, abort_flag, p.status, W_SFULL);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
@@ -274,11 +335,13 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 // The exponentials of the two query tiles take turns (tile 0 of key tile j, tile 1
                 // of j, tile 0 of j + 1, ...): each then has the arithmetic pipes to itself while
                 // the other tile's MMAs run, instead of both drifting into lock step.
-                // TURN + g is arrived on by group g when its exponentials of a key tile are done.  (Tile 0 waits for
+                // TURN + g is arrived on by group g when all but the last eight of its exponentials of a key tile are done: the
+                // hand-over takes about as long as those (after the last one: 33k-token clip 3.48 -> 3.42 ms, d = 64, 725-token
+                // frames 607 -> 572 us; at half time it cost 5 %).  (Tile 0 waits for
                 // tile 1's previous turn even at the start of an item: the barrier must never get two phases ahead of
                 // a group that has yet to wait on it.)
-                if (two && (g == 1 || n_turn > 0)) {
-                    ok = mbar_wait(bar(TURN + (g ^ 1)), (g == 1 ? n_turn : n_turn - 1) & 1, abort_flag, p.status, W_TURN);
+                if (two && (g == 1 || (bits & TURNED))) {
+                    ok = mbar_wait(bar(TURN + (g ^ 1)), ((bits & TURN_ODD) ? 1 : 0) ^ (g == 1 ? 0 : 1), abort_flag, p.status, W_TURN);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                 }
@@ -311,6 +374,13 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                         if (x & 1) sum_b = add2(sum_b, pack2(a0, a1));
                         else sum_a = add2(sum_a, pack2(a0, a1));
                         u[x] = bf16x2(a0, a1);
+                        if (ch == 3 && x == 11) {
+                            // (the compiler must neither put off what comes before nor bring forward what comes after)
+                            asm volatile("" ::"r"(u[x]), "r"(u[x - 1]), "r"(u[x - 2]) : "memory");
+                            if (two) mbar_arrive(bar(TURN + g));
+#pragma unroll
+                            for (int y = x + 1; y < 16; ++y) asm volatile("" : "+r"(v[3][2 * y]), "+r"(v[3][2 * y + 1]));
+                        }
                     }
                     tmem_st16(tP + ch * 16, u);
                     if (ch == 1) {
@@ -319,7 +389,6 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                         mbar_arrive(bar(P_HALF + g));
                     }
                 }
-                if (two) mbar_arrive(bar(TURN + g));
                 tmem_wait_st();
                 tc_fence_before();
                 mbar_arrive(bar(P_FULL + g));
@@ -327,44 +396,118 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 unpack2(add2(sum_a, sum_b), s0, s1);
                 l_run = l_run * alpha + (s0 + s1);
                 ++jt;
-                ++n_s;
-                if (two) ++n_turn;
+                bits ^= S_ODD;
+                if (two) bits = (bits ^ TURN_ODD) | TURNED;
             }
             if (!ok) break;
             // ---- epilogue
-            // The merge weights of the routed partials depend only on log-sum-exps: have them ready before
-            // the last P V lands.  wslot[s] = exp(lse_s - lse_total), w_own likewise for this pass's own part.
+            // what follows from the item's fields is worked out anew: kept from before the loop, it would take the loop's registers
+            // (d = 64, frames of 725 and 923 tokens: 588 -> 572, 562 -> 552 us)
+            int h_ = h, phase_ = it_.phase, first_ = first;
+            asm volatile("" : "+r"(h_), "+r"(phase_), "+r"(first_));
+            {
+            const int h = h_, group = phase_ >> 1, first = first_, h_loc = h - group * p.hg, LB = (p.L + 127) >> 7;
+            char *part = reinterpret_cast<char *>(p.part_o + (size_t)(group & 1) * p.part_stride);
+            // Results move in the 16 x 256-bit load shape of the tensor memory: of a 16-row half of the warp's rows, lane
+            // l holds rows l / 4 and l / 4 + 8, of every eight columns the two at 2 (l % 4).  Four lanes then write 128
+            // contiguous bytes of a row.  (A row per lane, 32 bytes at a time, a warp's store touched 32 lines, and the 64 of
+            // an item's partials kept the memory pipe busy for some 4000 cycles.)  A partial is stored with its columns in
+            // the order of the lanes; only O, in the end, is put in the order of the columns.
+            constexpr int CB = D / 64;                  // 64-column blocks
+            const int l4 = lane >> 2, l2 = lane & 3;
             const float inv_l = 1.f / l_run;
             const float lse_own = (m_run + log2f(l_run)) * kLn2;
-            float w_own = inv_l, big = lse_own, wsum = 1.f;
-            float wslot[KW];
-#pragma unroll
-            for (int s = 0; s < KW; ++s) wslot[s] = 0.f;
-            const float *pl = nullptr;
             // what this item depends on (an anchor item: the routed items of its group have stored all their partials;
             // a routed item: the anchor items two groups back have read the buffer it is about to store into) has been
-            // awaited by the bookkeeping lane, which then arrives on DEPEND, once per item
+            // awaited by the bookkeeping lane, which then arrives on DEPEND, once per phase of the queue
             if (dep) {
                 ok = mbar_wait(bar(DEPEND), dep_phase, abort_flag, p.status, W_DEPEND);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
             }
-            if (!routed && qi >= 0 && p.k > 0) {
-                pl = p.part_lse + part_lse_at(h, LB, p.k, qi, 0);        // slot s: pl[s * 128]
-                if (p.k <= KW) {
-                    float plv[KW];
+            if (routed) {
+                size_t line = 0;                        // where this row's partial goes
+                bool keep = false;
+                if (rt < rows) {
+                    const int q = p.kdiv.query(entry), slot = entry - q * p.k;
+                    (void)index_ok(entry >= 0 && q < p.L, p.status, IX_LIST_ENTRY);
+                    if (entry >= 0 && q < p.L) {         // never follow an entry that is not a row of this head
+                        line = part_line(h_loc, LB, p.k, CB, q, slot);
+                        keep = true;
+                        p.part_lse[part_lse_at(h, LB, p.k, q, slot)] = lse_own;
+                    }
+                }
+                ok = mbar_wait(bar(O_FULL + g), (bits & MINE_ODD) ? 1 : 0, abort_flag, p.status, W_OFULL);
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc_fence_after();
+                uint32_t o[2 * CB][32];
 #pragma unroll
-                    for (int s = 0; s < KW; ++s) plv[s] = s < p.k ? __ldcg(pl + s * 128) : -INFINITY;
+                for (int x = 0; x < 2 * CB; ++x) tmem_ld_16x256b(tO + ((x / CB) << 20) + (x % CB) * 64, o[x]);
+                tmem_wait_ld();
+                tc_fence_before();
+                mbar_arrive(bar(O_FREE + g));            // the issuer may start the next item's P V (which overwrites O)
 #pragma unroll
-                    for (int s = 0; s < KW; ++s) big = fmaxf(big, plv[s]);
-                    wsum = __expf(lse_own - big);
+                for (int j = 0; j < 4; ++j) {            // rows 8 j + l4 of the warp's 32
+                    const float w = __shfl_sync(0xffffffffu, inv_l, j * 8 + l4);
+                    const size_t at = __shfl_sync(0xffffffffu, line, j * 8 + l4);
+                    const bool some = __shfl_sync(0xffffffffu, keep, j * 8 + l4);
+                    const int q7 = (int)(at >> 7) & 7;       // the query modulo 8
+                    char *dst = part + at + ((kMergeInRegs ? l2 : l2 ^ (q7 >> 1)) << 5);
 #pragma unroll
-                    for (int s = 0; s < KW; ++s) { wslot[s] = __expf(plv[s] - big); wsum += wslot[s]; }     // exp(-inf) = 0: empty slot
+                    for (int cb = 0; cb < CB; ++cb) {
+                        const uint32_t (&v)[32] = o[(j >> 1) * CB + cb];
+                        uint32_t u[8];
 #pragma unroll
-                    for (int s = 0; s < KW; ++s) wslot[s] /= wsum;
-                } else {
+                        for (int x = 0; x < 8; ++x)
+                            u[x] = bf16x2(__uint_as_float(v[4 * x + 2 * (j & 1)]) * w, __uint_as_float(v[4 * x + 2 * (j & 1) + 1]) * w);
+                        if (!kMergeInRegs && (q7 & 1)) {
+#pragma unroll
+                            for (int x = 0; x < 4; ++x) { const uint32_t t = u[x]; u[x] = u[4 + x]; u[4 + x] = t; }
+                        }
+                        if (some) st_256(dst + (cb << 14), u);
+                    }
+                }
+            } else {
+                // The weights of the merge depend only on log-sum-exps: have their sum ready before the last P V lands.  Slot s of
+                // this lane's row counts exp(lse_s - big), its own part exp(lse_own - big) / l, and the sum is divided by wsum.
+                float big = lse_own, wsum = 1.f;
+                const bool merge = qi >= 0 && p.k > 0;
+                const float *pl = p.part_lse + part_lse_at(h, LB, p.k, max(qi, 0), 0);        // slot s: pl[s * 128]
+                // How the partials come.  With one loading warp, and at d = 64: by bulk copies, a 64-column block of one slot of the
+                // warp's 32 rows at a time, into the query tile's buffer, whose last S is done (at d = 64, where there is room, into
+                // space of the warp's own), two or three under way.  With short chunks at d = 128, where a row has many picks: by
+                // loads into registers, 400 to 800 bytes a thread under way, in the shape in which the partials are stored.  (Cycles
+                // for the epilogue of 256 rows, the loads of a row by its own thread before -> this: d = 128, 4 picks 15000 -> 13700 by
+                // copies, 22900 by register loads; d = 64, 25 picks 38500 -> 33000, 56900; the whole launch on 256-token chunks, 30 picks,
+                // 18.8 -> 13.8 ms by register loads, 15.2 by copies.)
+                const int q0 = first + g * 128 + (warp & 3) * 32, n_rows = min(32, first + rows - q0);   // the warp's rows
+                const int n_merge = n_rows > 0 ? p.k : 0;
+                const int qb = it_.qbuf + g < 3 ? it_.qbuf + g : it_.qbuf + g - 3;
+                const uint32_t m_base = D == 128 ? sQ + qb * TILE_BYTES + (warp & 3) * (TILE_BYTES / 4) : sbase + 7 * TILE_BYTES + warp * (kMergeStages * 4096);
+                int m_st = 0, m_next = 0, m_flight = 0;          // stage to read, block to ask for, blocks under way
+                int c_st = 0, c_slot = 0, c_cb = 0;
+                auto copy_next = [&]() {                         // the warp's next block
+                    if (lane == 0) {
+                        const uint32_t b = bar(MERGE + warp * kMergeStages + c_st), dst = m_base + c_st * 4096;
+                        const int n1 = min(n_rows, 128 - (q0 & 127));        // rows in the first block of 128 queries
+                        mbar_expect_tx(b, n_rows * 128);
+                        bulk_load(dst, part + part_line(h_loc, LB, p.k, CB, q0, c_slot) + ((size_t)c_cb << 14), n1 * 128, b);
+                        if (n1 < n_rows)
+                            bulk_load(dst + n1 * 128, part + part_line(h_loc, LB, p.k, CB, q0 + n1, c_slot) + ((size_t)c_cb << 14), (n_rows - n1) * 128, b);
+                    }
+                    ++m_next;
+                    ++m_flight;
+                    if (++c_st == kMergeStages) c_st = 0;
+                    if (++c_slot == p.k) { c_slot = 0; ++c_cb; }
+                };
+                if (!kMergeInRegs && n_merge > 0) {
+                    // other CTAs' stores, seen through DEPEND by the generic proxy, are read by the copy engine
+                    if (lane == 0) asm volatile("fence.proxy.async;" ::: "memory");
+                    for (int x = 0; x < kMergeStages && x < CB * p.k; ++x) copy_next();
+                }
+                if (merge) {
                     // eight slots requested together; running maximum and sum
-                    wsum = 1.f;
 #pragma unroll 1
                     for (int s0 = 0; s0 < p.k; s0 += 8) {
                         float plv[8], m = big;
@@ -378,137 +521,195 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                         for (int u = 0; u < 8; ++u) wsum += __expf(plv[u] - big);
                     }
                 }
-                w_own = __expf(lse_own - big) / wsum * inv_l;
-            }
-            ok = mbar_wait(bar(O_FULL + g), n_mine & 1, abort_flag, p.status, W_OFULL);
-            ok = __all_sync(0xffffffffu, ok);
-            if (!ok) break;
-            tc_fence_after();
-#pragma unroll 1
-            for (int ch = 0; ch < D / 32; ++ch) {
-                uint32_t v[32];
-                __syncwarp();
-                tmem_ld32(tO + ch * 32, v);
-                tmem_wait_ld();
-                if (ch == D / 32 - 1) {
-                    // O has been read: the issuer may start the next item's P V (which overwrites it)
-                    tc_fence_before();
-                    mbar_arrive(bar(O_FREE + g));
-                }
-                float acc[32];
+                const float inv_w = 1.f / wsum, w_own = __expf(lse_own - big) * inv_l, big_log2 = big * kLog2e;
+                if constexpr (kMergeInRegs) {
+                    // Four passes, eight of the warp's rows each, over the slots, a few at a time: the loads of the next few are on
+                    // their way while these are added up.
+                    constexpr int B = 3;
+                    const int row0 = first + g * 128 + (warp & 3) * 32 + l4, row_end = first + rows;   // query of row l4 of the warp's
+                    struct Batch { uint32_t v[B][CB][8]; float ls[B]; };
+                    int ask_pass = 0, ask_s = 0;
+                    auto ask = [&](Batch &b) __attribute__((always_inline)) {
+                        const int q = row0 + ask_pass * 8;
+                        const bool in = q < row_end;
+                        const char *src = part + part_line(h_loc, LB, p.k, CB, q, ask_s) + l2 * 32;
+                        const float *ls = p.part_lse + part_lse_at(h, LB, p.k, q, ask_s);
 #pragma unroll
-                for (int x = 0; x < 32; ++x) acc[x] = __uint_as_float(v[x]) * w_own;
-                if (pl && p.k <= KW) {
-                    // four slots' pieces of this column block are requested together: one round trip, not four
+                        for (int u = 0; u < B; ++u) {
+                            const bool some = in && ask_s + u < p.k;
+                            const float x = __ldcg(some ? ls + u * 128 : pl);
+                            b.ls[u] = some ? x : -INFINITY;
 #pragma unroll
-                    for (int s0 = 0; s0 < KW; s0 += 4) {
-                        if (s0 >= p.k) break;
-                        uint4 raw[4][4];
-#pragma unroll
-                        for (int s = 0; s < 4; ++s)
-#pragma unroll
-                            for (int q4 = 0; q4 < 4; q4 += 2) {
-                                raw[s][q4] = raw[s][q4 + 1] = make_uint4(0, 0, 0, 0);
-                                if (s0 + s < p.k && wslot[s0 + s] != 0.f)
-                                    ld_cg_256(part16 + part_piece(h_loc, LB, p.k, NP, qi, s0 + s, ch * 4 + q4), raw[s][q4], raw[s][q4 + 1]);
-                            }
-#pragma unroll
-                        for (int s = 0; s < 4; ++s) {
-                            const float w = wslot[s0 + s];
-#pragma unroll
-                            for (int q4 = 0; q4 < 4; ++q4) {
-                                const __nv_bfloat162 *b = reinterpret_cast<const __nv_bfloat162 *>(&raw[s][q4]);
-#pragma unroll
-                                for (int y = 0; y < 4; ++y) {
-                                    const float2 f = __bfloat1622float2(b[y]);
-                                    acc[q4 * 8 + 2 * y] = fmaf(w, f.x, acc[q4 * 8 + 2 * y]);
-                                    acc[q4 * 8 + 2 * y + 1] = fmaf(w, f.y, acc[q4 * 8 + 2 * y + 1]);
-                                }
-                            }
+                            for (int cb = 0; cb < CB; ++cb) ld_cg_256_if(some, src + ((size_t)(u * CB + cb) << 14), b.v[u][cb]);
                         }
-                    }
-                } else if (pl) {
-                    // Four slots requested together, their log-sum-exps a batch ahead.  (One slot at a time kept 16 KB in flight
-                    // per SM: 9 bytes a cycle, 220k cycles for the 2 MB of a 256-row item with 30 picks.)
-                    const float inv_w = 1.f / wsum;
-                    const uint4 *src = part16 + part_piece(h_loc, LB, p.k, NP, qi, 0, ch * 4);
-                    constexpr int SLOT = (NP / 2) * 256;       // pieces from one slot to the next
-                    float ls[4];
+                        ask_s += B;
+                        if (ask_s >= p.k) { ask_s = 0; ++ask_pass; }
+                    };
+                    uint64_t acc[CB][8];
+                    int pass = 0, s0 = 0;
+                    float row_big = 0.f;
+                    auto add = [&](const Batch &b) __attribute__((always_inline)) {
+                        const int src_lane = pass * 8 + l4;
+                        if (s0 == 0) {
+                            row_big = __shfl_sync(0xffffffffu, big_log2, src_lane);
+                            const float w = __shfl_sync(0xffffffffu, w_own, src_lane);
+                            const uint64_t w2 = pack2(w, w);
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) ls[u] = u < p.k ? __ldcg(pl + u * 128) : -INFINITY;
-#pragma unroll 1
-                    for (int s0 = 0; s0 < p.k; s0 += 4, src += 4 * SLOT) {
-                        uint4 raw[4][4];
-                        float w[4];
+                            for (int cb = 0; cb < CB; ++cb) {
+                                uint32_t o[32];
+                                tmem_ld_16x256b(tO + ((pass >> 1) << 20) + cb * 64, o);
+                                tmem_wait_ld();
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            w[u] = __expf(ls[u] - big) * inv_w;        // exp(-inf) = 0: empty slot
-#pragma unroll
-                            for (int q4 = 0; q4 < 4; q4 += 2) {
-                                raw[u][q4] = raw[u][q4 + 1] = make_uint4(0, 0, 0, 0);
-                                if (ls[u] != -INFINITY) ld_cg_256(src + u * SLOT + q4 * 128, raw[u][q4], raw[u][q4 + 1]);
+                                for (int x = 0; x < 8; ++x)
+                                    acc[cb][x] = mul2(pack2(__uint_as_float((pass & 1) ? o[x * 4 + 2] : o[x * 4]), __uint_as_float((pass & 1) ? o[x * 4 + 3] : o[x * 4 + 1])), w2);
+                            }
+                            if (pass == 3) {
+                                // O has been read: the issuer may start the next item's P V (which overwrites it)
+                                tc_fence_before();
+                                mbar_arrive(bar(O_FREE + g));
                             }
                         }
 #pragma unroll
-                        for (int u = 0; u < 4; ++u) ls[u] = s0 + 4 + u < p.k ? __ldcg(pl + (s0 + 4 + u) * 128) : -INFINITY;
+                        for (int u = 0; u < B; ++u) {
+                            // exp2(-inf) = 0: an empty slot, and what its place holds is not a number to use
+                            const float w = ex2(fmaf(b.ls[u], kLog2e, -row_big));
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
+                            for (int cb = 0; cb < CB; ++cb)
 #pragma unroll
-                            for (int q4 = 0; q4 < 4; ++q4) {
-                                const __nv_bfloat162 *b = reinterpret_cast<const __nv_bfloat162 *>(&raw[u][q4]);
+                                for (int x = 0; x < 8; ++x) add_weighted_if(w != 0.f, acc[cb][x], b.v[u][cb][x], w);
+                        }
+                        s0 += B;
+                        if (s0 >= p.k) {
+                            const float w = __shfl_sync(0xffffffffu, inv_w, src_lane);
+                            const int q = row0 + pass * 8;
 #pragma unroll
-                                for (int y = 0; y < 4; ++y) {
-                                    const float2 f = __bfloat1622float2(b[y]);
-                                    acc[q4 * 8 + 2 * y] = fmaf(w[u], f.x, acc[q4 * 8 + 2 * y]);
-                                    acc[q4 * 8 + 2 * y + 1] = fmaf(w[u], f.y, acc[q4 * 8 + 2 * y + 1]);
+                            for (int cb = 0; cb < CB; ++cb) {
+                                uint32_t u[8];
+#pragma unroll
+                                for (int x = 0; x < 8; ++x) {
+                                    float lo, hi;
+                                    unpack2(acc[cb][x], lo, hi);
+                                    u[x] = bf16x2(lo * w, hi * w);
                                 }
+                                quad_transpose(u, l2);                            // this lane: columns 16 l2 .. 16 l2 + 15
+                                if (q < row_end) st_256(p.O + ((size_t)h * p.L + q) * D + cb * 64 + l2 * 16, u);
                             }
+                            s0 = 0;
+                            ++pass;
+                        }
+                    };
+                    Batch even = {}, odd = {};
+                    ask(even);
+                    ok = mbar_wait(bar(O_FULL + g), (bits & MINE_ODD) ? 1 : 0, abort_flag, p.status, W_OFULL);
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    tc_fence_after();
+#pragma unroll 1
+                    while (pass < 4) {                           // an even number of passes, so of batches
+                        ask(odd);
+                        add(even);
+                        if (ask_pass < 4) ask(even);
+                        add(odd);
                     }
-                }
-                if (qi < 0) continue;
-                uint4 *dst_row = reinterpret_cast<uint4 *>(p.O + ((size_t)h * p.L + qi) * D + ch * 32);
-                uint4 out[4];
-#pragma unroll
-                for (int q4 = 0; q4 < 4; ++q4) {
-                    uint32_t *o32 = reinterpret_cast<uint32_t *>(&out[q4]);
-#pragma unroll
-                    for (int y = 0; y < 4; ++y) {
-                        __nv_bfloat162 b = __floats2bfloat162_rn(acc[q4 * 8 + 2 * y], acc[q4 * 8 + 2 * y + 1]);
-                        o32[y] = *reinterpret_cast<uint32_t *>(&b);
-                    }
-                }
-                if (routed) {            // whole 32-byte sectors
-                    st_256(part16 + part_piece(h_loc, LB, p.k, NP, qi, slot, ch * 4), out[0], out[1]);
-                    st_256(part16 + part_piece(h_loc, LB, p.k, NP, qi, slot, ch * 4 + 2), out[2], out[3]);
                 } else {
+                    ok = mbar_wait(bar(O_FULL + g), (bits & MINE_ODD) ? 1 : 0, abort_flag, p.status, W_OFULL);
+                    ok = __all_sync(0xffffffffu, ok);
+                    tc_fence_after();
+                    float ls1 = merge ? __ldcg(pl) : -INFINITY, ls2 = merge ? __ldcg(pl + min(1, p.k - 1) * 128) : -INFINITY;      // the next two slots'
+                    const int row7 = (q0 + lane) & 7;
+#pragma unroll 1
+                    for (int cb = 0; ok && cb < CB; ++cb) {
+                        uint64_t acc[32];                            // columns 2 x, 2 x + 1 of the block
+                        const uint64_t w2 = pack2(w_own, w_own);
 #pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) dst_row[q4] = out[q4];
+                        for (int x = 0; x < 2; ++x) {
+                            uint32_t o[32];
+                            __syncwarp();
+                            tmem_ld32(tO + cb * 64 + x * 32, o);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int y = 0; y < 16; ++y) acc[x * 16 + y] = mul2(pack2(__uint_as_float(o[2 * y]), __uint_as_float(o[2 * y + 1])), w2);
+                        }
+                        if (cb == CB - 1) {
+                            // O has been read: the issuer may start the next item's P V (which overwrites it)
+                            tc_fence_before();
+                            mbar_arrive(bar(O_FREE + g));
+                        }
+#pragma unroll 1
+                        for (int s = 0; s < n_merge; ++s) {
+                            const float w = ex2(fmaf(ls1, kLog2e, -big_log2));       // exp2(-inf) = 0: an empty slot
+                            ls1 = ls2;
+                            const int s2 = s + 2 < p.k ? s + 2 : s + 2 - p.k;       // (the next block's first slots after the last)
+                            ls2 = merge ? __ldcg(pl + min(s2, p.k - 1) * 128) : -INFINITY;
+                            ok = mbar_wait(bar(MERGE + warp * kMergeStages + m_st), (bits >> (MERGE_AT + m_st)) & 1, abort_flag, p.status, W_MERGE);
+                            ok = __all_sync(0xffffffffu, ok);
+                            if (!ok) break;
+                            const uint32_t src = m_base + m_st * 4096 + lane * 128;
+#pragma unroll
+                            for (int c16 = 0; c16 < 8; ++c16) {
+                                // what an empty slot's place holds is not a number to use
+                                uint32_t v[4];
+                                ld_shared_128(src + ((c16 ^ row7) << 4), v);
+#pragma unroll
+                                for (int y = 0; y < 4; ++y) add_weighted_if(w != 0.f, acc[((c16 & 1) * 4 + y) * 4 + (c16 >> 1)], v[y], w);
+                            }
+                            __syncwarp();
+                            bits ^= 1u << (MERGE_AT + m_st);
+                            --m_flight;
+                            if (m_next < CB * p.k) copy_next();
+                            if (++m_st == kMergeStages) m_st = 0;
+                        }
+                        if (ok && qi >= 0) {
+#pragma unroll
+                            for (int x = 0; x < 4; ++x) {
+                                uint32_t u[8];
+#pragma unroll
+                                for (int y = 0; y < 8; ++y) {
+                                    float lo, hi;
+                                    unpack2(acc[x * 8 + y], lo, hi);
+                                    u[y] = bf16x2(lo * inv_w, hi * inv_w);
+                                }
+                                st_256(p.O + ((size_t)h * p.L + qi) * D + cb * 64 + x * 16, u);
+                            }
+                        }
+                    }
+                    if (!ok) {       // copies under way must land before the shared memory is released
+                        int dummy_flag = 0;
+                        for (; m_flight > 0; --m_flight) {
+                            mbar_wait(bar(MERGE + warp * kMergeStages + m_st), (bits >> (MERGE_AT + m_st)) & 1, &dummy_flag, p.status, W_MERGE);
+                            bits ^= 1u << (MERGE_AT + m_st);
+                            if (++m_st == kMergeStages) m_st = 0;
+                        }
+                        break;
+                    }
+                    if (D == 128 && p.k > 0) {                   // the Q buffer is no longer in use
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(bar(MERGED + qb));
+                    }
                 }
+                if (qi >= 0) p.lse[(size_t)h * p.L + qi] = merge ? big + __logf(wsum) : lse_own;
             }
-            if (qi >= 0) {
-                if (routed) p.part_lse[part_lse_at(h, LB, p.k, qi, slot)] = lse_own;
-                else p.lse[(size_t)h * p.L + qi] = (pl ? big + __logf(wsum) : lse_own);
             }
             // this tile's rows are stored; the bookkeeping lane counts them once all 128 threads are here
             mbar_arrive(bar(ROWS_DONE + 2 * ((n_item - 1) & 3) + g));
-            ++n_mine;
+            bits ^= MINE_ODD;
         }
     } else if (warp == 8) {
-        if (LOADERS) asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        if (LOADERS) asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
         else asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         if (lane == 0) {
             // ------------------------------------------------------------ TMA producer of the K and V tiles
             prefetch_tensormap(&tmK);
             prefetch_tensormap(&tmV);
-            int n_item = 0, n_kv = 0;                         // items seen, K/V tiles issued
+            int n_kv = 0;                                     // K/V tiles issued
+            SlotIter slot_it;
             int k_last = -1, v_last = -1;                     // last tile whose K / V copy was issued
             bool ok = true;
             while (ok) {
-                const int sl = n_item & 1;
-                if (!mbar_wait(bar(ITEM_FULL + sl), (n_item >> 1) & 1, abort_flag, p.status, W_ITEMFULL)) break;
-                const ItemSlot it_ = s_item[sl];
-                mbar_arrive(bar(ITEM_EMPTY + sl));
-                ++n_item;
+                if (!mbar_wait(bar(ITEM_FULL + slot_it.at), slot_it.phase, abort_flag, p.status, W_ITEMFULL)) break;
+                const ItemSlot it_ = s_item[slot_it.at];
+                mbar_arrive(bar(ITEM_EMPTY + slot_it.at));
+                slot_it.next();
                 if (!it_.valid) break;
                 const int h = it_.h;
                 // the ring of stages runs on from the previous item
@@ -548,38 +749,49 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             // then, when the softmax groups have stored the item's rows, the rows join the phase's count.  The
             // groups' arrivals order their stores before this thread (CTA scope); its fence makes them visible
             // device-wide before the count moves.
-            // An item that depends on nothing does not go through DEPEND at all; the rows of an item are counted when
-            // the next item has been seen, so that the fence before the count (it waits for the item's stores to
-            // land) is not in the way of the next item.  DEPEND is arrived on after the previous item's rows were
-            // counted, that is after every softmax thread has passed its previous wait on it.
-            // Its fence may take longer than the groups need for two items, and a barrier must not complete two phases
-            // that nobody has waited for in between: the slot of item n + 2 is handed back only when item n + 1 has been
-            // counted, so item n + 4, the next to use the ROWS_DONE of item n, is not published before this lane has waited for
-            // item n.  (With one per slot, item n + 2 used it again, which is published while this lane may still be about to wait.)
-            int n_item = 0;
+            // An item that depends on nothing does not go through DEPEND at all, and of a phase's items only the first does: what
+            // it waited for stays true.  DEPEND is arrived on when the previous item's rows have been seen to be stored, that is after
+            // every softmax thread has passed its previous wait on it (a group without a tile in that item waits, and arrives
+            // on ROWS_DONE, all the same).
+            // The device-wide fence before the count waits for every store in flight, with short items longer than an item
+            // takes.  So an item's slot is handed back before it, and the rows of a few items are counted together: at the end of a
+            // phase, before a wait, and else every fourth item (256-token chunks, 30 picks, 6 heads: see the launch).
+            // A barrier must not complete two phases that nobody has waited for in between: the slot of item n + 1 is handed
+            // back when item n has been seen to be stored, and item n + 4, the next to use the ROWS_DONE of item n, goes into that
+            // slot.
+            SlotIter slot_it;
+            int n_item = 0, last_phase = -1;
             uint32_t rows_phase = 0;                            // bit 2 (item modulo 4) + tile: parity of the next phase of that ROWS_DONE
-            int pend_phase = -1, pend_rows = 0;                 // the item whose rows are still to be counted
+            int pend_tiles = 0, pend_item_rows = 0;             // the item before this one: barriers to wait for, rows
+            int pend_phase = -1, pend_rows = 0, pend_n = 0;     // rows stored and not yet counted, of how many items
+            auto count_rows = [&]() {
+                if (pend_n == 0) return;
+                __threadfence();
+                atomicAdd(&phase_tab[3 * pend_phase + 2], pend_rows);
+                pend_n = pend_rows = 0;
+            };
             bool ok = true;
             while (ok) {
-                const int sl = n_item & 1;
-                if (!mbar_wait(bar(ITEM_FULL + sl), (n_item >> 1) & 1, abort_flag, p.status, W_ITEMFULL)) break;
+                const int sl = slot_it.at;
+                if (!mbar_wait(bar(ITEM_FULL + sl), slot_it.phase, abort_flag, p.status, W_ITEMFULL)) break;
                 const ItemSlot it_ = s_item[sl];
+                slot_it.next();
                 ++n_item;
-                const int group = it_.phase >> 1;
-                const bool dep_anchor = it_.valid && !it_.routed && p.k > 0, dep_routed = it_.valid && it_.routed && group >= 2;
-                if (pend_phase >= 0) {
-                    const int n_qt = pend_rows > 128 ? 2 : 1;
-                    for (int g = 0; ok && g < n_qt; ++g) {
-                        const int b = 2 * ((n_item - 2) & 3) + g;          // the pending item is the one before this
-                        ok = mbar_wait(bar(ROWS_DONE + b), (rows_phase >> b) & 1, abort_flag, p.status, W_ROWSDONE);
-                        rows_phase ^= 1u << b;
-                    }
-                    if (!ok) break;
-                    __threadfence();
-                    atomicAdd(&phase_tab[3 * pend_phase + 2], pend_rows);
-                    pend_phase = -1;
+                for (int g = 0; ok && g < pend_tiles; ++g) {
+                    const int b = 2 * ((n_item - 2) & 3) + g;          // the pending item is the one before this
+                    ok = mbar_wait(bar(ROWS_DONE + b), (rows_phase >> b) & 1, abort_flag, p.status, W_ROWSDONE);
+                    rows_phase ^= 1u << b;
                 }
+                if (!ok) break;
                 mbar_arrive(bar(ITEM_EMPTY + sl));
+                if (pend_tiles) {
+                    pend_rows += pend_item_rows;
+                    ++pend_n;
+                }
+                const int group = it_.phase >> 1;
+                const bool first = it_.valid && it_.phase != last_phase;
+                const bool dep_anchor = first && !it_.routed && p.k > 0, dep_routed = first && it_.routed && group >= 2;
+                if (!it_.valid || first || pend_n >= 4) count_rows();
                 if (!it_.valid) break;
                 if (dep_anchor)
                     ok = wait_count(&phase_tab[3 * (2 * group) + 2], phase_tab[3 * (2 * group) + 1], abort_flag, p.status, W_DEPEND);
@@ -590,12 +802,13 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                     __threadfence();
                     mbar_arrive(bar(DEPEND));
                 }
-                pend_phase = it_.phase;
-                pend_rows = it_.rows;
+                pend_phase = last_phase = it_.phase;
+                pend_item_rows = it_.rows;
+                pend_tiles = it_.rows > 128 || dep_anchor || dep_routed ? 2 : 1;
             }
         }
     } else if (warp < 11) {
-        if (LOADERS) asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        if (LOADERS) asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
         else asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         // ------------------------------------------------------------ MMA issuers (one warp per query tile; the warp stays
         // together, one lane of it issues)
@@ -634,8 +847,8 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                     for (int ks = ks0; ks < ks1; ++ks) mma_ts_elect(d_o, a_p + ks * 8, v_lo + ks * (2048 >> 4), v_hi, IDESC_PV, accumulate || ks > ks0);
                 }
             };
-            // items seen, items with this tile, K/V tiles seen, P tiles consumed, query tiles loaded before this item
-            int n_item = 0, n_mine = 0, n_kv = 0, n_p = 0, n_qtile = 0;
+            // items with this tile, K/V tiles seen, P tiles consumed, query tiles loaded before this item
+            int n_mine = 0, n_kv = 0, n_p = 0, n_qtile = 0;
             uint32_t q_phase = 0;                         // bit b: parity of the next load of this tile into buffer b
             bool ok = true;
             // the whole warp waits, and goes on or gives up together
@@ -644,13 +857,14 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 return __all_sync(0xffffffffu, LOADERS ? mbar_wait_spin(bar(b), parity, abort_flag, p.status, code)
                                                        : mbar_wait(bar(b), parity, abort_flag, p.status, code)) != 0;
             };
+            SlotIter slot_it;
             while (ok) {
-                const int sl = n_item & 1;
-                if (!wait(ITEM_FULL + sl, (n_item >> 1) & 1, W_ITEMFULL)) break;
+                const int sl = slot_it.at;
+                if (!wait(ITEM_FULL + sl, slot_it.phase, W_ITEMFULL)) break;
                 const ItemSlot it_ = s_item[sl];
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(ITEM_EMPTY + sl));
-                ++n_item;
+                slot_it.next();
                 if (!uniform(it_.valid)) break;
                 const int rows = uniform(it_.rows), n_tiles = uniform(it_.ntiles);
                 const int q_seq = n_qtile + g;                      // this tile's place in the sequence of Q loads
@@ -721,7 +935,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             }
         }
     } else if (!LOADERS || warp == 11) {
-        if (LOADERS) asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        if (LOADERS) asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
         else asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
         // ------------------------------------------------------------ scheduler (lane 0 claims items in queue order) and
         // Q loader (the whole warp): a claimed item is published at once, then its query tiles are loaded as their
@@ -739,17 +953,24 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
         }
         int n_item = 0, n_qtile = 0, last_g = 0;       // last_g: query tile of the last one loaded or published
         uint32_t q_phase = 0;                          // bit 3 g + buffer: parity of the next phase of that Q_FULL
+        uint32_t m_used = 0, m_phase = 0;              // bit b: buffer b's tile merges partials in it; parity of the next phase of its MERGED
         bool ok = true, late = false;
+        SlotIter slot_it;
         while (ok) {
-            const int sl = n_item & 1;
+            const int sl = slot_it.at;
             ItemSlot s;
-            s.valid = 0; s.routed = 0; s.h = 0; s.first = 0; s.rows = 0; s.nrng = 0; s.ntiles = 0; s.phase = 0; s.rng = nullptr;
+            s.valid = 0; s.routed = 0; s.h = 0; s.first = 0; s.rows = 0; s.nrng = 0; s.ntiles = 0; s.phase = 0; s.qbuf = n_qtile % 3; s.rng = nullptr;
             if (lane == 0) {
-                if (n_item >= 2) ok = mbar_wait(bar(ITEM_EMPTY + sl), ((n_item - 2) >> 1) & 1, abort_flag, p.status, W_ITEMEMPTY);
+                if (n_item >= kItemSlots) ok = mbar_wait(bar(ITEM_EMPTY + sl), slot_it.phase ^ 1, abort_flag, p.status, W_ITEMEMPTY);
                 // Claimed early, an item's gathers are done before they are needed, but it is kept from a CTA that may be idle.
                 // After an anchor item (whose successors have plain tiles to load, and which end the queue), and when there
                 // are only a few items per CTA, the next one is claimed when the last S of this one has been issued.
-                if (ok && n_qtile > 0 && (late || total <= 2 * (int)gridDim.x)) {
+                const bool wait_for_s = n_qtile > 0 && (late || total <= 2 * (int)gridDim.x);
+                if (ok && wait_for_s && n_item >= 2) {       // every warp has seen the item before the last one
+                    const bool wrap = sl + 1 == kItemSlots;
+                    ok = mbar_wait(bar(ITEM_EMPTY + (wrap ? 0 : sl + 1)), slot_it.phase ^ (wrap ? 0 : 1), abort_flag, p.status, W_ITEMEMPTY);
+                }
+                if (ok && wait_for_s) {
                     const int qb = (n_qtile - 1) % 3, qf = 3 * last_g + qb;
                     // Where others load the tiles, the buffer's release before this one may be yet to come, and its phase would be
                     // taken for this one's.  It has come when the item's last tile is there.  (That barrier's own phase
@@ -785,6 +1006,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 late = !s.routed;
             }
             ++n_item;
+            slot_it.next();
             // the rest of the warp learns the item from lane 0
             const int valid = __shfl_sync(0xffffffffu, s.valid, 0), routed = __shfl_sync(0xffffffffu, s.routed, 0);
             const int h = __shfl_sync(0xffffffffu, s.h, 0), first = __shfl_sync(0xffffffffu, s.first, 0), rows = __shfl_sync(0xffffffffu, s.rows, 0);
@@ -798,7 +1020,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             }
             for (int g = 0; ok && g < n_qt; ++g) {
                 const int qb = n_qtile % 3, qf = 3 * g + qb;
-                ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.status, W_QEMPTY);
+                ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.status, W_QEMPTY) && merged(qb, !routed, m_used, m_phase);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 if (lane == 0) mbar_expect_tx(bar(Q_FULL + qf), TILE_BYTES);
@@ -838,23 +1060,25 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             for (int b = 0; b < 6; ++b) mbar_wait(bar(Q_FULL + b), ((q_phase >> b) & 1) ^ 1, &dummy_flag, p.status, W_QFULL);
         }
     } else {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 48;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
         // ------------------------------------------------------------ Q loaders: rows 32 lw .. 32 lw + 31 of every query tile.
         // All four warps load a part of every tile, so a buffer cannot be filled and released without one of them: none
         // can miss a phase of Q_EMPTY.
         const int lw = warp - 12;
-        int n_item = 0, n_qtile = 0;
+        int n_qtile = 0;
+        SlotIter slot_it;
+        uint32_t m_used = 0, m_phase = 0;              // as above
         uint32_t q_phase = 0;                          // bit 3 g + buffer: parity of the next phase of that Q_FULL
         bool ok = true;
         while (ok) {
-            const int sl = n_item & 1;
-            ok = mbar_wait(bar(ITEM_FULL + sl), (n_item >> 1) & 1, abort_flag, p.status, W_ITEMFULL);
+            const int sl = slot_it.at;
+            ok = mbar_wait(bar(ITEM_FULL + sl), slot_it.phase, abort_flag, p.status, W_ITEMFULL);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             const int valid = s_item[sl].valid, routed = s_item[sl].routed, h = s_item[sl].h, first = s_item[sl].first, rows = s_item[sl].rows;
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(ITEM_EMPTY + sl));
-            ++n_item;
+            slot_it.next();
             if (!valid) break;
             const int n_qt = rows > 128 ? 2 : 1;
             // the queries of this lane's rows (a row past the item's end fetches row 0 of the head: its result is never stored)
@@ -874,7 +1098,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 int row[4];
 #pragma unroll
                 for (int x = 0; x < 4; ++x) row[x] = h * p.L + __shfl_sync(0xffffffffu, qrow[g], (lane & 7) * 4 + x);
-                ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.status, W_QEMPTY);
+                ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.status, W_QEMPTY) && merged(qb, !routed, m_used, m_phase);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 if (lw == 0 && lane == 0) mbar_expect_tx(bar(Q_FULL + qf), TILE_BYTES);
@@ -964,6 +1188,7 @@ static int attend_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfl
     a.status = ws_ptr<int>(ws, p->ws.status);
     a.H = p->H; a.L = p->L; a.C = p->C; a.k = p->k; a.hg = p->heads_per_group; a.n_groups = n_groups;
     a.n_aitems = (int)p->qitems.size();
+    a.kdiv = SlotDiv::of(p->k);
     a.scale_log2 = p->scale * 1.4426950408889634f;
     a.cookie = p->cookie;
     // always the d = 128 footprint: more than half an SM's shared memory, so CTAs (which each
@@ -983,18 +1208,14 @@ int launch_attend_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloa
     // Who loads the query tiles.  A row gather costs the warp that issues it some 65 cycles for four rows of 128 bytes: with
     // one warp a 256-row routed item cannot start more often than every 13000 cycles (half that at d = 64), with four every
     // 3000 to 4000 - but four loading warps, one on every scheduler, are in the way of the softmax.  Measured, one warp -> four
-    // (d = 128; streams of 264k tokens):
-    //   two key tiles a chunk and less: 24 heads of a clip in 64-, 128- and 256-token frames 688 -> 602, 644 -> 551, 722 -> 667 us;
-    //     256-token chunks, 2, 6, 12 and 23 picks 4.46 -> 4.37, 6.66 -> 6.36, 10.1 -> 9.7, 18.2 -> 17.2 ms (6 heads);
-    //   three: 3 and 8 picks 11.52 -> 11.71, 18.08 -> 17.87 ms (12 heads); 2, 6, 10, 15 picks 5.14 -> 5.24, 7.63 -> 7.69, 10.12 -> 9.99,
-    //     13.35 -> 12.95 ms (6 heads);
-    //   four: 4, 8, 11, 14 picks 24.5 -> 25.1, 34.9 -> 35.9, 44.3 -> 44.1, 53.7 -> 52.2 ms (24 heads); 16, 24, 32 picks 14.21 -> 14.09, 20.8 -> 20.0,
-    //     26.6 -> 25.3 ms (6 heads); a clip, 4 picks 1136 -> 1184 us;
-    //   five to twelve: 1 to 3 % slower with fewer than 16 picks, within 1 % with more (five, 32 picks: 3 % faster, in runs that differ by 4).
-    // At d = 64 four are slower: 512-token chunks 16.0 -> 18.0 ms, a training step on 256-token chunks 429 -> 443 us.
-    if (p->d == 64) return attend_tc_d<64, false>(p, Q, K, V, O, lse, ws, s);
-    const long long up_to = p->k > 8 ? 4 : p->k > 6 ? 3 : 2;        // key tiles a chunk, on average
-    const bool loaders = p->k > 0 && p->routed_key_tiles <= up_to * p->ncol;
+    // (which at d = 128 also takes the merge through registers; streams of 131k tokens, 3 to 32 picks):
+    //   d = 64, 8 heads: chunks of 128 tokens 1.08 to 1.19 times faster, of 256 1.08 to 1.16 (24 picks 6.12 -> 5.28 ms), of 384 0.91 to
+    //     0.95 (6.24 -> 6.54 ms), of 512 0.96, of 640 0.91 to 0.94;
+    //   d = 128, 6 heads: 256 1.21 to 1.40 (32 picks 8.94 -> 6.59 ms), 384 1.02 to 1.19, 512 1.02 to 1.05 (9.57 -> 9.22 ms), 768 1.00 to 1.01,
+    //     1024 0.99 to 1.00; a clip of 1560-token frames, 24 heads, 0.97.
+    const int up_to = p->d == 64 ? 2 : 4;        // key tiles a chunk, on average
+    const bool loaders = p->k > 0 && p->routed_key_tiles <= (int64_t)up_to * p->ncol;
+    if (p->d == 64) return loaders ? attend_tc_d<64, true>(p, Q, K, V, O, lse, ws, s) : attend_tc_d<64, false>(p, Q, K, V, O, lse, ws, s);
     return loaders ? attend_tc_d<128, true>(p, Q, K, V, O, lse, ws, s) : attend_tc_d<128, false>(p, Q, K, V, O, lse, ws, s);
 }
 

@@ -190,6 +190,16 @@ __device__ __forceinline__ size_t part_piece(int hl, int LB, int k, int NP, int 
     return ((((((size_t)hl * LB + (qi >> 7)) * k + s) * (NP >> 1) + (c >> 1)) * 128 + (qi & 127)) << 1) + (c & 1);
 }
 
+// Layout of the forward's partial outputs: a row is d / 64 lines of 128 bytes, query-innermost within a block of 128 queries, so
+// that a slot's lines of consecutive queries, which a warp of an anchor item fetches together, are contiguous.  Byte offset of
+// the first line of (head-in-group hl, query qi, slot s); the next one is 16 KB (128 queries) further.  Within a line, the 16-byte
+// piece 2 i + z (i = 0..3, z = 0, 1) holds the columns 32 z + 8 x + 2 i and the one after (x = 0..3), the order in which the
+// tensor memory hands them out, and sits at place (2 i + z) ^ (qi mod 8), so that lanes reading a piece of eight rows meet no
+// bank twice.
+__device__ __forceinline__ size_t part_line(int hl, int LB, int k, int lines, int qi, int s) {
+    return ((((size_t)hl * LB + (qi >> 7)) * k + s) * lines << 14) + ((qi & 127) << 7);
+}
+
 // Index of the log-sum-exp of (head, query, slot): query-innermost like the partials, so that the lanes of an anchor
 // item, which hold consecutive queries, read 128 contiguous bytes per slot.
 __device__ __forceinline__ size_t part_lse_at(int h, int LB, int k, int qi, int s) {
