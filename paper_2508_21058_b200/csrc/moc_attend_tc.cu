@@ -123,29 +123,6 @@ __device__ __forceinline__ void add_weighted_if(bool cond, uint64_t &acc, uint32
     asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\t@p fma.rn.f32x2 %0, %1, %2, %0;\n\t}" : "+l"(acc) : "l"(v), "l"(w2), "r"((int)cond));
 }
 
-// Of a row's 64 columns lane i of four holds pairs 4 x + i (columns 8 x + 2 i, + 1) in word x; afterwards it holds
-// columns 16 i .. 16 i + 15.
-__device__ __forceinline__ void quad_transpose(uint32_t (&u)[8], int i) {
-    // word 2 y + z of lane i goes to word 4 z + i of lane y
-    uint32_t t[8];
-    // lanes two apart exchange the halves y / 2, then neighbours the words y % 2
-#pragma unroll
-    for (int x = 0; x < 4; ++x) {
-        const uint32_t other = __shfl_xor_sync(0xffffffffu, (i & 2) ? u[x] : u[4 + x], 2);
-        t[x] = (i & 2) ? other : u[x];                   // from the lane with bit 1 clear
-        t[4 + x] = (i & 2) ? u[4 + x] : other;           // from the lane with bit 1 set
-    }
-    // t[4 s + 2 b + z]: word 2 (2 (i / 2) + b) + z of lane (i & 1) + 2 s
-#pragma unroll
-    for (int s = 0; s < 2; ++s)
-#pragma unroll
-        for (int z = 0; z < 2; ++z) {
-            const uint32_t other = __shfl_xor_sync(0xffffffffu, (i & 1) ? t[4 * s + z] : t[4 * s + 2 + z], 1);
-            u[4 * z + 2 * s] = (i & 1) ? other : t[4 * s + z];
-            u[4 * z + 2 * s + 1] = (i & 1) ? t[4 * s + 2 + z] : other;
-        }
-}
-
 // LOADERS: four more warps load the query tiles, for short routed items (see the rule where the kernel is launched)
 template <int D, bool LOADERS>
 __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) attend_tc_kernel(const __grid_constant__ CUtensorMap tmQ,
@@ -591,8 +568,8 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                                     unpack2(acc[cb][x], lo, hi);
                                     u[x] = bf16x2(lo * w, hi * w);
                                 }
-                                quad_transpose(u, l2);                            // this lane: columns 16 l2 .. 16 l2 + 15
-                                if (q < row_end) st_256(p.O + ((size_t)h * p.L + q) * D + cb * 64 + l2 * 16, u);
+                                quad_transpose(u, l2);
+                                if (q < row_end) store_quad(p.O + ((size_t)h * p.L + q) * D + cb * 64, l2, u);
                             }
                             s0 = 0;
                             ++pass;
@@ -669,7 +646,9 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                                     unpack2(acc[x * 8 + y], lo, hi);
                                     u[y] = bf16x2(lo * inv_w, hi * inv_w);
                                 }
-                                st_256(p.O + ((size_t)h * p.L + qi) * D + cb * 64 + x * 16, u);
+                                uint4 *dst = reinterpret_cast<uint4 *>(p.O + ((size_t)h * p.L + qi) * D + cb * 64 + x * 16);
+                                dst[0] = make_uint4(u[0], u[1], u[2], u[3]);     // (O is 16-byte aligned, not 32)
+                                dst[1] = make_uint4(u[4], u[5], u[6], u[7]);
                             }
                         }
                     }

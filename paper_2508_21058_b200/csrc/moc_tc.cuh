@@ -330,6 +330,34 @@ __device__ __forceinline__ void st_256(void *ptr, const uint32_t (&u)[8]) {
                  : "memory");
 }
 
+// The four lanes of a row in tmem_ld_16x256b: of its 64 columns lane i holds pairs 4 x + i (columns 8 x + 2 i, + 1) in word x.
+// Afterwards words 0..3 of lane i are columns 8 i .. 8 i + 7 and words 4..7 columns 32 + 8 i .. 32 + 8 i + 7: two 16-byte pieces, of
+// which the four lanes' make 64 contiguous bytes each.
+__device__ __forceinline__ void quad_transpose(uint32_t (&u)[8], int i) {
+#pragma unroll
+    for (int z = 0; z < 8; z += 4) {
+        // neighbours exchange the words off the diagonal of their 2 x 2 blocks, then lanes two apart the blocks off the diagonal
+#pragma unroll
+        for (int y = 0; y < 4; y += 2) {
+            const uint32_t other = __shfl_xor_sync(0xffffffffu, (i & 1) ? u[z + y] : u[z + y + 1], 1);
+            if (i & 1) u[z + y] = other;
+            else u[z + y + 1] = other;
+        }
+#pragma unroll
+        for (int y = 0; y < 2; ++y) {
+            const uint32_t other = __shfl_xor_sync(0xffffffffu, (i & 2) ? u[z + y] : u[z + y + 2], 2);
+            if (i & 2) u[z + y] = other;
+            else u[z + y + 2] = other;
+        }
+    }
+}
+// what quad_transpose leaves, to a row's 64 columns at `row` (16-byte aligned: a caller's tensor promises no more)
+__device__ __forceinline__ void store_quad(__nv_bfloat16 *row, int i, const uint32_t (&u)[8]) {
+    uint4 *dst = reinterpret_cast<uint4 *>(row) + i;
+    dst[0] = make_uint4(u[0], u[1], u[2], u[3]);
+    dst[4] = make_uint4(u[4], u[5], u[6], u[7]);
+}
+
 }  // namespace tc
 
 // host: encode a 2-D bf16 tensor map [rows][cols], box {64 cols, box_rows}, 128-byte swizzle

@@ -56,3 +56,28 @@ def test_every_element_of_the_merge(shape):
         assert bool(torch.isfinite(run.O.float()).all())
         assert float((diff / norm.clamp(min=1e-3)).max()) < REL
         assert float((run.lse - lse).abs().max()) < 2e-3
+
+
+@pytest.mark.parametrize("d,frame", [(64, 130), (64, 400), (128, 130), (128, 600)])
+def test_tensors_on_16_byte_boundaries(d, frame):
+    """Every tensor of the boundary is 16-byte aligned and no more: the same bits as with 256-byte aligned ones."""
+    wl = W.Workload("align", 2, d, W.make_layout(2, 7, 6, frame), 3, 1, 1)
+    run = PU.GpuRun(wl, tensors=("q", "k", "v", "do")).forward()
+
+    def off(t):
+        flat = torch.empty(t.numel() + 8, dtype=t.dtype, device="cuda")
+        assert flat.data_ptr() % 32 == 0
+        return flat[8:].view(t.shape)
+
+    x = {n: off(t).copy_(t) for n, t in run.x.items()}
+    O, dQ, dK, dV = (off(run.O) for _ in range(4))
+    lse, p = torch.empty_like(run.lse), run.plan
+    p.moc_chunk_pool(x["k"], run.desc, run.ws)
+    p.moc_route(x["q"], run.desc, run.sel, run.ws)
+    run.attend_only()
+    run.backward()                                             # on the same lists: their order is the order of sums
+    p.moc_attend(x["q"], x["k"], x["v"], run.sel, O, lse, run.ws)
+    p.moc_attend_bwd(x["q"], x["k"], x["v"], O, lse, x["do"], run.sel, dQ, dK, dV, run.ws)
+    assert p.moc_get_status(run.ws)[0] == 0
+    for a, b in ((O, run.O), (dQ, run.dQ), (dK, run.dK), (dV, run.dV)):
+        assert torch.equal(a, b)
