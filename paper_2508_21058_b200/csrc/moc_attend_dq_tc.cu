@@ -6,7 +6,8 @@
 // the ANCHOR launch takes consecutive rows against their anchor ranges, adds the rows' partials and writes dQ.
 //
 //     T1 = Q K^T,  T2 = dO V^T          (both operands from shared memory, into TMEM)
-//     threads (two per TMEM lane) turn T1 into P, then (P, T2) into dS, written back to TMEM as bf16
+//     threads (two per TMEM lane) turn T1 into P, then (P, T2) into dS, written back to TMEM as bf16 over the columns of T2
+//     that the thread itself has read
 //     ACC += dS K                        (A from TMEM, the K tile as an MN-major operand)
 //
 // One CTA per SM walks its items (an equal share of the launch's, which but for the empty ones are much alike): the tensor memory, the
@@ -38,7 +39,7 @@ struct DqParams {
     const __nv_bfloat16 *Q, *dO;
     const float *lse, *delta;
     __nv_bfloat16 *dQ;
-    __nv_bfloat16 *part;          // routed dQ partials of the group of heads in flight (part_piece)
+    __nv_bfloat16 *part;          // routed dQ partials of the group of heads in flight (part_line)
     const float *part_lse;        // the forward's routed log-sum-exps (part_lse_at): -inf marks an empty slot
     const KeyRange *rng;          // key ranges the items index
     const WorkItem *items;        // up to 256 rows each: two of this kernel's items
@@ -54,6 +55,12 @@ struct DqParams {
 
 constexpr int kDqThreads = 512, kKStages = 3, kVStages = 2, kLoaders = 3;
 
+// acc += the bf16 pair u where cond holds
+__device__ __forceinline__ void add_if(bool cond, uint64_t &acc, uint32_t u) {
+    const uint64_t v = pack2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p add.rn.f32x2 %0, %0, %1;\n\t}" : "+l"(acc) : "l"(v), "r"((int)cond));
+}
+
 // description of an item, as the row loaders leave it for the other warps; rows = 0: no more items
 struct DqItem { int h, first, rows, nrng, ntiles, rng_off, t0, t1; };
 
@@ -66,7 +73,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
     constexpr int CH = D / 8;               // 16-byte pieces per row
     constexpr int N_TILES_SMEM = 2 + kKStages + kVStages;
     enum { X_FULL = 0, X_EMPTY, K_FULL, K_EMPTY = K_FULL + kKStages, V_FULL = K_EMPTY + kKStages, V_EMPTY = V_FULL + kVStages,
-           T1_FULL = V_EMPTY + kVStages, T1_READ, T2_FULL, RD2 = T2_FULL + 2, DS_DONE, ACC_FULL = DS_DONE + 2, ACC_FREE, N_BARS };
+           T1_FULL = V_EMPTY + kVStages, T1_READ, T2_FULL, DS_DONE = T2_FULL + 2, ACC_FULL = DS_DONE + 2, ACC_FREE, N_BARS };
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t bars[N_BARS];
     __shared__ __align__(16) float s_ld[2][2][128];      // per item parity: -lse * log2(e) and -delta of the item's rows
@@ -103,7 +110,6 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
         mbar_init(bar(T1_FULL), 1);
         mbar_init(bar(T1_READ), 256);
         for (int t = 0; t < 2; ++t) { mbar_init(bar(T2_FULL + t), 1); mbar_init(bar(DS_DONE + t), 256); }
-        mbar_init(bar(RD2), 256);
         mbar_init(bar(ACC_FULL), 1);
         mbar_init(bar(ACC_FREE), 256);
         fence_barrier_init();
@@ -159,14 +165,13 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
 
     if (warp < 8) {
         // ------------------------------------------------------------ lane threads
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 176;");
         const int r = threadIdx.x & 127;              // row of the item = TMEM lane
         const int half = warp >> 2;
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
         const uint64_t c2 = pack2(p.scale_log2, p.scale_log2);
-        constexpr int NP = D / 8;
         const int LB = (p.L + 127) >> 7;
-        uint4 *part16 = reinterpret_cast<uint4 *>(p.part);
+        char *part = reinterpret_cast<char *>(p.part);
         int g = 0;                                    // tiles processed
         bool ok = true;
         for (int n = 0; ok; ++n) {
@@ -180,20 +185,36 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
             const uint64_t nlse2 = pack2(nlse, nlse), ndlt2 = pack2(ndlt, ndlt);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(X_EMPTY));
-            // the destination of this row's result, wanted at the end
+            // the list entry of this row, wanted at the end
             int e = -1;
-            if (r < rows) e = ANCHOR ? first + r : p.qlist[(size_t)h * p.cap_total + first + r];
-            for (int jt = 0; jt < n_tiles; ++jt, ++g) {
-                const int st = g & 1;
-                int valid = 128, t0;
-                it.next(t0, valid);
+            if (!ANCHOR && r < rows) e = p.qlist[(size_t)h * p.cap_total + first + r];
+            float pv[64];
+            // P = exp2(scale log2(e) S - lse log2(e))
+            auto p_pair = [&](const uint32_t (&sv)[32], int x, float &p0, float &p1) {
+                unpack2(fma2(pack2(__uint_as_float(sv[x]), __uint_as_float(sv[x + 1])), c2, nlse2), p0, p1);
+                p0 = ex2(p0);
+                p1 = ex2(p1);
+            };
+            // dS = P (dP - delta)
+            auto ds_pair = [&](const uint32_t (&dp)[32], int rd, int x) {
+                float a0, a1;
+                unpack2(mul2(pack2(pv[rd * 32 + x], pv[rd * 32 + x + 1]), add2(pack2(__uint_as_float(dp[x]), __uint_as_float(dp[x + 1])), ndlt2)), a0, a1);
+                return bf16x2(a0, a1);
+            };
+            auto mask = [&](int valid) {                     // keys past the end of the range
+                if (valid < 128) {
+#pragma unroll
+                    for (int x = 0; x < 64; ++x)
+                        if (((x >> 5) * 2 + half) * 32 + (x & 31) >= valid) pv[x] = 0.f;
+                }
+            };
+            int valid, t0;
+            // P of the tile
+            auto form_p = [&]() __attribute__((always_inline)) -> bool {
                 ok = mbar_wait_spin(bar(T1_FULL), g & 1, abort_flag, p.status, DW_T1FULL);
                 ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
+                if (!ok) return false;
                 tc_fence_after();
-                // ---- P = exp2(scale log2(e) S - lse log2(e)) from T1
-                const uint32_t t2c = st ? 384u : 128u;       // T2 (then dS) of this tile
-                float pv[64];
                 uint32_t sv[2][32];
                 tmem_ld32(tmem + lane_off + half * 32, sv[0]);
                 tmem_ld32(tmem + lane_off + (2 + half) * 32, sv[1]);
@@ -201,120 +222,156 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
                 tc_fence_before();
                 mbar_arrive(bar(T1_READ));                   // T1 may be overwritten
 #pragma unroll
-                for (int rd = 0; rd < 2; ++rd) {
-                    const int ch = rd * 2 + half;
+                for (int rd = 0; rd < 2; ++rd)
 #pragma unroll
-                    for (int x = 0; x < 32; x += 2) {
-                        float p0, p1;
-                        unpack2(fma2(pack2(__uint_as_float(sv[rd][x]), __uint_as_float(sv[rd][x + 1])), c2, nlse2), p0, p1);
-                        pv[rd * 32 + x] = ex2(p0);
-                        pv[rd * 32 + x + 1] = ex2(p1);
-                    }
-                    if (valid < 128) {                       // keys past the end of the range
-#pragma unroll
-                        for (int x = 0; x < 32; ++x)
-                            if (ch * 32 + x >= valid) pv[rd * 32 + x] = 0.f;
-                    }
-                }
-                // ---- dS = P (dP - delta) from T2, written over T2 columns that have been read
+                    for (int x = 0; x < 32; x += 2) p_pair(sv[rd], x, pv[rd * 32 + x], pv[rd * 32 + x + 1]);
+                mask(valid);
+                return true;
+            };
+            // dS of the tile, and on to the next
+            auto form_ds = [&]() __attribute__((always_inline)) -> bool {
+                const int st = g & 1;
+                const uint32_t t2 = tmem + lane_off + (st ? 384u : 128u);
                 ok = mbar_wait_spin(bar(T2_FULL + st), (g >> 1) & 1, abort_flag, p.status, DW_T2FULL);
                 ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
+                if (!ok) return false;
                 tc_fence_after();
-                uint32_t dpv[2][32];
-                tmem_ld32(tmem + lane_off + t2c + half * 32, dpv[0]);
-                tmem_ld32(tmem + lane_off + t2c + (2 + half) * 32, dpv[1]);
+                uint32_t dp[2][32];
+                tmem_ld32(t2 + half * 32, dp[0]);
+                tmem_ld32(t2 + (2 + half) * 32, dp[1]);
                 tmem_wait_ld();
-                mbar_arrive(bar(RD2));                       // this thread's columns have been read
 #pragma unroll
                 for (int rd = 0; rd < 2; ++rd) {
-                    const int ch = rd * 2 + half;
                     uint32_t uds[16];
 #pragma unroll
-                    for (int x = 0; x < 32; x += 2) {
-                        float a0, a1;
-                        unpack2(mul2(pack2(pv[rd * 32 + x], pv[rd * 32 + x + 1]),
-                                     add2(pack2(__uint_as_float(dpv[rd][x]), __uint_as_float(dpv[rd][x + 1])), ndlt2)), a0, a1);
-                        uds[x >> 1] = bf16x2(a0, a1);
-                    }
-                    if (rd == 0) {                           // the other thread of the lane has read the columns stored over
-                        ok = mbar_wait_spin(bar(RD2), g & 1, abort_flag, p.status, DW_READ);
-                        ok = __all_sync(0xffffffffu, ok);
-                    }
-                    if (ok) tmem_st16(tmem + lane_off + t2c + ch * 16, uds);
+                    for (int x = 0; x < 32; x += 2) uds[x >> 1] = ds_pair(dp[rd], rd, x);
+                    // over the first half of the chunk's own columns, which this thread alone has read.  (With the chunks side by side
+                    // the two threads of a lane waited for each other: 10.69 -> 10.07 ms for the whole backward of the 33k-token
+                    // clip, 24 heads.)
+                    tmem_st16(t2 + (rd * 2 + half) * 32, uds);
                 }
-                if (!ok) break;
                 tmem_wait_st();
                 tc_fence_before();
                 mbar_arrive(bar(DS_DONE + st));
+                ++g;
+                return true;
+            };
+            it.next(t0, valid);
+            if (!form_p()) break;
+            for (int jt = 0; jt + 1 < n_tiles; ++jt) {
+                if (!form_ds()) break;
+                it.next(t0, valid);
+                if (!form_p()) break;
             }
-            if (!ok) break;
+            if (!ok || !form_ds()) break;
             // ---- epilogue
             ok = mbar_wait(bar(ACC_FULL), n & 1, abort_flag, p.status, DW_ACCFULL);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
-            uint32_t v[D / 64][32];
-#pragma unroll
-            for (int c = 0; c < D / 64; ++c) tmem_ld32(tmem + lane_off + 256 + (2 * c + half) * 32, v[c]);
-            tmem_wait_ld();
-            tc_fence_before();
-            mbar_arrive(bar(ACC_FREE));                      // the next item's dQ may be accumulated
-            if (ANCHOR) previous_done();                     // the routed launch's partials are complete
-            if (e < 0) continue;
-            int qi = e, slot = 0;
+            // Results move in the 16 x 256-bit load shape of the tensor memory: of a 16-row half of the warp's rows, lane l holds
+            // rows l / 4 and l / 4 + 8, of every eight columns the two at 2 (l % 4), so that four lanes write 128 contiguous bytes
+            // of a row.  (With a row per lane a warp's 32-byte stores touched 32 lines each.)  Of the two warps that share the TMEM
+            // lanes, each takes 64 columns of all rows (d = 128) or 16 rows (d = 64).  A partial keeps its columns in the order of the
+            // lanes; dQ is put in the order of the columns.
+            constexpr int NJ = D / 32;                       // groups of eight rows that this warp has
+            const int l4 = lane >> 2, l2 = lane & 3, cb = D == 128 ? half : 0, j0 = D == 128 ? 0 : 2 * half;
+            const uint32_t t_acc = tmem + lane_off + 256 + ((uint32_t)(j0 >> 1) << 20) + cb * 64;
             if (!ANCHOR) {
-                qi = p.kdiv.query(e);
-                slot = e - qi * p.k;
-                if (!index_ok((unsigned)qi < (unsigned)p.L, p.status, IX_BWD_LIST_ENTRY) || (unsigned)qi >= (unsigned)p.L) continue;
-            }
-#pragma unroll 1
-            for (int c = 0; c < D / 64; ++c) {
-                const int ch = 2 * c + half;
-                float acc[32];
+                uint32_t v[NJ / 2][32];
 #pragma unroll
-                for (int x = 0; x < 32; ++x) acc[x] = __uint_as_float(D == 64 || c == 0 ? v[0][x] : v[D / 64 - 1][x]) * p.scale;
-                if (ANCHOR) {
-                    // the routed partials of this query, four slots requested together; a slot is in use
-                    // if the forward left a finite log-sum-exp for it
-                    const float *pl = p.part_lse + part_lse_at(h, LB, p.k, qi, 0);      // slot s: pl[s * 128]
-#pragma unroll 1
-                    for (int s0 = 0; s0 < p.k; s0 += 4) {
-                        uint4 raw[4][4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const bool used = s0 + u < p.k && pl[(s0 + u) * 128] != -INFINITY;
-#pragma unroll
-                            for (int q4 = 0; q4 < 4; q4 += 2) {
-                                raw[u][q4] = raw[u][q4 + 1] = make_uint4(0, 0, 0, 0);
-                                if (used) ld_cg_256(part16 + part_piece(h - p.h0, LB, p.k, NP, qi, s0 + u, ch * 4 + q4), raw[u][q4], raw[u][q4 + 1]);
-                            }
-                        }
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-#pragma unroll
-                            for (int q4 = 0; q4 < 4; ++q4) {
-                                const __nv_bfloat162 *b = reinterpret_cast<const __nv_bfloat162 *>(&raw[u][q4]);
-#pragma unroll
-                                for (int y = 0; y < 4; ++y) {
-                                    const float2 f = __bfloat1622float2(b[y]);
-                                    acc[q4 * 8 + 2 * y] += f.x;
-                                    acc[q4 * 8 + 2 * y + 1] += f.y;
-                                }
-                            }
+                for (int x = 0; x < NJ / 2; ++x) tmem_ld_16x256b(t_acc + ((uint32_t)x << 20), v[x]);
+                tmem_wait_ld();
+                tc_fence_before();
+                mbar_arrive(bar(ACC_FREE));                  // the next item's dQ may be accumulated
+                size_t line = 0;                             // where this row's partial goes
+                bool keep = false;
+                if (e >= 0) {
+                    const int qi = p.kdiv.query(e), slot = e - qi * p.k;
+                    if (index_ok((unsigned)qi < (unsigned)p.L, p.status, IX_BWD_LIST_ENTRY) && (unsigned)qi < (unsigned)p.L) {
+                        line = part_line(h - p.h0, LB, p.k, D / 64, qi, slot);
+                        keep = true;
                     }
                 }
-                uint4 out[4];
-                uint32_t *o32 = reinterpret_cast<uint32_t *>(out);
 #pragma unroll
-                for (int x = 0; x < 16; ++x) o32[x] = bf16x2(acc[2 * x], acc[2 * x + 1]);
-                if (ANCHOR) {
-                    uint4 *dst = reinterpret_cast<uint4 *>(p.dQ + ((size_t)h * p.L + qi) * D + ch * 32);
+                for (int j = 0; j < NJ; ++j) {
+                    const size_t at = __shfl_sync(0xffffffffu, line, (j0 + j) * 8 + l4);
+                    const bool some = __shfl_sync(0xffffffffu, keep, (j0 + j) * 8 + l4);
+                    uint32_t u[8];
 #pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) dst[q4] = out[q4];
-                } else {                                     // whole 32-byte sectors (pairs of pieces)
-                    st_256(part16 + part_piece(h - p.h0, LB, p.k, NP, qi, slot, ch * 4), out[0], out[1]);
-                    st_256(part16 + part_piece(h - p.h0, LB, p.k, NP, qi, slot, ch * 4 + 2), out[2], out[3]);
+                    for (int x = 0; x < 8; ++x)
+                        u[x] = bf16x2(__uint_as_float(v[j >> 1][4 * x + 2 * (j & 1)]) * p.scale, __uint_as_float(v[j >> 1][4 * x + 2 * (j & 1) + 1]) * p.scale);
+                    if (some) st_256(part + at + ((size_t)cb << 14) + l2 * 32, u);
+                }
+            } else {
+                // the routed partials of a query, a few slots requested together, the next ones while these are added up; a slot is
+                // in use if the forward left a finite log-sum-exp for it
+                previous_done();                             // the routed launch's partials are complete
+                constexpr int B = 4;
+                struct Batch { uint32_t v[B][8]; float ls[B]; };
+                const int row0 = first + j0 * 8 + (warp & 3) * 32 + l4, row_end = first + rows;
+                int ask_j = 0, ask_s = 0;
+                auto ask = [&](Batch &b) __attribute__((always_inline)) {
+                    const int q = row0 + ask_j * 8;
+                    const bool in = q < row_end;
+                    const char *src = part + part_line(h - p.h0, LB, p.k, D / 64, q, ask_s) + ((size_t)cb << 14) + l2 * 32;
+                    const float *ls = p.part_lse + part_lse_at(h, LB, p.k, q, ask_s);
+#pragma unroll
+                    for (int u = 0; u < B; ++u) {
+                        const bool some = in && ask_s + u < p.k;
+                        const float x = *(some ? ls + u * 128 : p.part_lse);
+                        b.ls[u] = some ? x : -INFINITY;
+                        ld_cg_256_if(some, src + ((size_t)(u * (D / 64)) << 14), b.v[u]);
+                    }
+                    ask_s += B;
+                    if (ask_s >= p.k) { ask_s = 0; ++ask_j; }
+                };
+                uint64_t acc[8];
+                uint32_t v[32];
+                int j = 0, s0 = 0;
+                auto add = [&](const Batch &b) __attribute__((always_inline)) {
+                    if (s0 == 0) {
+                        if (!(j & 1)) {                      // two groups of rows at a time
+                            tmem_ld_16x256b(t_acc + ((uint32_t)(j >> 1) << 20), v);
+                            tmem_wait_ld();
+                            if (j == NJ - 2) {
+                                tc_fence_before();
+                                mbar_arrive(bar(ACC_FREE));  // the next item's dQ may be accumulated
+                            }
+                        }
+                        const uint64_t sc2 = pack2(p.scale, p.scale);
+#pragma unroll
+                        for (int x = 0; x < 8; ++x)
+                            acc[x] = mul2(pack2(__uint_as_float((j & 1) ? v[4 * x + 2] : v[4 * x]), __uint_as_float((j & 1) ? v[4 * x + 3] : v[4 * x + 1])), sc2);
+                    }
+#pragma unroll
+                    for (int u = 0; u < B; ++u)
+#pragma unroll
+                        for (int x = 0; x < 8; ++x) add_if(b.ls[u] != -INFINITY, acc[x], b.v[u][x]);
+                    s0 += B;
+                    if (s0 >= p.k) {
+                        uint32_t u[8];
+#pragma unroll
+                        for (int x = 0; x < 8; ++x) {
+                            float lo, hi;
+                            unpack2(acc[x], lo, hi);
+                            u[x] = bf16x2(lo, hi);
+                        }
+                        quad_transpose(u, l2);
+                        const int q = row0 + j * 8;
+                        if (q < row_end) store_quad(p.dQ + ((size_t)h * p.L + q) * D + cb * 64, l2, u);
+                        s0 = 0;
+                        ++j;
+                    }
+                };
+                Batch even = {}, odd = {};
+                ask(even);
+#pragma unroll 1
+                while (j < NJ) {                             // an even number of row groups, so of batches
+                    ask(odd);
+                    add(even);
+                    if (ask_j < NJ) ask(even);
+                    add(odd);
                 }
             }
         }
@@ -423,7 +480,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
         cp_async_wait_all();
     } else {
         // ------------------------------------------------------------ MMA issuers (a warp stays together, one lane of it issues)
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 88;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
         if (warp <= 13) {
             constexpr uint32_t IDESC_T = idesc_bf16_f32(128, 128, 0, 0);      // T = X Y^T, both K-major
             constexpr uint32_t IDESC_ACC = idesc_bf16_f32(128, D, 0, 1);      // ACC += dS K, K MN-major
@@ -488,8 +545,8 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
                         tc_fence_after();
                         const uint32_t ds = tmem + ((g & 1) ? 384u : 128u);
 #pragma unroll
-                        for (int ks = 0; ks < 8; ++ks)
-                            mma_ts_elect(tmem + 256, ds + ks * 8, lo(km) + s3 * STAGE + ks * (2048 >> 4), hi(km), IDESC_ACC, j > 0 || ks > 0);
+                        for (int ks = 0; ks < 8; ++ks)       // dS of 32 keys lies over the first half of their T2 columns
+                            mma_ts_elect(tmem + 256, ds + (ks >> 1) * 32 + (ks & 1) * 8, lo(km) + s3 * STAGE + ks * (2048 >> 4), hi(km), IDESC_ACC, j > 0 || ks > 0);
                         tc_commit_elect(bar(K_EMPTY + s3));
                         if (++s3 == kKStages) s3 = 0;
                         if (j + 2 < n_tiles) t2(g + 2, j + 3 == n_tiles);

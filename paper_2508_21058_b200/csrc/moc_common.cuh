@@ -177,25 +177,12 @@ __device__ __forceinline__ bool index_ok(bool cond, int *status, int code) {
 __device__ __forceinline__ bool index_ok(bool, int *, int) { return true; }
 #endif
 
-// Layout of the routed partial outputs.  The row of one (query, slot) is written by one thread of a routed item
-// and read by one thread of the query's anchor item, 16 bytes (a "piece": eight columns) at a time.  Anchor items
-// hold consecutive queries in consecutive lanes, so the pieces are laid out query-innermost: within a block of 128
-// queries, the pieces 2 c2 and 2 c2 + 1 (a pair: one 32-byte sector) of slot s of the block's queries are 128 x 32
-// contiguous bytes.  A warp's load of one pair for its 32 queries is then 1024 contiguous bytes instead of 32
-// scattered requests, and a routed item, whose rows are scattered queries, still writes whole sectors (a store of
-// half a sector makes the memory system read the other half first).
-//   index (in 16-byte units) of piece c of (head-in-group hl, query qi, slot s); NP = d / 8 pieces per row,
-//   LB = ceil(L / 128) blocks per head
-__device__ __forceinline__ size_t part_piece(int hl, int LB, int k, int NP, int qi, int s, int c) {
-    return ((((((size_t)hl * LB + (qi >> 7)) * k + s) * (NP >> 1) + (c >> 1)) * 128 + (qi & 127)) << 1) + (c & 1);
-}
-
-// Layout of the forward's partial outputs: a row is d / 64 lines of 128 bytes, query-innermost within a block of 128 queries, so
-// that a slot's lines of consecutive queries, which a warp of an anchor item fetches together, are contiguous.  Byte offset of
-// the first line of (head-in-group hl, query qi, slot s); the next one is 16 KB (128 queries) further.  Within a line, the 16-byte
-// piece 2 i + z (i = 0..3, z = 0, 1) holds the columns 32 z + 8 x + 2 i and the one after (x = 0..3), the order in which the
-// tensor memory hands them out, and sits at place (2 i + z) ^ (qi mod 8), so that lanes reading a piece of eight rows meet no
-// bank twice.
+// Layout of the routed partials (the forward's outputs, and dQ in the backward): a row is d / 64 lines of 128 bytes, query-innermost
+// within a block of 128 queries, so that a slot's lines of consecutive queries, which a warp of an anchor item fetches together,
+// are contiguous.  Byte offset of the first line of (head-in-group hl, query qi, slot s); the next one is 16 KB (128 queries)
+// further.  Within a line, the 16-byte piece 2 i + z (i = 0..3, z = 0, 1) holds the columns 32 z + 8 x + 2 i and the one after
+// (x = 0..3), the order in which the tensor memory hands them out.  Where the forward's merge reads lines from shared memory, a row
+// per lane, piece c sits at place c ^ (qi mod 8), so that lanes reading a piece of eight rows meet no bank twice; elsewhere at c.
 __device__ __forceinline__ size_t part_line(int hl, int LB, int k, int lines, int qi, int s) {
     return ((((size_t)hl * LB + (qi >> 7)) * k + s) * lines << 14) + ((qi & 127) << 7);
 }
