@@ -38,7 +38,7 @@ struct BwdParams {
     uint32_t cookie;              // what the workspace's status area must hold
     const KTile *ktiles;
     int n_ktiles, n_long;         // tiles per head, and how many of them come first for every head
-    const int32_t *off, *ranc_off, *ranc, *cap_off;
+    const KeyRange *qry_rng;
     const int *cnt;
     const int32_t *qlist;
     size_t cap_total;
@@ -67,7 +67,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
     __shared__ __align__(8) uint64_t bars[24];
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort;
-    __shared__ int w_valid, w_h, w_rows, w_ntiles, w_chunk, w_t0;
+    __shared__ int w_valid, w_h, w_ntiles, w_list;       // w_list: entries of the chunk's query list
+    __shared__ KTile s_kt;
     // per streamed query, (-lse * log2(e), -delta), for tiles j and j + 1
     __shared__ __align__(16) float s_ld[2][2][128];
 
@@ -77,80 +78,67 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
     const uint32_t sX = sbase, sY1 = sbase + 2 * TILE_BYTES, sY2 = sbase + (2 + kY1Stages) * TILE_BYTES;
     auto bar = [&](int i) { return smem_u32(&bars[i]); };
     constexpr int X_FULL = 0, Y1_FULL = 1, Y1_EMPTY = 4, Y2_FULL = 7, Y2_EMPTY = 9, T1_FULL = 11, T2_FULL = 13,
-                  P_HALF = 15, P_DONE = 16, DS_DONE = 17, ACC_FULL = 19, T1_ISSUED = 20, RD1 = 22, RD2 = 23;
+                  P_HALF = 15, P_DONE = 16, DS_DONE = 17, ACC_FULL = 19, T1_ISSUED = 20, RD1 = 22, RD2 = 23, N_BARS = 24;
 
-    if (threadIdx.x == 0) {
-        s_abort = 0;
-        int valid = (*(volatile int *)p.status == 0);
-        if (valid && (uint32_t)((volatile int *)p.status)[ST_COOKIE] != p.cookie) {
-            atomicCAS(p.status, 0, MOC_ERR_WORKSPACE);      // not this plan's lists: report, touch nothing else
-            valid = 0;
+    // What a block needs before its first load, each in a warp of its own, and one lookup deep.  (By one thread, one after
+    // another, with the chunk's anchors walked one by one: 3900 to 6000 cycles, of 45000 for a block of 13 query tiles.)
+    if (warp == 0) {
+        for (int b = lane; b < N_BARS; b += 32) {
+            const int n = b >= Y1_FULL && b < Y1_EMPTY ? 2                       // the ring's two producer warps
+                          : b >= Y2_FULL && b < T1_FULL ? 2                      // ... and T2 and ACC2, which both read the stage
+                          : b == ACC_FULL ? 2                                    // both issuers
+                          : b == P_HALF || b == P_DONE || (b >= DS_DONE && b < ACC_FULL) || b >= RD1 ? 256 : 1;
+            mbar_init(bar(b), n);
         }
-        uint32_t dyn_bytes;
-        asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn_bytes));
-        if (valid && (sbase - smem_u32(smem_raw)) + (uint32_t)N_TILES_SMEM * TILE_BYTES > dyn_bytes) {
-            // the launch gave less shared memory than the tiles need: report, touch nothing
-            if (atomicCAS(p.status, 0, MOC_ERR_TIMEOUT) == 0) p.status[1] = BW_SMEM;
-            valid = 0;
-        }
-        // block order: the long key tiles of every head, then the others head by head (tiles of one chunk next
-        // to each other: they stream the same query rows)
-        const int n_long_all = p.n_long * p.H;
-        int b = blockIdx.x, hh, ti;
-        if (b < n_long_all) { hh = b / p.n_long; ti = b - hh * p.n_long; }
-        else { b -= n_long_all; const int n_rest = p.n_ktiles - p.n_long; hh = b / n_rest; ti = p.n_long + b - hh * n_rest; }
-        const KTile kt = p.ktiles[ti];
-        w_h = hh;
-        w_chunk = kt.chunk;
-        w_t0 = kt.t0;
-        w_rows = kt.valid;
-        // query tiles: merged row ranges of the chunks that have this chunk as an anchor, then the routed list
-        int nt = 0;
-        const int a0 = p.ranc_off[kt.chunk], a1 = p.ranc_off[kt.chunk + 1];
-        for (int a = a0; a < a1;) {
-            int qc = p.ranc[a], r0 = p.off[qc], r1 = p.off[qc + 1];
-            for (++a; a < a1 && p.ranc[a] == qc + 1; ++a) { qc = p.ranc[a]; r1 = p.off[qc + 1]; }
-            nt += (r1 - r0 + 127) / 128;
-        }
-        nt += (p.cnt[w_h * p.C + kt.chunk] + 127) / 128;
-        w_ntiles = nt;
-        w_valid = valid;
-        mbar_init(bar(X_FULL), 1);
-        for (int t = 0; t < kY1Stages; ++t) {
-            mbar_init(bar(Y1_FULL + t), 2);       // the ring's two producer warps
-            mbar_init(bar(Y1_EMPTY + t), 1);
-        }
-        for (int t = 0; t < kY2Stages; ++t) {
-            mbar_init(bar(Y2_FULL + t), 2);
-            mbar_init(bar(Y2_EMPTY + t), 2);      // T2 and ACC2 both read the stage
-            mbar_init(bar(T1_FULL + t), 1);
-            mbar_init(bar(T2_FULL + t), 1);
-            mbar_init(bar(DS_DONE + t), 256);
-            mbar_init(bar(T1_ISSUED + t), 1);
-        }
-        mbar_init(bar(P_HALF), 256);
-        mbar_init(bar(P_DONE), 256);
-        mbar_init(bar(RD1), 256);
-        mbar_init(bar(RD2), 256);
-        mbar_init(bar(ACC_FULL), 2);                                // both issuers
         fence_barrier_init();
-    }
-    __syncthreads();
-    if (!w_valid) {
-        if (blockIdx.x == gridDim.x - 1) previous_done();
-        return;
-    }
-    if (warp == 8) {
+    } else if (warp == 1) {
+        if (lane == 0) {
+            s_abort = 0;
+            int valid = (*(volatile int *)p.status == 0);
+            if (valid && (uint32_t)((volatile int *)p.status)[ST_COOKIE] != p.cookie) {
+                atomicCAS(p.status, 0, MOC_ERR_WORKSPACE);      // not this plan's lists: report, touch nothing else
+                valid = 0;
+            }
+            uint32_t dyn_bytes;
+            asm volatile("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn_bytes));
+            if (valid && (sbase - smem_u32(smem_raw)) + (uint32_t)N_TILES_SMEM * TILE_BYTES > dyn_bytes) {
+                // the launch gave less shared memory than the tiles need: report, touch nothing
+                if (atomicCAS(p.status, 0, MOC_ERR_TIMEOUT) == 0) p.status[1] = BW_SMEM;
+                valid = 0;
+            }
+            w_valid = valid;
+        }
+    } else if (warp == 2) {
+        if (lane == 0) {
+            // block order: the long key tiles of every head, then the others head by head (tiles of one chunk next
+            // to each other: they stream the same query rows)
+            const int n_long_all = p.n_long * p.H;
+            int b = blockIdx.x, hh, ti;
+            if (b < n_long_all) { hh = b / p.n_long; ti = b - hh * p.n_long; }
+            else { b -= n_long_all; const int n_rest = p.n_ktiles - p.n_long; hh = b / n_rest; ti = p.n_long + b - hh * n_rest; }
+            const KTile kt = p.ktiles[ti];
+            const int n_list = p.cnt[hh * p.C + kt.chunk];
+            s_kt = kt;
+            w_h = hh;
+            w_list = n_list;
+            w_ntiles = kt.n_anc + (n_list + 127) / 128;
+        }
+    } else if (warp == 8) {
         tmem_alloc(smem_u32(&tmem_slot), 512);
         tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (!w_valid) {
+        if (warp == 8) tmem_dealloc(tmem_slot, 512);
+        if (blockIdx.x == gridDim.x - 1) previous_done();
+        return;
+    }
 
     // TMEM columns: T1 [0,128)  T2 [128,256)  ACC1 [256,384)  ACC2 [384,512)
     const uint32_t tmem = tmem_slot;
-    const int h = w_h, rows = w_rows, n_tiles = w_ntiles;
+    const int h = w_h, rows = s_kt.valid, n_tiles = w_ntiles, key0 = s_kt.t0;
     volatile int *abort_flag = &s_abort;
 
     if (warp < 8) {
@@ -262,34 +250,30 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
         }
         if (ok) {
             tc_fence_after();
+            // Four lanes write 128 contiguous bytes of a row (tmem_ld_16x256b).  Of the two warps that share the TMEM lanes, each
+            // takes 64 columns of all rows (d = 128) or 16 rows (d = 64).
+            constexpr int NJ = D / 32;                       // groups of eight rows that this warp has
+            const int l4 = lane >> 2, l2 = lane & 3, cb = D == 128 ? half : 0, j0 = D == 128 ? 0 : 2 * half;
 #pragma unroll 1
-            for (int ch = half; ch < D / 32; ch += 2) {
-                uint32_t v[32];
+            for (int side = 0; side < 2; ++side) {           // dK = scale ACC1, dV = ACC2
+                uint32_t v[NJ / 2][32];
                 __syncwarp();
-                tmem_ld32(tmem + lane_off + 256 + ch * 32, v);
+#pragma unroll
+                for (int x = 0; x < NJ / 2; ++x)
+                    tmem_ld_16x256b(tmem + lane_off + 256 + side * 128 + ((uint32_t)(x + (j0 >> 1)) << 20) + cb * 64, v[x]);
                 tmem_wait_ld();
-                float acc[32];
+                const float w = side ? 1.f : p.scale;
+                __nv_bfloat16 *dst = (side ? p.dV : p.dK) + ((size_t)h * p.L + key0) * D + cb * 64;
 #pragma unroll
-                for (int x = 0; x < 32; ++x) acc[x] = __uint_as_float(v[x]) * p.scale;
-                auto store_row = [&](__nv_bfloat16 *dst) {
+                for (int y = 0; y < NJ; ++y) {
+                    const int row = (warp & 3) * 32 + (j0 + y) * 8 + l4;
+                    uint32_t u[8];
 #pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {
-                        uint4 out;
-                        out.x = bf16x2(acc[q4 * 8 + 0], acc[q4 * 8 + 1]);
-                        out.y = bf16x2(acc[q4 * 8 + 2], acc[q4 * 8 + 3]);
-                        out.z = bf16x2(acc[q4 * 8 + 4], acc[q4 * 8 + 5]);
-                        out.w = bf16x2(acc[q4 * 8 + 6], acc[q4 * 8 + 7]);
-                        reinterpret_cast<uint4 *>(dst)[q4] = out;
-                    }
-                };
-                if (r < rows) store_row(p.dK + ((size_t)h * p.L + w_t0 + r) * D + ch * 32);
-                // dV = ACC2, not scaled
-                __syncwarp();
-                tmem_ld32(tmem + lane_off + 384 + ch * 32, v);
-                tmem_wait_ld();
-#pragma unroll
-                for (int x = 0; x < 32; ++x) acc[x] = __uint_as_float(v[x]);
-                if (r < rows) store_row(p.dV + ((size_t)h * p.L + w_t0 + r) * D + ch * 32);
+                    for (int x = 0; x < 8; ++x)
+                        u[x] = bf16x2(__uint_as_float(v[y >> 1][4 * x + 2 * (y & 1)]) * w, __uint_as_float(v[y >> 1][4 * x + 2 * (y & 1) + 1]) * w);
+                    quad_transpose(u, l2);
+                    if (row < rows) store_quad(dst + (size_t)row * D, l2, u);
+                }
             }
         }
     } else if (warp < 12) {
@@ -300,8 +284,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             mbar_expect_tx(bar(X_FULL), 2 * TILE_BYTES);
 #pragma unroll
             for (int sub = 0; sub < SUB; ++sub) {
-                tma_load_2d(sX + sub * SUB_BYTES, &tmK, sub * 64, h * p.L + w_t0, bar(X_FULL));
-                tma_load_2d(sX + TILE_BYTES + sub * SUB_BYTES, &tmV, sub * 64, h * p.L + w_t0, bar(X_FULL));
+                tma_load_2d(sX + sub * SUB_BYTES, &tmK, sub * 64, h * p.L + key0, bar(X_FULL));
+                tma_load_2d(sX + TILE_BYTES + sub * SUB_BYTES, &tmV, sub * 64, h * p.L + key0, bar(X_FULL));
             }
         }
         // The queries that attend to this chunk, 128 at a time: Q rows -> Y1 by the first two producer warps, dO rows -> Y2
@@ -311,21 +295,20 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
         // asynchronous copies (36 bytes a cycle and SM; TMA row gathers reach 24).
         const int pw = warp - 8, wsub = pw & 1;
         const bool y1 = pw < 2;
-        const int chunk = w_chunk;
-        const int a1 = p.ranc_off[chunk + 1];
-        int a = p.ranc_off[chunk], r0 = 0, r1 = 0;       // current row range [r0, r1)
-        const int n_list = p.cnt[h * p.C + chunk];
-        const int32_t *list = p.qlist + (size_t)h * p.cap_total + p.cap_off[chunk];
+        const KeyRange *rng = p.qry_rng + s_kt.rng;
+        int n_rng = s_kt.n_rng, r0 = 0, r1 = 0;          // ranges to come; current row range [r0, r1)
+        const int n_list = w_list, list0 = s_kt.list;
+        const int32_t *list = p.qlist + (size_t)h * p.cap_total + list0;
         int e0 = 0;                                        // next entry of the routed list
         bool ok = true;
         // This lane's two rows of a tile, in two steps so that no load is waited for: the list entries two tiles ahead,
         // then, one tile ahead, the queries with their lse and delta.
         int nx_whole = -1, nx_row = -1, nx_end = 0, nx_e[2] = {-1, -1};
         auto look_ahead = [&]() {
-            if (r0 >= r1 && a < a1) {                      // next merged range of anchor query rows
-                int qc = p.ranc[a];
-                r0 = p.off[qc]; r1 = p.off[qc + 1];
-                for (++a; a < a1 && p.ranc[a] == qc + 1; ++a) { qc = p.ranc[a]; r1 = p.off[qc + 1]; }
+            if (r0 >= r1 && n_rng > 0) {                   // next range of anchor query rows
+                r0 = rng->t0; r1 = rng->t1;
+                ++rng;
+                --n_rng;
             }
             const int i = wsub * 64 + lane;
             nx_whole = -1; nx_row = -1; nx_e[0] = nx_e[1] = -1;
@@ -338,7 +321,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
 #pragma unroll
                 for (int x = 0; x < 2; ++x) {
                     const int e = e0 + i + 32 * x;
-                    if (e < n_list && index_ok((size_t)p.cap_off[chunk] + e < p.cap_total, p.status, IX_BWD_LIST_POSITION)) nx_e[x] = list[e];
+                    if (e < n_list && index_ok((size_t)list0 + e < p.cap_total, p.status, IX_BWD_LIST_POSITION)) nx_e[x] = list[e];
                 }
                 e0 += 128;
             }
@@ -575,7 +558,7 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
     a.Q = Q; a.K = K; a.V = V; a.dO = dO; a.lse = lse; a.delta = delta;
     a.cookie = p->cookie;
     a.dK = dK; a.dV = dV;
-    a.ktiles = p->d_ktiles; a.n_ktiles = (int)p->ktiles.size(); a.n_long = p->n_long_ktiles; a.off = p->d_off; a.ranc_off = p->d_ranc_off; a.ranc = p->d_ranc; a.cap_off = p->d_cap_off;
+    a.ktiles = p->d_ktiles; a.n_ktiles = (int)p->ktiles.size(); a.n_long = p->n_long_ktiles; a.qry_rng = p->d_qry_rng;
     a.cnt = ws_ptr<int>(ws, p->ws.cnt);
     a.qlist = ws_ptr<int32_t>(ws, p->ws.qlist);
     a.cap_total = (size_t)p->cap_off[p->C];

@@ -29,8 +29,9 @@ struct KeyRange { int32_t t0, t1; };
 // offset, inside the head's list area, of the `rows` entries of one chunk's query list.
 struct WorkItem { int32_t h, first, rows, ntiles, rng_off, nrng, t0, t1; };
 
-// One tile of up to 128 consecutive key tokens of chunk c (backward, key-stationary pass).
-struct KTile { int32_t chunk, t0, valid, pad; };
+// One tile of up to 128 consecutive key tokens of a chunk (backward, key-stationary pass), with what its block looks up first:
+// the rows that have the chunk as an anchor (n_rng ranges from rng on, n_anc tiles of 128 rows) and where its query list starts.
+struct __align__(32) KTile { int32_t chunk, t0, valid, n_anc, rng, n_rng, list, pad; };
 
 struct WsLayout {
     size_t status;      // int32[kStatusWords], see StatusWord
@@ -67,6 +68,7 @@ struct moc_plan {
     std::vector<int64_t> anc_tokens;         // [C] anchor key tokens per query chunk
     std::vector<int32_t> ranc_off, ranc;     // reverse anchors: key chunk -> query chunks
     std::vector<moc::WorkItem> qitems;       // anchor-pass work items of one head
+    std::vector<moc::KeyRange> qry_rng;      // merged ranges of the query rows that have a chunk as an anchor, chunk by chunk
     std::vector<moc::KTile> ktiles;          // key tiles of one head: the long ones (see moc_plan_create) first, then chunk by chunk
     int n_long_ktiles = 0;
     std::vector<int32_t> pool_unit_off;      // [C+1] prefix of pool units per chunk
@@ -96,6 +98,7 @@ struct moc_plan {
     moc::WorkItem *d_qitems;
     moc::KeyRange *d_chunk_rng;              // [C] token range of every chunk
     moc::KTile *d_ktiles;
+    moc::KeyRange *d_qry_rng;
     moc::KeyRange *d_shot_chunks;            // [S]
     moc::WsLayout ws;
 };

@@ -190,11 +190,24 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
             tiles += nt;
         }
         const int64_t mean_rows = total / std::max<int64_t>(tiles, 1);
+        // the rows, as ranges: consecutive chunks are one
+        std::vector<int32_t> rng_off(C + 1, 0), rng_tiles(C, 0);
+        for (int c = 0; c < C; ++c) {
+            for (int a = p->ranc_off[c]; a < p->ranc_off[c + 1];) {
+                int qc = p->ranc[a];
+                KeyRange r{p->off[qc], p->off[qc + 1]};
+                for (++a; a < p->ranc_off[c + 1] && p->ranc[a] == qc + 1; ++a) r.t1 = p->off[++qc + 1];
+                p->qry_rng.push_back(r);
+                rng_tiles[c] += (r.t1 - r.t0 + 127) / 128;
+            }
+            rng_off[c + 1] = (int32_t)p->qry_rng.size();
+        }
         for (int pass = 0; pass < 2; ++pass) {
             for (int c = 0; c < C; ++c) {
                 const bool is_long = anc_rows[c] > 4 * mean_rows;
                 if (is_long != (pass == 0)) continue;
-                for (int t = p->off[c]; t < p->off[c + 1]; t += 128) p->ktiles.push_back(KTile{c, t, std::min(128, p->off[c + 1] - t), 0});
+                for (int t = p->off[c]; t < p->off[c + 1]; t += 128)
+                    p->ktiles.push_back(KTile{c, t, std::min(128, p->off[c + 1] - t), rng_tiles[c], rng_off[c], rng_off[c + 1] - rng_off[c], 0, 0});
             }
             if (pass == 0) p->n_long_ktiles = (int)p->ktiles.size();
         }
@@ -209,6 +222,7 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
         if (next >= 2147483647LL) { delete p; return MOC_ERR_SHAPE; }
         p->cap_off[c + 1] = (int32_t)next;
     }
+    for (KTile &kt : p->ktiles) kt.list = p->cap_off[kt.chunk];
     // score columns: the chunks that are not text; per query chunk its candidate columns (not an anchor, strictly
     // earlier if causal), whether they form a prefix of the columns (they do under the causal rule: everything
     // before the own shot's window), and how far any query up to that chunk can reach
@@ -252,7 +266,7 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     size_t o_off = take(4 * (C + 1)), o_shot = take(4 * C), o_mod = take(C), o_tok = take(4 * (size_t)L);
     size_t o_bits = take(4 * bits.size()), o_aoff = take(4 * (C + 1)), o_arng = take(sizeof(KeyRange) * p->anc_rng.size());
     size_t o_roff = take(4 * (C + 1)), o_ranc = take(4 * p->ranc.size()), o_qt = take(sizeof(WorkItem) * p->qitems.size());
-    size_t o_puo = take(4 * (C + 1)), o_puc = take(4 * unit_chunk.size()), o_cap = take(4 * (C + 1)), o_crng = take(sizeof(KeyRange) * C), o_kt = take(sizeof(KTile) * p->ktiles.size());
+    size_t o_puo = take(4 * (C + 1)), o_puc = take(4 * unit_chunk.size()), o_cap = take(4 * (C + 1)), o_crng = take(sizeof(KeyRange) * C), o_kt = take(sizeof(KTile) * p->ktiles.size()), o_qrng = take(sizeof(KeyRange) * p->qry_rng.size());
     size_t o_shots = take(sizeof(KeyRange) * p->shot_chunks.size());
     size_t o_candc = take(4 * cand_c.size()), o_lim = take(4 * C), o_reach = take(4 * C), o_colc = take(4 * std::max<size_t>(col_chunk.size(), 1));
     cudaError_t e = cudaMalloc(&p->d_blob, o);
@@ -276,6 +290,7 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     up(o_cap, p->cap_off.data(), 4 * (C + 1));
     up(o_crng, chunk_rng.data(), sizeof(KeyRange) * C);
     up(o_kt, p->ktiles.data(), sizeof(KTile) * p->ktiles.size());
+    up(o_qrng, p->qry_rng.data(), sizeof(KeyRange) * p->qry_rng.size());
     up(o_candc, cand_c.data(), 4 * cand_c.size());
     up(o_lim, lim.data(), 4 * C);
     up(o_reach, reach.data(), 4 * C);
@@ -294,6 +309,7 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     p->d_cap_off = (int32_t *)(b + o_cap);
     p->d_chunk_rng = (KeyRange *)(b + o_crng);
     p->d_ktiles = (KTile *)(b + o_kt);
+    p->d_qry_rng = (KeyRange *)(b + o_qrng);
     p->d_cand_c = (uint32_t *)(b + o_candc); p->d_lim = (int32_t *)(b + o_lim); p->d_reach = (int32_t *)(b + o_reach);
     p->d_col_chunk = (int32_t *)(b + o_colc);
     p->d_shot_chunks = (KeyRange *)(b + o_shots);
