@@ -255,10 +255,13 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 }
                 continue;
             }
-            const int rt = g * 128 + r;                 // row within the work item
+            // Row of the tile and of the item.  With four loading warps the rows of an anchor item's tile are dealt to the four
+            // softmax warps in equal parts, so that a tile of a few rows keeps all of them busy in the merge.
+            const int tile_rows = min(128, rows - g * 128), warp_rows = LOADERS && !routed ? (tile_rows + 3) >> 2 : 32;
+            const int row = (warp & 3) * warp_rows + lane, rt = g * 128 + row;
             // the list entry of a routed row is asked for here and looked at in the epilogue
             int qi = -1, entry = -1;
-            if (rt < rows) {
+            if (lane < warp_rows && row < tile_rows) {
                 if (!routed) qi = first + rt;
                 else if (index_ok((size_t)first + rt < p.cap_total, p.status, IX_LIST_POSITION))
                     entry = p.qlist[(size_t)h * p.cap_total + first + rt];
@@ -269,7 +272,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             if (!routed && qi >= 0 && p.k > 0) {
                 // the epilogue will merge this row's routed partials: start them on their way into L2 now
                 // (few picks only: what all CTAs ask for ahead has to stay in L2 until it is read)
-                if ((qi & 31) == 0 || r == 0)
+                if ((qi & 31) == 0 || lane == 0)
                     for (int s = 0; s < p.k; ++s) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.part_lse + part_lse_at(h, LB, p.k, qi, s)));
                 if (p.k <= 8)
                     for (int x = 0; x < p.k * (D / 64); ++x) asm volatile("prefetch.global.L2 [%0];" ::"l"(part + part_line(h_loc, LB, p.k, D / 64, qi, 0) + ((size_t)x << 14)));
@@ -405,7 +408,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             if (routed) {
                 size_t line = 0;                        // where this row's partial goes
                 bool keep = false;
-                if (rt < rows) {
+                if (g * 128 + r < rows) {
                     const int q = p.kdiv.query(entry), slot = entry - q * p.k;
                     (void)index_ok(entry >= 0 && q < p.L, p.status, IX_LIST_ENTRY);
                     if (entry >= 0 && q < p.L) {         // never follow an entry that is not a row of this head
@@ -458,7 +461,8 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 // for the epilogue of 256 rows, the loads of a row by its own thread before -> this: d = 128, 4 picks 15000 -> 13700 by
                 // copies, 22900 by register loads; d = 64, 25 picks 38500 -> 33000, 56900; the whole launch on 256-token chunks, 30 picks,
                 // 18.8 -> 13.8 ms by register loads, 15.2 by copies.)
-                const int q0 = first + g * 128 + (warp & 3) * 32, n_rows = min(32, first + rows - q0);   // the warp's rows
+                const int tile_rows = min(128, rows - g * 128), warp_rows = LOADERS ? (tile_rows + 3) >> 2 : 32;
+                const int q0 = first + g * 128 + (warp & 3) * warp_rows, n_rows = min(warp_rows, first + g * 128 + tile_rows - q0);   // the warp's rows
                 const int n_merge = n_rows > 0 ? p.k : 0;
                 const int qb = it_.qbuf + g < 3 ? it_.qbuf + g : it_.qbuf + g - 3;
                 const uint32_t m_base = D == 128 ? sQ + qb * TILE_BYTES + (warp & 3) * (TILE_BYTES / 4) : sbase + 7 * TILE_BYTES + warp * (kMergeStages * 4096);
@@ -500,10 +504,10 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 }
                 const float inv_w = 1.f / wsum, w_own = __expf(lse_own - big) * inv_l, big_log2 = big * kLog2e;
                 if constexpr (kMergeInRegs) {
-                    // Four passes, eight of the warp's rows each, over the slots, a few at a time: the loads of the next few are on
-                    // their way while these are added up.
+                    // Passes of eight of the warp's rows over the slots, a few at a time: the loads of the next few are on their way
+                    // while these are added up.
                     constexpr int B = 3;
-                    const int row0 = first + g * 128 + (warp & 3) * 32 + l4, row_end = first + rows;   // query of row l4 of the warp's
+                    const int row0 = q0 + l4, row_end = q0 + n_rows, n_pass = max(1, (n_rows + 7) >> 3);
                     struct Batch { uint32_t v[B][CB][8]; float ls[B]; };
                     int ask_pass = 0, ask_s = 0;
                     auto ask = [&](Batch &b) __attribute__((always_inline)) {
@@ -540,7 +544,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                                 for (int x = 0; x < 8; ++x)
                                     acc[cb][x] = mul2(pack2(__uint_as_float((pass & 1) ? o[x * 4 + 2] : o[x * 4]), __uint_as_float((pass & 1) ? o[x * 4 + 3] : o[x * 4 + 1])), w2);
                             }
-                            if (pass == 3) {
+                            if (pass == n_pass - 1) {
                                 // O has been read: the issuer may start the next item's P V (which overwrites it)
                                 tc_fence_before();
                                 mbar_arrive(bar(O_FREE + g));
@@ -582,11 +586,13 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                     if (!ok) break;
                     tc_fence_after();
 #pragma unroll 1
-                    while (pass < 4) {                           // an even number of passes, so of batches
+                    while (true) {                               // (past the last pass no row is asked for)
                         ask(odd);
                         add(even);
-                        if (ask_pass < 4) ask(even);
+                        if (pass == n_pass) break;
+                        ask(even);
                         add(odd);
+                        if (pass == n_pass) break;
                     }
                 } else {
                     ok = mbar_wait(bar(O_FULL + g), (bits & MINE_ODD) ? 1 : 0, abort_flag, p.status, W_OFULL);
@@ -1085,8 +1091,8 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 if (!routed) {
                     if (lane == 0) {
 #pragma unroll
-                        for (int sub = 0; sub < SUB; ++sub)
-                            tma_load_2d(dst + sub * SUB_BYTES, &tmQ, sub * 64, h * p.L + first + g * 128 + lw * 32, bar(Q_FULL + qf));
+                        for (int sub = 0; sub < SUB; ++sub)          // (32 rows, of which the tile's part for the warp comes first)
+                            tma_load_2d(dst + sub * SUB_BYTES, &tmQ, sub * 64, h * p.L + first + g * 128 + lw * ((min(128, rows - g * 128) + 3) >> 2), bar(Q_FULL + qf));
                     }
                 } else if (lane < 8) {                          // lane l gathers rows 4 l .. 4 l + 3 of the warp's 32
 #pragma unroll
