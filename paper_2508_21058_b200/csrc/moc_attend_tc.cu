@@ -149,6 +149,12 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                   O_FULL = 23, O_FREE = 25, TURN = 27, ROWS_DONE = 29, DEPEND = 37, ITEM_FULL = 38, ITEM_EMPTY = ITEM_FULL + kItemSlots,
                   MERGED = ITEM_EMPTY + kItemSlots, MERGE = MERGED + 3;
     constexpr int kMergeStages = D == 128 ? 2 : 3;                     // blocks of partials under way per softmax warp
+    // Registers of a thread after the split; warpgroup by warpgroup they add up to what the launch gave (3 x 168, 4 x 128).  (At
+    // d = 64 the issuing warps need more than the loading ones: 210-token chunks, 25 picks 8.54 -> 8.35 ms, a 576-token clip 15.7 ->
+    // 15.2 us; at d = 128 within half a per cent.)
+    constexpr int kRegsSoftmax = 224, kRegsIssue = !LOADERS ? 56 : D == 64 ? 40 : 32, kRegsLoad = D == 64 ? 24 : 32;
+    static_assert(!LOADERS || 2 * kRegsSoftmax + kRegsIssue + kRegsLoad == 512, "setmaxnreg would wait for registers that there are not");
+    static_assert(LOADERS || 2 * kRegsSoftmax + kRegsIssue == 504, "setmaxnreg would wait for registers that there are not");
     // Who merges the routed partials how: see the epilogue of the anchor items.
     constexpr bool kMergeInRegs = D == 128 && LOADERS;
     constexpr int kItemReaders = 2 + 2 + 256 + (LOADERS ? 4 : 0);      // producer and bookkeeping lanes, two issuing warps, every softmax thread, loading warps
@@ -216,7 +222,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
         // ------------------------------------------------------------ softmax / epilogue groups
         // the row-per-thread softmax holds a whole 128-key row of S in registers: take the
         // registers the third warpgroup gives up
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));
         const int g = warp >> 2;                       // query tile of this group
         const int r = threadIdx.x & 127;               // row within the tile = TMEM lane
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
@@ -680,8 +686,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             bits ^= MINE_ODD;
         }
     } else if (warp == 8) {
-        if (LOADERS) asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
-        else asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
         if (lane == 0) {
             // ------------------------------------------------------------ TMA producer of the K and V tiles
             prefetch_tensormap(&tmK);
@@ -793,8 +798,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             }
         }
     } else if (warp < 11) {
-        if (LOADERS) asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
-        else asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
         // ------------------------------------------------------------ MMA issuers (one warp per query tile; the warp stays
         // together, one lane of it issues)
         const int g = uniform(warp - 9);
@@ -920,8 +924,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             }
         }
     } else if (!LOADERS || warp == 11) {
-        if (LOADERS) asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
-        else asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsIssue));
         // ------------------------------------------------------------ scheduler (lane 0 claims items in queue order) and
         // Q loader (the whole warp): a claimed item is published at once, then its query tiles are loaded as their
         // buffers come free, which for the first tile is before the previous item has finished
@@ -1045,7 +1048,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             for (int b = 0; b < 6; ++b) mbar_wait(bar(Q_FULL + b), ((q_phase >> b) & 1) ^ 1, &dummy_flag, p.status, W_QFULL);
         }
     } else {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLoad));
         // ------------------------------------------------------------ Q loaders: rows 32 lw .. 32 lw + 31 of every query tile.
         // All four warps load a part of every tile, so a buffer cannot be filled and released without one of them: none
         // can miss a phase of Q_EMPTY.
