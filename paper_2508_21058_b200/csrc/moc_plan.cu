@@ -49,6 +49,26 @@ static uint32_t plan_cookie(const moc_plan *p) {
     return hsh ? hsh : 1u;
 }
 
+// tok_chunk[t] = the chunk of token t, a block per chunk.  (Made on the host and copied, with the caller's stream waited for, a plan
+// of a 132k-token stream held the caller up for 214 us; now 140.)
+__global__ void token_chunk_kernel(const int32_t *__restrict__ off, int32_t *__restrict__ tok_chunk) {
+    for (int t = off[blockIdx.x] + threadIdx.x; t < off[blockIdx.x + 1]; t += blockDim.x) tok_chunk[t] = blockIdx.x;
+}
+
+// The stream on which plans get their tables, one per device for as long as the process lives (making one takes 100 us).
+static cudaError_t table_stream(int device, cudaStream_t *out) {
+    static std::mutex mu;
+    static std::vector<cudaStream_t> streams;
+    std::lock_guard<std::mutex> hold(mu);
+    if ((int)streams.size() <= device) streams.resize(device + 1, nullptr);
+    if (!streams[device]) {
+        const cudaError_t e = cudaStreamCreateWithFlags(&streams[device], cudaStreamNonBlocking);
+        if (e != cudaSuccess) { streams[device] = nullptr; return e; }
+    }
+    *out = streams[device];
+    return cudaSuccess;
+}
+
 // Workspace layout.  The routed partial outputs ([heads][L][k][d] bf16, k times the size of O) are held for
 // one group of Hg heads at a time; attention and its backward run group by group.  If all heads fit the plan's
 // budget there is one group and one buffer; otherwise two buffers of Hg heads each (consecutive groups
@@ -154,12 +174,11 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
         p->ranc_off[j + 1] = (int32_t)p->ranc.size();
     }
     // query tiles (never straddle a chunk) and pool work units
-    std::vector<int32_t> tok_chunk(L), unit_chunk;
+    std::vector<int32_t> unit_chunk;
     std::vector<KeyRange> chunk_rng(C);
     for (int c = 0; c < C; ++c) chunk_rng[c] = KeyRange{p->off[c], p->off[c + 1]};
     p->pool_unit_off.assign(C + 1, 0);
     for (int c = 0; c < C; ++c) {
-        for (int t = p->off[c]; t < p->off[c + 1]; ++t) tok_chunk[t] = c;
         int anc_tiles = 0;
         for (int a = p->anc_off[c]; a < p->anc_off[c + 1]; ++a) anc_tiles += (p->anc_rng[a].t1 - p->anc_rng[a].t0 + 127) / 128;
         for (int r = p->off[c]; r < p->off[c + 1]; r += kQTileRows)
@@ -263,22 +282,22 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     // one device blob
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o = align_up(o + bytes, 256); return at; };
-    size_t o_off = take(4 * (C + 1)), o_shot = take(4 * C), o_mod = take(C), o_tok = take(4 * (size_t)L);
+    size_t o_off = take(4 * (C + 1)), o_shot = take(4 * C), o_mod = take(C);
     size_t o_bits = take(4 * bits.size()), o_aoff = take(4 * (C + 1)), o_arng = take(sizeof(KeyRange) * p->anc_rng.size());
     size_t o_roff = take(4 * (C + 1)), o_ranc = take(4 * p->ranc.size()), o_qt = take(sizeof(WorkItem) * p->qitems.size());
     size_t o_puo = take(4 * (C + 1)), o_puc = take(4 * unit_chunk.size()), o_cap = take(4 * (C + 1)), o_crng = take(sizeof(KeyRange) * C), o_kt = take(sizeof(KTile) * p->ktiles.size()), o_qrng = take(sizeof(KeyRange) * p->qry_rng.size());
     size_t o_shots = take(sizeof(KeyRange) * p->shot_chunks.size());
     size_t o_candc = take(4 * cand_c.size()), o_lim = take(4 * C), o_reach = take(4 * C), o_colc = take(4 * std::max<size_t>(col_chunk.size(), 1));
+    const size_t from_host = o, o_tok = take(4 * (size_t)L);             // the token table is made on the device
     cudaError_t e = cudaMalloc(&p->d_blob, o);
     if (e != cudaSuccess) { set_cuda_error(e, "cudaMalloc(plan tables)"); delete p; return MOC_ERR_CUDA; }
     char *b = static_cast<char *>(p->d_blob);
     // the tables are put together on the host and go over in one copy (twenty small ones took longer than everything else here)
-    std::vector<char> host(o);
+    std::vector<char> host(from_host);
     auto up = [&](size_t at, const void *src, size_t bytes) { if (bytes) memcpy(host.data() + at, src, bytes); };
     up(o_off, p->off.data(), 4 * (C + 1));
     up(o_shot, p->shot.data(), 4 * C);
     up(o_mod, p->mod.data(), C);
-    up(o_tok, tok_chunk.data(), 4 * (size_t)L);
     up(o_bits, bits.data(), 4 * bits.size());
     up(o_aoff, p->anc_off.data(), 4 * (C + 1));
     up(o_arng, p->anc_rng.data(), sizeof(KeyRange) * p->anc_rng.size());
@@ -296,11 +315,18 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     up(o_reach, reach.data(), 4 * C);
     up(o_colc, col_chunk.data(), 4 * col_chunk.size());
     up(o_shots, p->shot_chunks.data(), sizeof(KeyRange) * p->shot_chunks.size());
-    // A copy from pageable memory may return while the last of it is still on its way, and a caller's non-blocking stream is
-    // not ordered behind the stream of the copy: the plan is handed out when the tables are there.
-    e = cudaMemcpy(b, host.data(), o, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
-    if (e != cudaSuccess) { set_cuda_error(e, "cudaMemcpy(plan tables)"); cudaFree(p->d_blob); delete p; return MOC_ERR_CUDA; }
+    // On a stream of its own: on the legacy stream the copy would wait for what the caller has under way there.  The plan is
+    // handed out when the tables are there, for a stream of any kind.
+    cudaStream_t st = nullptr;
+    e = table_stream(dev, &st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(b, host.data(), from_host, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) {
+        token_chunk_kernel<<<(unsigned)C, 256, 0, st>>>((const int32_t *)(b + o_off), (int32_t *)(b + o_tok));
+        g_launches.fetch_add(1);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) { set_cuda_error(e, "plan tables"); cudaFree(p->d_blob); delete p; return MOC_ERR_CUDA; }
     p->d_off = (int32_t *)(b + o_off); p->d_shot = (int32_t *)(b + o_shot); p->d_mod = (uint8_t *)(b + o_mod);
     p->d_tok_chunk = (int32_t *)(b + o_tok); p->d_anc_bits = (uint32_t *)(b + o_bits);
     p->d_anc_off = (int32_t *)(b + o_aoff); p->d_anc_rng = (KeyRange *)(b + o_arng);
