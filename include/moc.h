@@ -229,7 +229,8 @@ int moc_outer_reduced_layout(const moc_plan *plan, const int32_t *sel_shot, int3
  * stream keeps (tok_map: DEVICE int32; out: DEVICE [H][n_out][d] bf16). */
 int moc_gather_tokens(const moc_plan *plan, const void *X, const int32_t *tok_map, int32_t n_out, void *out, void *stream);
 
-/* How many kernel launches the library has enqueued since it was loaded. */
+/* How many kernel launches the library's calls have enqueued since it was loaded (plan creation, which fills a
+ * table with one, not counted). */
 int64_t moc_launch_count(void);
 
 const char *moc_strerror(int status);

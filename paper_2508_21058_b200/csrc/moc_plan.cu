@@ -322,7 +322,6 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     if (e == cudaSuccess) e = cudaMemcpyAsync(b, host.data(), from_host, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
         token_chunk_kernel<<<(unsigned)C, 256, 0, st>>>((const int32_t *)(b + o_off), (int32_t *)(b + o_tok));
-        g_launches.fetch_add(1);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
