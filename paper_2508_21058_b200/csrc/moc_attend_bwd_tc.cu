@@ -38,6 +38,9 @@ struct BwdParams {
     uint32_t cookie;              // what the workspace's status area must hold
     const KTile *ktiles;
     int n_ktiles, n_long;         // tiles per head, and how many of them come first for every head
+    int n_split;                  // blocks that share the query tiles of one of those
+    float4 *split_sum;            // their sums, [tile][block][dK, dV], each as the lane threads hold it
+    int *split_done;              // [tile] blocks that have left theirs
     const KeyRange *qry_rng;
     const int *cnt;
     const int32_t *qlist;
@@ -68,6 +71,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort;
     __shared__ int w_valid, w_h, w_ntiles, w_list;       // w_list: entries of the chunk's query list
+    __shared__ int w_skip, w_part, w_split, s_last;      // query tiles of the blocks before this one, which shares tile w_split with others (-1: none)
     __shared__ KTile s_kt;
     // per streamed query, (-lse * log2(e), -delta), for tiles j and j + 1
     __shared__ __align__(16) float s_ld[2][2][128];
@@ -112,16 +116,24 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
         if (lane == 0) {
             // block order: the long key tiles of every head, then the others head by head (tiles of one chunk next
             // to each other: they stream the same query rows)
-            const int n_long_all = p.n_long * p.H;
-            int b = blockIdx.x, hh, ti;
-            if (b < n_long_all) { hh = b / p.n_long; ti = b - hh * p.n_long; }
-            else { b -= n_long_all; const int n_rest = p.n_ktiles - p.n_long; hh = b / n_rest; ti = p.n_long + b - hh * n_rest; }
+            const int n_long_all = p.n_long * p.H * p.n_split;
+            int b = blockIdx.x, hh, ti, part = 0, parts = 1;
+            if (b < n_long_all) {
+                parts = p.n_split;
+                part = b % parts;
+                b /= parts;
+                w_split = parts > 1 ? b : -1;
+                hh = b / p.n_long; ti = b - hh * p.n_long;
+            } else { w_split = -1; b -= n_long_all; const int n_rest = p.n_ktiles - p.n_long; hh = b / n_rest; ti = p.n_long + b - hh * n_rest; }
             const KTile kt = p.ktiles[ti];
             const int n_list = p.cnt[hh * p.C + kt.chunk];
             s_kt = kt;
             w_h = hh;
             w_list = n_list;
-            w_ntiles = kt.n_anc + (n_list + 127) / 128;
+            const int nt = kt.n_anc + (n_list + 127) / 128;
+            w_part = part;
+            w_skip = (int)((long long)nt * part / parts);
+            w_ntiles = (int)((long long)nt * (part + 1) / parts) - w_skip;
         }
     } else if (warp == 8) {
         tmem_alloc(smem_u32(&tmem_slot), 512);
@@ -254,14 +266,16 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             // takes 64 columns of all rows (d = 128) or 16 rows (d = 64).
             constexpr int NJ = D / 32;                       // groups of eight rows that this warp has
             const int l4 = lane >> 2, l2 = lane & 3, cb = D == 128 ? half : 0, j0 = D == 128 ? 0 : 2 * half;
-#pragma unroll 1
-            for (int side = 0; side < 2; ++side) {           // dK = scale ACC1, dV = ACC2
-                uint32_t v[NJ / 2][32];
+            const int slot = w_split, me = (half * 4 + (warp & 3)) * 32 + lane;
+            constexpr int NV = NJ / 2 * 8;                   // float4s of a thread and side
+            auto load = [&](int side, uint32_t (&v)[NJ / 2][32]) {
                 __syncwarp();
 #pragma unroll
                 for (int x = 0; x < NJ / 2; ++x)
                     tmem_ld_16x256b(tmem + lane_off + 256 + side * 128 + ((uint32_t)(x + (j0 >> 1)) << 20) + cb * 64, v[x]);
                 tmem_wait_ld();
+            };
+            auto store = [&](int side, const uint32_t (&v)[NJ / 2][32]) {       // dK = scale ACC1, dV = ACC2
                 const float w = side ? 1.f : p.scale;
                 __nv_bfloat16 *dst = (side ? p.dV : p.dK) + ((size_t)h * p.L + key0) * D + cb * 64;
 #pragma unroll
@@ -273,6 +287,64 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                         u[x] = bf16x2(__uint_as_float(v[y >> 1][4 * x + 2 * (y & 1)]) * w, __uint_as_float(v[y >> 1][4 * x + 2 * (y & 1) + 1]) * w);
                     quad_transpose(u, l2);
                     if (row < rows) store_quad(dst + (size_t)row * D, l2, u);
+                }
+            };
+            uint32_t v[NJ / 2][32];
+            if (slot < 0) {
+#pragma unroll 1
+                for (int side = 0; side < 2; ++side) {
+                    load(side, v);
+                    store(side, v);
+                }
+            } else {
+                // Shared with other blocks: each leaves its sums, and the last one adds them up, in the order of the blocks whichever
+                // is last.  They lie where dQ's routed partials were, which dQ's launches have done with.
+                previous_done();
+                auto sums = [&](int part, int side) { return p.split_sum + (((size_t)slot * p.n_split + part) * 2 + side) * (NV * 256) + me; };
+#pragma unroll 1
+                for (int side = 0; side < 2; ++side) {
+                    load(side, v);
+                    float4 *to = sums(w_part, side);
+#pragma unroll
+                    for (int x = 0; x < NV; ++x) {
+                        const uint32_t *f = &v[x >> 3][4 * (x & 7)];
+                        to[x * 256] = make_float4(__uint_as_float(f[0]), __uint_as_float(f[1]), __uint_as_float(f[2]), __uint_as_float(f[3]));
+                    }
+                }
+                // (the lane threads' own two barriers, once more: every wait here is bounded)
+                mbar_arrive(bar(RD1));
+                ok = mbar_wait_spin(bar(RD1), n_tiles & 1, abort_flag, p.status, BW_READ);
+                if (threadIdx.x == 0 && ok) {
+                    __threadfence();
+                    s_last = atomicAdd(p.split_done + slot, 1) == p.n_split - 1;
+                    __threadfence();
+                }
+                mbar_arrive(bar(RD2));
+                ok = ok && mbar_wait_spin(bar(RD2), n_tiles & 1, abort_flag, p.status, BW_READ);
+                ok = __all_sync(0xffffffffu, ok);
+                if (ok && s_last) {
+#pragma unroll 1
+                    for (int side = 0; side < 2; ++side) {
+                        __syncwarp();
+#pragma unroll
+                        for (int x = 0; x < NV; ++x)
+#pragma unroll
+                            for (int y = 0; y < 4; ++y) v[x >> 3][4 * (x & 7) + y] = 0u;
+#pragma unroll 1
+                        for (int part = 0; part < p.n_split; ++part) {
+                            const float4 *from = sums(part, side);
+#pragma unroll
+                            for (int x = 0; x < NV; ++x) {
+                                const float4 f = __ldcg(from + x * 256);
+                                uint32_t *a = &v[x >> 3][4 * (x & 7)];
+                                a[0] = __float_as_uint(__uint_as_float(a[0]) + f.x);
+                                a[1] = __float_as_uint(__uint_as_float(a[1]) + f.y);
+                                a[2] = __float_as_uint(__uint_as_float(a[2]) + f.z);
+                                a[3] = __float_as_uint(__uint_as_float(a[3]) + f.w);
+                            }
+                        }
+                        store(side, v);
+                    }
                 }
             }
         }
@@ -350,6 +422,15 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             }
             look_ahead();
         };
+        for (int skip = w_skip; skip > 0; --skip) {        // the query tiles of the blocks before this one
+            if (r0 >= r1 && n_rng > 0) {
+                r0 = rng->t0; r1 = rng->t1;
+                ++rng;
+                --n_rng;
+            }
+            if (r0 < r1) r0 += 128;
+            else e0 += 128;
+        }
         if (n_tiles > 0) { look_ahead(); next_rows(); }
         int st = 0, ph = 0;                                // stage of tile jt in this warp's ring, and its phase
         int issued = 0;                                    // tiles whose copies this warp has issued
@@ -548,7 +629,11 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
                            const __nv_bfloat16 *O, const float *lse, const __nv_bfloat16 *dO, const int32_t *sel,
                            __nv_bfloat16 *dQ, __nv_bfloat16 *dK, __nv_bfloat16 *dV, void *ws, cudaStream_t s) {
     float *delta = ws_ptr<float>(ws, p->ws.delta);
-    if (int r = launch_delta(p, O, dO, delta, s)) return r;
+    // split key tiles leave their sums in the space of the routed partials, if that is large enough
+    const size_t sums = 2 * sizeof(float) * 128 * (size_t)D * p->n_long_ktiles * p->H;
+    const int n_split = p->n_split > 1 && sums * p->n_split <= p->ws.part_lse - p->ws.part_o ? p->n_split : 1;
+    int *split_done = ws_ptr<int>(ws, p->ws.pool_done);
+    if (int r = launch_delta(p, O, dO, delta, split_done, n_split > 1 ? p->n_long_ktiles * p->H : 0, s)) return r;
     CUtensorMap tmK, tmV, tmQ, tmdO;       // Q and dO: tiles of 64 rows
     if (int r = make_tmap_2d_bf16(&tmK, K, (uint64_t)p->H * p->L, D, 128)) return r;
     if (int r = make_tmap_2d_bf16(&tmV, V, (uint64_t)p->H * p->L, D, 128)) return r;
@@ -558,7 +643,9 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
     a.Q = Q; a.K = K; a.V = V; a.dO = dO; a.lse = lse; a.delta = delta;
     a.cookie = p->cookie;
     a.dK = dK; a.dV = dV;
-    a.ktiles = p->d_ktiles; a.n_ktiles = (int)p->ktiles.size(); a.n_long = p->n_long_ktiles; a.qry_rng = p->d_qry_rng;
+    a.ktiles = p->d_ktiles; a.n_ktiles = (int)p->ktiles.size(); a.n_long = p->n_long_ktiles;
+    a.n_split = n_split; a.split_sum = ws_ptr<float4>(ws, p->ws.part_o); a.split_done = split_done;
+    a.qry_rng = p->d_qry_rng;
     a.cnt = ws_ptr<int>(ws, p->ws.cnt);
     a.qlist = ws_ptr<int32_t>(ws, p->ws.qlist);
     a.cap_total = (size_t)p->cap_off[p->C];
@@ -576,7 +663,7 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
     if (smem < tiles) return MOC_ERR_SHAPE;
     MOC_CUDA_TRY(cudaFuncSetAttribute(attend_dkv_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (int r = launch_dq_tc(p, Q, K, V, lse, delta, dO, dQ, ws, s)) return r;
-    MOC_CUDA_TRY(launch_early(backward_overlaps(p), attend_dkv_tc_kernel<D>, (unsigned)(p->ktiles.size() * (size_t)p->H), kBwdThreads, smem, s, tmK, tmV, tmQ, tmdO, a));
+    MOC_CUDA_TRY(launch_early(backward_overlaps(p), attend_dkv_tc_kernel<D>, (unsigned)((p->ktiles.size() + (size_t)(n_split - 1) * p->n_long_ktiles) * p->H), kBwdThreads, smem, s, tmK, tmV, tmQ, tmdO, a));
     MOC_LAUNCH_CHECK();
     return MOC_OK;
 }

@@ -135,7 +135,9 @@ __global__ void __launch_bounds__(128) attend_scalar_kernel(const __nv_bfloat16 
 // delta_i = sum_x dO_ix O_ix
 template <int D>
 __global__ void __launch_bounds__(128) delta_kernel(const __nv_bfloat16 *__restrict__ O, const __nv_bfloat16 *__restrict__ dO,
-                                                     float *__restrict__ delta, size_t n_rows) {
+                                                     float *__restrict__ delta, size_t n_rows, int *__restrict__ zero, int n_zero) {
+    if (blockIdx.x == 0)                                   // the counters of split dK/dV tiles
+        for (int x = threadIdx.x; x < n_zero; x += 128) zero[x] = 0;
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const size_t row = (size_t)blockIdx.x * 4 + warp;
     if (row >= n_rows) return;
@@ -284,7 +286,7 @@ static int attend_bwd_scalar_d(const moc_plan *p, const __nv_bfloat16 *Q, const 
     const size_t rows = (size_t)p->H * p->L;
     const unsigned grid = (unsigned)((rows + 3) / 4);
     float *delta = ws_ptr<float>(ws, p->ws.delta);
-    delta_kernel<D><<<grid, 128, 0, s>>>(O, dO, delta, rows);
+    delta_kernel<D><<<grid, 128, 0, s>>>(O, dO, delta, rows, nullptr, 0);
     MOC_LAUNCH_CHECK();
     dq_scalar_kernel<D><<<grid, 128, 0, s>>>(Q, K, V, dO, lse, delta, sel, dQ, p->d_off, p->d_tok_chunk, p->d_anc_off,
                                              p->d_anc_rng, p->H, p->L, p->k, p->scale);
@@ -297,11 +299,11 @@ static int attend_bwd_scalar_d(const moc_plan *p, const __nv_bfloat16 *Q, const 
     return MOC_OK;
 }
 
-int launch_delta(const moc_plan *p, const __nv_bfloat16 *O, const __nv_bfloat16 *dO, float *delta, cudaStream_t s) {
+int launch_delta(const moc_plan *p, const __nv_bfloat16 *O, const __nv_bfloat16 *dO, float *delta, int *zero, int n_zero, cudaStream_t s) {
     const size_t rows = (size_t)p->H * p->L;
     const unsigned grid = (unsigned)((rows + 3) / 4);
-    if (p->d == 128) delta_kernel<128><<<grid, 128, 0, s>>>(O, dO, delta, rows);
-    else delta_kernel<64><<<grid, 128, 0, s>>>(O, dO, delta, rows);
+    if (p->d == 128) delta_kernel<128><<<grid, 128, 0, s>>>(O, dO, delta, rows, zero, n_zero);
+    else delta_kernel<64><<<grid, 128, 0, s>>>(O, dO, delta, rows, zero, n_zero);
     MOC_LAUNCH_CHECK();
     return MOC_OK;
 }

@@ -745,7 +745,8 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             // on ROWS_DONE, all the same).
             // The device-wide fence before the count waits for every store in flight, with short items longer than an item
             // takes.  So an item's slot is handed back before it, and the rows of a few items are counted together: at the end of a
-            // phase, before a wait, and else every fourth item (256-token chunks, 30 picks, 6 heads: see the launch).
+            // phase, before a wait, and else every fourth item (with the ring of three slots, before the epilogue was cut: 256-token
+            // chunks, 118 picks 23.1 -> 22.3 ms, 30 picks 18.4 -> 17.9).
             // A barrier must not complete two phases that nobody has waited for in between: the slot of item n + 1 is handed
             // back when item n has been seen to be stored, and item n + 4, the next to use the ROWS_DONE of item n, goes into that
             // slot.

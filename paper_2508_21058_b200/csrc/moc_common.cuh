@@ -41,7 +41,7 @@ struct WsLayout {
     size_t qlist;       // int32[H][cap_total]  per (head, chunk) list at cap_off[c]: entries i*k+s of the picks of c
     size_t desc3;       // bf16 [H][3][Cpad][d]  descriptors split into three bf16 terms (hi + mid + lo)
     size_t pool_part;   // float[H][n_pool_units][d] partial key sums
-    size_t pool_done;   // int32[H][C] arrival counters (cleared at the start of every pooling call)
+    size_t pool_done;   // int32[H][C] arrival counters (cleared at the start of every pooling call; in the backward, of split key tiles)
     size_t queue;       // int32[kQueueHeader + 6 groups] work queue of the forward attention kernel
     size_t part_o;      // bf16 [1 or 2][Hg][L][k][d] routed partial outputs (normalised) of one group of Hg heads; with
                         // several groups, two buffers that consecutive groups alternate between
@@ -71,6 +71,7 @@ struct moc_plan {
     std::vector<moc::KeyRange> qry_rng;      // merged ranges of the query rows that have a chunk as an anchor, chunk by chunk
     std::vector<moc::KTile> ktiles;          // key tiles of one head: the long ones (see moc_plan_create) first, then chunk by chunk
     int n_long_ktiles = 0;
+    int n_split = 1;                         // blocks that share the query rows of a long key tile (see moc_plan_create)
     std::vector<int32_t> pool_unit_off;      // [C+1] prefix of pool units per chunk
     std::vector<moc::KeyRange> shot_chunks;  // [S] chunk range [t0, t1) of every shot (outer-loop routing)
     int words;                               // uint32 words per anchor bitmap row
@@ -249,7 +250,8 @@ int launch_attend_bwd_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_b
 inline bool backward_overlaps(const moc_plan *p) { return p->ktiles.size() * (size_t)p->H <= 16 * (size_t)p->n_sm; }
 int launch_dq_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat16 *K, const __nv_bfloat16 *V, const float *lse,
                  const float *delta, const __nv_bfloat16 *dO, __nv_bfloat16 *dQ, void *ws, cudaStream_t s);
-int launch_delta(const moc_plan *p, const __nv_bfloat16 *O, const __nv_bfloat16 *dO, float *delta, cudaStream_t s);
+// (also clears n_zero counters)
+int launch_delta(const moc_plan *p, const __nv_bfloat16 *O, const __nv_bfloat16 *dO, float *delta, int *zero, int n_zero, cudaStream_t s);
 int launch_attend_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat16 *K, const __nv_bfloat16 *V,
                      const int32_t *sel, __nv_bfloat16 *O, float *lse, void *ws, cudaStream_t s);
 

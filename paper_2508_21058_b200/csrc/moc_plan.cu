@@ -21,6 +21,8 @@ void set_cuda_error(cudaError_t e, const char *where) {
     (void)cudaGetLastError();
 }
 
+constexpr int kMaxSplit = 8;
+
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Sec. 3.2: text chunks are anchors of every query; so are the chunks of the query's shot
@@ -229,6 +231,19 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
                     p->ktiles.push_back(KTile{c, t, std::min(128, p->off[c + 1] - t), rng_tiles[c], rng_off[c], rng_off[c + 1] - rng_off[c], 0, 0});
             }
             if (pass == 0) p->n_long_ktiles = (int)p->ktiles.size();
+        }
+        // A long tile is one block's serial work.  Where that is more than an SM's share of the whole launch (short streams: a
+        // caption's block alone then takes as long as all else), its query rows are dealt to several blocks, each with about
+        // that share, or what the other blocks have if that is more.  From twice the share on.  (Whole backward passes, one block ->
+        // several: 2 heads of 4.6k tokens 108 -> 91 us, 3 heads of 3.3k tokens at d = 64 79 -> 68, three small scenes 73.5 -> 71.3; below
+        // the line 1 % slower, 6 heads of 3.7k tokens 128.8 -> 130.3.)
+        if (p->n_long_ktiles > 0) {
+            const int64_t routed = (int64_t)L * p->k / 128, n_kt = (int64_t)p->ktiles.size();        // (tiles of picks, all chunks)
+            int64_t all = 0, longest = 0;
+            for (const KTile &kt : p->ktiles) { all += kt.n_anc; longest = std::max<int64_t>(longest, kt.n_anc); }
+            all += routed * n_kt / std::max(C, 1);
+            const int64_t share = std::max<int64_t>(4, std::max(all * p->H / p->n_sm, all / n_kt));
+            p->n_split = longest < 2 * share ? 1 : (int)std::min<int64_t>(kMaxSplit, (longest + share - 1) / share);
         }
     }
     // Query-list capacities: chunk c can be picked by at most the rows after it (causal) or by

@@ -303,19 +303,8 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, int a_mn_maj
 // 128-byte rows whose base is 1024-byte aligned (the layout TMA SWIZZLE_128B produces)
 __device__ __forceinline__ uint32_t sw128_offset(int r, int c16) { return (uint32_t)(r * 128 + ((c16 ^ (r & 7)) << 4)); }
 
-// 32-byte (one sector) global load that is cached in L2 only, and 32-byte global store; addresses 32-byte aligned
-__device__ __forceinline__ void ld_cg_256(const void *ptr, uint4 &a, uint4 &b) {
-    asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-                 : "l"(ptr));
-}
-__device__ __forceinline__ void st_256(void *ptr, const uint4 &a, const uint4 &b) {
-    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                 ::"l"(ptr), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
-                 : "memory");
-}
-
-// the load where cond holds (predicated: as a branch around it, the values it leaves alone cost registers twice)
+// 32-byte (one sector) global load that is cached in L2 only, and 32-byte global store; addresses 32-byte aligned.
+// The load where cond holds (predicated: as a branch around it, the values it leaves alone cost registers twice)
 __device__ __forceinline__ void ld_cg_256_if(bool cond, const void *ptr, uint32_t (&u)[8]) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"

@@ -1,0 +1,47 @@
+"""dK and dV of a caption whose key tiles are shared by several blocks, against the CUDA-core kernels on the same selection: every
+element, and the same bits whichever block is last."""
+import pytest
+import torch
+
+from paper_2508_21058_b200 import MocPlan
+from paper_2508_21058_b200 import workloads as W
+
+import parity_utils as PU
+
+pytestmark = pytest.mark.gpu
+
+# heads, head_dim, (shots, caption, frames, frame length), k; by the rule of moc_plan_create the blocks of a caption's tile are
+SHAPES = {
+    "4 blocks, a tile of two rows": (2, 128, (1, 130, 24, 100), 2),
+    "8 blocks, two captions of 5": (1, 128, (2, 5, 20, 129), 1),
+    "6 blocks, one key": (1, 64, (1, 1, 40, 64), 1),
+    "7 blocks, d 64": (3, 64, (1, 40, 64, 97), 3),
+    "no room for their sums": (1, 128, (1, 140, 30, 100), 0),              # without picks there are no partials to take the place of
+}
+# P and dS are rounded to bf16 (half an ulp: 2^-9) on one side, the results on both: a few 1e-3 of the 2-norm of a block of rows
+# (seen: 4e-3).  Of at most 49 query tiles one left out, or taken twice, is off by sqrt(1 / 49) = 0.14.
+REL = 2e-2
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_every_gradient_of_a_shared_tile(shape):
+    heads, d, lay, k = SHAPES[shape]
+    wl = W.Workload("split", heads, d, W.make_layout(*lay), k, 1, 1)
+    run = PU.GpuRun(wl, tensors=("q", "k", "v", "do")).forward()
+    x, outs = run.x, []
+    ref = MocPlan.from_workload(wl, scalar_attend=True)
+    ws = ref.new_workspace(with_bwd=True)
+    ref.moc_lists_from_sel(run.sel, ws)
+    want = [torch.empty_like(run.O) for _ in range(3)]
+    ref.moc_attend_bwd(x["q"], x["k"], x["v"], run.O, run.lse, x["do"], run.sel, *want, ws)
+    for _ in range(20):
+        run.backward()
+        outs.append([t.clone() for t in (run.dQ, run.dK, run.dV)])
+    off = wl.layout.chunk_off
+    for got in outs:
+        for a, b, first in zip(got, want, outs[0]):
+            assert torch.equal(a, first)
+            for c in range(wl.n_chunks):
+                rows = slice(int(off[c]), int(off[c + 1]))
+                diff, norm = ((t[:, rows].float()).flatten(1).norm(dim=1) for t in (a.float() - b.float(), b))
+                assert float((diff / norm.clamp(min=1e-3)).max()) < REL, (c, float((diff / norm).max()))
