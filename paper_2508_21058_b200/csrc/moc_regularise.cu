@@ -138,10 +138,11 @@ int launch_context_drop(const moc_plan *p, int32_t *sel, float p_max, float lamb
     }
     const size_t rows = (size_t)p->H * p->L, row_bytes = sizeof(uint32_t) * ((size_t)p->k + p->words);
     // 128 rows a block, fewer where their slots and bitmaps do not fit
+    constexpr int kMost = 200 * 1024;        // (the attribute is the same for every call: another thread's may come between)
     unsigned block = 128;
-    while (block > 1 && block * row_bytes > 200 * 1024) block /= 2;
-    if (block * row_bytes > 200 * 1024) return MOC_ERR_SHAPE;
-    MOC_CUDA_TRY(cudaFuncSetAttribute(context_drop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(block * row_bytes)));
+    while (block > 1 && block * row_bytes > kMost) block /= 2;
+    if (block * row_bytes > kMost) return MOC_ERR_SHAPE;
+    MOC_CUDA_TRY(cudaFuncSetAttribute(context_drop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost));
     context_drop_kernel<<<(unsigned)((rows + block - 1) / block), block, block * row_bytes, s>>>(sel, p->d_tok_chunk, p->d_anc_bits, tab, p->H, p->L, p->C, p->k,
                                                                       p->words, (p->flags & MOC_FLAG_CAUSAL) ? 1 : 0, p_max,
                                                                       (uint32_t)seed, (uint32_t)(seed >> 32));

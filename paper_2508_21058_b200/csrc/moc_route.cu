@@ -1132,10 +1132,11 @@ int launch_lists_from_sel(const moc_plan *p, int32_t *sel, void *ws, cudaStream_
         // looking at the earlier entries, and the block's bitmaps fit.  (All calls, without -> with: 63 slots, 970 chunks, 251k rows
         // 283 -> 145 us; 47 slots, 144 chunks, 24k rows 76 -> 33; 14 slots, 45 chunks 21.5 -> 16.4; but 12 slots, 565 chunks 34.8 -> 36.9.)
         const size_t hist = 2 * sizeof(int) * (size_t)p->C, bits = 256 * sizeof(uint32_t) * (size_t)p->words;
-        const bool bitmap = (long long)p->k * p->k > 4LL * (p->words + 2 * p->k) && hist + bits <= 200 * 1024;
+        constexpr int kMost = 200 * 1024;    // (the attribute is the same for every call: another thread's may come between)
+        const bool bitmap = (long long)p->k * p->k > 4LL * (p->words + 2 * p->k) && hist + bits <= kMost;
         const size_t smem = hist + (bitmap ? bits : 0);
-        if (hist > 200 * 1024) return MOC_ERR_SHAPE;
-        MOC_CUDA_TRY(cudaFuncSetAttribute(lists_from_sel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (hist > kMost) return MOC_ERR_SHAPE;
+        MOC_CUDA_TRY(cudaFuncSetAttribute(lists_from_sel_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost));
         lists_from_sel_kernel<<<dim3((unsigned)((p->L + 255) / 256), (unsigned)p->H), 256, smem, s>>>(
             sel, ws_ptr<float>(ws, p->ws.part_lse), cnt, ws_ptr<int32_t>(ws, p->ws.qlist), p->d_tok_chunk, p->d_anc_bits,
             p->d_cap_off, status, p->L, p->C, p->k, p->words, (p->flags & MOC_FLAG_CAUSAL) ? 1 : 0, (size_t)p->cap_off[p->C], bitmap);
