@@ -64,6 +64,7 @@ def load_library():
     lib.moc_debug_use_cuda_core_attention.argtypes = [vp, i32]
     lib.moc_debug_set_wait_limit_us.argtypes = [vp, C.c_uint]
     lib.moc_debug_wait_probe.argtypes = [vp, vp, i32, vp]
+    lib.moc_debug_shared_key_tiles.argtypes = [C.POINTER(_Problem), i32, i32, C.POINTER(i32), vp, vp]
     lib.moc_attend.argtypes = [vp] * 9
     lib.moc_attend_bwd.argtypes = [vp] * 13
     lib.moc_selected_pairs.argtypes = [vp, vp, vp, C.POINTER(C.c_int64)]
@@ -98,6 +99,30 @@ def _stream():
     return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
+def _problem(n_heads, n_tokens, head_dim, chunk_off, chunk_shot, chunk_mod, top_k, win_back, win_fwd, causal, softmax_scale):
+    """The C problem statement, and the host arrays it points to."""
+    off = np.ascontiguousarray(chunk_off, np.int32)
+    shot = np.ascontiguousarray(chunk_shot, np.int32)
+    mod = np.ascontiguousarray(chunk_mod, np.uint8)
+    if len(off) != len(shot) + 1 or len(mod) != len(shot):
+        raise MocError(-3, "moc error -3: chunk tables have inconsistent lengths")
+    pr = _Problem(int(n_heads), int(n_tokens), int(head_dim), len(shot), int(top_k), int(win_back), int(win_fwd),
+                  FLAG_CAUSAL if causal else 0, float(softmax_scale), off.ctypes.data, shot.ctypes.data, mod.ctypes.data)
+    return pr, (off, shot, mod)
+
+
+def debug_shared_key_tiles(wl, n_sm):
+    """Test hook, host only: for each long key tile of a head in the dK/dV launch on n_sm SMs, the tiles of query rows that have it as
+    an anchor and the blocks that share it."""
+    lay = wl.layout
+    pr, tables = _problem(wl.n_heads, lay.n_tokens, wl.head_dim, lay.chunk_off, lay.chunk_shot, lay.chunk_mod, wl.top_k, wl.win_back,
+                          wl.win_fwd, wl.causal, 0.0)
+    cap = lay.n_tokens // 128 + lay.n_chunks
+    n, query_tiles, blocks = C.c_int(0), np.zeros(cap, np.int32), np.zeros(cap, np.int32)
+    _check(load_library().moc_debug_shared_key_tiles(C.byref(pr), int(n_sm), cap, C.byref(n), query_tiles.ctypes.data, blocks.ctypes.data))
+    return query_tiles[:n.value], blocks[:n.value]
+
+
 class MocPlan:
     """Owns a ``moc_plan``.  Methods mirror the C entry points and take torch CUDA tensors."""
 
@@ -105,16 +130,10 @@ class MocPlan:
                  win_back=0, win_fwd=0, causal=True, scalar_attend=False, softmax_scale=0.0):
         self._lib = load_library()
         self._h = C.c_void_p(0)
-        off = np.ascontiguousarray(chunk_off, np.int32)
-        shot = np.ascontiguousarray(chunk_shot, np.int32)
-        mod = np.ascontiguousarray(chunk_mod, np.uint8)
-        flags = FLAG_CAUSAL if causal else 0
-        pr = _Problem(int(n_heads), int(n_tokens), int(head_dim), len(shot), int(top_k), int(win_back), int(win_fwd),
-                      flags, float(softmax_scale), off.ctypes.data, shot.ctypes.data, mod.ctypes.data)
-        if len(off) != len(shot) + 1 or len(mod) != len(shot):
-            raise MocError(-3, "moc error -3: chunk tables have inconsistent lengths")
+        pr, tables = _problem(n_heads, n_tokens, head_dim, chunk_off, chunk_shot, chunk_mod, top_k, win_back, win_fwd, causal,
+                              softmax_scale)
         _check(self._lib.moc_plan_create(C.byref(pr), C.byref(self._h)))
-        self.H, self.L, self.d, self.C, self.k = int(n_heads), int(n_tokens), int(head_dim), len(shot), int(top_k)
+        self.H, self.L, self.d, self.C, self.k = int(n_heads), int(n_tokens), int(head_dim), pr.n_chunks, int(top_k)
         if scalar_attend:       # test hook: the in-library CUDA-core cross-check of the attention kernels
             _check(self._lib.moc_debug_use_cuda_core_attention(self._h, 1))
 

@@ -10,8 +10,10 @@
 //     T1 = K Q^T,  T2 = V dO^T          (both operands from shared memory, into TMEM)
 //     threads (two per TMEM lane) turn T1 into P, then (P, T2) into dS, written back to TMEM as bf16
 //     ACC1 += dS Q,  ACC2 += P dO       (A from TMEM, the streamed tile as an MN-major operand)
-// lse and delta belong to the column; ACC1 is dK, ACC2 is dV.  Each key tile is owned by one CTA: no atomics, no partial
-// sums.  Issue order: ACC2(j), T1(j+1), ACC1(j), T2(j+1), so that while the lanes form P(j+1) the pipe runs ACC1(j) and
+// lse and delta belong to the column; ACC1 is dK, ACC2 is dV.  A key tile is owned by one CTA, except that in short streams
+// several share the query tiles of one that most rows attend (derive_plan): each leaves its fp32 sums, and the last to leave, by an
+// atomic counter, adds them in the order of the CTAs.
+// Issue order: ACC2(j), T1(j+1), ACC1(j), T2(j+1), so that while the lanes form P(j+1) the pipe runs ACC1(j) and
 // T2(j+1), and T1 / T2 are rewritten only after the contraction that reads the P / dS stored over them; ACC2(j) starts on the
 // first half of P(j) while the lanes form the second.
 // A tile takes 3300 cycles (33k-token clip) for 2048 cycles of MMAs at the pipe's best rate: P, dS and the wait for T1(j+1)
@@ -38,7 +40,7 @@ struct BwdParams {
     uint32_t cookie;              // what the workspace's status area must hold
     const KTile *ktiles;
     int n_ktiles, n_long;         // tiles per head, and how many of them come first for every head
-    int n_split;                  // blocks that share the query tiles of one of those
+    int n_split;                  // blocks that are launched for each of those; the tile says how many of them share it
     float4 *split_sum;            // their sums, [tile][block][dK, dV], each as the lane threads hold it
     int *split_done;              // [tile] blocks that have left theirs
     const KeyRange *qry_rng;
@@ -71,7 +73,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort;
     __shared__ int w_valid, w_h, w_ntiles, w_list;       // w_list: entries of the chunk's query list
-    __shared__ int w_skip, w_part, w_split, s_last;      // query tiles of the blocks before this one, which shares tile w_split with others (-1: none)
+    __shared__ int w_skip, w_part, w_parts, w_split, s_last;      // query tiles of the blocks before this one, which is one of w_parts on tile w_split
     __shared__ KTile s_kt;
     // per streamed query, (-lse * log2(e), -delta), for tiles j and j + 1
     __shared__ __align__(16) float s_ld[2][2][128];
@@ -117,21 +119,22 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             // block order: the long key tiles of every head, then the others head by head (tiles of one chunk next
             // to each other: they stream the same query rows)
             const int n_long_all = p.n_long * p.H * p.n_split;
-            int b = blockIdx.x, hh, ti, part = 0, parts = 1;
+            int b = blockIdx.x, hh, ti, part = 0;
             if (b < n_long_all) {
-                parts = p.n_split;
-                part = b % parts;
-                b /= parts;
-                w_split = parts > 1 ? b : -1;
+                part = b % p.n_split;
+                b /= p.n_split;
+                w_split = b;
                 hh = b / p.n_long; ti = b - hh * p.n_long;
-            } else { w_split = -1; b -= n_long_all; const int n_rest = p.n_ktiles - p.n_long; hh = b / n_rest; ti = p.n_long + b - hh * n_rest; }
+            } else { b -= n_long_all; const int n_rest = p.n_ktiles - p.n_long; hh = b / n_rest; ti = p.n_long + b - hh * n_rest; }
             const KTile kt = p.ktiles[ti];
             const int n_list = p.cnt[hh * p.C + kt.chunk];
             s_kt = kt;
             w_h = hh;
             w_list = n_list;
             const int nt = kt.n_anc + (n_list + 127) / 128;
+            const int parts = min(kt.parts, p.n_split);
             w_part = part;
+            w_parts = parts;
             w_skip = (int)((long long)nt * part / parts);
             w_ntiles = (int)((long long)nt * (part + 1) / parts) - w_skip;
         }
@@ -142,7 +145,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (!w_valid) {
+    if (!w_valid || w_part >= w_parts) {                   // ... or a block that its tile has no use for
         if (warp == 8) tmem_dealloc(tmem_slot, 512);
         if (blockIdx.x == gridDim.x - 1) previous_done();
         return;
@@ -266,7 +269,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             // takes 64 columns of all rows (d = 128) or 16 rows (d = 64).
             constexpr int NJ = D / 32;                       // groups of eight rows that this warp has
             const int l4 = lane >> 2, l2 = lane & 3, cb = D == 128 ? half : 0, j0 = D == 128 ? 0 : 2 * half;
-            const int slot = w_split, me = (half * 4 + (warp & 3)) * 32 + lane;
+            const int slot = w_split, parts = w_parts, me = (half * 4 + (warp & 3)) * 32 + lane;
             constexpr int NV = NJ / 2 * 8;                   // float4s of a thread and side
             auto load = [&](int side, uint32_t (&v)[NJ / 2][32]) {
                 __syncwarp();
@@ -290,7 +293,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                 }
             };
             uint32_t v[NJ / 2][32];
-            if (slot < 0) {
+            if (parts == 1) {
 #pragma unroll 1
                 for (int side = 0; side < 2; ++side) {
                     load(side, v);
@@ -316,7 +319,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                 ok = mbar_wait_spin(bar(RD1), n_tiles & 1, abort_flag, p.status, BW_READ);
                 if (threadIdx.x == 0 && ok) {
                     __threadfence();
-                    s_last = atomicAdd(p.split_done + slot, 1) == p.n_split - 1;
+                    s_last = atomicAdd(p.split_done + slot, 1) == parts - 1;
                     __threadfence();
                 }
                 mbar_arrive(bar(RD2));
@@ -331,7 +334,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
 #pragma unroll
                             for (int y = 0; y < 4; ++y) v[x >> 3][4 * (x & 7) + y] = 0u;
 #pragma unroll 1
-                        for (int part = 0; part < p.n_split; ++part) {
+                        for (int part = 0; part < parts; ++part) {
                             const float4 *from = sums(part, side);
 #pragma unroll
                             for (int x = 0; x < NV; ++x) {
@@ -629,9 +632,7 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
                            const __nv_bfloat16 *O, const float *lse, const __nv_bfloat16 *dO, const int32_t *sel,
                            __nv_bfloat16 *dQ, __nv_bfloat16 *dK, __nv_bfloat16 *dV, void *ws, cudaStream_t s) {
     float *delta = ws_ptr<float>(ws, p->ws.delta);
-    // split key tiles leave their sums in the space of the routed partials, if that is large enough
-    const size_t sums = 2 * sizeof(float) * 128 * (size_t)D * p->n_long_ktiles * p->H;
-    const int n_split = p->n_split > 1 && sums * p->n_split <= p->ws.part_lse - p->ws.part_o ? p->n_split : 1;
+    const int n_split = dkv_split(p);
     int *split_done = ws_ptr<int>(ws, p->ws.pool_done);
     if (int r = launch_delta(p, O, dO, delta, split_done, n_split > 1 ? p->n_long_ktiles * p->H : 0, s)) return r;
     CUtensorMap tmK, tmV, tmQ, tmdO;       // Q and dO: tiles of 64 rows

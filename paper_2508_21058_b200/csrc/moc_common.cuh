@@ -30,8 +30,9 @@ struct KeyRange { int32_t t0, t1; };
 struct WorkItem { int32_t h, first, rows, ntiles, rng_off, nrng, t0, t1; };
 
 // One tile of up to 128 consecutive key tokens of a chunk (backward, key-stationary pass), with what its block looks up first:
-// the rows that have the chunk as an anchor (n_rng ranges from rng on, n_anc tiles of 128 rows) and where its query list starts.
-struct __align__(32) KTile { int32_t chunk, t0, valid, n_anc, rng, n_rng, list, pad; };
+// the rows that have the chunk as an anchor (n_rng ranges from rng on, n_anc tiles of 128 rows), where its query list starts, and
+// how many blocks share its query tiles (no more than n_anc: each has one).
+struct __align__(32) KTile { int32_t chunk, t0, valid, n_anc, rng, n_rng, list, parts; };
 
 struct WsLayout {
     size_t status;      // int32[kStatusWords], see StatusWord
@@ -69,9 +70,9 @@ struct moc_plan {
     std::vector<int32_t> ranc_off, ranc;     // reverse anchors: key chunk -> query chunks
     std::vector<moc::WorkItem> qitems;       // anchor-pass work items of one head
     std::vector<moc::KeyRange> qry_rng;      // merged ranges of the query rows that have a chunk as an anchor, chunk by chunk
-    std::vector<moc::KTile> ktiles;          // key tiles of one head: the long ones (see moc_plan_create) first, then chunk by chunk
+    std::vector<moc::KTile> ktiles;          // key tiles of one head: the long ones (see derive_plan) first, then chunk by chunk
     int n_long_ktiles = 0;
-    int n_split = 1;                         // blocks that share the query rows of a long key tile (see moc_plan_create)
+    int n_split = 1;                         // the largest number of blocks that share the query rows of a long key tile (see derive_plan)
     std::vector<int32_t> pool_unit_off;      // [C+1] prefix of pool units per chunk
     std::vector<moc::KeyRange> shot_chunks;  // [S] chunk range [t0, t1) of every shot (outer-loop routing)
     int words;                               // uint32 words per anchor bitmap row
@@ -248,6 +249,12 @@ int launch_attend_bwd_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_b
 // in turn (one after another -> overlapping): 0.7 blocks per SM 158 -> 134 us, 4 447 -> 428 us; at 20, 45 and 111 the two are alike
 // (6.64 / 6.64, 14.16 / 14.16 and 102.9 / 102.3 ms, where the runs of one side differ by 0.7 %).
 inline bool backward_overlaps(const moc_plan *p) { return p->ktiles.size() * (size_t)p->H <= 16 * (size_t)p->n_sm; }
+// Blocks per long key tile that dK/dV is launched with (a tile's own number may be smaller): the plan's, if the shared tiles' sums fit
+// into the space of the routed partials, else one.
+inline int dkv_split(const moc_plan *p) {
+    const size_t sums = 2 * sizeof(float) * 128 * (size_t)p->d * p->n_long_ktiles * p->H;
+    return p->n_split > 1 && sums * p->n_split <= p->ws.part_lse - p->ws.part_o ? p->n_split : 1;
+}
 int launch_dq_tc(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat16 *K, const __nv_bfloat16 *V, const float *lse,
                  const float *delta, const __nv_bfloat16 *dO, __nv_bfloat16 *dQ, void *ws, cudaStream_t s);
 // (also clears n_zero counters)
@@ -267,4 +274,7 @@ int moc_debug_set_wait_limit_us(moc_plan *plan, unsigned us);
 // one block whose only wait is on a barrier that nothing ever arrives on: it must give up after the limit,
 // record MOC_ERR_TIMEOUT with detail `code` in ws, and return
 int moc_debug_wait_probe(const moc_plan *plan, void *ws, int code, void *stream);
+// host only: the long key tiles of dK/dV of a problem on a GPU with n_sm SMs (up to cap of them written): tiles of query rows that
+// a tile has whatever is picked, and blocks that share them
+int moc_debug_shared_key_tiles(const moc_problem *problem, int n_sm, int cap, int *n_tiles, int *query_tiles, int *blocks);
 }

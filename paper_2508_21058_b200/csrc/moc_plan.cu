@@ -108,13 +108,14 @@ void layout_workspace(moc_plan *p) {
     p->cookie = plan_cookie(p);
 }
 
-}  // namespace moc
+// What the derivation leaves for the device alone.
+struct DeviceTables {
+    std::vector<uint32_t> bits, cand_c;
+    std::vector<int32_t> unit_chunk, lim, reach, col_chunk;
+    std::vector<KeyRange> chunk_rng;
+};
 
-using namespace moc;
-
-extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
-    if (!pr || !out) return MOC_ERR_NULL;
-    *out = nullptr;
+static int check_problem(const moc_problem *pr) {
     if (!pr->chunk_off || !pr->chunk_shot || !pr->chunk_mod) return MOC_ERR_NULL;
     if (pr->n_heads < 1 || pr->n_tokens < 1 || pr->n_chunks < 1 || pr->n_chunks > pr->n_tokens) return MOC_ERR_SHAPE;
     // heads index grid.y; head * L + token is a 32-bit row coordinate of the tensor maps
@@ -133,27 +134,24 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
         if (pr->chunk_mod[c] > 1) return MOC_ERR_CHUNK_TABLE;
         if (c > 0 && pr->chunk_shot[c] < pr->chunk_shot[c - 1]) return MOC_ERR_CHUNK_TABLE;
     }
-    int dev = 0;
-    MOC_CUDA_TRY(cudaGetDevice(&dev));
-    // two attributes, not the whole property structure, which takes the driver a millisecond or two to fill in
-    int cc_major = 0, n_sm = 0;
-    MOC_CUDA_TRY(cudaDeviceGetAttribute(&cc_major, cudaDevAttrComputeCapabilityMajor, dev));
-    MOC_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
-    if (cc_major != 10) return MOC_ERR_ARCH;
+    return MOC_OK;
+}
 
-    moc_plan *p = new (std::nothrow) moc_plan();
-    if (!p) return MOC_ERR_CUDA;
+// Everything of a plan that a checked problem and the number of SMs determine; no device work.
+static int derive_plan(moc_plan *p, const moc_problem *pr, int n_sm, DeviceTables &tab) {
+    const int C = pr->n_chunks, L = pr->n_tokens;
     p->H = pr->n_heads; p->L = L; p->d = pr->head_dim; p->C = C; p->k = pr->top_k;
     p->win_back = pr->win_back; p->win_fwd = pr->win_fwd; p->flags = pr->flags;
     p->scale = pr->softmax_scale > 0.f ? pr->softmax_scale : 1.0f / sqrtf((float)pr->head_dim);
-    p->device = dev; p->n_sm = n_sm;
+    p->n_sm = n_sm;
     p->off.assign(pr->chunk_off, pr->chunk_off + C + 1);
     p->shot.assign(pr->chunk_shot, pr->chunk_shot + C);
     p->mod.assign(pr->chunk_mod, pr->chunk_mod + C);
 
     // anchor bitmaps, merged anchor key ranges, reverse anchors
     p->words = (C + 31) / 32;
-    std::vector<uint32_t> bits((size_t)C * p->words, 0u);
+    std::vector<uint32_t> &bits = tab.bits;
+    bits.assign((size_t)C * p->words, 0u);
     std::vector<std::vector<int32_t>> rev(C);
     p->anc_off.assign(C + 1, 0);
     p->anc_tokens.assign(C, 0);
@@ -176,9 +174,8 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
         p->ranc_off[j + 1] = (int32_t)p->ranc.size();
     }
     // query tiles (never straddle a chunk) and pool work units
-    std::vector<int32_t> unit_chunk;
-    std::vector<KeyRange> chunk_rng(C);
-    for (int c = 0; c < C; ++c) chunk_rng[c] = KeyRange{p->off[c], p->off[c + 1]};
+    std::vector<int32_t> &unit_chunk = tab.unit_chunk;
+    for (int c = 0; c < C; ++c) tab.chunk_rng.push_back(KeyRange{p->off[c], p->off[c + 1]});
     p->pool_unit_off.assign(C + 1, 0);
     for (int c = 0; c < C; ++c) {
         int anc_tiles = 0;
@@ -228,22 +225,27 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
                 const bool is_long = anc_rows[c] > 4 * mean_rows;
                 if (is_long != (pass == 0)) continue;
                 for (int t = p->off[c]; t < p->off[c + 1]; t += 128)
-                    p->ktiles.push_back(KTile{c, t, std::min(128, p->off[c + 1] - t), rng_tiles[c], rng_off[c], rng_off[c + 1] - rng_off[c], 0, 0});
+                    p->ktiles.push_back(KTile{c, t, std::min(128, p->off[c + 1] - t), rng_tiles[c], rng_off[c], rng_off[c + 1] - rng_off[c], 0, 1});
             }
             if (pass == 0) p->n_long_ktiles = (int)p->ktiles.size();
         }
         // A long tile is one block's serial work.  Where that is more than an SM's share of the whole launch (short streams: a
         // caption's block alone then takes as long as all else), its query rows are dealt to several blocks, each with about
-        // that share, or what the other blocks have if that is more.  From twice the share on.  (Whole backward passes, one block ->
-        // several: 2 heads of 4.6k tokens 108 -> 91 us, 3 heads of 3.3k tokens at d = 64 79 -> 68, three small scenes 73.5 -> 71.3; below
-        // the line 1 % slower, 6 heads of 3.7k tokens 128.8 -> 130.3.)
+        // that share, or what the other blocks have if that is more.  From twice the share on.  Tile by tile: next to a caption that
+        // every row attends, a chunk that is much longer than its neighbours may have fewer query tiles than the caption has blocks,
+        // and a block must have one.  (Whole backward passes, one block -> several: 2 heads of 4.6k tokens 108 -> 91 us, 3 heads of 3.3k
+        // tokens at d = 64 79 -> 68, three small scenes 73.5 -> 71.3; below the line 1 % slower, 6 heads of 3.7k tokens 128.8 -> 130.3.)
         if (p->n_long_ktiles > 0) {
             const int64_t routed = (int64_t)L * p->k / 128, n_kt = (int64_t)p->ktiles.size();        // (tiles of picks, all chunks)
-            int64_t all = 0, longest = 0;
-            for (const KTile &kt : p->ktiles) { all += kt.n_anc; longest = std::max<int64_t>(longest, kt.n_anc); }
+            int64_t all = 0;
+            for (const KTile &kt : p->ktiles) all += kt.n_anc;
             all += routed * n_kt / std::max(C, 1);
             const int64_t share = std::max<int64_t>(4, std::max(all * p->H / p->n_sm, all / n_kt));
-            p->n_split = longest < 2 * share ? 1 : (int)std::min<int64_t>(kMaxSplit, (longest + share - 1) / share);
+            for (int x = 0; x < p->n_long_ktiles; ++x) {
+                KTile &kt = p->ktiles[x];
+                if (kt.n_anc >= 2 * share) kt.parts = (int32_t)std::min<int64_t>(kMaxSplit, (kt.n_anc + share - 1) / share);
+                p->n_split = std::max(p->n_split, kt.parts);
+            }
         }
     }
     // Query-list capacities: chunk c can be picked by at most the rows after it (causal) or by
@@ -253,14 +255,14 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     for (int c = 0; c < C; ++c) {
         const int64_t cap = p->k == 0 ? 0 : ((p->flags & MOC_FLAG_CAUSAL) ? L - p->off[c + 1] : L);
         const int64_t next = (int64_t)p->cap_off[c] + cap;
-        if (next >= 2147483647LL) { delete p; return MOC_ERR_SHAPE; }
+        if (next >= 2147483647LL) return MOC_ERR_SHAPE;
         p->cap_off[c + 1] = (int32_t)next;
     }
     for (KTile &kt : p->ktiles) kt.list = p->cap_off[kt.chunk];
     // score columns: the chunks that are not text; per query chunk its candidate columns (not an anchor, strictly
     // earlier if causal), whether they form a prefix of the columns (they do under the causal rule: everything
     // before the own shot's window), and how far any query up to that chunk can reach
-    std::vector<int32_t> col_chunk, col_of(C, -1);
+    std::vector<int32_t> &col_chunk = tab.col_chunk, col_of(C, -1);
     for (int j = 0; j < C; ++j)
         if (p->mod[j] != 1) { col_of[j] = (int32_t)col_chunk.size(); col_chunk.push_back(j); }
     p->ncol = (int)col_chunk.size();
@@ -268,8 +270,11 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     for (int j : col_chunk) p->routed_key_tiles += (p->off[j + 1] - p->off[j] + 127) / 128;
     p->cwords = std::max(1, (p->ncol + 31) / 32);
     p->c_pad = std::max(16, (p->ncol + 15) / 16 * 16);
-    std::vector<uint32_t> cand_c((size_t)C * p->cwords, 0u);
-    std::vector<int32_t> lim(C, 0), reach(C, 0);
+    std::vector<uint32_t> &cand_c = tab.cand_c;
+    std::vector<int32_t> &lim = tab.lim, &reach = tab.reach;
+    cand_c.assign((size_t)C * p->cwords, 0u);
+    lim.assign(C, 0);
+    reach.assign(C, 0);
     p->prefix_mode = 1;
     for (int c = 0; c < C; ++c) {
         int n_cand = 0, top = 0;
@@ -291,6 +296,33 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     p->partials_budget = (size_t)6 << 30;
     p->wait_us = 0;
     layout_workspace(p);
+    return MOC_OK;
+}
+
+}  // namespace moc
+
+using namespace moc;
+
+extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
+    if (!pr || !out) return MOC_ERR_NULL;
+    *out = nullptr;
+    if (int r = check_problem(pr)) return r;
+    const int C = pr->n_chunks, L = pr->n_tokens;
+    int dev = 0;
+    MOC_CUDA_TRY(cudaGetDevice(&dev));
+    // two attributes, not the whole property structure, which takes the driver a millisecond or two to fill in
+    int cc_major = 0, n_sm = 0;
+    MOC_CUDA_TRY(cudaDeviceGetAttribute(&cc_major, cudaDevAttrComputeCapabilityMajor, dev));
+    MOC_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+    if (cc_major != 10) return MOC_ERR_ARCH;
+
+    moc_plan *p = new (std::nothrow) moc_plan();
+    if (!p) return MOC_ERR_CUDA;
+    p->device = dev;
+    DeviceTables tab;
+    if (int r = derive_plan(p, pr, n_sm, tab)) { delete p; return r; }
+    const std::vector<uint32_t> &bits = tab.bits, &cand_c = tab.cand_c;
+    const std::vector<int32_t> &unit_chunk = tab.unit_chunk, &lim = tab.lim, &reach = tab.reach, &col_chunk = tab.col_chunk;
     // the fixed scratch of moc_chunk_pool_noalloc: its address is looked up here, where allocating is allowed
     if (int r = pool_scratch_prepare(dev)) { delete p; return r; }
 
@@ -322,7 +354,7 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     up(o_puo, p->pool_unit_off.data(), 4 * (C + 1));
     up(o_puc, unit_chunk.data(), 4 * unit_chunk.size());
     up(o_cap, p->cap_off.data(), 4 * (C + 1));
-    up(o_crng, chunk_rng.data(), sizeof(KeyRange) * C);
+    up(o_crng, tab.chunk_rng.data(), sizeof(KeyRange) * C);
     up(o_kt, p->ktiles.data(), sizeof(KTile) * p->ktiles.size());
     up(o_qrng, p->qry_rng.data(), sizeof(KeyRange) * p->qry_rng.size());
     up(o_candc, cand_c.data(), 4 * cand_c.size());
@@ -514,6 +546,22 @@ extern "C" int moc_debug_use_cuda_core_attention(moc_plan *p, int on) {
 extern "C" int moc_debug_set_wait_limit_us(moc_plan *p, unsigned us) {
     if (!p) return MOC_ERR_NULL;
     p->wait_us = us;
+    return MOC_OK;
+}
+
+extern "C" int moc_debug_shared_key_tiles(const moc_problem *pr, int n_sm, int cap, int *n_tiles, int *query_tiles, int *blocks) {
+    if (!pr || !n_tiles || !query_tiles || !blocks) return MOC_ERR_NULL;
+    if (int r = check_problem(pr)) return r;
+    if (n_sm < 1) return MOC_ERR_SHAPE;
+    moc_plan p;
+    DeviceTables tab;
+    if (int r = derive_plan(&p, pr, n_sm, tab)) return r;
+    const int most = dkv_split(&p);
+    *n_tiles = p.n_long_ktiles;
+    for (int x = 0; x < std::min(cap, p.n_long_ktiles); ++x) {
+        query_tiles[x] = p.ktiles[x].n_anc;
+        blocks[x] = std::min(p.ktiles[x].parts, most);
+    }
     return MOC_OK;
 }
 

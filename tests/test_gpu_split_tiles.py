@@ -7,6 +7,7 @@ from paper_2508_21058_b200 import MocPlan
 from paper_2508_21058_b200 import workloads as W
 
 import parity_utils as PU
+from test_shared_key_tiles import LONG_CHUNK
 
 pytestmark = pytest.mark.gpu
 
@@ -23,10 +24,7 @@ SHAPES = {
 REL = 2e-2
 
 
-@pytest.mark.parametrize("shape", SHAPES)
-def test_every_gradient_of_a_shared_tile(shape):
-    heads, d, lay, k = SHAPES[shape]
-    wl = W.Workload("split", heads, d, W.make_layout(*lay), k, 1, 1)
+def check_every_gradient(wl, passes, spoil=None):
     run = PU.GpuRun(wl, tensors=("q", "k", "v", "do")).forward()
     x, outs = run.x, []
     ref = MocPlan.from_workload(wl, scalar_attend=True)
@@ -34,7 +32,9 @@ def test_every_gradient_of_a_shared_tile(shape):
     ref.moc_lists_from_sel(run.sel, ws)
     want = [torch.empty_like(run.O) for _ in range(3)]
     ref.moc_attend_bwd(x["q"], x["k"], x["v"], run.O, run.lse, x["do"], run.sel, *want, ws)
-    for _ in range(20):
+    for _ in range(passes):
+        if spoil:
+            spoil.backward()
         run.backward()
         outs.append([t.clone() for t in (run.dQ, run.dK, run.dV)])
     off = wl.layout.chunk_off
@@ -45,3 +45,17 @@ def test_every_gradient_of_a_shared_tile(shape):
                 rows = slice(int(off[c]), int(off[c + 1]))
                 diff, norm = ((t[:, rows].float()).flatten(1).norm(dim=1) for t in (a.float() - b.float(), b))
                 assert float((diff / norm.clamp(min=1e-3)).max()) < REL, (c, float((diff / norm).max()))
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_every_gradient_of_a_shared_tile(shape):
+    heads, d, lay, k = SHAPES[shape]
+    check_every_gradient(W.Workload("split", heads, d, W.make_layout(*lay), k, 1, 1), 20)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("stream", LONG_CHUNK)
+def test_a_long_chunk_with_fewer_query_tiles_than_the_caption_has_blocks(stream, d):
+    """After the backward of another stream, which leaves sums in every SM's tensor memory."""
+    other = PU.GpuRun(W.Workload("spoil", 8, d, W.make_layout(1, 64, 12, 512), 2, 1, 1), tensors=("q", "k", "v", "do")).forward()
+    check_every_gradient(LONG_CHUNK[stream](d), 3, other)
