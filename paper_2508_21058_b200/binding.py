@@ -64,7 +64,7 @@ def load_library():
     lib.moc_debug_use_cuda_core_attention.argtypes = [vp, i32]
     lib.moc_debug_set_wait_limit_us.argtypes = [vp, C.c_uint]
     lib.moc_debug_wait_probe.argtypes = [vp, vp, i32, vp]
-    lib.moc_debug_shared_key_tiles.argtypes = [C.POINTER(_Problem), i32, i32, C.POINTER(i32), vp, vp]
+    lib.moc_debug_shared_key_tiles.argtypes = [C.POINTER(_Problem), i32, i32, C.POINTER(i32), vp, vp, C.POINTER(sz)]
     lib.moc_attend.argtypes = [vp] * 9
     lib.moc_attend_bwd.argtypes = [vp] * 13
     lib.moc_selected_pairs.argtypes = [vp, vp, vp, C.POINTER(C.c_int64)]
@@ -113,14 +113,15 @@ def _problem(n_heads, n_tokens, head_dim, chunk_off, chunk_shot, chunk_mod, top_
 
 def debug_shared_key_tiles(wl, n_sm):
     """Test hook, host only: for each long key tile of a head in the dK/dV launch on n_sm SMs, the tiles of query rows that have it as
-    an anchor and the blocks that share it."""
+    an anchor and the blocks that share it; and the bytes there are for the counters of all heads' tiles."""
     lay = wl.layout
     pr, tables = _problem(wl.n_heads, lay.n_tokens, wl.head_dim, lay.chunk_off, lay.chunk_shot, lay.chunk_mod, wl.top_k, wl.win_back,
                           wl.win_fwd, wl.causal, 0.0)
     cap = lay.n_tokens // 128 + lay.n_chunks
-    n, query_tiles, blocks = C.c_int(0), np.zeros(cap, np.int32), np.zeros(cap, np.int32)
-    _check(load_library().moc_debug_shared_key_tiles(C.byref(pr), int(n_sm), cap, C.byref(n), query_tiles.ctypes.data, blocks.ctypes.data))
-    return query_tiles[:n.value], blocks[:n.value]
+    n, room, query_tiles, blocks = C.c_int(0), C.c_size_t(0), np.zeros(cap, np.int32), np.zeros(cap, np.int32)
+    _check(load_library().moc_debug_shared_key_tiles(C.byref(pr), int(n_sm), cap, C.byref(n), query_tiles.ctypes.data, blocks.ctypes.data,
+                                                     C.byref(room)))
+    return query_tiles[:n.value], blocks[:n.value], room.value
 
 
 class MocPlan:

@@ -42,7 +42,8 @@ struct WsLayout {
     size_t qlist;       // int32[H][cap_total]  per (head, chunk) list at cap_off[c]: entries i*k+s of the picks of c
     size_t desc3;       // bf16 [H][3][Cpad][d]  descriptors split into three bf16 terms (hi + mid + lo)
     size_t pool_part;   // float[H][n_pool_units][d] partial key sums
-    size_t pool_done;   // int32[H][C] arrival counters (cleared at the start of every pooling call; in the backward, of split key tiles)
+    size_t pool_done;   // int32 arrival counters: of pooling, [H][C] (cleared at the start of every call), or in the backward, [H][n_long_ktiles], of
+                        // the key tiles that several blocks share
     size_t queue;       // int32[kQueueHeader + 6 groups] work queue of the forward attention kernel
     size_t part_o;      // bf16 [1 or 2][Hg][L][k][d] routed partial outputs (normalised) of one group of Hg heads; with
                         // several groups, two buffers that consecutive groups alternate between
@@ -275,6 +276,6 @@ int moc_debug_set_wait_limit_us(moc_plan *plan, unsigned us);
 // record MOC_ERR_TIMEOUT with detail `code` in ws, and return
 int moc_debug_wait_probe(const moc_plan *plan, void *ws, int code, void *stream);
 // host only: the long key tiles of dK/dV of a problem on a GPU with n_sm SMs (up to cap of them written): tiles of query rows that
-// a tile has whatever is picked, and blocks that share them
-int moc_debug_shared_key_tiles(const moc_problem *problem, int n_sm, int cap, int *n_tiles, int *query_tiles, int *blocks);
+// a tile has whatever is picked, and blocks that share them; and the bytes there are for the counters of all heads' tiles
+int moc_debug_shared_key_tiles(const moc_problem *problem, int n_sm, int cap, int *n_tiles, int *query_tiles, int *blocks, size_t *counter_room);
 }

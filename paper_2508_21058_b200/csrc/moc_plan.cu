@@ -98,7 +98,7 @@ void layout_workspace(moc_plan *p) {
     w.qlist = take(sizeof(int32_t) * H * (size_t)std::max(p->cap_off[C], 1));
     w.desc3 = take(sizeof(__nv_bfloat16) * H * 3 * (size_t)p->c_pad * d);
     w.pool_part = take(sizeof(float) * H * (size_t)p->n_pool_units * d);
-    w.pool_done = take(sizeof(int32_t) * H * C);
+    w.pool_done = take(sizeof(int32_t) * H * std::max<size_t>(C, p->n_split > 1 ? p->n_long_ktiles : 0));
     w.queue = take(sizeof(int32_t) * (kQueueHeader + 6 * groups));
     w.part_o = take(per_head * (size_t)p->heads_per_group * buffers);
     w.part_lse = take(sizeof(float) * H * ((L + 127) / 128 * 128) * (k ? k : 1));
@@ -549,8 +549,9 @@ extern "C" int moc_debug_set_wait_limit_us(moc_plan *p, unsigned us) {
     return MOC_OK;
 }
 
-extern "C" int moc_debug_shared_key_tiles(const moc_problem *pr, int n_sm, int cap, int *n_tiles, int *query_tiles, int *blocks) {
-    if (!pr || !n_tiles || !query_tiles || !blocks) return MOC_ERR_NULL;
+extern "C" int moc_debug_shared_key_tiles(const moc_problem *pr, int n_sm, int cap, int *n_tiles, int *query_tiles, int *blocks,
+                                           size_t *counter_room) {
+    if (!pr || !n_tiles || !query_tiles || !blocks || !counter_room) return MOC_ERR_NULL;
     if (int r = check_problem(pr)) return r;
     if (n_sm < 1) return MOC_ERR_SHAPE;
     moc_plan p;
@@ -558,6 +559,7 @@ extern "C" int moc_debug_shared_key_tiles(const moc_problem *pr, int n_sm, int c
     if (int r = derive_plan(&p, pr, n_sm, tab)) return r;
     const int most = dkv_split(&p);
     *n_tiles = p.n_long_ktiles;
+    *counter_room = p.ws.queue - p.ws.pool_done;
     for (int x = 0; x < std::min(cap, p.n_long_ktiles); ++x) {
         query_tiles[x] = p.ktiles[x].n_anc;
         blocks[x] = std::min(p.ktiles[x].parts, most);

@@ -27,7 +27,7 @@ LONG_CHUNK = {
 
 @pytest.mark.parametrize("stream", LONG_CHUNK)
 def test_a_long_chunk_has_no_more_blocks_than_query_tiles(stream):
-    query_tiles, blocks = debug_shared_key_tiles(LONG_CHUNK[stream](128), N_SM)
+    query_tiles, blocks, _ = debug_shared_key_tiles(LONG_CHUNK[stream](128), N_SM)
     assert query_tiles.min() < blocks.max()                    # the case: the caption's number would be too many
     assert np.all(blocks >= 1) and np.all(blocks <= query_tiles)
 
@@ -45,7 +45,7 @@ def test_every_block_has_a_query_tile_whatever_the_stream():
             shots, window = np.sort(rng.randint(rng.choice([1, 3, n]), size=n)), rng.choice([0, 1, 3, W.WHOLE_SHOT], 2)
         sizes[list(captions)] = rng.choice([1, 5, 64, 128, 256, 1000])
         wl = ragged(rng.choice([1, 2, 4]), rng.choice([64, 128]), sizes, rng.choice([1, 2, 4, 9, 20]), *window, captions, shots)
-        query_tiles, blocks = debug_shared_key_tiles(wl, N_SM)
+        query_tiles, blocks, _ = debug_shared_key_tiles(wl, N_SM)
         assert np.all((blocks >= 1) & (blocks <= 8) & (blocks <= query_tiles)), (sizes, shots, query_tiles, blocks)
         # tiles first..last of block p: floor(n p / blocks) to floor(n (p + 1) / blocks), with n at least the query tiles
         for n_qt, b in zip(query_tiles, blocks):
@@ -53,3 +53,11 @@ def test_every_block_has_a_query_tile_whatever_the_stream():
             assert np.all(np.diff(cuts) >= 1)
         uneven += len(blocks) > 0 and query_tiles.min() < blocks.max()
     assert uneven > 20
+
+
+@pytest.mark.parametrize("heads,caption,chunks,size,n_sm", [(1, 5000, 30, 608, 148), (2, 6656, 30, 1560, 2000), (2, 12800, 30, 1560, 2000)])
+def test_the_counters_of_shared_tiles_fit_their_area(heads, caption, chunks, size, n_sm):
+    """A caption of many key tiles before few chunks: more counters than the stream has chunks, which the work queue follows."""
+    query_tiles, blocks, room = debug_shared_key_tiles(ragged(heads, 128, [caption] + [size] * chunks, 4), n_sm)
+    assert blocks.max() > 1 and len(blocks) > chunks + 1
+    assert 4 * heads * len(blocks) <= room
