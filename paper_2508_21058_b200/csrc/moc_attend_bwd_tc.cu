@@ -100,6 +100,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
     } else if (warp == 1) {
         if (lane == 0) {
             s_abort = 0;
+            s_last = 0;                                    // (stays so if thread 0 gives up before it has counted the block)
             int valid = (*(volatile int *)p.status == 0);
             if (valid && (uint32_t)((volatile int *)p.status)[ST_COOKIE] != p.cookie) {
                 atomicCAS(p.status, 0, MOC_ERR_WORKSPACE);      // not this plan's lists: report, touch nothing else

@@ -183,3 +183,46 @@ def test_the_model_sees_a_barrier_that_gets_two_phases_ahead():
     one = [[op.replace("T1_ISSUED + (j & 1), (j >> 1) & 1", "T1_ISSUED, j & 1").replace("T1_ISSUED + (j & 1)", "T1_ISSUED") for op in ops]
            for ops in (SIDE1, SIDE2)]
     assert not all(list(_schedules(*one)))
+
+
+def shared_tile_epilogue(seed, s_last, initialised):
+    """The end of a block that shares its key tile (two barriers of the lane warps, the count of the blocks that have left their sums in
+    between), in which waits for a barrier that is not complete may run out.  Whether a warp stored although the block has not
+    counted itself, and so does not know that it is the last."""
+    rng, bars, state = random.Random(seed), (Barrier(8), Barrier(8)), {"last": 0 if initialised else s_last, "counted": False}
+    stored = []
+
+    def warp(w):
+        ok = True
+        bars[0].arrive()
+        yield 0, lambda: bars[0].done(0)
+        ok = ok and bars[0].done(0)
+        if w == 0 and ok:
+            state.update(last=1, counted=True)               # this block is the last one
+        bars[1].arrive()
+        if ok:
+            yield 1, lambda: bars[1].done(0)
+            ok = bars[1].done(0)
+        if ok and state["last"]:
+            stored.append(state["counted"])
+
+    agents = {w: warp(w) for w in range(8)}
+    waits, slow = dict.fromkeys(agents), rng.randrange(8)
+    while agents:
+        able = [w for w in agents if waits[w] is None or waits[w][1]()]
+        late = [w for w in agents if w not in able and rng.random() < 0.2]      # ... and these run out
+        who = rng.choice([w for w in able + late if w != slow] or able or list(agents))
+        try:
+            waits[who] = next(agents[who])
+        except StopIteration:
+            del agents[who]
+    return not all(stored)
+
+
+def test_a_block_that_gives_up_on_a_shared_tile_stores_nothing():
+    with open(SRC) as f:
+        text = f.read()
+    before = text[:text.index("__syncthreads();")]
+    assert any(shared_tile_epilogue(seed, 1, False) for seed in range(500))      # the model sees what an unset flag does
+    assert not any(shared_tile_epilogue(seed, 1, True) for seed in range(500))
+    assert re.search(r"\bs_last = 0;", before)                                   # and the kernel sets it before the barriers are used
