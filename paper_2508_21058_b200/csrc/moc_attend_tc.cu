@@ -115,8 +115,6 @@ __device__ __forceinline__ bool wait_count(const int *ctr, int need, volatile in
     }
 }
 
-constexpr float kLog2e = 1.4426950408889634f;
-
 // acc += w x (the bf16 pair u) where cond holds
 __device__ __forceinline__ void add_weighted_if(bool cond, uint64_t &acc, uint32_t u, float w) {
     const uint64_t v = pack2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u)), w2 = pack2(w, w);
@@ -508,7 +506,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                         for (int u = 0; u < 8; ++u) wsum += __expf(plv[u] - big);
                     }
                 }
-                const float inv_w = 1.f / wsum, w_own = __expf(lse_own - big) * inv_l, big_log2 = big * kLog2e;
+                const float inv_w = 1.f / wsum, w_own = __expf(lse_own - big) * inv_l;
                 if constexpr (kMergeInRegs) {
                     // Passes of eight of the warp's rows over the slots, a few at a time: the loads of the next few are on their way
                     // while these are added up.
@@ -538,7 +536,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                     auto add = [&](const Batch &b) __attribute__((always_inline)) {
                         const int src_lane = pass * 8 + l4;
                         if (s0 == 0) {
-                            row_big = __shfl_sync(0xffffffffu, big_log2, src_lane);
+                            row_big = __shfl_sync(0xffffffffu, big, src_lane);
                             const float w = __shfl_sync(0xffffffffu, w_own, src_lane);
                             const uint64_t w2 = pack2(w, w);
 #pragma unroll
@@ -558,8 +556,9 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                         }
 #pragma unroll
                         for (int u = 0; u < B; ++u) {
-                            // exp2(-inf) = 0: an empty slot, and what its place holds is not a number to use
-                            const float w = ex2(fmaf(b.ls[u], kLog2e, -row_big));
+                            // exp(-inf) = 0: an empty slot, and what its place holds is not a number to use.  (Formed as for wsum: with
+                            // big * log2(e) rounded beforehand the weights of scores around 1e5 did not sum to one.)
+                            const float w = __expf(b.ls[u] - row_big);
 #pragma unroll
                             for (int cb = 0; cb < CB; ++cb)
 #pragma unroll
@@ -626,7 +625,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                         }
 #pragma unroll 1
                         for (int s = 0; s < n_merge; ++s) {
-                            const float w = ex2(fmaf(ls1, kLog2e, -big_log2));       // exp2(-inf) = 0: an empty slot
+                            const float w = __expf(ls1 - big);       // as for wsum; exp(-inf) = 0: an empty slot
                             ls1 = ls2;
                             const int s2 = s + 2 < p.k ? s + 2 : s + 2 - p.k;       // (the next block's first slots after the last)
                             ls2 = merge ? __ldcg(pl + min(s2, p.k - 1) * 128) : -INFINITY;

@@ -81,3 +81,17 @@ def test_tensors_on_16_byte_boundaries(d, frame):
     assert p.moc_get_status(run.ws)[0] == 0
     for a, b in ((O, run.O), (dQ, run.dQ), (dK, run.dK), (dV, run.dV)):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("d,frame,k", [(128, 130, 3), (128, 600, 5), (64, 130, 3), (64, 400, 5)])
+def test_weights_of_large_scores_sum_to_one(d, frame, k):
+    """Scores with a common part of some 4e5: values of one come out as one.  The partials and O are sums of P rounded to bf16 over the
+    sum of P (half an ulp each: 2^-9), so O is one or the bf16 below."""
+    wl = W.Workload("large", 2, d, W.make_layout(1, 16, 16, frame), k, 0, 0)
+    run = PU.GpuRun(wl)
+    for n in ("q", "k"):
+        run.x[n][..., 0] = 2000.0
+    run.x["v"].fill_(1.0)
+    run.forward()
+    assert float(run.lse.min()) > 3e5
+    assert float((run.O.float() - 1).abs().max()) <= 2 ** -8
