@@ -126,7 +126,8 @@ def _clean_like_the_contract(wl, orc, sel):
     return out
 
 
-@pytest.mark.parametrize("name", ["mini2", "mini9", "mini5"])
+# (repeats are found by comparing with up to 4 picks, by a bitmap of the row's picks with 12 and 20)
+@pytest.mark.parametrize("name", ["mini2", "mini9", "mini5", "mini6", "mini10"])
 def test_edited_selection_is_honoured_after_lists_from_sel(name):
     wl = W.workload(name)
     run = PU.GpuRun(wl, tensors=("q", "k", "v", "do")).forward()
