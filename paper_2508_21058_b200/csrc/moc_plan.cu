@@ -1,5 +1,6 @@
 // Plan object (validated problem + derived chunk tables on the device), workspace layout,
 // argument checking and the C entry points.
+#include <cuda.h>
 #include <math.h>
 #include <algorithm>
 #include <string.h>
@@ -57,18 +58,30 @@ __global__ void token_chunk_kernel(const int32_t *__restrict__ off, int32_t *__r
     for (int t = off[blockIdx.x] + threadIdx.x; t < off[blockIdx.x + 1]; t += blockDim.x) tok_chunk[t] = blockIdx.x;
 }
 
-// The stream on which plans get their tables, one per device for as long as the process lives (making one takes 100 us).
-static cudaError_t table_stream(int device, cudaStream_t *out) {
+// The stream on which plans get their tables, one per context for as long as the process lives (making one takes 100 us).  A stream
+// belongs to the context it was made in, and a device can have several, or a new one after cudaDeviceReset.
+static cudaError_t table_stream(cudaStream_t *out) {
+    typedef CUresult (*CtxGetIdFn)(CUcontext, unsigned long long *);
+    struct Entry { unsigned long long ctx; cudaStream_t stream; };
     static std::mutex mu;
-    static std::vector<cudaStream_t> streams;
+    static std::vector<Entry> streams;
+    static CtxGetIdFn ctx_id = nullptr;
     std::lock_guard<std::mutex> hold(mu);
-    if ((int)streams.size() <= device) streams.resize(device + 1, nullptr);
-    if (!streams[device]) {
-        const cudaError_t e = cudaStreamCreateWithFlags(&streams[device], cudaStreamNonBlocking);
-        if (e != cudaSuccess) { streams[device] = nullptr; return e; }
+    if (!ctx_id) {
+        void *sym = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const cudaError_t e = cudaGetDriverEntryPoint("cuCtxGetId", &sym, cudaEnableDefault, &q);
+        if (e != cudaSuccess) return e;
+        if (!sym || q != cudaDriverEntryPointSuccess) return cudaErrorSymbolNotFound;
+        ctx_id = (CtxGetIdFn)sym;
     }
-    *out = streams[device];
-    return cudaSuccess;
+    unsigned long long id = 0;                                   // of the current context; never used twice
+    if (ctx_id(nullptr, &id) != CUDA_SUCCESS) return cudaErrorInvalidResourceHandle;
+    for (const Entry &x : streams)
+        if (x.ctx == id) { *out = x.stream; return cudaSuccess; }
+    const cudaError_t e = cudaStreamCreateWithFlags(out, cudaStreamNonBlocking);
+    if (e == cudaSuccess) streams.push_back(Entry{id, *out});
+    return e;
 }
 
 // Workspace layout.  The routed partial outputs ([heads][L][k][d] bf16, k times the size of O) are held for
@@ -365,7 +378,7 @@ extern "C" int moc_plan_create(const moc_problem *pr, moc_plan **out) {
     // On a stream of its own: on the legacy stream the copy would wait for what the caller has under way there.  The plan is
     // handed out when the tables are there, for a stream of any kind.
     cudaStream_t st = nullptr;
-    e = table_stream(dev, &st);
+    e = table_stream(&st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b, host.data(), from_host, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
         token_chunk_kernel<<<(unsigned)C, 256, 0, st>>>((const int32_t *)(b + o_off), (int32_t *)(b + o_tok));

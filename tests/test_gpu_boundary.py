@@ -1,6 +1,7 @@
 """Contract of the C ABI beyond plain parity: a workspace that does not hold the plan's lists is refused
 on the device without a fault, an edited selection is honoured after moc_lists_from_sel, a bounded wait
 that runs out is reported and leaves the GPU usable, the workspace budget, and the debug build."""
+import ctypes
 import os
 import subprocess
 import sys
@@ -297,3 +298,20 @@ def test_a_new_plans_tables_are_there_for_a_stream_of_any_kind(name):
             *got, ws = plan.forward(x["q"], x["k"], x["v"])
             assert plan.moc_get_status(ws)[0] == 0               # waits for the side stream alone
             assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+def test_plans_are_made_in_every_context_of_the_device():
+    """A plan's tables go over on a stream that is kept; a stream belongs to one context.  (Only made and destroyed in the second one:
+    the tensors of this process belong to the first.)"""
+    cu, ctx, wl = ctypes.CDLL("libcuda.so.1"), ctypes.c_void_p(), W.workload("mini2")
+    before = PU.GpuRun(wl).forward()
+    assert cu.cuCtxCreate_v2(ctypes.byref(ctx), 0, torch.cuda.current_device()) == 0
+    try:
+        for _ in range(2):
+            MocPlan.from_workload(wl).close()
+    finally:
+        assert cu.cuCtxDestroy_v2(ctx) == 0
+    after = PU.GpuRun(wl).forward()
+    for n in ("desc", "sel"):
+        assert torch.equal(getattr(before, n), getattr(after, n)), n
+    assert float((before.O.float() - after.O.float()).abs().max()) <= 1e-2          # the same rows, grouped into other tiles
