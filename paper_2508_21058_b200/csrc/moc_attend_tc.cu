@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
         // What gives every barrier's phase: of the running counts only the low bits, in one register.  (A row of S fills most of
         // the registers: each one that lives through the loop over the tiles is one the loop lacks.)
         enum : uint32_t { S_ODD = 1, TURN_ODD = 2, TURNED = 4, MINE_ODD = 8, DEP_ODD = 16, MERGE_AT = 5 };      // key tiles; key tiles in
-                                                       // two-tile items, any at all; items with this tile; DEPENDs; MERGE phases
+                                                       // two-tile items, any at all; items with this tile; DEPENDs; MERGE phases; from bit 16 on, see `slots`
         uint32_t bits = 0;
         int n_item = 0, last_phase = -1;               // items seen, modulo 12 (three slots, four ROWS_DONE)
         bool ok = true;
@@ -467,7 +467,10 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 // 18.8 -> 13.8 ms by register loads, 15.2 by copies.)
                 const int tile_rows = min(128, rows - g * 128), warp_rows = LOADERS ? (tile_rows + 3) >> 2 : 32;
                 const int q0 = first + g * 128 + (warp & 3) * warp_rows, n_rows = min(warp_rows, first + g * 128 + tile_rows - q0);   // the warp's rows
-                const int n_merge = n_rows > 0 ? p.k : 0;
+                // Slots up to the last one that a row of the warp uses: early in a stream, and wherever rows may route to few chunks, most of
+                // many are empty.  (All k slots -> these: 3 heads of 2.2k tokens, 512-token chunks, 30 picks 59.6 -> 43.4 us, d = 64 44.4 ->
+                // 29.5; 12 heads of 66k tokens, 800-token chunks, 30 picks 11.41 -> 10.94 ms; with all in use within 2 %.)
+                int n_slots = p.k, used = 0;
                 const int qb = it_.qbuf + g < 3 ? it_.qbuf + g : it_.qbuf + g - 3;
                 const uint32_t m_base = D == 128 ? sQ + qb * TILE_BYTES + (warp & 3) * (TILE_BYTES / 4) : sbase + 7 * TILE_BYTES + warp * (kMergeStages * 4096);
                 int m_st = 0, m_next = 0, m_flight = 0;          // stage to read, block to ask for, blocks under way
@@ -484,9 +487,9 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                     ++m_next;
                     ++m_flight;
                     if (++c_st == kMergeStages) c_st = 0;
-                    if (++c_slot == p.k) { c_slot = 0; ++c_cb; }
+                    if (++c_slot == n_slots) { c_slot = 0; ++c_cb; }
                 };
-                if (!kMergeInRegs && n_merge > 0) {
+                if (!kMergeInRegs && n_rows > 0 && p.k > 0) {
                     // other CTAs' stores, seen through DEPEND by the generic proxy, are read by the copy engine
                     if (lane == 0) asm volatile("fence.proxy.async;" ::: "memory");
                     for (int x = 0; x < kMergeStages && x < CB * p.k; ++x) copy_next();
@@ -503,25 +506,43 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                         wsum *= __expf(big - m);
                         big = m;
 #pragma unroll
-                        for (int u = 0; u < 8; ++u) wsum += __expf(plv[u] - big);
+                        for (int u = 0; u < 8; ++u) {
+                            wsum += __expf(plv[u] - big);
+                            if (plv[u] != -INFINITY) used = s0 + u + 1;
+                        }
                     }
+                }
+                if (kMergeInRegs) {
+                    bits = (bits & 0xffff) | (uint32_t)__reduce_max_sync(0xffffffffu, used) << 16;
+                } else {                                         // (the first few have been asked for already)
+                    n_slots = max(__reduce_max_sync(0xffffffffu, used), min(kMergeStages, p.k));
+                    if (c_slot >= n_slots) { c_slot = 0; ++c_cb; }
+                    if (n_rows <= 0) n_slots = 0;
                 }
                 const float inv_w = 1.f / wsum, w_own = __expf(lse_own - big) * inv_l;
                 if constexpr (kMergeInRegs) {
                     // Passes of eight of the warp's rows over the slots, a few at a time: the loads of the next few are on their way
                     // while these are added up.
                     constexpr int B = 3;
+                    // The slots in use are kept beside the phases and taken out where they are wanted: in a register of their own, or as the
+                    // bound of the loops (whose counters then are not the whole warp's), they made the loop over the tiles spill.
+                    auto slots = [&]() __attribute__((always_inline)) {
+                        int n;
+                        asm volatile("shr.u32 %0, %1, 16;" : "=r"(n) : "r"(bits));
+                        return n;
+                    };
                     const int row0 = q0 + l4, row_end = q0 + n_rows, n_pass = max(1, (n_rows + 7) >> 3);
                     struct Batch { uint32_t v[B][CB][8]; float ls[B]; };
                     int ask_pass = 0, ask_s = 0;
                     auto ask = [&](Batch &b) __attribute__((always_inline)) {
                         const int q = row0 + ask_pass * 8;
                         const bool in = q < row_end;
+                        const int n = slots();
                         const char *src = part + part_line(h_loc, LB, p.k, CB, q, ask_s) + l2 * 32;
                         const float *ls = p.part_lse + part_lse_at(h, LB, p.k, q, ask_s);
 #pragma unroll
                         for (int u = 0; u < B; ++u) {
-                            const bool some = in && ask_s + u < p.k;
+                            const bool some = in && ask_s + u < n;
                             const float x = __ldcg(some ? ls + u * 128 : pl);
                             b.ls[u] = some ? x : -INFINITY;
 #pragma unroll
@@ -554,15 +575,17 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                                 mbar_arrive(bar(O_FREE + g));
                             }
                         }
+                        if (s0 < slots()) {
 #pragma unroll
-                        for (int u = 0; u < B; ++u) {
-                            // exp(-inf) = 0: an empty slot, and what its place holds is not a number to use.  (Formed as for wsum: with
-                            // big * log2(e) rounded beforehand the weights of scores around 1e5 did not sum to one.)
-                            const float w = __expf(b.ls[u] - row_big);
+                            for (int u = 0; u < B; ++u) {
+                                // exp(-inf) = 0: an empty slot, and what its place holds is not a number to use.  (Formed as for wsum: with
+                                // big * log2(e) rounded beforehand the weights of scores around 1e5 did not sum to one.)
+                                const float w = __expf(b.ls[u] - row_big);
 #pragma unroll
-                            for (int cb = 0; cb < CB; ++cb)
+                                for (int cb = 0; cb < CB; ++cb)
 #pragma unroll
-                                for (int x = 0; x < 8; ++x) add_weighted_if(w != 0.f, acc[cb][x], b.v[u][cb][x], w);
+                                    for (int x = 0; x < 8; ++x) add_weighted_if(w != 0.f, acc[cb][x], b.v[u][cb][x], w);
+                            }
                         }
                         s0 += B;
                         if (s0 >= p.k) {
@@ -624,10 +647,10 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                             mbar_arrive(bar(O_FREE + g));
                         }
 #pragma unroll 1
-                        for (int s = 0; s < n_merge; ++s) {
+                        for (int s = 0; s < n_slots; ++s) {
                             const float w = __expf(ls1 - big);       // as for wsum; exp(-inf) = 0: an empty slot
                             ls1 = ls2;
-                            const int s2 = s + 2 < p.k ? s + 2 : s + 2 - p.k;       // (the next block's first slots after the last)
+                            const int s2 = s + 2 < n_slots ? s + 2 : s + 2 - n_slots;       // (the next block's first slots after the last)
                             ls2 = merge ? __ldcg(pl + min(s2, p.k - 1) * 128) : -INFINITY;
                             ok = mbar_wait(bar(MERGE + warp * kMergeStages + m_st), (bits >> (MERGE_AT + m_st)) & 1, abort_flag, p.status, W_MERGE);
                             ok = __all_sync(0xffffffffu, ok);
@@ -644,7 +667,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                             __syncwarp();
                             bits ^= 1u << (MERGE_AT + m_st);
                             --m_flight;
-                            if (m_next < CB * p.k) copy_next();
+                            if (m_next < CB * n_slots) copy_next();
                             if (++m_st == kMergeStages) m_st = 0;
                         }
                         if (ok && qi >= 0) {

@@ -25,6 +25,13 @@ SHAPES = {
     "d 64, 3 picks": (2, 64, (2, 1, 9, 65), 3, False),                    # as many as stages
     "d 64, 4 picks, empty slots": (2, 64, (3, 5, 9, 129), 4, True),
     "d 64, 9 picks, one loading warp": (2, 64, (2, 3, 14, 300), 9, True),
+    # more slots than chunks to pick: rows that use none, fewer than are asked for ahead, or some of them
+    "register merge, 3 of 12 slots": (2, 128, (1, 16, 5, 130), 12, False),
+    "register merge, 5 of 20 slots, some empty": (2, 128, (1, 16, 7, 140), 20, True),
+    "block copies, 3 of 12 slots": (2, 128, (1, 16, 5, 577), 12, False),
+    "block copies, 5 of 20 slots, some empty": (1, 128, (1, 16, 7, 530), 20, True),
+    "d 64, 3 of 12 slots": (2, 64, (1, 16, 5, 130), 12, False),
+    "d 64, 5 of 20 slots, some empty, one loading warp": (2, 64, (1, 16, 7, 300), 20, True),
 }
 # P and the partials are rounded to bf16 on one side and not on the other (half an ulp: 2^-9), as is O on both: three such steps, 6e-3,
 # on the 2-norm of a block of rows; a slot missed, taken twice or weighed wrongly is off by more than a tenth (at most 9 picks).
