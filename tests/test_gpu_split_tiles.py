@@ -5,22 +5,25 @@ import torch
 
 from paper_2508_21058_b200 import MocPlan
 from paper_2508_21058_b200 import workloads as W
+from paper_2508_21058_b200.binding import debug_shared_key_tiles
 
 import parity_utils as PU
 from test_shared_key_tiles import LONG_CHUNK
 
 pytestmark = pytest.mark.gpu
 
-# heads, head_dim, (shots, caption, frames, frame length), k; by the rule of moc_plan_create the blocks of a caption's tile are
+# heads, head_dim, (shots, caption, frames, frame length), k, blocks that share a caption's tile on 148 SMs
 SHAPES = {
-    "4 blocks, a tile of two rows": (2, 128, (1, 130, 24, 100), 2),
-    "8 blocks, two captions of 5": (1, 128, (2, 5, 20, 129), 1),
-    "6 blocks, one key": (1, 64, (1, 1, 40, 64), 1),
-    "7 blocks, d 64": (3, 64, (1, 40, 64, 97), 3),
-    "no room for their sums": (1, 128, (1, 140, 30, 100), 0),              # without picks there are no partials to take the place of
+    "4 blocks, a tile of two rows": (2, 128, (1, 130, 24, 100), 2, 4),
+    "8 blocks, two captions of 5": (1, 128, (2, 5, 40, 129), 1, 8),
+    "8 blocks, three captions of two tiles": (1, 128, (3, 130, 30, 129), 3, 8),
+    "6 blocks, one key": (1, 64, (1, 1, 40, 64), 2, 6),
+    "7 blocks, d 64": (3, 64, (1, 40, 64, 97), 3, 7),
+    "no room for the sums of two captions": (1, 128, (2, 5, 20, 129), 1, 1),
+    "no room for their sums": (1, 128, (1, 140, 30, 100), 0, 1),           # without picks there are no partials to take the place of
 }
 # P and dS are rounded to bf16 (half an ulp: 2^-9) on one side, the results on both: a few 1e-3 of the 2-norm of a block of rows
-# (seen: 4e-3).  Of at most 49 query tiles one left out, or taken twice, is off by sqrt(1 / 49) = 0.14.
+# (seen: 4e-3).  Of at most 94 query tiles one left out, or taken twice, is off by sqrt(1 / 94) = 0.10.
 REL = 2e-2
 
 
@@ -49,8 +52,11 @@ def check_every_gradient(wl, passes, spoil=None):
 
 @pytest.mark.parametrize("shape", SHAPES)
 def test_every_gradient_of_a_shared_tile(shape):
-    heads, d, lay, k = SHAPES[shape]
-    check_every_gradient(W.Workload("split", heads, d, W.make_layout(*lay), k, 1, 1), 20)
+    heads, d, lay, k, blocks = SHAPES[shape]
+    wl = W.Workload("split", heads, d, W.make_layout(*lay), k, 1, 1)
+    n_sm = torch.cuda.get_device_properties(0).multi_processor_count
+    assert n_sm != 148 or set(debug_shared_key_tiles(wl, n_sm)[1]) == {blocks}
+    check_every_gradient(wl, 20)
 
 
 @pytest.mark.parametrize("d", [64, 128])

@@ -13,13 +13,13 @@ pytestmark = pytest.mark.gpu
 # heads, head_dim, (shots, caption, frames, frame length), k
 SHAPES = {
     "whole tiles only": (5, 128, (3, 128, 6, 128), 4),                 # one key tile a chunk; every dK/dV query tile from consecutive rows
-    "four key tiles a chunk": (2, 128, (2, 16, 4, 512), 2),            # one query-loading warp: few picks
-    "four key tiles and one key": (2, 128, (2, 16, 4, 513), 2),        # one, whatever the picks
-    "two key tiles a chunk": (2, 128, (2, 16, 6, 256), 2),             # the last size with four loading warps whatever the picks
-    "two key tiles and one key": (2, 128, (2, 16, 8, 257), 6),         # the first size with one for up to 6 picks
-    "three key tiles, 7 picks": (2, 128, (2, 16, 8, 384), 7),          # the last size with four for 7 and 8
-    "four key tiles, 8 picks": (1, 128, (2, 16, 8, 512), 8),           # the last number of picks with one at this size
-    "four key tiles, 9 picks": (1, 128, (2, 16, 8, 512), 9),           # the first with four
+    "four key tiles a chunk": (2, 128, (2, 16, 4, 512), 2),            # the last size with four query-loading warps
+    "four key tiles and one key": (2, 128, (2, 16, 4, 513), 2),        # the first with one
+    "two key tiles a chunk": (2, 128, (2, 16, 6, 256), 2),
+    "two key tiles and one key": (2, 128, (2, 16, 8, 257), 6),         # three key tiles, the last with one key; whole batches of the merge
+    "three key tiles, 7 picks": (2, 128, (2, 16, 8, 384), 7),          # a last merge batch with one slot
+    "four key tiles, 8 picks": (1, 128, (2, 16, 8, 512), 8),           # ... with two
+    "four key tiles, 9 picks": (1, 128, (2, 16, 8, 512), 9),
     "one row past a tile": (7, 128, (2, 1, 11, 129), 9),               # items of 256 rows and of a few; a merge of 8 + 1 picks
     "one row short of two tiles": (2, 64, (2, 31, 9, 255), 8),         # a full merge batch
     "17 picks": (3, 64, (2, 1, 13, 65), 17),                           # the shortest sorted list, 26 columns
