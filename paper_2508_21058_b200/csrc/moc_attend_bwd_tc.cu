@@ -163,7 +163,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
         // 2 + half, so that the first two chunks - the first half of P for ACC2 - are finished first.  A thread
         // keeps its 64 P values between the two halves of a tile.
         asm volatile("setmaxnreg.inc.sync.aligned.u32 168;");
-        const int r = threadIdx.x & 127;              // row of the stationary tile = TMEM lane
         const int half = warp >> 2;
         const uint32_t lane_off = (uint32_t)((warp & 3) * 32) << 16;
         const uint64_t c2 = pack2(p.scale_log2, p.scale_log2);

@@ -246,8 +246,8 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
 #pragma unroll
                     for (int x = 0; x < 32; x += 2) uds[x >> 1] = ds_pair(dp[rd], rd, x);
                     // over the first half of the chunk's own columns, which this thread alone has read.  (With the chunks side by side
-                    // the two threads of a lane waited for each other: 10.69 -> 10.07 ms for the whole backward of the 33k-token
-                    // clip, 24 heads.)
+                    // the two threads of a lane waited for each other.  Without that, and with the partials as whole lines: 10.75 -> 10.21 ms
+                    // for the whole backward of the 33k-token clip, 24 heads, by itself.)
                     tmem_st16(t2 + (rd * 2 + half) * 32, uds);
                 }
                 tmem_wait_st();

@@ -51,7 +51,7 @@ struct AttendParams {
     __nv_bfloat16 *O;
     float *lse;
     __nv_bfloat16 *part_o;      // [2 or 1] buffers of the group in flight's partials (even / odd groups alternate), laid
-                                // out query-innermost in blocks of 128 queries (part_piece)
+                                // out query-innermost in blocks of 128 queries (part_line)
     float *part_lse;            // log-sum-exps of the partials, query-innermost (part_lse_at)
     size_t part_stride;         // elements between the two partial buffers (0 with a single group)
     const KeyRange *chunk_rng;  // [C] key range of a routed item (its chunk)
@@ -320,8 +320,8 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 // of j, tile 0 of j + 1, ...): each then has the arithmetic pipes to itself while
                 // the other tile's MMAs run, instead of both drifting into lock step.
                 // TURN + g is arrived on by group g when all but the last eight of its exponentials of a key tile are done: the
-                // hand-over takes about as long as those (after the last one: 33k-token clip 3.48 -> 3.42 ms, d = 64, 725-token
-                // frames 607 -> 572 us; at half time it cost 5 %).  (Tile 0 waits for
+                // hand-over takes about as long as those.  (After the last one instead, with the epilogue as it is now, the same within
+                // 0.3 %: 33k-token clip 3.407 and 3.404 ms, d = 64, 725-token frames 643.5 and 643.7 us; at half time it cost 5 %.)  (Tile 0 waits for
                 // tile 1's previous turn even at the start of an item: the barrier must never get two phases ahead of
                 // a group that has yet to wait on it.)
                 if (two && (g == 1 || (bits & TURNED))) {
