@@ -26,16 +26,6 @@ constexpr int kMaxSplit = 8;
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-// Sec. 3.2: text chunks are anchors of every query; so are the chunks of the query's shot
-// inside the window around its own chunk.
-static bool is_anchor(const moc_plan *p, int c, int j) {
-    if (p->mod[j] == 1) return true;
-    if (p->shot[j] != p->shot[c]) return false;
-    if (j < c && p->win_back != MOC_WHOLE_SHOT && c - j > p->win_back) return false;
-    if (j > c && p->win_fwd != MOC_WHOLE_SHOT && j - c > p->win_fwd) return false;
-    return true;
-}
-
 // FNV-1a over the problem and the heads per group: a workspace routed by one plan is not accepted by a plan of another problem,
 // nor under another budget (routing lays the attention's work queue out by groups of heads)
 static uint32_t plan_cookie(const moc_plan *p) {
@@ -161,17 +151,27 @@ static int derive_plan(moc_plan *p, const moc_problem *pr, int n_sm, DeviceTable
     p->shot.assign(pr->chunk_shot, pr->chunk_shot + C);
     p->mod.assign(pr->chunk_mod, pr->chunk_mod + C);
 
+    // Sec. 3.2: text chunks are anchors of every query; so are the chunks of the query's shot
+    // inside the window around its own chunk.  (Asked C * C times, twice: on values that no store can change.)
+    const auto is_anchor = [mod = p->mod.data(), shot = p->shot.data(), back = p->win_back, fwd = p->win_fwd](int c, int j) {
+        if (mod[j] == 1) return true;
+        if (shot[j] != shot[c]) return false;
+        if (j < c && back != MOC_WHOLE_SHOT && c - j > back) return false;
+        if (j > c && fwd != MOC_WHOLE_SHOT && j - c > fwd) return false;
+        return true;
+    };
     // anchor bitmaps, merged anchor key ranges, reverse anchors
     p->words = (C + 31) / 32;
-    std::vector<uint32_t> &bits = tab.bits;
-    bits.assign((size_t)C * p->words, 0u);
+    tab.bits.assign((size_t)C * p->words, 0u);
+    uint32_t *bits = tab.bits.data();
     std::vector<std::vector<int32_t>> rev(C);
     p->anc_off.assign(C + 1, 0);
     p->anc_tokens.assign(C, 0);
     for (int c = 0; c < C; ++c) {
+        uint32_t *row = bits + (size_t)c * p->words;
         for (int j = 0; j < C; ++j) {
-            if (!is_anchor(p, c, j)) continue;
-            bits[(size_t)c * p->words + j / 32] |= 1u << (j % 32);
+            if (!is_anchor(c, j)) continue;
+            row[j / 32] |= 1u << (j % 32);
             rev[j].push_back(c);
             p->anc_tokens[c] += p->off[j + 1] - p->off[j];
             if ((int)p->anc_rng.size() > p->anc_off[c] && p->anc_rng.back().t1 == p->off[j])
@@ -283,18 +283,20 @@ static int derive_plan(moc_plan *p, const moc_problem *pr, int n_sm, DeviceTable
     for (int j : col_chunk) p->routed_key_tiles += (p->off[j + 1] - p->off[j] + 127) / 128;
     p->cwords = std::max(1, (p->ncol + 31) / 32);
     p->c_pad = std::max(16, (p->ncol + 15) / 16 * 16);
-    std::vector<uint32_t> &cand_c = tab.cand_c;
-    std::vector<int32_t> &lim = tab.lim, &reach = tab.reach;
-    cand_c.assign((size_t)C * p->cwords, 0u);
-    lim.assign(C, 0);
-    reach.assign(C, 0);
+    tab.cand_c.assign((size_t)C * p->cwords, 0u);
+    tab.lim.assign(C, 0);
+    tab.reach.assign(C, 0);
+    uint32_t *cand_c = tab.cand_c.data();
+    int32_t *lim = tab.lim.data(), *reach = tab.reach.data();
+    const bool causal = p->flags & MOC_FLAG_CAUSAL;
     p->prefix_mode = 1;
     for (int c = 0; c < C; ++c) {
         int n_cand = 0, top = 0;
-        for (int j = 0; j < C; ++j) {
-            if (is_anchor(p, c, j) || ((p->flags & MOC_FLAG_CAUSAL) && j >= c)) continue;
+        uint32_t *row = cand_c + (size_t)c * p->cwords;
+        for (int j = 0; j < (causal ? c : C); ++j) {
+            if (is_anchor(c, j)) continue;
             const int col = col_of[j];          // a non-anchor is never text
-            cand_c[(size_t)c * p->cwords + col / 32] |= 1u << (col % 32);
+            row[col / 32] |= 1u << (col % 32);
             ++n_cand;
             top = col + 1;
         }
