@@ -17,8 +17,8 @@
 //                 (warp 1 the even units, warp 10 the odd ones);
 //     warps 2-5 / 6-9   selection groups (one, two or four: the units in turn), one query per thread (TMEM
 //                 lane = query): read the scores 32 chunks at a time, drop non-candidates,
-//                 keep a sorted top-k in registers (at most 64 entries; more picks are taken in
-//                 passes of 64 over recomputed scores), then write sel_idx and append the picks
+//                 keep a sorted top-k in registers (at most 32 entries; where more are picked, and with
+//                 more than 16 of many chunks: moc_route_long.cu), then write sel_idx and append the picks
 //                 to the per-(head, chunk) query lists (tile-local ranks from a shared-memory
 //                 histogram, one global atomic per (tile, chunk) to reserve the range).
 //   The head's descriptors stay in shared memory for the CTA's lifetime (C <= 192) and are scored
@@ -34,6 +34,7 @@
 #include <algorithm>
 
 #include "moc_common.cuh"
+#include "moc_route.cuh"
 #include "moc_tc.cuh"
 
 namespace moc {
@@ -137,7 +138,6 @@ struct RouteParams {
     int dual;               // two issuers (resident block, two accumulators or more).  The Q stages are then even in number: each
                             // stage serves one issuer, which so waits for every use of it (an issuer that left out a use could
                             // take the phase of a load still on its way for the one it waits for)
-    int n_pass;             // selection passes over a tile's scores: 64 picks each (the scores are recomputed per pass)
     int surv_cap;           // threshold selection: survivor slots per query row in shared memory (0 = not used)
     int *tile_off;          // [H C + 1] running tile counts, written by the last block to finish
     uint32_t cookie;
@@ -266,7 +266,6 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
     auto qparity_of = [&](int n) { return (int)((s_unit[n] >> 28) & 1u); };
     __syncthreads();
     constexpr int ACC_COLS = 512 / NG;   // TMEM columns per accumulator (NG = 4 only with sb_rows <= 128)
-    const int n_pass = KMAX == 64 ? p.n_pass : 1;     // only the 64-entry list is used for more picks than it holds
     const bool resident = p.d_rows == p.c_pad;       // every chunk's descriptor is held: loaded once, two MMA issuers
 
     if (warp == 0) {
@@ -294,7 +293,6 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                         tma_load_2d(sQ + st * Q_TILE_BYTES + sub * Q_SUB_BYTES, &tmQ, sub * 64, h * p.L + unit_of(n) * kRtRows, bar(Q_FULL + st));
                     ++qn;
                 }
-                for (int rep = 0; ok && rep < n_pass; ++rep)
                 for (int sb = 0; ok && sb < n_sb; ++sb) {
                     if (resident ? dn == 0 : sb != res_sb) {
                         ok = mbar_wait(bar(D_EMPTY), (dn & 1) ^ 1, abort_flag, p.status, RW_DEMPTY);
@@ -356,7 +354,6 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                 for (int n = n0; n < n1; ++n) n_sb = max(n_sb, steps_of(n));
                 for (int n = n0; ok && n < n1; ++n)
                     ok = wait(Q_FULL + qstage_of(n), qparity_of(n), RW_QFULL);
-                for (int rep = 0; ok && rep < n_pass; ++rep)
                 for (int sb = 0; ok && sb < n_sb; ++sb) {
                     if (resident ? dn == 0 : sb != res_sb) {
                         ok = wait(D_FULL, dn & 1, RW_DFULL);
@@ -405,10 +402,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                     // streamed blocks: the next step, if it needs another block, may overwrite this one once
                     // these MMAs are done
                     if (ok && !resident) {
-                        int nsb = sb + 1;
-                        bool more = true;
-                        if (nsb >= n_sb) { nsb = 0; more = rep + 1 < n_pass || n1 < nu; }
-                        if (more && nsb != sb) tc_commit_elect(bar(D_EMPTY));
+                        if (sb + 1 < n_sb || (n1 < nu && sb != 0)) tc_commit_elect(bar(D_EMPTY));
                     }
                 }
                 for (int n = n0; ok && n < n1; ++n) tc_commit_elect(bar(Q_EMPTY + qstage_of(n)));
@@ -430,7 +424,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
             ++ngs;
             return o;
         };
-        // the sorted list of this pass's picks lives in registers (a 64-entry list leaves room for one selection group)
+        // the sorted list of picks lives in registers
         constexpr int KR = KMAX;
         // With at most kRtDeferredChunks chunks the list append of a unit is finished after the next unit's selection,
         // so the round trip of the range-reserving atomics is hidden; `pend` is the unit whose append is open.
@@ -503,13 +497,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                 }
                 return j0 == 0 ? w0 : (live ? p.cand_c[(size_t)ci * p.cwords + (j0 >> 5)] : 0u);
             };
-            // More than 64 picks are taken 64 at a time: every pass sees the tile's scores again (the issuer
-            // recomputes them) and considers only the columns that come after the previous pass's last pick in
-            // the order of the result (score descending, then column ascending).
-            [[maybe_unused]] float prev_s = INFINITY;
-            [[maybe_unused]] int prev_j = -1;
-            for (int pass = 0; ok && pass < n_pass; ++pass) {
-            const int kp = min(p.k - pass * 64, KMAX);      // picks of this pass
+            const int kp = p.k;
             TopK<KMAX> top;
             top.init();
             [[maybe_unused]] float kth = -INFINITY;
@@ -582,13 +570,6 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                         float f[32];
 #pragma unroll
                         for (int c = 0; c < 32; ++c) f[c] = ((cand >> c) & 1u) ? __uint_as_float(v[c]) : -INFINITY;
-                        if (KMAX == 64 && pass > 0) {
-#pragma unroll
-                            for (int c = 0; c < 32; ++c) {
-                                const bool after = f[c] < prev_s || (f[c] == prev_s && j0 + c > prev_j);
-                                f[c] = after ? f[c] : -INFINITY;
-                            }
-                        }
 #pragma unroll 1
                         for (int round = 0; round < kp; ++round) {
                             float m8[4];
@@ -707,21 +688,12 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                         if (two) tmem_ld32(acc + ch, vh);
                         const uint32_t cand_l = cand_bits(jb + cl), cand_h = two ? cand_bits(jb + ch) : 0u;
                         tmem_wait_ld();
-                        const bool later_pass = KMAX == 64 && pass > 0;
-                        const bool plain = !later_pass && __all_sync(0xffffffffu, cand_l == 0xffffffffu && (!two || cand_h == 0xffffffffu));
+                        const bool plain = __all_sync(0xffffffffu, cand_l == 0xffffffffu && (!two || cand_h == 0xffffffffu));
                         if (!plain) {
 #pragma unroll
                             for (int c = 0; c < 32; ++c) {
                                 vl[c] = ((cand_l >> c) & 1u) ? vl[c] : 0xff800000u;      // -inf
                                 vh[c] = ((cand_h >> c) & 1u) ? vh[c] : 0xff800000u;
-                            }
-                            if (later_pass) {               // only what comes after the previous pass's last pick
-#pragma unroll
-                                for (int c = 0; c < 32; ++c) {
-                                    const float fl = __uint_as_float(vl[c]), fh = __uint_as_float(vh[c]);
-                                    vl[c] = (fl < prev_s || (fl == prev_s && jb + cl + c > prev_j)) ? vl[c] : 0xff800000u;
-                                    vh[c] = (fh < prev_s || (fh == prev_s && jb + ch + c > prev_j)) ? vh[c] : 0xff800000u;
-                                }
                             }
                         }
                         if (two) {
@@ -797,14 +769,12 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                         for (int b = 0; b < half; ++b) scan(b * 32, (b + half) * 32, b + half < nblk);
                         fast = drain();
                     } else {
-                        // Long lists: no group maxima (a list of k needs more groups than registers hold); the columns are
+                        // Lists of 17 to 32: no group maxima (a list of k needs more groups than registers hold); the columns are
                         // scanned against the list's own k-th score, which rises as they go: after n columns about k / n of
-                        // the next ones survive.  64 columns at a time, with a 64-entry queue from the start; with the
-                        // shorter queue of the 32-entry lists the first 32 columns are sorted by a network and are the
-                        // list, and the next ones go 32 at a time, which always fit, until 4 k have been seen.  (Taken best
-                        // first, as pairs of blocks whose survivors do not fit still are, the first 64 columns cost two thirds of
-                        // the selection: up to k rounds of 350 instructions a block.  264k tokens, 30 picks of 1008
-                        // columns, 6 heads: 4.26 -> 3.25 ms.)
+                        // the next ones survive.  The first 32 columns are sorted by a network and are the list, and the next ones go 32 at a
+                        // time, which always fit, until 4 k have been seen, then 64.  (Taken best first, as pairs of blocks whose
+                        // survivors do not fit still are, the first 64 columns cost two thirds of the selection: up to k rounds of 350
+                        // instructions a block.)
                         int b0 = 0;
                         if constexpr (KMAX == 32) {
                             if (sb == 0) {
@@ -829,7 +799,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
 #pragma unroll 1
                         while (b0 < nblk) {
                             thr = fmaxf(kth, -FLT_MAX);
-                            const bool two = b0 + 1 < nblk && (KMAX == 64 || jb + b0 * 32 >= 4 * kp);
+                            const bool two = b0 + 1 < nblk && jb + b0 * 32 >= 4 * kp;
                             scan(b0 * 32, (b0 + 1) * 32, two);
                             if (!drain()) extract_blocks(b0 * 32, min(rows_sb, (b0 + 1 + two) * 32));
                             b0 += 1 + two;
@@ -843,16 +813,11 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
             }
             if (!ok) break;
             fetch_cand(live2);
-            if (KMAX == 64) {                           // the next pass starts after this pass's last pick
-#pragma unroll
-                for (int x = 0; x < KR; ++x)
-                    if (x == kp - 1) { prev_s = top.s[x]; prev_j = top.j[x]; }
-            }
             // columns -> chunks; sel_idx and the empty slots' partial log-sum-exp
 #pragma unroll
             for (int x = 0; x < KR; ++x) top.j[x] = top.j[x] >= 0 ? s_col[top.j[x]] : -1;
-            int32_t *out = p.sel + ((size_t)h * p.L + i) * p.k + pass * 64;
-            float *pl = p.part_lse + part_lse_at(h, (p.L + 127) >> 7, p.k, i, pass * 64);     // slot x: pl[x * 128]
+            int32_t *out = p.sel + ((size_t)h * p.L + i) * p.k;
+            float *pl = p.part_lse + part_lse_at(h, (p.L + 127) >> 7, p.k, i, 0);     // slot x: pl[x * 128]
             if (live) {
 #pragma unroll
                 for (int x = 0; x < KR; ++x)
@@ -918,13 +883,12 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                     for (int x = 0; x < KR; ++x)
                         if (pend.j[x] >= 0) {
                             const size_t at = (size_t)s_cap[pend.j[x]] + hist[pend.j[x]] + pend.rank[x];
-                            if (index_ok(at < p.cap_total, p.status, IX_APPEND_POSITION)) list[at] = i * p.k + pass * 64 + x;
+                            if (index_ok(at < p.cap_total, p.status, IX_APPEND_POSITION)) list[at] = i * p.k + x;
                         }
                 }
                 ok = group_sync();
                 if (!ok) break;
             }
-            }   // pass
         }
         if (ok && pend.open) {                 // the last unit's entries
             write_bases();
@@ -934,40 +898,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, 512);
-    // The last block to get here turns the pick counts into the running counts of attention tiles over the (head,
-    // chunk) pairs and marks the workspace (what route_tiles_kernel does on the paths that have no such block): one
-    // launch less.  Every block's counts are in place before it arrives (the atomics that made them have
-    // returned), and the fence orders them before the arrival.
-    __shared__ int s_last, s_wsum[32];
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(&p.status[ST_ARRIVE], 1) == (int)gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    const int HC = p.H * p.C, T = kRtThreads, t = threadIdx.x;
-    const int per = (HC + T - 1) / T, i0 = min(t * per, HC), i1 = min(i0 + per, HC);
-    int mine = 0;
-    for (int i = i0; i < i1; ++i) mine += (__ldcg(p.cnt + i) + kQTileRows - 1) / kQTileRows;
-    int incl = mine;                                     // inclusive scan over the block: warps by shuffles, then warp totals
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int up = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += up;
-    }
-    if (lane == 31) s_wsum[warp] = incl;
-    __syncthreads();
-    int at = incl - mine;
-    for (int w = 0; w < warp; ++w) at += s_wsum[w];
-    for (int i = i0; i < i1; ++i) {
-        p.tile_off[i] = at;
-        at += (__ldcg(p.cnt + i) + kQTileRows - 1) / kQTileRows;
-    }
-    if (t == T - 1) {
-        p.tile_off[HC] = at;
-        p.status[ST_COOKIE] = (int)p.cookie;
-    }
+    finish_route(p.status, p.cnt, p.tile_off, p.H * p.C, p.cookie, kRtThreads);
 }
 
 // gtile[i] = attention tiles (of kQTileRows picks) before (head, chunk) pair i, with a final total;
@@ -1162,6 +1093,10 @@ static int launch_route_d(const moc_plan *p, const __nv_bfloat16 *Q, const float
         route_prep_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(desc, desc3, cnt, status, p->d_col_chunk, p->H, p->C, p->ncol, p->c_pad, D, p->wait_us);
         MOC_LAUNCH_CHECK();
     }
+    if (route_is_long(p)) {
+        if (int r = launch_route_long(p, Q, desc3, sel, ws, s)) return r;
+        return finish_lists(p, ws, s, false);       // the routing kernel's last block has counted the tiles
+    }
     if (p->k > 0) {
         RouteParams a;
         a.desc = fused_prep ? desc : nullptr; a.wait_us = p->wait_us;
@@ -1182,11 +1117,9 @@ static int launch_route_d(const moc_plan *p, const __nv_bfloat16 *Q, const float
         const size_t q_tile = (size_t)kRtRows * D * 2, d_block = ((size_t)3 * a.d_rows * D * 2 + 1023) & ~(size_t)1023;
         a.ctas_per_head = std::max(1, std::min(p->n_sm / p->H, a.tiles_per_head));
         const unsigned grid = (unsigned)(p->H * a.ctas_per_head);
-        // Four selection groups with few chunks (more warps to hide the selection's latencies); one when the
-        // 64-entry list takes nearly all of a thread's registers; two otherwise.
-        const int ng = few ? 4 : p->k > 32 ? 1 : 2;
-        a.n_pass = p->k > 64 ? (p->k + 63) / 64 : 1;
-        // one histogram per group, the list offsets, and one byte per unit of a CTA
+        // Four selection groups with few chunks (more warps to hide the selection's latencies), two otherwise.
+        const int ng = few ? 4 : 2;
+                // one histogram per group, the list offsets, and one byte per unit of a CTA
         const size_t hist = (ng * (p->k <= 8 && p->C <= kRtDeferredChunks ? 4 : 1) + 1) * sizeof(int) * (size_t)p->C + sizeof(int) * (size_t)p->ncol +
                             4 * (size_t)(a.tiles_per_head / a.ctas_per_head + 16),
                      budget = 227 * 1024 - 1024 - 512;      // what an SM has, less the alignment slack and the kernel's static variables
@@ -1197,8 +1130,8 @@ static int launch_route_d(const moc_plan *p, const __nv_bfloat16 *Q, const float
         size_t surv = 0;
         if (!few && budget > d_block + hist + 2 * q_tile + 16) {
             const size_t room = budget - d_block - hist - 2 * q_tile - 16, per_slot = (size_t)ng * 160 * sizeof(float);
-            // short lists: one scan per scoring step, a few more than k survive; long lists: 64 columns at a time,
-            // all of which survive at first
+            // up to 16 picks: one scan per scoring step, a few more than k survive; beyond: up to 64 columns at a time, all of which
+            // may survive
             const int want = p->k <= 16 ? std::max(12, 2 * p->k + 12) : 64, need = p->k <= 16 ? p->k + 4 : 32;
             const int have = (int)std::min<size_t>(room / per_slot, 255);
             if (have >= need) a.surv_cap = std::min(want, have);
@@ -1221,8 +1154,7 @@ static int launch_route_d(const moc_plan *p, const __nv_bfloat16 *Q, const float
         else if (p->k <= 6 && !few) MOC_ROUTE_CASE(6, 2, false);
         else if (p->k <= 8) { if (few) MOC_ROUTE_CASE(8, 4, true); else MOC_ROUTE_CASE(8, 2, false); }
         else if (p->k <= 16) MOC_ROUTE_CASE(16, 2, false);
-        else if (p->k <= 32) MOC_ROUTE_CASE(32, 2, false);
-        else MOC_ROUTE_CASE(64, 1, false);                 // beyond 64 picks: several passes of 64
+        else MOC_ROUTE_CASE(32, 2, false);
 #undef MOC_ROUTE_CASE
         MOC_LAUNCH_CHECK();
         return finish_lists(p, ws, s, false);       // the routing kernel's last block has counted the tiles

@@ -1,0 +1,97 @@
+"""Routing with many picks per query (csrc/moc_route_long.cu): the picks against the oracle at the edges of its sizes, and where counting
+by a threshold is hard: equal scores, chunks that repeat, rows with few candidates, scores that are not normally distributed."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import Oracle
+from paper_2508_21058_b200 import workloads as W
+
+import parity_utils as PU
+
+pytestmark = pytest.mark.gpu
+
+
+def ragged(heads, d, n_chunks, size, k, captions=(0,), shots=1, causal=True, window=(0, 0)):
+    sizes = np.full(n_chunks, size)
+    sizes[::3] += 1
+    lay = W.Layout(np.concatenate([[0], np.cumsum(sizes)]).astype(np.int32), (np.arange(n_chunks) * shots // n_chunks).astype(np.int32),
+                   np.isin(np.arange(n_chunks), captions).astype(np.uint8))
+    return W.Workload("many picks", heads, d, lay, k, *window, causal=causal)
+
+
+def routed(wl, spoil=None):
+    run = PU.GpuRun(wl)
+    if spoil:
+        spoil(run.x)
+    run.forward()
+    return run
+
+
+def check(run):
+    wl = run.wl
+    orc = Oracle.from_workload(wl)
+    h = run.host_inputs()
+    sel = run.sel.cpu().numpy()
+    PU.assert_routing(wl, orc, h["q"], orc.chunk_pool(h["k"]), sel)
+    # the lists hold every pick once: the selection's pairs, as the counts in the workspace have them, are those of sel_idx
+    size = np.diff(wl.layout.chunk_off).astype(np.int64)
+    assert run.plan.moc_selected_pairs(run.ws) == anchor_pairs(wl) + int(size[sel[sel >= 0]].sum())
+
+
+def anchor_pairs(wl):
+    """Anchor pairs, by the rule."""
+    lay = wl.layout
+    size, text, shot, idx = np.diff(lay.chunk_off).astype(np.int64), lay.chunk_mod == 1, lay.chunk_shot, np.arange(lay.n_chunks)
+    back, fwd = (lay.n_chunks if w == W.WHOLE_SHOT else w for w in (wl.win_back, wl.win_fwd))
+    return wl.n_heads * sum(int(size[c]) * int(size[text | ((shot == shot[c]) & (idx >= c - back) & (idx <= c + fwd))].sum()) for c in range(lay.n_chunks))
+
+
+@pytest.mark.parametrize("k", [17, 24, 25, 56, 57, 64, 120, 121, 128, 240, 241, 512])
+def test_every_length_of_list(k):
+    check(routed(ragged(1, 64 if k % 2 else 128, 300 if k <= 240 else 600, 5, k)))
+
+
+@pytest.mark.parametrize("n_chunks,k", [(18, 33), (34, 40), (50, 40), (130, 64), (131, 64), (146, 20), (147, 20), (514, 20), (515, 30), (1026, 20), (1500, 24)])
+def test_every_number_of_columns(n_chunks, k):
+    check(routed(ragged(2, 64, n_chunks, 3, k, captions=(0, n_chunks // 2))))
+
+
+@pytest.mark.parametrize("wl", [ragged(2, 128, 90, 17, 33, causal=False), ragged(1, 64, 1100, 3, 40, causal=False, shots=5, window=(1, 1)),
+                                ragged(3, 128, 140, 20, 18, shots=7, window=(2, 0)), ragged(1, 128, 200, 9, 130, shots=4, window=(W.WHOLE_SHOT, W.WHOLE_SHOT))],
+                         ids=["not causal", "not causal, 1100 chunks", "window behind", "whole shots"])
+def test_candidates_that_are_not_a_prefix_or_few(wl):
+    check(routed(wl))
+
+
+@pytest.mark.parametrize("k,n_chunks", [(20, 200), (100, 300), (40, 1200)])
+def test_equal_scores_go_to_the_earlier_chunk(k, n_chunks):
+    """All scores equal: the first candidates, whatever the threshold."""
+    run = routed(ragged(1, 64, n_chunks, 4, k), lambda x: x["q"].zero_())
+    sel, tc = run.sel.cpu().numpy()[0], run.wl.layout.token_chunk()
+    for i in range(0, len(sel), 7):
+        n = min(k, max(0, int(tc[i]) - 1))                     # (chunk 0 is a caption, the row's own chunk an anchor)
+        assert np.array_equal(sel[i], np.concatenate([np.arange(1, n + 1), np.full(k - n, -1)]))
+
+
+def test_groups_of_equal_chunks():
+    """Keys that repeat every six chunks: scores in groups of fifty equal ones, of which some are taken."""
+    def repeat(x):
+        off = 0
+        for c, n in enumerate(np.diff(wl.layout.chunk_off)):
+            x["k"][:, off:off + n] = (0.25 * base[c % 6])[:, None]
+            off += n
+    wl = ragged(1, 128, 301, 4, 60)
+    base = torch.randint(-3, 4, (6, 1, 128), device="cuda").to(torch.bfloat16)
+    run = routed(wl, repeat)
+    check(run)
+
+
+def test_scores_far_from_normal():
+    """Scores of nine magnitudes, from a sixty-fourth to four times the usual."""
+    def spread(x):
+        off = np.asarray(wl.layout.chunk_off)
+        for c in range(wl.n_chunks):
+            x["k"][:, off[c]:off[c + 1]] *= 2.0 ** (2 - 7 * c % 9)
+    wl = ragged(1, 128, 400, 4, 70)
+    check(routed(wl, spread))
