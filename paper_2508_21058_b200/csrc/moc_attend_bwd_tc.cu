@@ -51,6 +51,7 @@ struct BwdParams {
     int H, L, C, k;
     SlotDiv kdiv;
     float scale, scale_log2;
+    WaitBound wait;
 };
 
 constexpr int kY1Stages = 3, kY2Stages = 2;   // stages of the streamed tiles Y1 (read twice per tile) and Y2
@@ -170,8 +171,8 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
         int s3 = 0, ph3 = 0;                          // Y1 stage of tile jt and its phase
         for (int jt = 0; jt < n_tiles; ++jt) {
             const int st = jt & 1;
-            ok = mbar_wait_spin(bar(T1_FULL + st), (jt >> 1) & 1, abort_flag, p.status, BW_T1FULL);
-            ok = ok && mbar_wait(bar(Y1_FULL + s3), ph3, abort_flag, p.status, BW_YFULL);
+            ok = mbar_wait_spin(bar(T1_FULL + st), (jt >> 1) & 1, abort_flag, p.wait, BW_T1FULL);
+            ok = ok && mbar_wait(bar(Y1_FULL + s3), ph3, abort_flag, p.wait, BW_YFULL);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
@@ -207,7 +208,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
 #pragma unroll
                     for (int x = 0; x < 16; ++x) ups[x] = bf16x2(pv[rd * 32 + 2 * x], pv[rd * 32 + 2 * x + 1]);
                     if (rd == 0) {
-                        ok = mbar_wait_spin(bar(RD1), jt & 1, abort_flag, p.status, BW_READ);
+                        ok = mbar_wait_spin(bar(RD1), jt & 1, abort_flag, p.wait, BW_READ);
                         ok = __all_sync(0xffffffffu, ok);
                     }
                     if (ok) {
@@ -220,7 +221,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             }
             if (!ok) break;
             // ---- dS = P (dP - delta) from T2, written over T2 columns that have been read
-            ok = mbar_wait_spin(bar(T2_FULL + st), (jt >> 1) & 1, abort_flag, p.status, BW_T2FULL);
+            ok = mbar_wait_spin(bar(T2_FULL + st), (jt >> 1) & 1, abort_flag, p.wait, BW_T2FULL);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
@@ -247,7 +248,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                     }
                 }
                 if (rd == 0) {
-                    ok = mbar_wait_spin(bar(RD2), jt & 1, abort_flag, p.status, BW_READ);
+                    ok = mbar_wait_spin(bar(RD2), jt & 1, abort_flag, p.wait, BW_READ);
                     ok = __all_sync(0xffffffffu, ok);
                 }
                 if (ok) tmem_st16(tmem + lane_off + t2c + ch * 16, uds);
@@ -260,7 +261,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
         }
         // ---- epilogue
         if (ok) {
-            ok = mbar_wait(bar(ACC_FULL), 0, abort_flag, p.status, BW_ACCFULL);
+            ok = mbar_wait(bar(ACC_FULL), 0, abort_flag, p.wait, BW_ACCFULL);
             ok = __all_sync(0xffffffffu, ok);
         }
         if (ok) {
@@ -316,14 +317,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                 }
                 // (the lane threads' own two barriers, once more: every wait here is bounded)
                 mbar_arrive(bar(RD1));
-                ok = mbar_wait_spin(bar(RD1), n_tiles & 1, abort_flag, p.status, BW_READ);
+                ok = mbar_wait_spin(bar(RD1), n_tiles & 1, abort_flag, p.wait, BW_READ);
                 if (threadIdx.x == 0 && ok) {
                     __threadfence();
                     s_last = atomicAdd(p.split_done + slot, 1) == parts - 1;
                     __threadfence();
                 }
                 mbar_arrive(bar(RD2));
-                ok = ok && mbar_wait_spin(bar(RD2), n_tiles & 1, abort_flag, p.status, BW_READ);
+                ok = ok && mbar_wait_spin(bar(RD2), n_tiles & 1, abort_flag, p.wait, BW_READ);
                 ok = __all_sync(0xffffffffu, ok);
                 if (ok && s_last) {
 #pragma unroll 1
@@ -448,7 +449,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             const int t_whole = whole, t_q[2] = {q[0], q[1]};
             const float t_lse[2] = {q_lse[0], q_lse[1]}, t_del[2] = {q_del[0], q_del[1]};
             if (jt + 1 < n_tiles) next_rows();
-            ok = mbar_wait(bar(b_empty + st), ph ^ 1, abort_flag, p.status, BW_YEMPTY);
+            ok = mbar_wait(bar(b_empty + st), ph ^ 1, abort_flag, p.wait, BW_YEMPTY);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             const uint32_t dst = ring + st * TILE_BYTES;
@@ -472,7 +473,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             ++issued;
             if (y1) {
                 // the lanes have finished with the lse / delta of tile jt - 2
-                if (jt >= 2) ok = mbar_wait(bar(DS_DONE + (jt & 1)), ((jt - 2) >> 1) & 1, abort_flag, p.status, BW_DSDONE);
+                if (jt >= 2) ok = mbar_wait(bar(DS_DONE + (jt & 1)), ((jt - 2) >> 1) & 1, abort_flag, p.wait, BW_DSDONE);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
 #pragma unroll
@@ -497,7 +498,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             cp_async_wait_all();
             int dummy_flag = 0;
             for (int b = 1; b <= n_st; ++b)
-                if (issued - b >= 0) mbar_wait(bar(b_full + (issued - b) % n_st), ((issued - b) / n_st) & 1, &dummy_flag, p.status, BW_YFULL);
+                if (issued - b >= 0) mbar_wait(bar(b_full + (issued - b) % n_st), ((issued - b) / n_st) & 1, &dummy_flag, p.wait, BW_YFULL);
         }
     } else {
         // ------------------------------------------------------------ MMA issuers: warp 12 owns the T1 / P side
@@ -519,7 +520,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             auto lo = [](uint64_t d) { return (uint32_t)d; };
             auto hi = [](uint64_t d) { return (uint32_t)(d >> 32); };
             bool ok = true;
-            auto wait = [&](int b, int parity, int code) { ok = ok && __all_sync(0xffffffffu, mbar_wait_spin(bar(b), parity, abort_flag, p.status, code)); };
+            auto wait = [&](int b, int parity, int code) { ok = ok && __all_sync(0xffffffffu, mbar_wait_spin(bar(b), parity, abort_flag, p.wait, code)); };
             // the MMA groups, without their waits and commits
             // (s3 = j mod the Y1 stage count is carried along by the callers: no division on this warp)
             auto t1 = [&](int j, int s3) {  // T1(j) = X1 Y1(j)^T
@@ -624,6 +625,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
     tc_fence_before();
     __syncthreads();
     if (warp == 8) tmem_dealloc(tmem, 512);
+    if (threadIdx.x == 0) report_abort(p.status, s_abort);
     if (blockIdx.x == gridDim.x - 1) previous_done();    // nothing here depends on dQ's launches, but what follows may
 }
 
@@ -643,6 +645,7 @@ static int attend_bwd_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv
     BwdParams a;
     a.Q = Q; a.K = K; a.V = V; a.dO = dO; a.lse = lse; a.delta = delta;
     a.cookie = p->cookie;
+    a.wait = WaitBound::of(p->wait_us);
     a.dK = dK; a.dV = dV;
     a.ktiles = p->d_ktiles; a.n_ktiles = (int)p->ktiles.size(); a.n_long = p->n_long_ktiles;
     a.n_split = n_split; a.split_sum = ws_ptr<float4>(ws, p->ws.part_o); a.split_done = split_done;

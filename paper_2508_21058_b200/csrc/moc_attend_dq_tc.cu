@@ -51,6 +51,7 @@ struct DqParams {
     SlotDiv kdiv;
     float scale, scale_log2;
     uint32_t cookie;
+    WaitBound wait;
 };
 
 constexpr int kDqThreads = 512, kKStages = 3, kVStages = 2, kLoaders = 3;
@@ -175,7 +176,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
         int g = 0;                                    // tiles processed
         bool ok = true;
         for (int n = 0; ok; ++n) {
-            ok = mbar_wait(bar(X_FULL), n & 1, abort_flag, p.status, DW_XFULL);
+            ok = mbar_wait(bar(X_FULL), n & 1, abort_flag, p.wait, DW_XFULL);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             const int rows = s_item[n & 1].rows, h = s_item[n & 1].h, first = s_item[n & 1].first, n_tiles = s_item[n & 1].ntiles;
@@ -211,7 +212,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
             int valid, t0;
             // P of the tile
             auto form_p = [&]() __attribute__((always_inline)) -> bool {
-                ok = mbar_wait_spin(bar(T1_FULL), g & 1, abort_flag, p.status, DW_T1FULL);
+                ok = mbar_wait_spin(bar(T1_FULL), g & 1, abort_flag, p.wait, DW_T1FULL);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) return false;
                 tc_fence_after();
@@ -232,7 +233,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
             auto form_ds = [&]() __attribute__((always_inline)) -> bool {
                 const int st = g & 1;
                 const uint32_t t2 = tmem + lane_off + (st ? 384u : 128u);
-                ok = mbar_wait_spin(bar(T2_FULL + st), (g >> 1) & 1, abort_flag, p.status, DW_T2FULL);
+                ok = mbar_wait_spin(bar(T2_FULL + st), (g >> 1) & 1, abort_flag, p.wait, DW_T2FULL);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) return false;
                 tc_fence_after();
@@ -265,7 +266,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
             }
             if (!ok || !form_ds()) break;
             // ---- epilogue
-            ok = mbar_wait(bar(ACC_FULL), n & 1, abort_flag, p.status, DW_ACCFULL);
+            ok = mbar_wait(bar(ACC_FULL), n & 1, abort_flag, p.wait, DW_ACCFULL);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
@@ -389,14 +390,14 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
                 int t0, valid;
                 while (it.next(t0, valid)) {
                     const int s2 = n_v & 1;
-                    ok = mbar_wait(bar(K_EMPTY + s3), ph3 ^ 1, abort_flag, p.status, DW_YEMPTY);
+                    ok = mbar_wait(bar(K_EMPTY + s3), ph3 ^ 1, abort_flag, p.wait, DW_YEMPTY);
                     if (!ok) break;
                     mbar_expect_tx(bar(K_FULL + s3), TILE_BYTES);
 #pragma unroll
                     for (int sub = 0; sub < SUB; ++sub)
                         tma_load_2d(sK + s3 * TILE_BYTES + sub * SUB_BYTES, &tmK, sub * 64, w.h * p.L + t0, bar(K_FULL + s3));
                     ++n_k;
-                    ok = mbar_wait(bar(V_EMPTY + s2), ((n_v >> 1) & 1) ^ 1, abort_flag, p.status, DW_YEMPTY);
+                    ok = mbar_wait(bar(V_EMPTY + s2), ((n_v >> 1) & 1) ^ 1, abort_flag, p.wait, DW_YEMPTY);
                     if (!ok) break;
                     mbar_expect_tx(bar(V_FULL + s2), TILE_BYTES);
 #pragma unroll
@@ -409,9 +410,9 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
             if (*abort_flag) {      // copies already issued must land before the shared memory is released
                 int dummy_flag = 0;
                 for (int b = 1; b <= kKStages; ++b)
-                    if (n_k - b >= 0) mbar_wait(bar(K_FULL + (n_k - b) % kKStages), ((n_k - b) / kKStages) & 1, &dummy_flag, p.status, DW_YFULL);
+                    if (n_k - b >= 0) mbar_wait(bar(K_FULL + (n_k - b) % kKStages), ((n_k - b) / kKStages) & 1, &dummy_flag, p.wait, DW_YFULL);
                 for (int b = 1; b <= kVStages; ++b)
-                    if (n_v - b >= 0) mbar_wait(bar(V_FULL + ((n_v - b) & 1)), ((n_v - b) >> 1) & 1, &dummy_flag, p.status, DW_YFULL);
+                    if (n_v - b >= 0) mbar_wait(bar(V_FULL + ((n_v - b) & 1)), ((n_v - b) >> 1) & 1, &dummy_flag, p.wait, DW_YFULL);
             }
         }
     } else if (warp < 12) {
@@ -446,7 +447,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
                 }
             }
             if (n > 0) {
-                ok = mbar_wait(bar(X_EMPTY), (n - 1) & 1, abort_flag, p.status, DW_XEMPTY);
+                ok = mbar_wait(bar(X_EMPTY), (n - 1) & 1, abort_flag, p.wait, DW_XEMPTY);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
             }
@@ -488,7 +489,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
             auto lo = [](uint64_t d) { return (uint32_t)d; };
             auto hi = [](uint64_t d) { return (uint32_t)(d >> 32); };
             bool ok = true;
-            auto wait = [&](int b, int parity, int code) { ok = ok && __all_sync(0xffffffffu, mbar_wait_spin(bar(b), parity, abort_flag, p.status, code)); };
+            auto wait = [&](int b, int parity, int code) { ok = ok && __all_sync(0xffffffffu, mbar_wait_spin(bar(b), parity, abort_flag, p.wait, code)); };
             int g = 0, s3 = 0, ph3 = 0;                        // tile, its K stage and phase
             if (uniform(warp) == 12) {
                 const uint64_t x1 = smem_desc_sw128(sX, 16, 1024), kk = smem_desc_sw128(sK, 16, 1024);
@@ -559,6 +560,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
     tc_fence_before();
     __syncthreads();
     if (warp == 8) tmem_dealloc(tmem, 512);
+    if (threadIdx.x == 0) report_abort(p.status, s_abort);
     if (ANCHOR && blockIdx.x == 0) previous_done();      // an abandoned launch has not waited yet
 }
 
@@ -579,6 +581,7 @@ static int dq_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfloat1
     a.n_items = (int)p->qitems.size();
     a.scale = p->scale; a.scale_log2 = p->scale * 1.4426950408889634f;
     a.cookie = p->cookie;
+    a.wait = WaitBound::of(p->wait_us);
     // seven tiles (Q, dO, three K and two V stages; always the d = 128 footprint, so that CTAs, which each take all of the
     // tensor memory, never share an SM): all an SM has, so the request is what the static variables leave of the limit
     const size_t tiles = (size_t)(2 + kKStages + kVStages) * 128 * 128 * 2;

@@ -67,6 +67,7 @@ struct AttendParams {
     SlotDiv kdiv;
     float scale_log2;           // softmax scale * log2(e)
     uint32_t cookie;
+    WaitBound wait;
 };
 
 constexpr int kBN = 128;               // keys per tile
@@ -97,22 +98,13 @@ struct SlotIter {
     }
 };
 
-// a bounded wait on a counter in global memory (another CTA adds to it)
-__device__ __forceinline__ bool wait_count(const int *ctr, int need, volatile int *abort_flag, int *status, int code) {
-    if (*(volatile const int *)ctr >= need) return true;
-    const uint64_t t0 = global_timer_ns();
-    for (uint32_t it = 1;; ++it) {
-        if (*(volatile const int *)ctr >= need) return true;
+// a bounded wait on a counter in global memory (another CTA adds to it); a look takes half a microsecond or more
+__device__ __forceinline__ bool wait_count(const int *ctr, int need, volatile int *abort_flag, const WaitBound &bound, int code) {
+    for (uint32_t it = 0; *(volatile const int *)ctr < need;) {
         __nanosleep(200);
-        if ((it & 0x3f) == 0) {
-            if (*abort_flag) return false;
-            if (global_timer_ns() - t0 > wait_limit_ns(status)) {
-                *abort_flag = 1;
-                if (atomicCAS(status, 0, MOC_ERR_TIMEOUT) == 0) status[ST_DETAIL] = code;
-                return false;
-            }
-        }
+        if (++it > 2 * bound.us) return gave_up(abort_flag, code);
     }
+    return true;
 }
 
 // acc += w x (the bf16 pair u) where cond holds
@@ -209,7 +201,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
         if (D != 128 || kMergeInRegs) return true;
         bool done = true;
         if ((used >> qb) & 1) {
-            done = mbar_wait(bar(MERGED + qb), (phase >> qb) & 1, abort_flag, p.status, W_MERGE);
+            done = mbar_wait(bar(MERGED + qb), (phase >> qb) & 1, abort_flag, p.wait, W_MERGE);
             phase ^= 1u << qb;
         }
         used = (used & ~(1u << qb)) | ((uint32_t)(merges && p.k > 0) << qb);
@@ -235,7 +227,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
         bool ok = true;
         while (ok) {
             const int sl = n_item % kItemSlots;
-            ok = mbar_wait(bar(ITEM_FULL + sl), (n_item / kItemSlots) & 1, abort_flag, p.status, W_ITEMFULL);
+            ok = mbar_wait(bar(ITEM_FULL + sl), (n_item / kItemSlots) & 1, abort_flag, p.wait, W_ITEMFULL);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             const ItemSlot it_ = s_item[sl];
@@ -252,7 +244,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             if (dep) bits ^= DEP_ODD;
             if (g == 1 && !two) {                       // this item has one query tile
                 if (dep) {                              // ... and every thread sees every phase of DEPEND
-                    ok = mbar_wait(bar(DEPEND), dep_phase, abort_flag, p.status, W_DEPEND);
+                    ok = mbar_wait(bar(DEPEND), dep_phase, abort_flag, p.wait, W_DEPEND);
                     ok = __all_sync(0xffffffffu, ok);
                     const int b = ROWS_DONE + 2 * ((n_item - 1) & 3) + 1;
                     mbar_arrive(bar(b));
@@ -286,7 +278,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             TileIter it(it_.rng, it_.nrng);
             int t0, valid, jt = 0;
             while (it.next(t0, valid)) {
-                ok = mbar_wait(bar(S_FULL + g), bits & S_ODD, abort_flag, p.status, W_SFULL);
+                ok = mbar_wait(bar(S_FULL + g), bits & S_ODD, abort_flag, p.wait, W_SFULL);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
@@ -325,7 +317,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 // tile 1's previous turn even at the start of an item: the barrier must never get two phases ahead of
                 // a group that has yet to wait on it.)
                 if (two && (g == 1 || (bits & TURNED))) {
-                    ok = mbar_wait(bar(TURN + (g ^ 1)), ((bits & TURN_ODD) ? 1 : 0) ^ (g == 1 ? 0 : 1), abort_flag, p.status, W_TURN);
+                    ok = mbar_wait(bar(TURN + (g ^ 1)), ((bits & TURN_ODD) ? 1 : 0) ^ (g == 1 ? 0 : 1), abort_flag, p.wait, W_TURN);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                 }
@@ -405,7 +397,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             // a routed item: the anchor items two groups back have read the buffer it is about to store into) has been
             // awaited by the bookkeeping lane, which then arrives on DEPEND, once per phase of the queue
             if (dep) {
-                ok = mbar_wait(bar(DEPEND), dep_phase, abort_flag, p.status, W_DEPEND);
+                ok = mbar_wait(bar(DEPEND), dep_phase, abort_flag, p.wait, W_DEPEND);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
             }
@@ -421,7 +413,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                         p.part_lse[part_lse_at(h, LB, p.k, q, slot)] = lse_own;
                     }
                 }
-                ok = mbar_wait(bar(O_FULL + g), (bits & MINE_ODD) ? 1 : 0, abort_flag, p.status, W_OFULL);
+                ok = mbar_wait(bar(O_FULL + g), (bits & MINE_ODD) ? 1 : 0, abort_flag, p.wait, W_OFULL);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc_fence_after();
@@ -609,7 +601,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                     };
                     Batch even = {}, odd = {};
                     ask(even);
-                    ok = mbar_wait(bar(O_FULL + g), (bits & MINE_ODD) ? 1 : 0, abort_flag, p.status, W_OFULL);
+                    ok = mbar_wait(bar(O_FULL + g), (bits & MINE_ODD) ? 1 : 0, abort_flag, p.wait, W_OFULL);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     tc_fence_after();
@@ -623,7 +615,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                         if (pass == n_pass) break;
                     }
                 } else {
-                    ok = mbar_wait(bar(O_FULL + g), (bits & MINE_ODD) ? 1 : 0, abort_flag, p.status, W_OFULL);
+                    ok = mbar_wait(bar(O_FULL + g), (bits & MINE_ODD) ? 1 : 0, abort_flag, p.wait, W_OFULL);
                     ok = __all_sync(0xffffffffu, ok);
                     tc_fence_after();
                     float ls1 = merge ? __ldcg(pl) : -INFINITY, ls2 = merge ? __ldcg(pl + min(1, p.k - 1) * 128) : -INFINITY;      // the next two slots'
@@ -652,7 +644,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                             ls1 = ls2;
                             const int s2 = s + 2 < n_slots ? s + 2 : s + 2 - n_slots;       // (the next block's first slots after the last)
                             ls2 = merge ? __ldcg(pl + min(s2, p.k - 1) * 128) : -INFINITY;
-                            ok = mbar_wait(bar(MERGE + warp * kMergeStages + m_st), (bits >> (MERGE_AT + m_st)) & 1, abort_flag, p.status, W_MERGE);
+                            ok = mbar_wait(bar(MERGE + warp * kMergeStages + m_st), (bits >> (MERGE_AT + m_st)) & 1, abort_flag, p.wait, W_MERGE);
                             ok = __all_sync(0xffffffffu, ok);
                             if (!ok) break;
                             const uint32_t src = m_base + m_st * 4096 + lane * 128;
@@ -689,7 +681,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                     if (!ok) {       // copies under way must land before the shared memory is released
                         int dummy_flag = 0;
                         for (; m_flight > 0; --m_flight) {
-                            mbar_wait(bar(MERGE + warp * kMergeStages + m_st), (bits >> (MERGE_AT + m_st)) & 1, &dummy_flag, p.status, W_MERGE);
+                            mbar_wait(bar(MERGE + warp * kMergeStages + m_st), (bits >> (MERGE_AT + m_st)) & 1, &dummy_flag, p.wait, W_MERGE);
                             bits ^= 1u << (MERGE_AT + m_st);
                             if (++m_st == kMergeStages) m_st = 0;
                         }
@@ -718,7 +710,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             int k_last = -1, v_last = -1;                     // last tile whose K / V copy was issued
             bool ok = true;
             while (ok) {
-                if (!mbar_wait(bar(ITEM_FULL + slot_it.at), slot_it.phase, abort_flag, p.status, W_ITEMFULL)) break;
+                if (!mbar_wait(bar(ITEM_FULL + slot_it.at), slot_it.phase, abort_flag, p.wait, W_ITEMFULL)) break;
                 const ItemSlot it_ = s_item[slot_it.at];
                 mbar_arrive(bar(ITEM_EMPTY + slot_it.at));
                 slot_it.next();
@@ -730,13 +722,13 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 while (it.next(t0, valid)) {
                     const int st = n_kv & 1;
                     const uint32_t ph = (n_kv >> 1) & 1;
-                    if (!mbar_wait(bar(K_EMPTY + st), ph ^ 1, abort_flag, p.status, W_KEMPTY)) { ok = false; break; }
+                    if (!mbar_wait(bar(K_EMPTY + st), ph ^ 1, abort_flag, p.wait, W_KEMPTY)) { ok = false; break; }
                     mbar_expect_tx(bar(K_FULL + st), TILE_BYTES);
 #pragma unroll
                     for (int sub = 0; sub < SUB; ++sub)
                         tma_load_2d(sK + st * TILE_BYTES + sub * SUB_BYTES, &tmK, sub * 64, h * p.L + t0, bar(K_FULL + st));
                     k_last = n_kv;
-                    if (!mbar_wait(bar(V_EMPTY + st), ph ^ 1, abort_flag, p.status, W_VEMPTY)) { ok = false; break; }
+                    if (!mbar_wait(bar(V_EMPTY + st), ph ^ 1, abort_flag, p.wait, W_VEMPTY)) { ok = false; break; }
                     mbar_expect_tx(bar(V_FULL + st), TILE_BYTES);
 #pragma unroll
                     for (int sub = 0; sub < SUB; ++sub)
@@ -750,8 +742,8 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 int dummy_flag = 0;
                 for (int b = 0; b < 2; ++b) {
                     const int kj = k_last - b, vj = v_last - b;
-                    if (kj >= 0) mbar_wait(bar(K_FULL + (kj & 1)), (kj >> 1) & 1, &dummy_flag, p.status, W_KFULL);
-                    if (vj >= 0) mbar_wait(bar(V_FULL + (vj & 1)), (vj >> 1) & 1, &dummy_flag, p.status, W_VFULL);
+                    if (kj >= 0) mbar_wait(bar(K_FULL + (kj & 1)), (kj >> 1) & 1, &dummy_flag, p.wait, W_KFULL);
+                    if (vj >= 0) mbar_wait(bar(V_FULL + (vj & 1)), (vj >> 1) & 1, &dummy_flag, p.wait, W_VFULL);
                 }
             }
         } else if (lane == 16) {
@@ -786,13 +778,13 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             bool ok = true;
             while (ok) {
                 const int sl = slot_it.at;
-                if (!mbar_wait(bar(ITEM_FULL + sl), slot_it.phase, abort_flag, p.status, W_ITEMFULL)) break;
+                if (!mbar_wait(bar(ITEM_FULL + sl), slot_it.phase, abort_flag, p.wait, W_ITEMFULL)) break;
                 const ItemSlot it_ = s_item[sl];
                 slot_it.next();
                 ++n_item;
                 for (int g = 0; ok && g < pend_tiles; ++g) {
                     const int b = 2 * ((n_item - 2) & 3) + g;          // the pending item is the one before this
-                    ok = mbar_wait(bar(ROWS_DONE + b), (rows_phase >> b) & 1, abort_flag, p.status, W_ROWSDONE);
+                    ok = mbar_wait(bar(ROWS_DONE + b), (rows_phase >> b) & 1, abort_flag, p.wait, W_ROWSDONE);
                     rows_phase ^= 1u << b;
                 }
                 if (!ok) break;
@@ -807,9 +799,9 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 if (!it_.valid || first || pend_n >= 4) count_rows();
                 if (!it_.valid) break;
                 if (dep_anchor)
-                    ok = wait_count(&phase_tab[3 * (2 * group) + 2], phase_tab[3 * (2 * group) + 1], abort_flag, p.status, W_DEPEND);
+                    ok = wait_count(&phase_tab[3 * (2 * group) + 2], phase_tab[3 * (2 * group) + 1], abort_flag, p.wait, W_DEPEND);
                 if (dep_routed)
-                    ok = wait_count(&phase_tab[3 * (2 * (group - 2) + 1) + 2], phase_tab[3 * (2 * (group - 2) + 1) + 1], abort_flag, p.status, W_DEPEND);
+                    ok = wait_count(&phase_tab[3 * (2 * (group - 2) + 1) + 2], phase_tab[3 * (2 * (group - 2) + 1) + 1], abort_flag, p.wait, W_DEPEND);
                 if (!ok) break;
                 if (dep_anchor || dep_routed) {
                     __threadfence();
@@ -866,8 +858,8 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             // the whole warp waits, and goes on or gives up together
             auto wait = [&](int b, uint32_t parity, int code) {
                 // (with the loaders' traffic on every scheduler a parked issuer wakes later still: it polls)
-                return __all_sync(0xffffffffu, LOADERS ? mbar_wait_spin(bar(b), parity, abort_flag, p.status, code)
-                                                       : mbar_wait(bar(b), parity, abort_flag, p.status, code)) != 0;
+                return __all_sync(0xffffffffu, LOADERS ? mbar_wait_spin(bar(b), parity, abort_flag, p.wait, code)
+                                                       : mbar_wait(bar(b), parity, abort_flag, p.wait, code)) != 0;
             };
             SlotIter slot_it;
             while (ok) {
@@ -972,22 +964,22 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             ItemSlot s;
             s.valid = 0; s.routed = 0; s.h = 0; s.first = 0; s.rows = 0; s.nrng = 0; s.ntiles = 0; s.phase = 0; s.qbuf = n_qtile % 3; s.rng = nullptr;
             if (lane == 0) {
-                if (n_item >= kItemSlots) ok = mbar_wait(bar(ITEM_EMPTY + sl), slot_it.phase ^ 1, abort_flag, p.status, W_ITEMEMPTY);
+                if (n_item >= kItemSlots) ok = mbar_wait(bar(ITEM_EMPTY + sl), slot_it.phase ^ 1, abort_flag, p.wait, W_ITEMEMPTY);
                 // Claimed early, an item's gathers are done before they are needed, but it is kept from a CTA that may be idle.
                 // After an anchor item (whose successors have plain tiles to load, and which end the queue), and when there
                 // are only a few items per CTA, the next one is claimed when the last S of this one has been issued.
                 const bool wait_for_s = n_qtile > 0 && (late || total <= 2 * (int)gridDim.x);
                 if (ok && wait_for_s && n_item >= 2) {       // every warp has seen the item before the last one
                     const bool wrap = sl + 1 == kItemSlots;
-                    ok = mbar_wait(bar(ITEM_EMPTY + (wrap ? 0 : sl + 1)), slot_it.phase ^ (wrap ? 0 : 1), abort_flag, p.status, W_ITEMEMPTY);
+                    ok = mbar_wait(bar(ITEM_EMPTY + (wrap ? 0 : sl + 1)), slot_it.phase ^ (wrap ? 0 : 1), abort_flag, p.wait, W_ITEMEMPTY);
                 }
                 if (ok && wait_for_s) {
                     const int qb = (n_qtile - 1) % 3, qf = 3 * last_g + qb;
                     // Where others load the tiles, the buffer's release before this one may be yet to come, and its phase would be
                     // taken for this one's.  It has come when the item's last tile is there.  (That barrier's own phase
                     // before was of an item that the softmax warps have left, and the next is of one not yet published.)
-                    if (LOADERS) ok = mbar_wait(bar(Q_FULL + qf), ((q_phase >> qf) & 1) ^ 1, abort_flag, p.status, W_QFULL);
-                    ok = ok && mbar_wait(bar(Q_EMPTY + qb), ((n_qtile - 1) / 3) & 1, abort_flag, p.status, W_QEMPTY);
+                    if (LOADERS) ok = mbar_wait(bar(Q_FULL + qf), ((q_phase >> qf) & 1) ^ 1, abort_flag, p.wait, W_QFULL);
+                    ok = ok && mbar_wait(bar(Q_EMPTY + qb), ((n_qtile - 1) / 3) & 1, abort_flag, p.wait, W_QEMPTY);
                 }
                 const int t = (ok && usable && !*abort_flag && *(volatile int *)p.status == 0) ? atomicAdd(&p.queue[0], 1) : total;
                 if (t < total) {
@@ -1031,7 +1023,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             }
             for (int g = 0; ok && g < n_qt; ++g) {
                 const int qb = n_qtile % 3, qf = 3 * g + qb;
-                ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.status, W_QEMPTY) && merged(qb, !routed, m_used, m_phase);
+                ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.wait, W_QEMPTY) && merged(qb, !routed, m_used, m_phase);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 if (lane == 0) mbar_expect_tx(bar(Q_FULL + qf), TILE_BYTES);
@@ -1068,7 +1060,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             // drain: the Q copies already issued must land before the CTA's shared memory is released
             int dummy_flag = 0;
             // (a barrier that was never used is past the phase before its first)
-            for (int b = 0; b < 6; ++b) mbar_wait(bar(Q_FULL + b), ((q_phase >> b) & 1) ^ 1, &dummy_flag, p.status, W_QFULL);
+            for (int b = 0; b < 6; ++b) mbar_wait(bar(Q_FULL + b), ((q_phase >> b) & 1) ^ 1, &dummy_flag, p.wait, W_QFULL);
         }
     } else {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLoad));
@@ -1083,7 +1075,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
         bool ok = true;
         while (ok) {
             const int sl = slot_it.at;
-            ok = mbar_wait(bar(ITEM_FULL + sl), slot_it.phase, abort_flag, p.status, W_ITEMFULL);
+            ok = mbar_wait(bar(ITEM_FULL + sl), slot_it.phase, abort_flag, p.wait, W_ITEMFULL);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             const int valid = s_item[sl].valid, routed = s_item[sl].routed, h = s_item[sl].h, first = s_item[sl].first, rows = s_item[sl].rows;
@@ -1109,7 +1101,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 int row[4];
 #pragma unroll
                 for (int x = 0; x < 4; ++x) row[x] = h * p.L + __shfl_sync(0xffffffffu, qrow[g], (lane & 7) * 4 + x);
-                ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.status, W_QEMPTY) && merged(qb, !routed, m_used, m_phase);
+                ok = mbar_wait(bar(Q_EMPTY + qb), ((n_qtile / 3) & 1) ^ 1, abort_flag, p.wait, W_QEMPTY) && merged(qb, !routed, m_used, m_phase);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 if (lw == 0 && lane == 0) mbar_expect_tx(bar(Q_FULL + qf), TILE_BYTES);
@@ -1134,12 +1126,13 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
             // drain: the Q copies already issued must land before the CTA's shared memory is released
             int dummy_flag = 0;
             // (a barrier that was never used is past the phase before its first)
-            for (int b = 0; b < 6; ++b) mbar_wait(bar(Q_FULL + b), ((q_phase >> b) & 1) ^ 1, &dummy_flag, p.status, W_QFULL);
+            for (int b = 0; b < 6; ++b) mbar_wait(bar(Q_FULL + b), ((q_phase >> b) & 1) ^ 1, &dummy_flag, p.wait, W_QFULL);
         }
     }
     tc_fence_before();
     __syncthreads();
     if (warp == 8) tmem_dealloc(tmem, kTmemCols);
+    if (threadIdx.x == 0) report_abort(p.status, s_abort);
     // the last CTA to leave rewinds the queue, so that the next call on this workspace needs no launch that prepares it
     if (threadIdx.x == 0 && s_usable) {
         __threadfence();
@@ -1202,6 +1195,7 @@ static int attend_tc_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bfl
     a.kdiv = SlotDiv::of(p->k);
     a.scale_log2 = p->scale * 1.4426950408889634f;
     a.cookie = p->cookie;
+    a.wait = WaitBound::of(p->wait_us);
     // always the d = 128 footprint: more than half an SM's shared memory, so CTAs (which each
     // take all 512 TMEM columns) never share an SM
     const size_t smem = 7 * (size_t)128 * 128 * 2 + 1024;      // Q ring of three, K and V two stages each

@@ -15,10 +15,20 @@ constexpr int kQTileRows = 256;     // query rows per attention work item (two 1
 constexpr int kPoolSlice = 256;     // tokens per chunk-pool work unit
 constexpr int kStatusWords = 16;    // status area at the head of the workspace (int32 each):
 // [0] device status (a moc_status), [1] detail code, [2] cookie of the plan whose lists the workspace holds,
-// [3] limit of every bounded wait in microseconds (0 = the default of one second), [4] routing blocks that have finished
-enum StatusWord { ST_STATUS = 0, ST_DETAIL = 1, ST_COOKIE = 2, ST_WAIT_US = 3, ST_ARRIVE = 4 };
+// [4] routing blocks that have finished
+enum StatusWord { ST_STATUS = 0, ST_DETAIL = 1, ST_COOKIE = 2, ST_ARRIVE = 4 };
 constexpr int kQueueHeader = 4;     // queue area: [0] next item to claim, [1] items, [2] phases, [3] CTAs that have left; then 3 ints per phase
 constexpr unsigned kPrivFlagCudaCoreAttend = 0x80000000u;   // plan flag outside the public header: test hook
+
+// How often a kernel's waits look before they give up: about a second's worth, or `us` microseconds' (tests; never more than the default).
+struct WaitBound {
+    uint32_t parked, polled;
+    uint32_t us;
+    static WaitBound of(unsigned us) {
+        if (us == 0 || us > 1000000u) us = 1000000u;
+        return WaitBound{us / 4 + 1, us * 32u, us};
+    }
+};
 
 // One contiguous range of key tokens [t0, t1).
 struct KeyRange { int32_t t0, t1; };
@@ -270,7 +280,7 @@ extern "C" {
 // attention and its backward on the plain fp32 CUDA-core kernels (an in-library cross-check that reads
 // the selection straight from sel_idx)
 int moc_debug_use_cuda_core_attention(moc_plan *plan, int on);
-// limit of every bounded device-side wait, in microseconds, for workspaces routed from now on (0 = default)
+// limit of every bounded device-side wait, in microseconds, of the launches from now on (0 = default)
 int moc_debug_set_wait_limit_us(moc_plan *plan, unsigned us);
 // one block whose only wait is on a barrier that nothing ever arrives on: it must give up after the limit,
 // record MOC_ERR_TIMEOUT with detail `code` in ws, and return

@@ -11,13 +11,11 @@
 
 namespace moc {
 
-__global__ void __launch_bounds__(32) wait_probe_kernel(int *status, int code, unsigned wait_us) {
+__global__ void __launch_bounds__(32) wait_probe_kernel(int *status, int code, WaitBound bound) {
     __shared__ __align__(8) uint64_t bar;
     __shared__ int s_abort;
     if (threadIdx.x == 0) {
         s_abort = 0;
-        status[ST_WAIT_US] = (int)wait_us;      // what routing with this plan would have stated
-        __threadfence();
         tc::mbar_init(tc::smem_u32(&bar), 1);
         tc::fence_barrier_init();
     }
@@ -25,7 +23,8 @@ __global__ void __launch_bounds__(32) wait_probe_kernel(int *status, int code, u
     if (threadIdx.x == 0) {
         volatile int *abort_flag = &s_abort;
         // phase 0 of a freshly initialised barrier completes only after one arrival: none comes
-        (void)tc::mbar_wait(tc::smem_u32(&bar), 0, abort_flag, status, code);
+        (void)tc::mbar_wait(tc::smem_u32(&bar), 0, abort_flag, bound, code);
+        tc::report_abort(status, s_abort);
     }
     __syncwarp();
 }
@@ -37,7 +36,7 @@ extern "C" int moc_debug_wait_probe(const moc_plan *p, void *ws, int code, void 
     if (!p) return MOC_ERR_NULL;
     if (!ws) return MOC_ERR_WORKSPACE;
     if (p->wait_us == 0 || p->wait_us > 100000u) return MOC_ERR_SHAPE;   // a probe never waits longer than 0.1 s
-    wait_probe_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(ws_ptr<int>(ws, p->ws.status), code, p->wait_us);
+    wait_probe_kernel<<<1, 32, 0, (cudaStream_t)stream>>>(ws_ptr<int>(ws, p->ws.status), code, WaitBound::of(p->wait_us));
     MOC_LAUNCH_CHECK();
     return MOC_OK;
 }

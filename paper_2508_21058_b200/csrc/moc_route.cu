@@ -91,14 +91,14 @@ __device__ __forceinline__ void sort32(uint64_t (&a)[32]) {
 
 // desc3[h][t][col][:] for t = 0, 1, 2: bf16 terms of the descriptor of score column col (the col-th non-text
 // chunk; rows beyond the last column are zero); also clears the pick counters and the status words (the workspace holds no plan's lists until they
-// are complete) and states the limit of the bounded waits.  With desc == nullptr only the clearing is done.
+// are complete).  With desc == nullptr only the clearing is done.
 __global__ void route_prep_kernel(const float *__restrict__ desc, __nv_bfloat16 *__restrict__ desc3, int *__restrict__ cnt,
                                   int *__restrict__ status, const int32_t *__restrict__ col_chunk, int H, int C, int ncol,
-                                  int c_pad, int d, unsigned wait_us) {
+                                  int c_pad, int d) {
     const size_t n = desc ? (size_t)H * c_pad * d : 0;
     const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     if (i < (size_t)H * C) cnt[i] = 0;
-    if (i < kStatusWords) status[i] = i == ST_WAIT_US ? (int)wait_us : 0;
+    if (i < kStatusWords) status[i] = 0;
     if (i >= n) return;
     const int x = (int)(i % d);
     const int c = (int)((i / d) % c_pad);
@@ -117,7 +117,7 @@ __global__ void route_prep_kernel(const float *__restrict__ desc, __nv_bfloat16 
 
 struct RouteParams {
     const float *desc;      // few-chunk case: the fp32 descriptors, split into their three terms by the kernel itself (else nullptr)
-    unsigned wait_us;       // limit of the bounded waits, stated in the status words by the kernel in that case
+    WaitBound wait;
     int32_t *sel;
     float *part_lse;
     int *cnt;
@@ -189,7 +189,6 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
 
     if (threadIdx.x == 0) {
         s_abort = 0;
-        if (FEW && p.desc) p.status[ST_WAIT_US] = (int)p.wait_us;       // every block writes the same value, before any of its waits
         for (int t = 0; t < kMaxStages; ++t) { mbar_init(bar(Q_FULL + t), 1); mbar_init(bar(Q_EMPTY + t), 1); }
         mbar_init(bar(D_FULL), 1);
         mbar_init(bar(D_EMPTY), 1);
@@ -285,7 +284,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                 for (int n = n0; n < n1; ++n) n_sb = max(n_sb, steps_of(n));   // blocks that hold a column in reach
                 for (int n = n0; ok && n < n1; ++n) {
                     const int st = qstage_of(n);                          // qn == n: one Q tile per unit, in unit order
-                    ok = mbar_wait(bar(Q_EMPTY + st), qparity_of(n) ^ 1, abort_flag, p.status, RW_QEMPTY);
+                    ok = mbar_wait(bar(Q_EMPTY + st), qparity_of(n) ^ 1, abort_flag, p.wait, RW_QEMPTY);
                     if (!ok) break;
                     mbar_expect_tx(bar(Q_FULL + st), Q_TILE_BYTES);
 #pragma unroll
@@ -295,7 +294,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                 }
                 for (int sb = 0; ok && sb < n_sb; ++sb) {
                     if (resident ? dn == 0 : sb != res_sb) {
-                        ok = mbar_wait(bar(D_EMPTY), (dn & 1) ^ 1, abort_flag, p.status, RW_DEMPTY);
+                        ok = mbar_wait(bar(D_EMPTY), (dn & 1) ^ 1, abort_flag, p.wait, RW_DEMPTY);
                         if (!ok) break;
                         if (FEW && p.desc) {
                             mbar_arrive(bar(D_FULL));       // the block wrote the terms itself, before the roles parted
@@ -317,9 +316,9 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                 int dummy_flag = 0;
                 for (int b = 1; b <= p.q_stages; ++b) {
                     const int qj = qn - b;
-                    if (qj >= 0) mbar_wait(bar(Q_FULL + qj % p.q_stages), (qj / p.q_stages) & 1, &dummy_flag, p.status, RW_QFULL);
+                    if (qj >= 0) mbar_wait(bar(Q_FULL + qj % p.q_stages), (qj / p.q_stages) & 1, &dummy_flag, p.wait, RW_QFULL);
                 }
-                if (dn > 0) mbar_wait(bar(D_FULL), (dn - 1) & 1, &dummy_flag, p.status, RW_DFULL);
+                if (dn > 0) mbar_wait(bar(D_FULL), (dn - 1) & 1, &dummy_flag, p.wait, RW_DFULL);
             }
         }
     } else if (warp == 1 || warp == 2 + 4 * NG) {
@@ -343,7 +342,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
             bool ok = true;
             // the whole warp waits, and goes on or gives up together
             auto wait = [&](int b, uint32_t parity, int code) {
-                return __all_sync(0xffffffffu, mbar_wait(bar(b), parity, abort_flag, p.status, code)) != 0;
+                return __all_sync(0xffffffffu, mbar_wait(bar(b), parity, abort_flag, p.wait, code)) != 0;
             };
             // a round: one unit (resident block; the two issuers take alternate units), or NG consecutive units that
             // share every streamed block
@@ -420,7 +419,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
         bool ok = true;
         auto group_sync = [&]() {     // all 128 threads of the group, bounded
             mbar_arrive(bar(GROUP + sg));
-            bool o = mbar_wait_spin(bar(GROUP + sg), ngs & 1, abort_flag, p.status, RW_GROUP);   // polled: a parked thread wakes late
+            bool o = mbar_wait_spin(bar(GROUP + sg), ngs & 1, abort_flag, p.wait, RW_GROUP);   // polled: a parked thread wakes late
             ++ngs;
             return o;
         };
@@ -524,7 +523,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                 for (int x = 1; x < KR; ++x) kth = (x < kp) ? top.s[x] : kth;
             };
             for (int sb = 0; ok && sb < n_sb; ++sb) {
-                ok = mbar_wait_spin(bar(ACC_FULL + sg), nacc & 1, abort_flag, p.status, RW_ACCFULL);
+                ok = mbar_wait_spin(bar(ACC_FULL + sg), nacc & 1, abort_flag, p.wait, RW_ACCFULL);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 ++nacc;
@@ -898,6 +897,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, 512);
+    if (threadIdx.x == 0) report_abort(p.status, s_abort);
     finish_route(p.status, p.cnt, p.tile_off, p.H * p.C, p.cookie, kRtThreads);
 }
 
@@ -1056,7 +1056,7 @@ int launch_lists_from_sel(const moc_plan *p, int32_t *sel, void *ws, cudaStream_
     int *cnt = ws_ptr<int>(ws, p->ws.cnt);
     int *status = ws_ptr<int>(ws, p->ws.status);
     const size_t n = std::max((size_t)p->H * p->C, (size_t)kStatusWords);
-    route_prep_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(nullptr, nullptr, cnt, status, nullptr, p->H, p->C, p->ncol, p->c_pad, p->d, p->wait_us);
+    route_prep_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(nullptr, nullptr, cnt, status, nullptr, p->H, p->C, p->ncol, p->c_pad, p->d);
     MOC_LAUNCH_CHECK();
     if (p->k > 0) {
         // Whether an entry repeats an earlier one: by a bitmap of the row's picks where clearing and marking it is less work than
@@ -1090,7 +1090,7 @@ static int launch_route_d(const moc_plan *p, const __nv_bfloat16 *Q, const float
         MOC_CUDA_TRY(cudaMemsetAsync(status, 0, (p->ws.cnt - p->ws.status) + sizeof(int) * (size_t)p->H * p->C, s));
     } else {
         const size_t n = std::max((size_t)p->H * p->c_pad * D, (size_t)kStatusWords);   // covers H * C too
-        route_prep_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(desc, desc3, cnt, status, p->d_col_chunk, p->H, p->C, p->ncol, p->c_pad, D, p->wait_us);
+        route_prep_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(desc, desc3, cnt, status, p->d_col_chunk, p->H, p->C, p->ncol, p->c_pad, D);
         MOC_LAUNCH_CHECK();
     }
     if (route_is_long(p)) {
@@ -1099,7 +1099,8 @@ static int launch_route_d(const moc_plan *p, const __nv_bfloat16 *Q, const float
     }
     if (p->k > 0) {
         RouteParams a;
-        a.desc = fused_prep ? desc : nullptr; a.wait_us = p->wait_us;
+        a.desc = fused_prep ? desc : nullptr;
+        a.wait = WaitBound::of(p->wait_us);
         a.sel = sel; a.part_lse = ws_ptr<float>(ws, p->ws.part_lse); a.cnt = cnt;
         a.qlist = ws_ptr<int32_t>(ws, p->ws.qlist);
         a.tok_chunk = p->d_tok_chunk; a.cand_c = p->d_cand_c; a.lim = p->d_lim; a.reach = p->d_reach;

@@ -61,6 +61,7 @@ struct RouteLongParams {
     int *tile_off;
     uint32_t cookie;
     size_t cap_total;
+    WaitBound wait;
 };
 
 // Scores ordered as unsigned integers (-0 below +0), and back.
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
                 const int t = u / p.H, h = u - t * p.H, steps = steps_of(reach_of(t));
                 const int st = p.q_stages == 2 ? qn & 1 : 0;
                 const uint32_t ph = (p.q_stages == 2 ? qn >> 1 : qn) & 1;
-                ok = mbar_wait(bar(Q_EMPTY + st), ph ^ 1, abort_flag, p.status, RL_QEMPTY);
+                ok = mbar_wait(bar(Q_EMPTY + st), ph ^ 1, abort_flag, p.wait, RL_QEMPTY);
                 if (!ok) break;
                 mbar_expect_tx(bar(Q_FULL + st), Q_TILE_BYTES);
 #pragma unroll
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
                 ++qn;
                 for (int x = 0; x < 3 * steps; ++x) {
                     const int sb = x / 3, term = x - 3 * sb;
-                    ok = mbar_wait(bar(D_EMPTY + slot), dph ^ 1, abort_flag, p.status, RL_DEMPTY);
+                    ok = mbar_wait(bar(D_EMPTY + slot), dph ^ 1, abort_flag, p.wait, RL_DEMPTY);
                     if (!ok) break;
                     mbar_expect_tx(bar(D_FULL + slot), SUB * d_sub_bytes);
 #pragma unroll
@@ -194,9 +195,9 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
                 // drain: copies already issued must land before the CTA's shared memory is released
                 int dummy_flag = 0;
                 for (int b = 1; b <= p.q_stages; ++b)
-                    if (qn - b >= 0) mbar_wait(bar(Q_FULL + (qn - b) % p.q_stages), ((qn - b) / p.q_stages) & 1, &dummy_flag, p.status, RL_QFULL);
+                    if (qn - b >= 0) mbar_wait(bar(Q_FULL + (qn - b) % p.q_stages), ((qn - b) / p.q_stages) & 1, &dummy_flag, p.wait, RL_QFULL);
                 for (int b = 1; b <= p.d_slots; ++b)
-                    if (dn - b >= 0) mbar_wait(bar(D_FULL + (dn - b) % p.d_slots), ((dn - b) / p.d_slots) & 1, &dummy_flag, p.status, RL_DFULL);
+                    if (dn - b >= 0) mbar_wait(bar(D_FULL + (dn - b) % p.d_slots), ((dn - b) / p.d_slots) & 1, &dummy_flag, p.wait, RL_DFULL);
             }
         }
     } else if (warp == kLongSel + 1) {
@@ -205,7 +206,7 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
         int qn = 0, slot = 0;
         uint32_t dph = 0, acc_phase = 0;
         bool ok = true;
-        auto wait = [&](int b, uint32_t parity, int code) { return __all_sync(ALL, mbar_wait(bar(b), parity, abort_flag, p.status, code)) != 0; };
+        auto wait = [&](int b, uint32_t parity, int code) { return __all_sync(ALL, mbar_wait(bar(b), parity, abort_flag, p.wait, code)) != 0; };
         for (int u = blockIdx.x; ok && u < p.n_units; u += gridDim.x) {
             const int reach = uniform(reach_of(u / p.H)), steps = steps_of(reach);
             const int st = p.q_stages == 2 ? qn & 1 : 0;
@@ -248,7 +249,7 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
         auto meet = [&](int b, uint32_t bit) {                // warps that meet, bounded
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(b));
-            const bool o = mbar_wait(bar(b), (sync_phase & bit) ? 1 : 0, abort_flag, p.status, RL_SYNC);
+            const bool o = mbar_wait(bar(b), (sync_phase & bit) ? 1 : 0, abort_flag, p.wait, RL_SYNC);
             sync_phase ^= bit;
             return __all_sync(ALL, o) != 0;
         };
@@ -316,7 +317,7 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
                         f(v, j0, cand);
                     }
                 };
-                for (int s = 0; ok && s < n_st; ++s) ok = mbar_wait(bar(ACC_FULL + s), (acc_phase >> s) & 1, abort_flag, p.status, RL_ACCFULL);
+                for (int s = 0; ok && s < n_st; ++s) ok = mbar_wait(bar(ACC_FULL + s), (acc_phase >> s) & 1, abort_flag, p.wait, RL_ACCFULL);
                 ok = __all_sync(ALL, ok);
                 if (!ok) break;
                 acc_phase ^= (1u << n_st) - 1;
@@ -557,6 +558,7 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
     tc_fence_before();
     __syncthreads();
     if (warp == kLongSel) tmem_dealloc(tmem, 512);
+    if (threadIdx.x == 0) report_abort(p.status, s_abort);
     finish_route(p.status, p.cnt, p.tile_off, p.H * p.C, p.cookie, kLongThreads);
 }
 
@@ -590,6 +592,7 @@ static int route_long_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bf
     a.d_rows = std::min(p->c_pad, kLongStep);
     a.tile_off = ws_ptr<int>(ws, p->ws.tile_off);
     a.cookie = p->cookie;
+    a.wait = WaitBound::of(p->wait_us);
     a.cap_total = (size_t)p->cap_off[p->C];
     // Survivors that are sorted: more than k, so that the first threshold is often good enough (30 of 504: any of 30 to 64), at most 512;
     // or all the columns there are.  With more columns than an accumulator holds each 512 of them have thresholds of their own, and a
