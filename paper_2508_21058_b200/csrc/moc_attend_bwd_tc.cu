@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
     // per streamed query, (-lse * log2(e), -delta), for tiles j and j + 1
     __shared__ __align__(16) float s_ld[2][2][128];
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     // shared tiles: X1 X2 | Y1 stages | Y2 stages
     const uint32_t sX = sbase, sY1 = sbase + 2 * TILE_BYTES, sY2 = sbase + (2 + kY1Stages) * TILE_BYTES;
@@ -462,12 +462,17 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             } else {
                 constexpr int RP = 32 / CH;                // rows per instruction
                 const int c16 = lane % CH;
+                // (eight rows at a time, in which the swizzle repeats: all 64 of them unrolled were 10 KB of code)
+#pragma unroll 1
+                for (int r8 = 0; r8 < 64; r8 += 8) {
+                    const int rows_q = r8 < 32 ? t_q[0] : t_q[1];
 #pragma unroll
-                for (int rb = 0; rb < 64; rb += RP) {
-                    const int rl = rb + lane / CH;
-                    const int qq = __shfl_sync(0xffffffffu, t_q[rb >> 5], rl & 31);
-                    cp_async16(dst + (c16 >> 3) * SUB_BYTES + sw128_offset(wsub * 64 + rl, c16 & 7),
-                               rows_src + (size_t)max(qq, 0) * D + c16 * 8, qq >= 0 ? 16u : 0u);
+                    for (int rb = 0; rb < 8; rb += RP) {
+                        const int rl = rb + lane / CH;
+                        const int qq = __shfl_sync(0xffffffffu, rows_q, (r8 + rl) & 31);
+                        cp_async16(dst + (c16 >> 3) * SUB_BYTES + (wsub * 64 + r8) * 128 + sw128_offset(rl, c16 & 7),
+                                   rows_src + (size_t)max(qq, 0) * D + c16 * 8, qq >= 0 ? 16u : 0u);
+                    }
                 }
             }
             ++issued;

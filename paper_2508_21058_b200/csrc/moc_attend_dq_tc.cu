@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort, s_lo, s_total;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     // shared tiles: X1 (Q) X2 (dO) | K stages | V stages
     const uint32_t sX = sbase, sK = sbase + 2 * TILE_BYTES, sV = sbase + (2 + kKStages) * TILE_BYTES;
@@ -460,12 +460,14 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
                     const uint32_t dst = sX + (b >> 2) * TILE_BYTES;
                     constexpr int RP = 32 / CH;                // rows per instruction
                     const int c16 = lane % CH;
+#pragma unroll 1
+                    for (int r8 = 0; r8 < 32; r8 += 8)          // (eight rows at a time, in which the swizzle repeats)
 #pragma unroll
-                    for (int rb = 0; rb < 32; rb += RP) {
-                        const int rl = rb + lane / CH, qq = __shfl_sync(0xffffffffu, q[y], rl);
-                        cp_async16(dst + (c16 >> 3) * SUB_BYTES + sw128_offset((b & 3) * 32 + rl, c16 & 7), src + (size_t)max(qq, 0) * D + c16 * 8,
-                                   qq >= 0 ? 16u : 0u);
-                    }
+                        for (int rb = 0; rb < 8; rb += RP) {
+                            const int rl = rb + lane / CH, qq = __shfl_sync(0xffffffffu, q[y], r8 + rl);
+                            cp_async16(dst + (c16 >> 3) * SUB_BYTES + ((b & 3) * 32 + r8) * 128 + sw128_offset(rl, c16 & 7),
+                                       src + (size_t)max(qq, 0) * D + c16 * 8, qq >= 0 ? 16u : 0u);
+                        }
                     if (b < 4) {                               // a row without a query gets lse = +inf: P and dS are zero
                         s_ld[n & 1][0][b * 32 + lane] = lse[y] * -1.4426950408889634f;
                         s_ld[n & 1][1][b * 32 + lane] = -del[y];

@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
     __shared__ int s_abort, s_usable;      // s_usable: the workspace holds this plan's lists
     __shared__ ItemSlot s_item[kItemSlots];
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     // shared tiles: Q ring of three | K stage 0,1 | V stage 0,1
     const uint32_t sQ = sbase, sK = sbase + 3 * TILE_BYTES, sV = sbase + 5 * TILE_BYTES;

@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *gbase = smem_raw + (sbase - smem_u32(smem_raw));
     // shared memory: descriptor block (3 terms x SUB sub-tiles of d_rows x 128 bytes) | Q stages | histograms
@@ -934,7 +934,7 @@ __global__ void __launch_bounds__(1024) route_tiles_kernel(const int *__restrict
 // rewound.  One block: a warp adds up a group's pick counts, one thread then lays the phases out.
 __device__ void write_queue(int *__restrict__ queue, const int *__restrict__ cnt, const int *__restrict__ gtile, int H, int L, int C, int k,
                             int hg, int n_groups, int n_aitems) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     for (int g = warp; g < n_groups; g += blockDim.x >> 5) {
         const int h0 = g * hg, h1 = min(H, h0 + hg);
         int entries = 0;

@@ -125,7 +125,7 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
     __shared__ float s_stat[3][4][kLongRows];
     __shared__ int s_count[2][4][kLongRows];
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *gbase = smem_raw + (sbase - smem_u32(smem_raw));
     // shared memory: descriptor ring (a slot: SUB sub-tiles of d_rows x 128 bytes) | Q stages | survivors, CAP per row | one or two histograms

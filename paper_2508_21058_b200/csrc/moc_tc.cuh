@@ -152,7 +152,13 @@ __device__ __forceinline__ void tc_commit_elect(uint32_t bar) {
         "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
         : "memory");
 }
-// a value that every lane of the warp holds, as one the compiler knows to be the same in all of them
+// A value that every lane of the warp holds, as one the compiler knows to be the same in all of them.
+// The warp's number in the block is taken through it in the kernels whose warps have roles: with threadIdx.x >> 5 alone a role's
+// branch counts as one that the lanes may part at, and the issuers' loops were written out with a guard around each of their
+// instructions (some 33 a tcgen05.mma).  The code of the kernels is what it saves, which in these is what bounds the
+// loops (a few roles' loops share the instruction cache).  Plain -> through this, with the backward's row loaders looped: the code
+// of the dK/dV kernel 96 -> 55 KB, of dQ 89 -> 57 (d = 128); 24 heads of 6.7k tokens, 4 picks, backward 9.95 -> 9.69 ms, 6 heads
+// 2.21 -> 2.14 ms, routing 64 -> 58 us; 2 heads of 115k tokens, 30 picks, routing 690 -> 652 us; the forward as before.
 __device__ __forceinline__ int uniform(int v) { return __shfl_sync(0xffffffffu, v, 0); }
 
 // 32 consecutive fp32 columns of this thread's TMEM lane
