@@ -169,10 +169,18 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
         const uint64_t c2 = pack2(p.scale_log2, p.scale_log2);
         bool ok = true;
         int s3 = 0, ph3 = 0;                          // Y1 stage of tile jt and its phase
+        // A barrier that has completed is looked at some hundred cycles before its wait, behind other work: a wait costs the lanes
+        // that much even then, and their chain, P, ACC2, T1 of the next tile, P again, is what a tile takes.  P and dS lie over the first half
+        // of the chunk's own columns, which the thread alone has read; side by side, the two threads of a lane waited for each other twice a
+        // tile.  (Both, with the same looks ahead in the dQ kernel, the whole backward: 4 heads of 33k tokens 1450 -> 1425 us, 24 heads
+        // at the power limit 9.77 -> 9.64 ms, 8 heads of 42k tokens 4.04 -> 3.97, 12 heads of 6.3k, d = 64, 240 -> 234 us, 3 heads of
+        // 3.1k 70 -> 67.5.)  What is left of a tile's 2500 cycles (d = 128): 1024 of exponentials, the products after them, and 64 KB of
+        // query rows out of L2, 25 bytes a cycle and SM.
+        bool t1_early = false, y1_early = false;
         for (int jt = 0; jt < n_tiles; ++jt) {
             const int st = jt & 1;
-            ok = mbar_wait_spin(bar(T1_FULL + st), (jt >> 1) & 1, abort_flag, p.wait, BW_T1FULL);
-            ok = ok && mbar_wait(bar(Y1_FULL + s3), ph3, abort_flag, p.wait, BW_YFULL);
+            ok = t1_early || mbar_wait_spin(bar(T1_FULL + st), (jt >> 1) & 1, abort_flag, p.wait, BW_T1FULL);
+            ok = ok && (y1_early || mbar_wait(bar(Y1_FULL + s3), ph3, abort_flag, p.wait, BW_YFULL));
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
@@ -183,13 +191,12 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             tmem_ld32(tmem + lane_off + half * 32, sv[0]);
             tmem_ld32(tmem + lane_off + (2 + half) * 32, sv[1]);
             tmem_wait_ld();
-            // P goes over T1 columns that the other thread of the lane reads; that read is announced here and waited
-            // for (bounded, like every wait) just before the first store
-            mbar_arrive(bar(RD1));
+            bool t2_early = false;
 #pragma unroll
             for (int rd = 0; rd < 2; ++rd) {
                 const int ch = rd * 2 + half;
                 const uint32_t (&s)[32] = sv[rd];
+                if (rd == 1) t2_early = mbar_test_wait(bar(T2_FULL + st), (jt >> 1) & 1);
                 // two columns per packed instruction; four columns' (negated) lse per shared-memory load
 #pragma unroll
                 for (int x = 0; x < 32; x += 4) {
@@ -207,21 +214,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                     uint32_t ups[16];
 #pragma unroll
                     for (int x = 0; x < 16; ++x) ups[x] = bf16x2(pv[rd * 32 + 2 * x], pv[rd * 32 + 2 * x + 1]);
-                    if (rd == 0) {
-                        ok = mbar_wait_spin(bar(RD1), jt & 1, abort_flag, p.wait, BW_READ);
-                        ok = __all_sync(0xffffffffu, ok);
-                    }
-                    if (ok) {
-                        tmem_st16(tmem + lane_off + ch * 16, ups);
-                        tmem_wait_st();
-                        tc_fence_before();
-                        mbar_arrive(bar(rd == 0 ? P_HALF : P_DONE));      // the first, then the second 64 columns of P
-                    }
+                    tmem_st16(tmem + lane_off + ch * 32, ups);
+                    tmem_wait_st();
+                    tc_fence_before();
+                    mbar_arrive(bar(rd == 0 ? P_HALF : P_DONE));      // the first, then the second 64 columns of P
                 }
             }
-            if (!ok) break;
             // ---- dS = P (dP - delta) from T2, written over T2 columns that have been read
-            ok = mbar_wait_spin(bar(T2_FULL + st), (jt >> 1) & 1, abort_flag, p.wait, BW_T2FULL);
+            ok = t2_early || mbar_wait_spin(bar(T2_FULL + st), (jt >> 1) & 1, abort_flag, p.wait, BW_T2FULL);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
@@ -229,7 +229,6 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
             tmem_ld32(tmem + lane_off + t2c + half * 32, dpv[0]);
             tmem_ld32(tmem + lane_off + t2c + (2 + half) * 32, dpv[1]);
             tmem_wait_ld();
-            mbar_arrive(bar(RD2));                                      // this thread's columns have been read
 #pragma unroll
             for (int rd = 0; rd < 2; ++rd) {
                 const int ch = rd * 2 + half;
@@ -247,17 +246,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                         uds[(x >> 1) + y] = bf16x2(a0, a1);
                     }
                 }
-                if (rd == 0) {
-                    ok = mbar_wait_spin(bar(RD2), jt & 1, abort_flag, p.wait, BW_READ);
-                    ok = __all_sync(0xffffffffu, ok);
-                }
-                if (ok) tmem_st16(tmem + lane_off + t2c + ch * 16, uds);
+                tmem_st16(tmem + lane_off + t2c + ch * 32, uds);
             }
-            if (!ok) break;
+            if (++s3 == kY1Stages) { s3 = 0; ph3 ^= 1; }
+            t1_early = mbar_test_wait(bar(T1_FULL + (st ^ 1)), ((jt + 1) >> 1) & 1);
+            y1_early = mbar_test_wait(bar(Y1_FULL + s3), ph3);
             tmem_wait_st();
             tc_fence_before();
             mbar_arrive(bar(DS_DONE + st));
-            if (++s3 == kY1Stages) { s3 = 0; ph3 ^= 1; }
         }
         // ---- epilogue
         if (ok) {
@@ -317,14 +313,14 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                 }
                 // (the lane threads' own two barriers, once more: every wait here is bounded)
                 mbar_arrive(bar(RD1));
-                ok = mbar_wait_spin(bar(RD1), n_tiles & 1, abort_flag, p.wait, BW_READ);
+                ok = mbar_wait_spin(bar(RD1), 0, abort_flag, p.wait, BW_READ);
                 if (threadIdx.x == 0 && ok) {
                     __threadfence();
                     s_last = atomicAdd(p.split_done + slot, 1) == parts - 1;
                     __threadfence();
                 }
                 mbar_arrive(bar(RD2));
-                ok = ok && mbar_wait_spin(bar(RD2), n_tiles & 1, abort_flag, p.wait, BW_READ);
+                ok = ok && mbar_wait_spin(bar(RD2), 0, abort_flag, p.wait, BW_READ);
                 ok = __all_sync(0xffffffffu, ok);
                 if (ok && s_last) {
 #pragma unroll 1
@@ -548,13 +544,13 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                 const uint32_t ds = tmem + 128;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)
-                    mma_ts_elect(tmem + 256, ds + ks * 8, lo(y1m) + s3 * (uint32_t)STAGE + ks * (2048 >> 4), hi(y1m), IDESC_ACC, j > 0 || ks > 0);
+                    mma_ts_elect(tmem + 256, ds + (ks >> 1) * 32 + (ks & 1) * 8, lo(y1m) + s3 * (uint32_t)STAGE + ks * (2048 >> 4), hi(y1m), IDESC_ACC, j > 0 || ks > 0);
             };
             auto acc2 = [&](int j, int half) {   // ACC2 += P(j) Y2(j), the K steps of one half of P
                 const int s2 = j & 1;
 #pragma unroll
                 for (int ks = 0; ks < 4; ++ks)
-                    mma_ts_elect(tmem + 384, tmem + (half * 4 + ks) * 8, lo(y2m) + s2 * (uint32_t)STAGE + (half * 4 + ks) * (2048 >> 4), hi(y2m),
+                    mma_ts_elect(tmem + 384, tmem + (half * 2 + (ks >> 1)) * 32 + (ks & 1) * 8, lo(y2m) + s2 * (uint32_t)STAGE + (half * 4 + ks) * (2048 >> 4), hi(y2m),
                               IDESC_ACC, j > 0 || half > 0 || ks > 0);
             };
             // MMAs queue up behind one another, so a group goes out as soon as what it reads is there

@@ -210,9 +210,10 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
                 }
             };
             int valid, t0;
+            bool t1_early = false, t2_early = false;         // looked at behind other work: see the dK/dV kernel
             // P of the tile
             auto form_p = [&]() __attribute__((always_inline)) -> bool {
-                ok = mbar_wait_spin(bar(T1_FULL), g & 1, abort_flag, p.wait, DW_T1FULL);
+                ok = t1_early || mbar_wait_spin(bar(T1_FULL), g & 1, abort_flag, p.wait, DW_T1FULL);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) return false;
                 tc_fence_after();
@@ -222,6 +223,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
                 tmem_wait_ld();
                 tc_fence_before();
                 mbar_arrive(bar(T1_READ));                   // T1 may be overwritten
+                t2_early = mbar_test_wait(bar(T2_FULL + (g & 1)), (g >> 1) & 1);
 #pragma unroll
                 for (int rd = 0; rd < 2; ++rd)
 #pragma unroll
@@ -233,13 +235,14 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
             auto form_ds = [&]() __attribute__((always_inline)) -> bool {
                 const int st = g & 1;
                 const uint32_t t2 = tmem + lane_off + (st ? 384u : 128u);
-                ok = mbar_wait_spin(bar(T2_FULL + st), (g >> 1) & 1, abort_flag, p.wait, DW_T2FULL);
+                ok = t2_early || mbar_wait_spin(bar(T2_FULL + st), (g >> 1) & 1, abort_flag, p.wait, DW_T2FULL);
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) return false;
                 tc_fence_after();
                 uint32_t dp[2][32];
                 tmem_ld32(t2 + half * 32, dp[0]);
                 tmem_ld32(t2 + (2 + half) * 32, dp[1]);
+                t1_early = mbar_test_wait(bar(T1_FULL), (g + 1) & 1);
                 tmem_wait_ld();
 #pragma unroll
                 for (int rd = 0; rd < 2; ++rd) {
