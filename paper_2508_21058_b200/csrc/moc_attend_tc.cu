@@ -300,6 +300,10 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
 #pragma unroll
                     for (int x = 0; x < 32; x += 2) m4[ch] = max3(m4[ch], __uint_as_float(v[ch][x]), __uint_as_float(v[ch][x + 1]));
                 }
+                // The turn is looked at here and awaited below, where a wait costs some hundred cycles even if it has come.  (At d = 64,
+                // where it has rarely come by now, the look cost 2 %; at d = 128, 4 heads of 33k tokens 537 -> 526 us, 2 heads of 42k 411 -> 403,
+                // 2 heads of 32k tokens, 512-token chunks, 1273 -> 1255, 24 heads of 33k at the power limit 3.33 -> 3.29 ms.)
+                const bool my_turn = D == 128 && (!two || (g == 0 && !(bits & TURNED)) || mbar_test_wait(bar(TURN + (g ^ 1)), ((bits & TURN_ODD) ? 1 : 0) ^ (g == 1 ? 0 : 1)));
                 const float m_new = fmaxf(m_run, fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])) * c);
                 float alpha = 1.f;
                 if (jt == 0) {
@@ -316,7 +320,7 @@ __global__ void __launch_bounds__(LOADERS ? kThreadsLoaders : kThreads, 1) atten
                 // 0.3 %: 33k-token clip 3.407 and 3.404 ms, d = 64, 725-token frames 643.5 and 643.7 us; at half time it cost 5 %.)  (Tile 0 waits for
                 // tile 1's previous turn even at the start of an item: the barrier must never get two phases ahead of
                 // a group that has yet to wait on it.)
-                if (two && (g == 1 || (bits & TURNED))) {
+                if (D == 128 ? !__all_sync(0xffffffffu, my_turn) : two && (g == 1 || (bits & TURNED))) {
                     ok = mbar_wait(bar(TURN + (g ^ 1)), ((bits & TURN_ODD) ? 1 : 0) ^ (g == 1 ? 0 : 1), abort_flag, p.wait, W_TURN);
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
