@@ -213,14 +213,15 @@ class MocPlan:
     def moc_outer_reduced_layout(self, sel_shot, q_tok0, q_tok1):
         """Host only: (chunk_off, chunk_shot, chunk_mod, tok_map) of the reduced stream for one row of sel_shot."""
         sel = np.ascontiguousarray(sel_shot, np.int32).reshape(-1)
-        off = np.zeros(self.C + 1, np.int32)
-        shot = np.zeros(self.C, np.int32)
-        mod = np.zeros(self.C, np.uint8)
-        tok = np.zeros(self.L, np.int32)
+        # only what the call fills in is touched, and no part is copied: clearing and copying a map of 264k tokens took longer than making it
+        off = np.empty(self.C + 1, np.int32)
+        shot = np.empty(self.C, np.int32)
+        mod = np.empty(self.C, np.uint8)
+        tok = np.empty(self.L, np.int32)
         nc, nt = C.c_int32(0), C.c_int32(0)
         _check(self._lib.moc_outer_reduced_layout(self._h, sel.ctypes.data, len(sel), int(q_tok0), int(q_tok1), C.byref(nc),
                                                   C.byref(nt), off.ctypes.data, shot.ctypes.data, mod.ctypes.data, tok.ctypes.data))
-        return off[:nc.value + 1].copy(), shot[:nc.value].copy(), mod[:nc.value].copy(), tok[:nt.value].copy()
+        return off[:nc.value + 1], shot[:nc.value], mod[:nc.value], tok[:nt.value]
 
     def moc_gather_tokens(self, X, tok_map, out):
         _check(self._lib.moc_gather_tokens(self._h, _ptr(X), _ptr(tok_map), int(tok_map.numel()), _ptr(out), _stream()))
