@@ -4,7 +4,7 @@
 // the block records MOC_ERR_TIMEOUT and a code in the workspace's status area and returns normally.
 // Nothing in a healthy run makes a wait run out, so this probe does it on purpose in the one way that is
 // harmless: a block waits on a barrier that no thread, copy or tensor-core operation will ever arrive
-// on, through the same bounded wait as every other kernel, with the limit the workspace states.  It
+// on, through the same bounded wait as every other kernel, with the limit that its launch is given.  It
 // touches no other memory, holds no tensor memory and has no copy in flight, so giving up is all it does.
 #include "moc_common.cuh"
 #include "moc_tc.cuh"
