@@ -183,7 +183,7 @@ struct SlotDiv {
 // work-item fields) is checked before it is used as an address; a bad one records MOC_ERR_INDEX with `code`
 // in the status area and the access is skipped.  In the release build the checks cost nothing.
 enum IndexCheck { IX_ITEM_FIELDS = 200, IX_LIST_POSITION, IX_LIST_ENTRY, IX_APPEND_POSITION, IX_BWD_ITEM_FIELDS,
-                  IX_BWD_LIST_POSITION, IX_BWD_LIST_ENTRY };
+                  IX_BWD_LIST_POSITION, IX_BWD_LIST_ENTRY, IX_ROUTE_SURVIVORS, IX_ROUTE_COLUMN };
 #ifdef MOC_DEBUG
 __device__ __forceinline__ bool index_ok(bool cond, int *status, int code) {
     if (!cond && atomicCAS(status, 0, MOC_ERR_INDEX) == 0) status[ST_DETAIL] = code;

@@ -5,7 +5,7 @@
 // twenty entries on that, and not the scores, is the time of routing (264k tokens, 1008 columns, 2 heads, 118 picks: 6.7 ms).  Here a
 // row's threads only count: of the scores in tensor memory those that reach a threshold, until a few more than k do, two or three times; those
 // alone are kept, and sorted by a whole warp.  (2 heads, a thread per row -> this, us: 264k tokens, 1008 columns: 20 picks 971 -> 755, 30 1122 ->
-// 823, 60 3063 -> 1340, 118 6706 -> 1870; 504 columns: 20 680 -> 487, 32 802 -> 597, 64 2173 -> 998; 40k tokens, 200 columns, 20 picks 96 -> 82.)
+// 805, 60 3063 -> 1300, 118 6706 -> 1800; 504 columns: 20 680 -> 493, 32 802 -> 592, 64 2173 -> 998; 40k tokens, 200 columns, 20 picks 96 -> 82.)
 // What bounds it now (118 picks, per tile of 130,000 cycles): the sorts 41,000, counting 31,000, the list entries, four bytes here and there, 25,000.
 // Scores through a scratch in L2, so that a warp could hold a row, took 1.4 times as long: 64 KB a step each way.
 //
@@ -53,8 +53,8 @@ struct RouteLongParams {
     const int32_t *col_chunk;   // [ncol] chunk of a score column
     const int32_t *cap_off;
     int *status;
-    int H, L, C, c_pad, k, cwords, prefix;
-    int tiles_per_head, n_units;
+    int H, L, C, c_pad, ncol, k, cwords, prefix;
+    int n_units;
     int d_rows;                 // columns per step of the ring: 128, or all of them
     int q_stages, d_slots;
     int hists;                  // pick counters of two units (a unit's list entries are written behind the next one's scores), or of one
@@ -64,12 +64,33 @@ struct RouteLongParams {
     WaitBound wait;
 };
 
-// Scores ordered as unsigned integers (-0 below +0), and back.
+// Scores are counted, stored, thinned and sorted in one order: numbers, subnormal ones and -0 all taken as zero.  It is written out here, so
+// that it does not hang on the compiler's flags: a store that told a subnormal threshold from zero, where the count did not, left
+// fewer survivors than had been counted.
+__device__ __forceinline__ int reaches(float f, float thr) {
+    int r;
+    asm("{\n\t.reg .pred p;\n\tsetp.ge.ftz.f32 p, %1, %2;\n\tselp.s32 %0, 1, 0, p;\n\t}" : "=r"(r) : "f"(f), "f"(thr));
+    return r;
+}
+// (and, of equal ones, in the columns before `before`)
+__device__ __forceinline__ int reaches(float f, int col, float thr, int before) {
+    int r;
+    asm("{\n\t.reg .pred p, q;\n\tsetp.lt.s32 p, %2, %4;\n\tsetp.eq.and.ftz.f32 p, %1, %3, p;\n\tsetp.gt.or.ftz.f32 q, %1, %3, p;\n\tselp.s32 %0, 1, 0, q;\n\t}"
+        : "=r"(r) : "f"(f), "r"(col), "f"(thr), "r"(before));
+    return r;
+}
+// Scores as unsigned integers of the same order (of those that count as zero, subnormal ones keep theirs), and back.
 __device__ __forceinline__ uint32_t ordered(float f) {
     const uint32_t b = __float_as_uint(f);
     return b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u);
 }
 __device__ __forceinline__ float from_ordered(uint32_t u) { return __uint_as_float((u & 0x80000000u) ? u ^ 0x80000000u : ~u); }
+// ... and with all that count as zero as +0.
+__device__ __forceinline__ uint32_t sort_key(float f) {
+    float z;
+    asm("add.ftz.f32 %0, %1, 0f00000000;" : "=f"(z) : "f"(f));
+    return ordered(z);
+}
 
 // The value that a standard normal variable exceeds with probability p (Abramowitz and Stegun 26.2.23, error below 5e-4).
 __device__ __forceinline__ float normal_above(float p) {
@@ -370,17 +391,17 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
                     if (!ties) {
                         each_block(0xff800000u, [&](const uint32_t (&v)[32], int, uint32_t) {
 #pragma unroll
-                            for (int c = 0; c < 32; ++c) c_new += __uint_as_float(v[c]) >= thr;
+                            for (int c = 0; c < 32; ++c) c_new += reaches(__uint_as_float(v[c]), thr);
                         });
                     } else {
                         each_block(0xff800000u, [&](const uint32_t (&v)[32], int j0, uint32_t) {
 #pragma unroll
-                            for (int c = 0; c < 32; ++c) c_new += __uint_as_float(v[c]) > thr || (__uint_as_float(v[c]) == thr && j0 + c < before);
+                            for (int c = 0; c < 32; ++c) c_new += reaches(__uint_as_float(v[c]), j0 + c, thr, before);
                         });
                     }
 #pragma unroll 4
                     for (int e = part; e < max_len; e += 4)
-                        if (e < len) c_old += sc_at(row, e) > thr || (sc_at(row, e) == thr && co_at(row, e) < before);
+                        if (e < len) c_old += ties ? reaches(sc_at(row, e), co_at(row, e), thr, before) : reaches(sc_at(row, e), thr);
                     s_count[pass_no & 1][part][row] = c_new | c_old << 16;
                     ok = same_rows();
                     if (!ok) break;
@@ -436,37 +457,38 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
                             }
 #pragma unroll
                             for (int x = 0; x < 8; ++x)
-                                if (e0 + x < len && (f[x] > thr || (f[x] == thr && c[x] < before))) { sc_at(row, to) = f[x]; co_at(row, to) = (uint16_t)c[x]; ++to; }
+                                if (e0 + x < len && reaches(f[x], c[x], thr, before)) { sc_at(row, to) = f[x]; co_at(row, to) = (uint16_t)c[x]; ++to; }
                         }
                     }
                     ok = same_rows();
                     if (!ok) break;
                 }
-                if (!ties && N <= kQueueShared) {
-                    uint32_t a_sc = smem_u32(&sc_at(row, at)), a_co = smem_u32(&co_at(row, at));
+                // (where this thread's entries have to end: survivors are stored by the rule that they were counted by)
+                const int end = at + (s_count[(pass_no - 1) & 1][part][row] & 0xffff);
+                // a survivor's score and column, and the places of the next one's
+                auto store = [](auto &a_sc, auto &a_co, float f, int col, int take) __attribute__((always_inline)) {
+                    if constexpr (N <= kQueueShared)
+                        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %4, 0;\n\t@p st.shared.f32 [%0], %2;\n\t@p st.shared.u16 [%1], %3;\n\t"
+                                     "@p add.u32 %0, %0, 4;\n\t@p add.u32 %1, %1, 2;\n\t}" : "+r"(a_sc), "+r"(a_co) : "f"(f), "h"((uint16_t)col), "r"(take) : "memory");
+                    else
+                        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %4, 0;\n\t@p st.global.f32 [%0], %2;\n\t@p st.global.u16 [%1], %3;\n\t"
+                                     "@p add.u64 %0, %0, 4;\n\t@p add.u64 %1, %1, 2;\n\t}" : "+l"(a_sc), "+l"(a_co) : "f"(f), "h"((uint16_t)col), "r"(take) : "memory");
+                };
+                auto place = [](auto &x) { if constexpr (N <= kQueueShared) return smem_u32(&x); else return (uint64_t)__cvta_generic_to_global(&x); };
+                auto a_sc = place(sc_at(row, at));
+                auto a_co = place(co_at(row, at));
+                if (!ties) {
                     each_block(0xff800000u, [&](const uint32_t (&v)[32], int j0, uint32_t) {
 #pragma unroll
-                        for (int c = 0; c < 32; ++c)
-                            asm volatile(
-                                "{\n\t.reg .pred p;\n\t"
-                                "setp.ge.f32 p, %2, %3;\n\t"
-                                "@p st.shared.f32 [%0], %2;\n\t"
-                                "@p st.shared.u16 [%1], %4;\n\t"
-                                "@p add.u32 %0, %0, 4;\n\t"
-                                "@p add.u32 %1, %1, 2;\n\t}"
-                                : "+r"(a_sc), "+r"(a_co)
-                                : "f"(__uint_as_float(v[c])), "f"(thr), "h"((uint16_t)(j0 + c))
-                                : "memory");
+                        for (int c = 0; c < 32; ++c) store(a_sc, a_co, __uint_as_float(v[c]), j0 + c, reaches(__uint_as_float(v[c]), thr));
                     });
                 } else {
                     each_block(0xff800000u, [&](const uint32_t (&v)[32], int j0, uint32_t) {
 #pragma unroll
-                        for (int c = 0; c < 32; ++c) {
-                            const float f = __uint_as_float(v[c]);
-                            if (f > thr || (f == thr && j0 + c < before)) { sc_at(row, at) = f; co_at(row, at) = (uint16_t)(j0 + c); ++at; }
-                        }
+                        for (int c = 0; c < 32; ++c) store(a_sc, a_co, __uint_as_float(v[c]), j0 + c, reaches(__uint_as_float(v[c]), j0 + c, thr, before));
                     });
                 }
+                index_ok(a_sc == place(sc_at(row, end)), p.status, IX_ROUTE_SURVIVORS);
                 len = total;
                 tc_fence_before();
                 __syncwarp();
@@ -479,7 +501,7 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
             ok = all_warps();
             if (!ok) break;
             if (last_t >= 0) write_entries(last_h, last_t, other);
-            // a warp per row, two rows at a time: the survivors sorted, score descending (-0 as +0), then column ascending
+            // a warp per row, two rows at a time: the survivors sorted, score descending, then column ascending
             constexpr int R = N <= 4 ? 2 : 1;
 #pragma unroll 1
             for (int y = 0; y < 8; y += R) {
@@ -494,7 +516,7 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
                     for (int e = 0; e < N; ++e) {
                         const int x = lane * N + e;
                         key[b][e] = 0;
-                        if (x < n_surv[b]) key[b][e] = (uint64_t)ordered(sc_at(r0 + 4 * b, x) + 0.f) << 32 | (uint32_t)~(uint32_t)co_at(r0 + 4 * b, x);
+                        if (x < n_surv[b]) key[b][e] = (uint64_t)sort_key(sc_at(r0 + 4 * b, x)) << 32 | (uint32_t)~(uint32_t)co_at(r0 + 4 * b, x);
                     }
                 }
                 warp_sort<R, N>(key, lane);
@@ -508,8 +530,9 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
                         const int x = lane * N + e;
                         if (x >= p.k || i >= p.L) continue;
                         int j = -1;
-                        if (x < n_surv[b]) {
-                            j = p.col_chunk[(int)~(uint32_t)key[b][e]];
+                        const uint32_t col = ~(uint32_t)key[b][e];
+                        if (x < n_surv[b] && index_ok(col < (uint32_t)p.ncol, p.status, IX_ROUTE_COLUMN) && col < (uint32_t)p.ncol) {
+                            j = p.col_chunk[col];
                             atomicAdd(&hist[j], 1);
                         } else {
                             pl[x * 128] = -INFINITY;
@@ -586,9 +609,8 @@ static int route_long_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bf
     a.qlist = ws_ptr<int32_t>(ws, p->ws.qlist);
     a.tok_chunk = p->d_tok_chunk; a.cand_c = p->d_cand_c; a.lim = p->d_lim; a.reach = p->d_reach;
     a.col_chunk = p->d_col_chunk; a.cap_off = p->d_cap_off; a.status = ws_ptr<int>(ws, p->ws.status);
-    a.H = p->H; a.L = p->L; a.C = p->C; a.c_pad = p->c_pad; a.k = p->k; a.cwords = p->cwords; a.prefix = p->prefix_mode;
-    a.tiles_per_head = (p->L + kLongRows - 1) / kLongRows;
-    a.n_units = p->H * a.tiles_per_head;
+    a.H = p->H; a.L = p->L; a.C = p->C; a.c_pad = p->c_pad; a.ncol = p->ncol; a.k = p->k; a.cwords = p->cwords; a.prefix = p->prefix_mode;
+    a.n_units = p->H * ((p->L + kLongRows - 1) / kLongRows);
     a.d_rows = std::min(p->c_pad, kLongStep);
     a.tile_off = ws_ptr<int>(ws, p->ws.tile_off);
     a.cookie = p->cookie;

@@ -1,5 +1,9 @@
 """Routing with many picks per query (csrc/moc_route_long.cu): the picks against the oracle at the edges of its sizes, and where counting
 by a threshold is hard: equal scores, chunks that repeat, rows with few candidates, scores that are not normally distributed."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -95,3 +99,39 @@ def test_scores_far_from_normal():
             x["k"][:, off[c]:off[c + 1]] *= 2.0 ** (2 - 7 * c % 9)
     wl = ragged(1, 128, 400, 4, 70)
     check(routed(wl, spread))
+
+
+def blank(wl):
+    """Every tenth chunk's keys zero, and scores about a negative mean: the k-th largest is often a zero, or close to it."""
+    def spoil(x):
+        x["q"] += 0.25
+        x["k"] -= 0.25
+        off = np.asarray(wl.layout.chunk_off)
+        for c in range(3, wl.n_chunks, 10):
+            x["k"][:, off[c]:off[c + 1]] = 0
+    return spoil
+
+
+BLANK = [(64, 300, 20), (128, 300, 28), (128, 400, 60), (64, 504, 118), (128, 1000, 20), (64, 1100, 52), (128, 1300, 118), (128, 700, 130)]
+
+
+@pytest.mark.parametrize("d,n_chunks,k", BLANK)
+def test_some_chunks_are_blank(d, n_chunks, k):
+    wl = ragged(2, d, n_chunks, 4, k)
+    check(routed(wl, blank(wl)))
+
+
+def test_debug_build_finds_every_survivor_where_it_was_counted():
+    """The build with -DMOC_DEBUG compares what a thread stores with what it counted.  (In a child process: a process loads one variant.)"""
+    code = ("import sys; sys.path[:0] = %r\n"
+            "import test_gpu_route_long as T\n"
+            "from paper_2508_21058_b200 import lib_path\n"
+            "assert lib_path().endswith('libmoc_debug.so')\n"
+            "for d, n, k in T.BLANK:\n"
+            "    wl = T.ragged(2, d, n, 4, k)\n"
+            "    T.routed(wl, T.blank(wl))\n"
+            "print('DEBUG_BUILD_OK')\n") % [PU.ROOT, os.path.join(PU.ROOT, "tests")]
+    from paper_2508_21058_b200 import build as libbuild
+    libbuild.build(debug=True)
+    res = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, env=dict(os.environ, MOC_LIBRARY="debug"), timeout=600)
+    assert res.returncode == 0 and "DEBUG_BUILD_OK" in res.stdout, res.stdout[-2000:] + res.stderr[-4000:]
