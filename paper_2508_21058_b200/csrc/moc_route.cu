@@ -1115,15 +1115,16 @@ static int launch_route_d(const moc_plan *p, const __nv_bfloat16 *Q, const float
         a.cap_total = (size_t)p->cap_off[p->C];
         a.tile_off = ws_ptr<int>(ws, p->ws.tile_off);
         a.cookie = p->cookie;
+        constexpr int kMost = 227 * 1024 - 512;      // what an SM has, less the kernel's static variables (the attribute is the same for every plan, as above)
         const size_t q_tile = (size_t)kRtRows * D * 2, d_block = ((size_t)3 * a.d_rows * D * 2 + 1023) & ~(size_t)1023;
         a.ctas_per_head = std::max(1, std::min(p->n_sm / p->H, a.tiles_per_head));
         const unsigned grid = (unsigned)(p->H * a.ctas_per_head);
         // Four selection groups with few chunks (more warps to hide the selection's latencies), two otherwise.
         const int ng = few ? 4 : 2;
-                // one histogram per group, the list offsets, and one byte per unit of a CTA
+        // one histogram per group, the list offsets, and one byte per unit of a CTA
         const size_t hist = (ng * (p->k <= 8 && p->C <= kRtDeferredChunks ? 4 : 1) + 1) * sizeof(int) * (size_t)p->C + sizeof(int) * (size_t)p->ncol +
                             4 * (size_t)(a.tiles_per_head / a.ctas_per_head + 16),
-                     budget = 227 * 1024 - 1024 - 512;      // what an SM has, less the alignment slack and the kernel's static variables
+                     budget = kMost - 1024;     // less the slack that aligns the tiles
         if (d_block + q_tile + hist > budget) return MOC_ERR_SHAPE;
         // threshold selection (not the few-chunk case): survivor slots per row, as many as fit beside two Q stages
         // (too few: the best-first extraction alone is used)
@@ -1148,7 +1149,7 @@ static int launch_route_d(const moc_plan *p, const __nv_bfloat16 *Q, const float
         if (int r = make_tmap_2d_bf16(&tmD, desc3, (uint64_t)p->H * 3 * p->c_pad, D, (uint32_t)a.d_rows)) return r;
 #define MOC_ROUTE_CASE(KM, NG, FW)                                                                                          \
     do {                                                                                                                \
-        MOC_CUDA_TRY(cudaFuncSetAttribute(route_tc_kernel<D, KM, NG, FW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+        MOC_CUDA_TRY(cudaFuncSetAttribute(route_tc_kernel<D, KM, NG, FW>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost)); \
         route_tc_kernel<D, KM, NG, FW><<<grid, rt_threads(NG), smem, s>>>(tmQ, tmD, a);                                     \
     } while (0)
         if (p->k <= 4) { if (few) MOC_ROUTE_CASE(4, 4, true); else MOC_ROUTE_CASE(4, 2, false); }

@@ -585,9 +585,13 @@ __global__ void __launch_bounds__(kLongThreads, 1) route_long_kernel(const __gri
     finish_route(p.status, p.cnt, p.tile_off, p.H * p.C, p.cookie, kLongThreads);
 }
 
+// What an SM has, less the kernel's static variables.  The attribute is the same for every plan: another thread's call may come between it and the
+// launch, and with the size of a plan of fewer chunks the launch would fail.
+constexpr int kLongMost = 227 * 1024 - 11 * 1024;
+
 template <int D, int N>
-static int route_long_n(const moc_plan *p, const RouteLongParams &a, const CUtensorMap &tmQ, const CUtensorMap &tmD, unsigned grid, size_t smem, cudaStream_t s) {
-    MOC_CUDA_TRY(cudaFuncSetAttribute(route_long_kernel<D, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+static int route_long_n(const RouteLongParams &a, const CUtensorMap &tmQ, const CUtensorMap &tmD, unsigned grid, size_t smem, cudaStream_t s) {
+    MOC_CUDA_TRY(cudaFuncSetAttribute(route_long_kernel<D, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, kLongMost));
     route_long_kernel<D, N><<<grid, kLongThreads, smem, s>>>(tmQ, tmD, a);
     MOC_LAUNCH_CHECK();
     return MOC_OK;
@@ -622,7 +626,7 @@ static int route_long_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bf
     const bool one = p->c_pad <= kLongStep * kLongAcc;
     const int want = std::min(p->k <= (one ? 28 : 20) ? 32 : p->k <= (one ? 60 : 52) ? 64 : p->k <= 120 ? 128 : p->k <= 240 ? 256 : 512, p->c_pad);
     const int n = want <= 32 ? 1 : want <= 64 ? 2 : want <= 128 ? 4 : want <= 256 ? 8 : 16;
-    const size_t budget = 227 * 1024 - 1024 - 11 * 1024;    // what an SM has, less the alignment slack and the kernel's static variables
+    const size_t budget = kLongMost - 1024;     // less the slack that aligns the tiles
     const size_t q_tile = (size_t)kLongRows * D * 2, slot = ((size_t)a.d_rows * D * 2 + 1023) & ~(size_t)1023;
     const size_t row_queue = (32 * n + 1) * 4 + (32 * n + 2) * 2, queue = n <= kQueueShared ? kLongRows * row_queue : 0, hist = sizeof(int) * (size_t)p->C;
     a.hists = q_tile + slot + queue + 2 * hist <= budget ? 2 : 1;
@@ -640,11 +644,11 @@ static int route_long_d(const moc_plan *p, const __nv_bfloat16 *Q, const __nv_bf
     if (int r = make_tmap_2d_bf16(&tmQ, Q, (uint64_t)p->H * p->L, D, kLongRows)) return r;
     if (int r = make_tmap_2d_bf16(&tmD, desc3, (uint64_t)p->H * 3 * p->c_pad, D, (uint32_t)a.d_rows)) return r;
     switch (n) {
-        case 1: return route_long_n<D, 1>(p, a, tmQ, tmD, grid, smem, s);
-        case 2: return route_long_n<D, 2>(p, a, tmQ, tmD, grid, smem, s);
-        case 4: return route_long_n<D, 4>(p, a, tmQ, tmD, grid, smem, s);
-        case 8: return route_long_n<D, 8>(p, a, tmQ, tmD, grid, smem, s);
-        default: return route_long_n<D, 16>(p, a, tmQ, tmD, grid, smem, s);
+        case 1: return route_long_n<D, 1>(a, tmQ, tmD, grid, smem, s);
+        case 2: return route_long_n<D, 2>(a, tmQ, tmD, grid, smem, s);
+        case 4: return route_long_n<D, 4>(a, tmQ, tmD, grid, smem, s);
+        case 8: return route_long_n<D, 8>(a, tmQ, tmD, grid, smem, s);
+        default: return route_long_n<D, 16>(a, tmQ, tmD, grid, smem, s);
     }
 }
 

@@ -5,6 +5,7 @@ import ctypes
 import os
 import subprocess
 import sys
+import threading
 
 import numpy as np
 import pytest
@@ -315,3 +316,40 @@ def test_plans_are_made_in_every_context_of_the_device():
     for n in ("desc", "sel"):
         assert torch.equal(getattr(before, n), getattr(after, n)), n
     assert float((before.O.float() - after.O.float()).abs().max()) <= 1e-2          # the same rows, grouped into other tiles
+
+
+@pytest.mark.parametrize("k,calls", [(4, 20000), (40, 3000)])
+def test_plans_of_different_sizes_route_from_several_threads(k, calls):
+    """One kernel serves plans whose tables take different amounts of shared memory; a thread's call may come between another's
+    preparation and its launch.  (With the size of the plan as the kernel's attribute one launch in 6000 failed.)"""
+    runs, failed = [], []
+    for n_chunks in (60, 60, 600, 600):
+        lay = W.Layout(np.arange(n_chunks + 1, dtype=np.int32), np.zeros(n_chunks, np.int32), (np.arange(n_chunks) == 0).astype(np.uint8))
+        wl = W.Workload("threads", 1, 64, lay, k, 0, 0)
+        plan, x = MocPlan.from_workload(wl), W.generate(wl, "cuda", ("q", "k"))
+        ws, desc = plan.new_workspace(), torch.empty((1, plan.C, 64), dtype=torch.float32, device="cuda")
+        sel = torch.empty((1, plan.L, k), dtype=torch.int32, device="cuda")
+        plan.moc_chunk_pool(x["k"], desc, ws)
+        plan.moc_route(x["q"], desc, sel, ws)
+        runs.append((plan, x["q"], desc, sel, ws, sel.clone()))
+    torch.cuda.synchronize()
+
+    def many(plan, q, desc, sel, ws, _):
+        stream = torch.cuda.Stream()
+        args = (plan._h, *(t.data_ptr() for t in (q, desc, sel, ws)), stream.cuda_stream)
+        for n in range(calls):
+            code = plan._lib.moc_route(*args)                    # (as bare as can be: the threads shall meet inside the call)
+            if code:
+                failed.append((n, code))
+            if n % 256 == 0:
+                stream.synchronize()
+
+    threads = [threading.Thread(target=many, args=r) for r in runs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not failed
+    for plan, q, desc, sel, ws, want in runs:
+        assert plan.moc_get_status(ws)[0] == 0 and torch.equal(sel, want)

@@ -155,3 +155,13 @@ def test_dq_rows_are_dealt_evenly_to_the_blocks(chunk):
                 pos = (pos + step) % grid
         assert sorted(seen) == list(range(2 * items))
         assert max(load) <= 1.03 * sum(load) / grid + 2
+
+
+@pytest.mark.parametrize("name", ["moc_route.cu", "moc_route_long.cu", "moc_regularise.cu"])
+def test_shared_memory_limits_are_the_same_for_every_plan(name):
+    """Kernels whose tables depend on the plan: the limit that is set before a launch is a constant, so that it does not matter
+    whose call set it last."""
+    with open(os.path.join(ROOT, "paper_2508_21058_b200", "csrc", name)) as f:
+        text = f.read()
+    limits = re.findall(r"cudaFuncAttributeMaxDynamicSharedMemorySize, (.*?)\)\)?;", text)
+    assert limits and all(re.search(rf"constexpr int {re.escape(x)} = [\d\s*+-]+;", text) for x in limits), limits
