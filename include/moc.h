@@ -211,7 +211,8 @@ int moc_get_status(const moc_plan *plan, const void *ws, void *stream, int *devi
  *   scores     = <x_g, phi(Psi_s)> for every shot ([H][S], fp32); shot_desc [H][S][d] fp32;
  *   sel_shot   = [H][top_m] int32: the top_m best shots among those that END before the block begins (a
  *                shot holding a token >= q_tok0 is not history), best first, equal scores to the earlier
- *                shot, -1 padded.  ws: scratch of moc_workspace_bytes (its pooling area is used). */
+ *                shot, -1 padded.  ws: scratch of moc_workspace_bytes (its pooling area is used).
+ * MOC_ERR_SHAPE with more than 12160 shots (d = 128) or 12224 (d = 64). */
 int moc_outer_num_shots(const moc_plan *plan, int32_t *n_shots);
 int moc_outer_route(const moc_plan *plan, const void *Xq, const float *desc, int32_t q_tok0, int32_t q_tok1, int32_t top_m,
                     float *shot_desc, float *scores, int32_t *sel_shot, void *ws, void *stream);

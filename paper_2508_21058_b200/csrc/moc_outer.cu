@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(256) block_sum_kernel(const __nv_bfloat16 *__r
 // each term and each candidate waited for: 8 shots of 22 chunks, a block of 33k queries, this launch and
 // the one before 36.9 -> 21.5 us; 12 shots of 7 chunks 27.7 -> 16.5.)
 constexpr int kScoreShots = 8;
+constexpr int most_shots(int d) { return (48 * 1024 - 4 * d) / 4; }      // whose scores a block keeps in shared memory, as the header states
 template <int D>
 __global__ void __launch_bounds__(D *kScoreShots) outer_score_kernel(const float *__restrict__ part, const float *__restrict__ desc,
                                                         const int32_t *__restrict__ off, const KeyRange *__restrict__ shot_chunks,
@@ -126,6 +127,16 @@ __global__ void __launch_bounds__(D *kScoreShots) outer_score_kernel(const float
     }
 }
 
+// (The scores and the kernel's own 4.6 KB may be more than a block gets unasked.  The limit is the same for every call: another thread's may come between.)
+template <int D>
+static int start_score(unsigned H, cudaStream_t s, const float *part, const float *desc, const int32_t *off, const KeyRange *shot_chunks, float *shot_desc,
+                       float *scores, int32_t *sel, int C, int S, int n_slices, int q0, int q1, int M) {
+    const size_t smem = sizeof(float) * (size_t)S;
+    if (smem > 40 * 1024) MOC_CUDA_TRY(cudaFuncSetAttribute(outer_score_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * most_shots(D)));
+    outer_score_kernel<D><<<H, D * kScoreShots, smem, s>>>(part, desc, off, shot_chunks, shot_desc, scores, sel, C, S, n_slices, q0, q1, M);
+    return MOC_OK;
+}
+
 template <int D>
 __global__ void __launch_bounds__(256) gather_rows_kernel(const __nv_bfloat16 *__restrict__ X, const int32_t *__restrict__ tok_map,
                                                           __nv_bfloat16 *__restrict__ out, int L, int n_out) {
@@ -162,24 +173,17 @@ extern "C" int moc_outer_route(const moc_plan *p, const void *Xq, const float *d
     if (!ws) return MOC_ERR_WORKSPACE;
     if (!aligned(ws, 256)) return MOC_ERR_ALIGN;
     const int S = (int)p->shot_chunks.size();
-    if (q_tok0 < 0 || q_tok1 <= q_tok0 || q_tok1 > p->L || top_m < 0 || top_m > S) return MOC_ERR_SHAPE;
+    if (q_tok0 < 0 || q_tok1 <= q_tok0 || q_tok1 > p->L || top_m < 0 || top_m > S || S > most_shots(p->d)) return MOC_ERR_SHAPE;
     cudaStream_t s = (cudaStream_t)stream;
     const int n_slices = (q_tok1 - q_tok0 + kPoolSlice - 1) / kPoolSlice;      // never more than the pooling units
     float *part = ws_ptr<float>(ws, p->ws.pool_part);
     const __nv_bfloat16 *X = static_cast<const __nv_bfloat16 *>(Xq);
     const dim3 grid((unsigned)n_slices, (unsigned)p->H);
-    const size_t smem = sizeof(float) * (size_t)S;
-    if (p->d == 128) {
-        block_sum_kernel<128><<<grid, 256, 0, s>>>(X, part, p->L, q_tok0, q_tok1, n_slices);
-        MOC_LAUNCH_CHECK();
-        outer_score_kernel<128><<<(unsigned)p->H, 128 * kScoreShots, smem, s>>>(part, desc, p->d_off, p->d_shot_chunks, shot_desc, scores, sel_shot,
-                                                                 p->C, S, n_slices, q_tok0, q_tok1, top_m);
-    } else {
-        block_sum_kernel<64><<<grid, 256, 0, s>>>(X, part, p->L, q_tok0, q_tok1, n_slices);
-        MOC_LAUNCH_CHECK();
-        outer_score_kernel<64><<<(unsigned)p->H, 64 * kScoreShots, smem, s>>>(part, desc, p->d_off, p->d_shot_chunks, shot_desc, scores, sel_shot,
-                                                               p->C, S, n_slices, q_tok0, q_tok1, top_m);
-    }
+    if (p->d == 128) block_sum_kernel<128><<<grid, 256, 0, s>>>(X, part, p->L, q_tok0, q_tok1, n_slices);
+    else block_sum_kernel<64><<<grid, 256, 0, s>>>(X, part, p->L, q_tok0, q_tok1, n_slices);
+    MOC_LAUNCH_CHECK();
+    const auto start = p->d == 128 ? start_score<128> : start_score<64>;
+    if (int r = start((unsigned)p->H, s, part, desc, p->d_off, p->d_shot_chunks, shot_desc, scores, sel_shot, p->C, S, n_slices, q_tok0, q_tok1, top_m)) return r;
     MOC_LAUNCH_CHECK();
     return MOC_OK;
 }

@@ -1,8 +1,9 @@
 """Scores of whole shots: as many as a block takes at a time, one more, one fewer, and several times as many."""
+import numpy as np
 import pytest
 import torch
 
-from paper_2508_21058_b200 import MocPlan
+from paper_2508_21058_b200 import MocError, MocPlan
 from paper_2508_21058_b200 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -27,3 +28,26 @@ def test_every_shot(shots, caption, frames, d):
     assert float((scores - (want * xg[:, None]).sum(2)).abs().max()) < 4 * (n + d) * 2 ** -24
     left = scores[:, :M].clone()                             # the block is the last shot
     assert torch.equal(sel.long(), torch.argsort(left, dim=1, descending=True, stable=True))
+
+
+@pytest.mark.parametrize("d,most", [(64, 12224), (128, 12160)])
+def test_as_many_shots_as_the_header_states(d, most):
+    """Shots of one token.  One more than the limit is refused before anything is written."""
+    for S in (most, most + 1):
+        lay = W.Layout(np.arange(S + 1, dtype=np.int32), np.arange(S, dtype=np.int32), np.zeros(S, np.uint8))
+        plan = MocPlan.from_workload(W.Workload("shots", 1, d, lay, 1, 0, 0))
+        x = torch.randn(1, S, d, device="cuda", generator=torch.Generator("cuda").manual_seed(d)).bfloat16()
+        ws, desc, M = plan.new_workspace(), x.float(), 5
+        shot_desc, scores, sel = torch.full((1, S, d), 7.0, device="cuda"), torch.full((1, S), 7.0, device="cuda"), torch.full((1, M), 7, dtype=torch.int32, device="cuda")
+        if S > most:
+            ws.fill_(9)
+            with pytest.raises(MocError) as e:
+                plan.moc_outer_route(x, desc, S - 300, S, M, shot_desc, scores, sel, ws)
+            torch.cuda.synchronize()
+            assert e.value.code == -2 and all(bool((t == 7).all()) for t in (shot_desc, scores, sel)) and bool((ws == 9).all())
+            continue
+        plan.moc_outer_route(x, desc, S - 300, S, M, shot_desc, scores, sel, ws)
+        want = (x[0].double() * x[0, S - 300:].double().mean(0)).sum(1)
+        # means of 300 terms and sums of d products of size about 1 in fp32, half an ulp each
+        assert torch.equal(shot_desc, desc) and float((scores[0] - want).abs().max()) < (300 + d) * 2 ** -22
+        assert torch.equal(sel[0].long(), torch.argsort(scores[0, :S - 300], descending=True, stable=True)[:M])
