@@ -64,6 +64,7 @@ def load_library():
     lib.moc_debug_use_cuda_core_attention.argtypes = [vp, i32]
     lib.moc_debug_set_wait_limit_us.argtypes = [vp, C.c_uint]
     lib.moc_debug_wait_probe.argtypes = [vp, vp, i32, vp]
+    lib.moc_debug_wait_probe_form.argtypes = [vp, vp, i32, i32, vp]
     lib.moc_debug_shared_key_tiles.argtypes = [C.POINTER(_Problem), i32, i32, C.POINTER(i32), vp, vp, C.POINTER(sz)]
     lib.moc_attend.argtypes = [vp] * 9
     lib.moc_attend_bwd.argtypes = [vp] * 13
@@ -230,8 +231,8 @@ class MocPlan:
     def debug_set_wait_limit_us(self, us: int):
         _check(self._lib.moc_debug_set_wait_limit_us(self._h, int(us)))
 
-    def debug_wait_probe(self, ws, code: int):
-        _check(self._lib.moc_debug_wait_probe(self._h, _ptr(ws), int(code), _stream()))
+    def debug_wait_probe(self, ws, code: int, form: int = 0):
+        _check(self._lib.moc_debug_wait_probe_form(self._h, _ptr(ws), int(form), int(code), _stream()))
 
     # convenience: allocate outputs and run the forward path
     def forward(self, Q, K, V, ws=None):

@@ -98,15 +98,6 @@ struct SlotIter {
     }
 };
 
-// a bounded wait on a counter in global memory (another CTA adds to it); a look takes half a microsecond or more
-__device__ __forceinline__ bool wait_count(const int *ctr, int need, volatile int *abort_flag, const WaitBound &bound, int code) {
-    for (uint32_t it = 0; *(volatile const int *)ctr < need;) {
-        __nanosleep(200);
-        if (++it > 2 * bound.us) return gave_up(abort_flag, code);
-    }
-    return true;
-}
-
 // acc += w x (the bf16 pair u) where cond holds
 __device__ __forceinline__ void add_weighted_if(bool cond, uint64_t &acc, uint32_t u, float w) {
     const uint64_t v = pack2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u)), w2 = pack2(w, w);

@@ -20,13 +20,14 @@ enum StatusWord { ST_STATUS = 0, ST_DETAIL = 1, ST_COOKIE = 2, ST_ARRIVE = 4 };
 constexpr int kQueueHeader = 4;     // queue area: [0] next item to claim, [1] items, [2] phases, [3] CTAs that have left; then 3 ints per phase
 constexpr unsigned kPrivFlagCudaCoreAttend = 0x80000000u;   // plan flag outside the public header: test hook
 
-// How often a kernel's waits look before they give up: about a second's worth, or `us` microseconds' (tests; never more than the default).
+// How often a kernel's waits look before they give up: one to two seconds' worth, or one to two times `us` microseconds' (tests; never more than the
+// default).  Measured with waits that nothing ends (moc_debug_wait_probe_form): a look takes 32.8 us where the thread parks, 86 ns
+// where it polls (46 in a loop of nothing else), 257 to 512 ns where it looks at a counter in global memory; the default is 2.05, 1.4 and 1 to 2 s.
 struct WaitBound {
-    uint32_t parked, polled;
-    uint32_t us;
+    uint32_t parked, polled, looks;
     static WaitBound of(unsigned us) {
         if (us == 0 || us > 1000000u) us = 1000000u;
-        return WaitBound{us / 4 + 1, us * 32u, us};
+        return WaitBound{us / 16 + 1, us * 16u, us * 4u};
     }
 };
 
@@ -283,8 +284,9 @@ int moc_debug_use_cuda_core_attention(moc_plan *plan, int on);
 // limit of every bounded device-side wait, in microseconds, of the launches from now on (0 = default)
 int moc_debug_set_wait_limit_us(moc_plan *plan, unsigned us);
 // one block whose only wait is on a barrier that nothing ever arrives on: it must give up after the limit,
-// record MOC_ERR_TIMEOUT with detail `code` in ws, and return
-int moc_debug_wait_probe(const moc_plan *plan, void *ws, int code, void *stream);
+// record MOC_ERR_TIMEOUT with detail `code` in ws, and return.  `form`: 0 the wait parks, 1 it polls, 2 it looks at a counter in global memory
+int moc_debug_wait_probe_form(const moc_plan *plan, void *ws, int form, int code, void *stream);
+int moc_debug_wait_probe(const moc_plan *plan, void *ws, int code, void *stream);      // form 0
 // host only: the long key tiles of dK/dV of a problem on a GPU with n_sm SMs (up to cap of them written): tiles of query rows that
 // a tile has whatever is picked, and blocks that share them; and the bytes there are for the counters of all heads' tiles
 int moc_debug_shared_key_tiles(const moc_problem *problem, int n_sm, int cap, int *n_tiles, int *query_tiles, int *blocks, size_t *counter_room);

@@ -37,11 +37,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Every wait is bounded, by a number of polls (WaitBound): some 4 us each where the thread is parked (measured, whatever the hint above says beyond
-// that), 16 ns and more where it polls.  The first wait of a CTA to run out leaves its code in the CTA's abort flag, which the CTA reports
-// when it leaves (report_abort).  There are some forty waits in a kernel, and the loops of its warps share an instruction cache: what stands
-// behind each is as short as can be.  (With a clock, the limit read from the workspace and the report at every wait the forward kernels were 20 KB
-// longer: 264k tokens in 256-token chunks, 2 heads, 3.89 -> 4.23 ms; 33k-token clip at d = 64 1.20 -> 1.29; its backward 3.59 -> 3.62.)
+// Every wait is bounded, by a number of polls (WaitBound).  The first wait of a CTA to run out leaves its code in the CTA's abort flag, which the CTA
+// reports when it leaves (report_abort); its other waits run out by themselves, so that a CTA that is stuck leaves within a few seconds.  There are
+// some forty waits in a kernel, and the loops of its warps share an instruction cache: what stands behind each is as short as
+// can be.  (With a clock, the limit read from the workspace and the report at every wait the forward kernels were 20 KB
+// longer: 264k tokens in 256-token chunks, 2 heads, 3.89 -> 4.23 ms; 33k-token clip at d = 64 1.20 -> 1.29; its backward 3.59 -> 3.62.  With nothing but a look
+// at the flag beside the limit, 6 heads in 512-token chunks, the whole forward, 18.83 -> 19.10 ms, in 256-token chunks 14.28 -> 14.56; in the
+// parked waits alone 19.30 and 14.41; with 32 bits of the clock besides 19.7 and 14.95.)
 __device__ __forceinline__ bool gave_up(volatile int *abort_flag, int code) {
     if (*abort_flag == 0) *abort_flag = code;
     return false;
@@ -71,6 +73,15 @@ __device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity) {
 __device__ __forceinline__ bool mbar_wait_spin(uint32_t bar, uint32_t parity, volatile int *abort_flag, const WaitBound &bound, int code) {
     for (uint32_t it = 0; !mbar_test_wait(bar, parity);)
         if (++it > bound.polled) return gave_up(abort_flag, code);
+    return true;
+}
+
+// The same for a counter in global memory that another CTA adds to.
+__device__ __forceinline__ bool wait_count(const int *ctr, int need, volatile int *abort_flag, const WaitBound &bound, int code) {
+    for (uint32_t it = 0; *(volatile const int *)ctr < need;) {
+        __nanosleep(200);
+        if (++it > bound.looks) return gave_up(abort_flag, code);
+    }
     return true;
 }
 

@@ -196,6 +196,22 @@ def test_a_wait_that_runs_out_is_reported_and_the_gpu_stays_usable():
     assert float((run.O.float() - O0.float()).abs().max()) <= 1e-2
 
 
+@pytest.mark.parametrize("form", [0, 1, 2])
+def test_every_form_of_wait_gives_up_after_its_limit(form):
+    """A wait that parks, one that polls, one on a counter, each for something that never comes, with a limit of 4 ms."""
+    run = PU.GpuRun(W.workload("mini2")).forward()
+    run.plan.debug_set_wait_limit_us(4000)
+    for code in (700, 701):                                      # (the first call loads the kernel)
+        run.ws[:64] = 0
+        t0, t1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        t0.record()
+        run.plan.debug_wait_probe(run.ws, code, form)
+        t1.record()
+        torch.cuda.synchronize()
+        assert run.plan.moc_get_status(run.ws) == (ERR_TIMEOUT, code)
+    assert 3.5 <= t0.elapsed_time(t1) <= 20.0                    # once to twice the limit as measured, and room for another clock
+
+
 def test_workspace_budget_groups_heads_and_results_do_not_change():
     wl = W.workload("mini2")
     wl.n_heads = 5
