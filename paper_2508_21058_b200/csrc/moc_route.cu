@@ -672,7 +672,8 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                     // down from slot cap - 1.  A survivor is stored while its stream's cursor is inside the queue and the
                     // cursor moves whether it was stored or not, so the count stays exact; the two streams have run into
                     // each other (or out of the queue) exactly when the counts add up to more than cap.  The stores are
-                    // predicated instructions, written out so that no branch is made of them.
+                    // predicated instructions, written out so that no branch is made of them; they compare as the maxima above
+                    // were taken, subnormal numbers as zero (or a row of nothing else would lose picks).
                     const uint32_t q_v = smem_u32(sv), q_j = smem_u32(sj);
                     uint32_t lo_v = q_v, lo_j = q_j, hi_v = q_v + (cap - 1) * 512, hi_j = q_j + (cap - 1) * 128;
                     const uint32_t lo_end = q_v + cap * 512;
@@ -700,7 +701,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                             for (int c = 0; c < 32; ++c) {
                                 asm volatile(
                                     "{\n\t.reg .pred p, q;\n\t"
-                                    "setp.ge.f32 p, %3, %4;\n\t"
+                                    "setp.ge.ftz.f32 p, %3, %4;\n\t"
                                     "setp.lt.and.u32 q, %0, %5, p;\n\t"
                                     "@q st.shared.f32 [%0], %3;\n\t"
                                     "@q st.shared.u8 [%1], %2;\n\t"
@@ -711,7 +712,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                                     : "memory");
                                 asm volatile(
                                     "{\n\t.reg .pred p, q;\n\t"
-                                    "setp.ge.f32 p, %3, %4;\n\t"
+                                    "setp.ge.ftz.f32 p, %3, %4;\n\t"
                                     "setp.ge.and.s32 q, %0, %5, p;\n\t"
                                     "@q st.shared.f32 [%0], %3;\n\t"
                                     "@q st.shared.u8 [%1], %2;\n\t"
@@ -726,7 +727,7 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                             for (int c = 0; c < 32; ++c)
                                 asm volatile(
                                     "{\n\t.reg .pred p, q;\n\t"
-                                    "setp.ge.f32 p, %3, %4;\n\t"
+                                    "setp.ge.ftz.f32 p, %3, %4;\n\t"
                                     "setp.lt.and.u32 q, %0, %5, p;\n\t"
                                     "@q st.shared.f32 [%0], %3;\n\t"
                                     "@q st.shared.u8 [%1], %2;\n\t"
