@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(kBwdThreads, 1) attend_dkv_tc_kernel(const __g
                         to[x * 256] = make_float4(__uint_as_float(f[0]), __uint_as_float(f[1]), __uint_as_float(f[2]), __uint_as_float(f[3]));
                     }
                 }
-                // (the lane threads' own two barriers, once more: every wait here is bounded)
+                // (two barriers of the lane threads that serve here alone, once a block, and not a __syncthreads of theirs: every wait here is bounded)
                 mbar_arrive(bar(RD1));
                 ok = mbar_wait_spin(bar(RD1), 0, abort_flag, p.wait, BW_READ);
                 if (threadIdx.x == 0 && ok) {

@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(kDqThreads, 1) attend_dq_tc_kernel(const __gri
 #pragma unroll
                         for (int ks = 0; ks < 8; ++ks)
                             if (ks < steps)                  // dS of 32 keys lies over the first half of their T2 columns
-                            mma_ts_elect(tmem + 256, ds + (ks >> 1) * 32 + (ks & 1) * 8, lo(km) + s3 * STAGE + ks * (2048 >> 4), hi(km), IDESC_ACC, j > 0 || ks > 0);
+                                mma_ts_elect(tmem + 256, ds + (ks >> 1) * 32 + (ks & 1) * 8, lo(km) + s3 * STAGE + ks * (2048 >> 4), hi(km), IDESC_ACC, j > 0 || ks > 0);
                         tc_commit_elect(bar(K_EMPTY + s3));
                         if (++s3 == kKStages) s3 = 0;
                         if (j + 2 < n_tiles) t2(g + 2, j + 3 == n_tiles);

@@ -775,31 +775,27 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                         // time, which always fit, until 4 k have been seen, then 64.  (Taken best first, as pairs of blocks whose
                         // survivors do not fit still are, the first 64 columns cost two thirds of the selection: up to k rounds of 350
                         // instructions a block.)
-                        int b0 = 0;
-                        if constexpr (KMAX == 32) {
-                            if (sb == 0) {
-                                uint32_t v[32];
-                                uint64_t key[32];
-                                tmem_ld32(acc, v);
-                                const uint32_t cand = cand_bits(0);
-                                tmem_wait_ld();
+                        // (Such lists are kept with at most 144 columns, which are one step: route_is_long.)
+                        uint32_t v[32];
+                        uint64_t key[32];
+                        tmem_ld32(acc, v);
+                        const uint32_t cand = cand_bits(0);
+                        tmem_wait_ld();
 #pragma unroll
-                                for (int c = 0; c < 32; ++c) key[c] = score_key(((cand >> c) & 1u) ? __uint_as_float(v[c]) : -INFINITY, c);
-                                sort32(key);
+                        for (int c = 0; c < 32; ++c) key[c] = score_key(((cand >> c) & 1u) ? __uint_as_float(v[c]) : -INFINITY, c);
+                        sort32(key);
 #pragma unroll
-                                for (int x = 0; x < 32; ++x) {
-                                    const bool some = (uint32_t)(key[x] >> 32) != kNoScore;
-                                    top.s[x] = some ? key_score(key[x]) : -INFINITY;
-                                    top.j[x] = some ? (int)~(uint32_t)key[x] : -1;
-                                }
-                                update_kth();
-                                b0 = 1;
-                            }
+                        for (int x = 0; x < KR; ++x) {
+                            const bool some = (uint32_t)(key[x] >> 32) != kNoScore;
+                            top.s[x] = some ? key_score(key[x]) : -INFINITY;
+                            top.j[x] = some ? (int)~(uint32_t)key[x] : -1;
                         }
+                        update_kth();
+                        int b0 = 1;
 #pragma unroll 1
                         while (b0 < nblk) {
                             thr = fmaxf(kth, -FLT_MAX);
-                            const bool two = b0 + 1 < nblk && jb + b0 * 32 >= 4 * kp;
+                            const bool two = b0 + 1 < nblk && b0 * 32 >= 4 * kp;
                             scan(b0 * 32, (b0 + 1) * 32, two);
                             if (!drain()) extract_blocks(b0 * 32, min(rows_sb, (b0 + 1 + two) * 32));
                             b0 += 1 + two;
