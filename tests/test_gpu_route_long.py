@@ -56,6 +56,39 @@ def test_every_length_of_list(k):
     check(routed(ragged(1, 64 if k % 2 else 128, 300 if k <= 240 else 600, 5, k)))
 
 
+# (survivors that are kept, by picks: 32, 64, 128, 256, 512; the first two lines lie elsewhere with more than 512 columns)
+@pytest.mark.parametrize("n_chunks,k", [(300, 20), (300, 21), (300, 28), (300, 29), (300, 52), (300, 53), (300, 60), (300, 61), (600, 20), (600, 21), (600, 28), (600, 29),
+                                        (600, 52), (600, 53), (600, 60), (600, 61), (600, 120), (600, 121), (600, 240), (600, 241)])
+def test_every_number_of_survivors(n_chunks, k):
+    check(routed(ragged(1, 128 if k % 2 else 64, n_chunks, 5, k)))
+
+
+def test_one_table_of_counters():
+    """So many chunks that the pick counters of a single unit fit beside the survivors; some blocks have two units and some one.  The picks against
+    scores in 64 bits, the lists against those made from the selection."""
+    H, C, k, d = 4, 7200, 118, 128
+    lay = W.Layout(np.arange(C + 1, dtype=np.int32), np.zeros(C, np.int32), (np.arange(C) == 0).astype(np.uint8))
+    run = PU.GpuRun(W.Workload("many chunks", H, d, lay, k, 0, 0)).forward()
+    sel, idx = run.sel.long(), torch.arange(C, device="cuda")
+    for h in range(H):
+        score = run.x["q"][h].double() @ run.desc[h].double().T
+        score.masked_fill_((idx[None] >= idx[:, None]) | (idx[None] == 0), -torch.inf)      # earlier chunks, but not the caption
+        want = (idx - 1).clamp(0, k)
+        assert torch.equal((sel[h] >= 0).sum(1), want)
+        mine = torch.where(sel[h] >= 0, score.gather(1, sel[h].clamp(min=0)), torch.inf)
+        kth = torch.where(want > 0, score.sort(1, descending=True).values.gather(1, (want - 1).clamp(min=0)[:, None])[:, 0], -torch.inf)
+        assert bool((mine >= kth[:, None] - PU.NEAR_TIE).all())                               # none that is not among the largest
+        ordered = sel[h].masked_fill(sel[h] < 0, C).sort(1).values
+        assert bool(((ordered[:, 1:] > ordered[:, :-1]) | (ordered[:, 1:] == C)).all())       # none twice
+        live = (sel[h, :, 1:] >= 0)
+        assert bool((mine[:, :-1] >= mine[:, 1:] - PU.NEAR_TIE)[live].all())                  # best first
+    O, lse, before = run.O.clone(), run.lse.clone(), run.sel.clone()
+    run.plan.moc_lists_from_sel(run.sel, run.ws)
+    run.attend_only()
+    assert torch.equal(run.sel, before)
+    assert float((run.O.float() - O.float()).abs().max()) <= 1e-2 and float((run.lse - lse).abs().max()) <= 1e-3      # the same rows, grouped into other tiles
+
+
 @pytest.mark.parametrize("n_chunks,k", [(18, 33), (34, 40), (50, 40), (130, 64), (131, 64), (146, 20), (147, 20), (514, 20), (515, 30), (1026, 20), (1500, 24)])
 def test_every_number_of_columns(n_chunks, k):
     check(routed(ragged(2, 64, n_chunks, 3, k, captions=(0, n_chunks // 2))))
