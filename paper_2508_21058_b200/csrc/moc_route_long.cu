@@ -6,7 +6,7 @@
 // row's threads only count: of the scores in tensor memory those that reach a threshold, until a few more than k do, two or three times; those
 // alone are kept, and sorted by a whole warp.  (2 heads, a thread per row -> this, us: 264k tokens, 1008 columns: 20 picks 971 -> 755, 30 1122 ->
 // 805, 60 3063 -> 1300, 118 6706 -> 1800; 504 columns: 20 680 -> 493, 32 802 -> 592, 64 2173 -> 998; 40k tokens, 200 columns, 20 picks 96 -> 82.)
-// What bounds it now (118 picks, per tile of 130,000 cycles): the sorts 41,000, counting 31,000, the list entries, four bytes here and there, 25,000.
+// What bounds it now (118 picks, per tile of 122,000 cycles): the sorts 44,500, the list entries, four bytes here and there, 26,600, counting 17,900.
 // Scores through a scratch in L2, so that a warp could hold a row, took 1.4 times as long: 64 KB a step each way.
 //
 // Persistent, one CTA per SM; the 128-query tiles ("units") are dealt round-robin, all heads' first tiles first (so that a query list is
