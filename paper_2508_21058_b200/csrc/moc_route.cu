@@ -59,12 +59,19 @@ struct TopK {
     }
 };
 
+// A score, or -inf if it is not a number (written out, whatever the compiler may assume of its operands)
+__device__ __forceinline__ float number_or_none(float f) {
+    asm("max.f32 %0, %0, 0fff800000;" : "+f"(f));
+    return f;
+}
+
 // ---- the first columns of a list of 17 to 32 picks: candidates as 64-bit keys, high word the score as an integer of
 // the same order (-0 and +0 alike, and a NaN, which is never picked, as -inf), low word the complement of the column, so that one
 // integer compare orders them as the result is ordered (score descending, then column ascending).
 constexpr uint32_t kNoScore = 0x007fffffu;      // high word of a score of -inf: nothing there
 __device__ __forceinline__ uint64_t score_key(float f, int col) {
-    asm("max.f32 %0, %0, 0fff800000;\n\tadd.rn.f32 %0, %0, 0f00000000;" : "+f"(f));
+    f = number_or_none(f);
+    asm("add.rn.f32 %0, %0, 0f00000000;" : "+f"(f));
     const int b = __float_as_int(f);
     return (uint64_t)((uint32_t)b ^ ((uint32_t)(b >> 31) | 0x80000000u)) << 32 | (uint32_t)~col;
 }
@@ -551,7 +558,9 @@ __global__ void __launch_bounds__(rt_threads(NG), 1) route_tc_kernel(const __gri
                             }
 #pragma unroll
                             for (int c = 0; c < 8; ++c) {
-                                insert(((cand >> (g * 8 + c)) & 1u) ? f[c] : -INFINITY, g * 8 + c);     // -inf changes nothing
+                                // -inf changes nothing, and a score that is not a number becomes that: once in the list, where no
+                                // entry is at least as large as it, it would let columns in that are not candidates, or no columns at all
+                                insert(((cand >> (g * 8 + c)) & 1u) ? number_or_none(f[c]) : -INFINITY, g * 8 + c);
                             }
                         }
                     }

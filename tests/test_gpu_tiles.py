@@ -1,5 +1,6 @@
 """The attention and routing kernels at the edges of their tiles, lists and variants, against the CPU oracle, with the
 tolerances of the other parity tests; and a workspace used again gives the same bits."""
+import numpy as np
 import pytest
 import torch
 
@@ -107,3 +108,37 @@ def test_a_nan_score_is_never_picked(k):
         want[i, :len(picks)] = picks
     assert torch.equal(run.sel[1], want)
     assert bool((run.sel[0, row] == -1).all())
+
+
+@pytest.mark.parametrize("frames,causal", [(1, True), (7, True), (15, False), (16, True), (17, True), (31, False), (32, True)])
+@pytest.mark.parametrize("k", [1, 4, 8])
+def test_scores_that_are_not_numbers_among_few_chunks(frames, causal, k):
+    """Up to 32 score columns and 8 picks, where the three terms of a score are added up by the selection: queries and keys with a NaN or an
+    infinity, or whose scores overflow.  No score that is not a number is picked, and no chunk that is not a candidate."""
+    lay = W.make_layout(1, 5, frames, 9)
+    for spoil in ("nan query", "nan key", "inf key", "overflow"):
+        run = PU.GpuRun(W.Workload("few", 2, 64, lay, k, 0, 0, causal=causal))
+        p, q, key = run.plan, run.x["q"], run.x["k"]
+        run.forward()
+        clean = run.sel.clone()
+        if spoil == "nan query":
+            q[:, ::3, 7] = float("nan")
+        elif spoil == "nan key":
+            key[:, 5 + 9 * (frames // 2), 3] = float("nan")
+        elif spoil == "inf key":
+            key[:, 5 + 9 * (frames // 2), 3] = float("inf")
+        else:
+            q.mul_(2.0 ** 70)
+            key.mul_(2.0 ** 70)
+        p.moc_chunk_pool(key, run.desc, run.ws)
+        p.moc_route(q, run.desc, run.sel, run.ws)
+        run.check_status()
+        sel = run.sel.cpu().numpy()
+        own = lay.token_chunk()[None, :, None]
+        assert np.all((sel >= -1) & (sel < lay.n_chunks) & (sel != 0) & (sel != own) & ((sel < own) if causal else True)), spoil
+        ordered = np.sort(np.where(sel < 0, 10 ** 6 + np.arange(k), sel), axis=2)
+        assert np.all(ordered[..., 1:] > ordered[..., :-1]), spoil                        # none twice
+        if spoil == "nan query":
+            assert np.all(sel[:, ::3] == -1) and torch.equal(run.sel[:, 1::3], clean[:, 1::3])
+        elif spoil in ("nan key", "inf key"):
+            assert not np.any(sel == 1 + frames // 2)         # (an infinite key's terms add up to no number)
